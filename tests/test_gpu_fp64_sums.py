@@ -1,0 +1,69 @@
+"""The FP64 direct sum at the edges of its work split (sinks per block, slices of the sources) against
+plain FP64 sums."""
+import numpy as np
+import pytest
+
+from paper_1405_2255_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+# a sum of up to 6000 FP64 terms in any order, each term good to a few ulp: (6000 + 10) 2^-53 of the
+# sum of the terms' magnitudes is 7e-13
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def g():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1405_2255_gb300 import build
+    build.build()
+    from paper_1405_2255_gb300 import gb3fmm
+    gb3fmm.load()
+    return gb3fmm
+
+
+def _dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+
+
+def _sums(x, mu, sinks):
+    """psi, acc, f and the sums of the magnitudes of acc's terms, by numpy."""
+    psi, acc, f = np.zeros(len(sinks)), np.zeros((len(sinks), 3)), np.zeros(len(sinks))
+    for b in range(0, len(sinks), 500):
+        d = x[None] - x[sinks[b:b + 500], None]
+        r2 = (d * d).sum(2)
+        ri = np.where(r2 > 0, 1.0 / np.sqrt(np.where(r2 > 0, r2, 1.0)), 0.0)
+        psi[b:b + 500] = (mu * ri).sum(1)
+        f[b:b + 500] = (mu * ri * ri).sum(1)
+        acc[b:b + 500] = ((mu * ri ** 3)[:, :, None] * d).sum(1)
+    return psi, acc, f
+
+
+def _check(psi, acc, ref):
+    p, a, f = ref
+    scale = np.maximum(f, 1e-300)  # sum of |terms| of each component of acc is at most f
+    assert np.max(np.abs(psi - p) / np.maximum(p, 1e-300)) < TOL
+    assert np.max(np.abs(acc - a) / scale[:, None]) < TOL
+
+
+@pytest.mark.parametrize("n,ns", [(1, 1), (31, 1), (257, 3), (1000, 33), (999, 250), (2049, 1217), (300, 9728),
+                                  (257, 38912), (130, 40001)])
+@pytest.mark.parametrize("want_f", [False, True])
+def test_direct_splits(g, n, ns, want_f):
+    x, mu = inputs.plummer(n, 900 + n)
+    if n > 300:
+        mu[::7] = 0.0
+        x[11] = x[12]  # a coincident pair
+    sinks = (np.arange(ns) * 7919) % n
+    ctx = g.Context()
+    out = ctx.fmm_direct(_dev(x), _dev(mu), 1.0, sinks=_dev(sinks.astype(np.int64)), want_f=want_f)
+    ref = _sums(x, mu, np.arange(n))
+    ref = tuple(v[sinks] for v in ref)
+    _check(out[0].cpu().numpy(), out[1].cpu().numpy(), ref)
+    if want_f:
+        assert np.max(np.abs(out[2].cpu().numpy() - ref[2]) / np.maximum(ref[2], 1e-300)) < TOL
+    ctx.close()
+
