@@ -441,6 +441,35 @@ static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t 
     return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
 }
 
+// FP64 P2P (want_f: the near sums of f into psi_near) with a work plan; without room for the plan's
+// scratch, or beyond its index ranges, the form that needs none.  *planned: which one ran
+static int run_p2p_fp64(fmm_ctx* ctx, const int2* list, bool want_f, bool* planned, cudaStream_t s) {
+    Cells c = cells_of(ctx);
+    *planned = false;
+    size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (ensure(ctx->p2p_tmp, need)) return 0;
+        need = launch_p2p_f64_plan(P<d4>(ctx->xm), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
+                                   P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near),
+                                   P<double>(ctx->acc_near), want_f, ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
+                                   ctx->h_counters + 8, s);
+        if (need == ~(size_t)0) return 0;
+        if (need <= ctx->p2p_tmp.bytes) {
+            *planned = true;
+            return 0;
+        }
+    }
+    return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
+}
+static int p2p_fp64(fmm_ctx* ctx, const int2* list, cudaStream_t s) {
+    bool planned;
+    TRY(run_p2p_fp64(ctx, list, false, &planned, s));
+    if (!planned)
+        launch_p2p_fp64(P<d4>(ctx->xm), cells_of(ctx), list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
+                        P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), s);
+    return 0;
+}
+
 // ------------------------------------------------------------------ the low-order scale (A7)
 static int estimate_scale(fmm_ctx* ctx, cudaStream_t s) {
     const int nc = ctx->ncells;
@@ -488,16 +517,20 @@ static int estimate_scale(fmm_ctx* ctx, cudaStream_t s) {
         launch_f_m2l(P<int2>(ctx->est_m2l), P<int>(ctx->m2l_seg_start), P<int>(ctx->m2l_seg_end), nc, c,
                      P<double>(ctx->Ff), s);
         for (int L = 1; L < nlev; ++L) launch_f_down_level(c, ctx->lev_start[L], ctx->lev_start[L + 1], P<double>(ctx->Ff), s);
-        launch_f_p2p(P<d4>(ctx->xm), c, P<int2>(ctx->est_p2p), P<int>(ctx->seg_start), P<int>(ctx->seg_end),
-                     P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->Ff), scale, s);
+        bool planned;
+        TRY(run_p2p_fp64(ctx, P<int2>(ctx->est_p2p), true, &planned, s));
+        if (planned)
+            launch_f_add(c, P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->Ff), P<double>(ctx->psi_near), scale, s);
+        else
+            launch_f_p2p(P<d4>(ctx->xm), c, P<int2>(ctx->est_p2p), P<int>(ctx->seg_start), P<int>(ctx->seg_end),
+                         P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->Ff), scale, s);
         return 0;
     }
     // (the p = 1 L2L is folded into launch_est_scale)
     if (mixed)
         TRY(run_p2p_mixed(ctx, P<int2>(ctx->est_p2p), 0, s));
     else
-        launch_p2p_fp64(P<d4>(ctx->xm), c, P<int2>(ctx->est_p2p), P<int>(ctx->seg_start), P<int>(ctx->seg_end),
-                        P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), s);
+        TRY(p2p_fp64(ctx, P<int2>(ctx->est_p2p), s));
     CU(cudaStreamWaitEvent(s, ctx->ev_est_m2l, 0));
     launch_est_scale(c, P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->F1), P<double>(ctx->acc_near), scale, s);
     return 0;
@@ -755,8 +788,7 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
         kernel_marks(nullptr);
         TRY(rc);
     } else
-        launch_p2p_fp64(P<d4>(ctx->xm), c, P<int2>(ctx->p2p), P<int>(ctx->seg_start), P<int>(ctx->seg_end),
-                        P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), s);
+        TRY(p2p_fp64(ctx, P<int2>(ctx->p2p), s));
     launch_coincident(P<d4>(ctx->xm), P<uint64_t>(ctx->keys), n, P<unsigned long long>(ctx->coin), s,
                       ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
     if (tidal) {  // Sec. 7.4: the near part over the same sources as the P2P

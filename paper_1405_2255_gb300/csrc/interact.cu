@@ -751,6 +751,7 @@ void launch_l2p(const d4* xm, Cells c, const d4* cen, const int* leaves, int nle
 }
 
 // ---------------------------------------------------------------- P2P, FP64
+// The form without a work plan (p2p.cu has the planned one): for callers without the scratch it needs.
 // One warp per chunk of up to 32 sinks of a leaf (lane = sink).  The sources are
 // the P2P segments of the leaf and of all its ancestors (a pair (A, B) with B
 // internal covers every leaf below B); they pass through a warp-private tile of
@@ -1086,6 +1087,23 @@ void launch_f_p2p(const d4* xm, Cells c, const int2* list, const int* seg_start,
                   const int* leaves, int nleaves, const double* Ff, double* f_sorted, cudaStream_t s) {
     if (nleaves <= 0) return;
     k_f_p2p<<<p2p_grid(nleaves), kP2PWarps * 32, 0, s>>>(xm, c, list, seg_start, seg_end, leaves, nleaves, Ff, f_sorted);
+    note_launch();
+}
+
+__global__ void k_f_add(Cells c, const int* __restrict__ leaves, int nleaves, const double* __restrict__ Ff,
+                        const double* __restrict__ fn, double* __restrict__ fout) {
+    const int lane = threadIdx.x & 31, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nleaves; t += nw) {
+        const int leaf = leaves[t];
+        if (!cell_active(c, leaf)) continue;
+        const double f = Ff[leaf];
+        for (int i = c.first[leaf] + lane, e = c.first[leaf] + c.count[leaf]; i < e; i += 32) fout[i] = f + fn[i];
+    }
+}
+void launch_f_add(Cells c, const int* leaves, int nleaves, const double* Ff, const double* fn, double* f_sorted,
+                  cudaStream_t s) {
+    if (nleaves <= 0) return;
+    k_f_add<<<grid_for((long long)nleaves * 32, 256, 16), 256, 0, s>>>(c, leaves, nleaves, Ff, fn, f_sorted);
     note_launch();
 }
 

@@ -219,7 +219,8 @@ void launch_l2p_split(const d4* xm, Cells c, const d4* cen, const int* leaves, i
 void launch_m2m_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M, cudaStream_t s);
 void launch_l2l_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* F, cudaStream_t s);
 // P2P (eq. 1) into psi_near/acc_near (sorted order): every leaf takes the sources of
-// its own P2P segment and those of its ancestors' segments.
+// its own P2P segment and those of its ancestors' segments.  This form needs no scratch; where
+// there is room for a work plan, launch_p2p_f64_plan is several times faster.
 void launch_p2p_fp64(const d4* xm, Cells c, const int2* list, const int* seg_start,
                      const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, cudaStream_t s);
 // Mixed P2P (p2p.cu).  mode (fmm_params.p2p_two_float): 0 dx from the FP32 high parts (the
@@ -233,6 +234,11 @@ size_t p2p_plan_fixed_bytes(int nleaves);
 size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
                         const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, int mode,
                         void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
+// FP64 P2P with a work plan as launch_p2p_mixed's (the same scratch, return value and host read);
+// want_f: psi receives sum mu / r^2 instead (eq. 6; acc is scratch)
+size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,
+                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, void* tmp,
+                           size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
 // ordered pairs of distinct particles at distance 0 (sorted keys and positions); with
 // an ensemble (off != nullptr) only pairs inside one system count
 void launch_coincident(const d4* xm, const uint64_t* keys, int n, unsigned long long* coincident, cudaStream_t s,
@@ -246,6 +252,9 @@ void launch_f_m2l(const int2* list, const int* seg_start, const int* seg_end, in
 void launch_f_down_level(Cells c, int lev_begin, int lev_end, double* Ff, cudaStream_t s);
 void launch_f_p2p(const d4* xm, Cells c, const int2* list, const int* seg_start, const int* seg_end,
                   const int* leaves, int nleaves, const double* Ff, double* f_sorted, cudaStream_t s);
+// the last step with a planned P2P: f = Ff of the leaf + the near sums fn
+void launch_f_add(Cells c, const int* leaves, int nleaves, const double* Ff, const double* fn, double* f_sorted,
+                  cudaStream_t s);
 // p = 1 M2L of the acceleration estimate from the monopoles about the centres of mass
 // (the dipole vanishes there) into F1[nc][4]
 void launch_est_m2l(const int2* list, const int* seg_start, const int* seg_end, int ncells, Cells c, double* F1,

@@ -169,27 +169,64 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// (k items, R replicas, S slots) for a leaf of c sinks, two sinks per slot: the least cost
-// k (2 / R + 0.6) per source over k >= ceil(c / 64) (the lanes' pair work and the staging of
-// the sources, in units of a lane's pair), then k = ceil(c / (2 S)) so that no item is empty
-__host__ __device__ inline void p2p_chunking(int c, int& k, int& R, int& S) {
-    k = R = S = 1;
-    if (c <= 0) return;
-    const int kmin = (c + 63) / 64;
-    float best = 3.0e38f;
-    for (int kk = kmin; kk < kmin + 12; ++kk) {
-        const int SS = (c + 2 * kk - 1) / (2 * kk);
-        const int RR = 32 / SS < kP2PRmax ? 32 / SS : kP2PRmax;
-        const float cost = (float)kk * (2.0f / (float)RR + 0.6f);
-        if (cost < best) {
-            best = cost;
-            k = kk;
-            R = RR;
-            S = SS;
+// How a leaf of c sinks is cut into work items: k items of at most Q S sinks, each replicated R
+// times across a warp (lane = replica * S + slot; slot s of an item holds its sinks s, S + s, ...,
+// (Q - 1) S + s).  A source costs an item Q / R steps of the warp.
+struct Chunk {
+    int k, R, S, Q;
+};
+// The mixed P2P: two sinks per slot; the least cost k (2 / R + 0.6) per source over
+// k >= ceil(c / 64) (the lanes' pair work and the staging of the sources, in units of a lane's
+// pair), then k = ceil(c / (2 S)) so that no item is empty.  Items longer than piece_steps steps
+// are split (see below).
+struct PlanMixed {
+    static constexpr unsigned piece_steps = 8192;
+    static constexpr int max_pieces = 64;
+    __device__ static inline Chunk chunk(int c) {
+        Chunk r{1, 1, 1, 2};
+        if (c <= 0) return r;
+        const int kmin = (c + 63) / 64;
+        float best = 3.0e38f;
+        for (int kk = kmin; kk < kmin + 12; ++kk) {
+            const int SS = (c + 2 * kk - 1) / (2 * kk);
+            const int RR = 32 / SS < kP2PRmax ? 32 / SS : kP2PRmax;
+            const float cost = (float)kk * (2.0f / (float)RR + 0.6f);
+            if (cost < best) {
+                best = cost;
+                r.k = kk;
+                r.R = RR;
+                r.S = SS;
+            }
         }
+        r.k = (c + 2 * r.S - 1) / (2 * r.S);
+        return r;
     }
-    k = (c + 2 * S - 1) / (2 * S);
-}
+};
+// The FP64 P2P is bound by the FP64 pipe alone (an instruction costs the same however many lanes
+// are active, staging runs beside it): the fewest steps k Q / R per source over S <= 32 slots and
+// Q <= 4 sinks per slot.  Short pieces (a step of 18 FP64 instructions holds a quarter of an SM for
+// 1152 cycles, so 256 steps are 0.14 ms) keep every SM busy to the end.
+struct PlanF64 {
+    static constexpr unsigned piece_steps = 256;
+    static constexpr int max_pieces = 1024;
+    __device__ static inline Chunk chunk(int c) {
+        Chunk r{1, 1, 1, 1};
+        if (c <= 0) return r;
+        float best = 3.0e38f;
+        for (int S = min(c, 32); S >= 1; --S) {
+            const int R = min(32 / S, 16);
+            for (int Q = 1; Q <= 4; ++Q) {
+                const int k = (c + Q * S - 1) / (Q * S);
+                const float cost = (float)(k * Q) / (float)R + 0.02f * (float)k;
+                if (cost < best) {
+                    best = cost;
+                    r = Chunk{k, R, S, Q};
+                }
+            }
+        }
+        return r;
+    }
+};
 
 // class of source cell A for sink leaf B (see the file comment); mode 1 only
 __device__ inline bool p2p_near(const d4& a, const d4& b) {
@@ -198,20 +235,21 @@ __device__ inline bool p2p_near(const d4& a, const d4& b) {
     return dx * dx + dy * dy + dz * dz < lim * lim;
 }
 
-// Long items are split: a leaf whose item would take a lane more than kP2PPieceSteps pair steps
-// (2 sources / R) has its stream of source cells cut into P = ceil(steps / kP2PPieceSteps) <=
-// kP2PMaxPieces pieces of about equal numbers of source cells, each with its own ranges, items
+// Long items are split: a leaf whose item would take a lane more than piece_steps steps
+// (Q sources / R) has its stream of source cells cut into P = ceil(steps / piece_steps) <=
+// max_pieces pieces of about equal numbers of source cells, each with its own ranges, items
 // and FP64 partial sums, which k_p2p_reduce adds in piece order.  The split depends on the leaf
 // alone, so a system gives the same result in an ensemble as alone.
-constexpr int kP2PMaxPieces = 64;
-constexpr unsigned kP2PPieceSteps = 8192;
 
 // per leaf index t (one warp each): the number of its source cells nb[t] (the ranges it can need
-// at most: its own and its ancestors' segment lengths) and the length of its items (a lane's
-// pair steps, 2 source particles / R; 0 for a leaf without active particles); tot[0] += nb
+// at most: its own and its ancestors' segment lengths), its pieces np[t] and its sort key,
+// descending in the length of a piece's items (a lane's steps, Q source particles / R; 0 for a leaf
+// without active particles); tot[0] += nb
+template <class PL>
 __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                             const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves,
-                            int* __restrict__ nb, unsigned* __restrict__ len, unsigned long long* __restrict__ tot) {
+                            int* __restrict__ nb, int* __restrict__ np, uint64_t* __restrict__ keys,
+                            unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long my = 0;
@@ -228,60 +266,81 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
         if (lane == 0) {
             nb[t] = (int)e;
             my += (unsigned long long)e;
-            int k, R, S;
-            p2p_chunking(c.count[leaf], k, R, S);
-            const unsigned long long l = 2ull * (unsigned long long)src / (unsigned long long)R + 1;
-            const unsigned w32 = !cell_active(c, leaf) ? 0u : (l > 0xfffffffeull ? 0xfffffffeu : (unsigned)l);
-            len[t] = w32;
+            const Chunk ch = PL::chunk(c.count[leaf]);
+            const unsigned long long l = (unsigned long long)ch.Q * (unsigned long long)src / (unsigned long long)ch.R + 1;
+            const unsigned len = !cell_active(c, leaf) ? 0u : (l > 0xfffffffeull ? 0xfffffffeu : (unsigned)l);
+            int P = (int)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
+            const int cap = e < PL::max_pieces ? (int)e : PL::max_pieces;
+            P = P < 1 ? 1 : (P > cap ? (cap > 0 ? cap : 1) : P);
+            np[t] = P;
+            const unsigned w32 = len ? (unsigned)(((unsigned long long)len + P - 1) / P) : 0u;
+            keys[t] = ((uint64_t)(255u - qlen8(w32)) << 32) | (unsigned)t;
         }
     }
     if (lane == 0 && my) atomicAdd(&tot[0], my);
 }
 
-// per leaf index t: its pieces np[t] and its sort key, descending in the length of a piece's items
-__global__ void k_p2p_pieces(const unsigned* __restrict__ len, const int* __restrict__ nb, int nleaves,
-                             int* __restrict__ np, uint64_t* __restrict__ keys) {
-    const unsigned long long lmax = kP2PPieceSteps;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nleaves; t += gridDim.x * blockDim.x) {
-        const unsigned l = len[t];
-        int P = (int)(((unsigned long long)l + lmax - 1) / lmax);
-        const int cap = nb[t] < kP2PMaxPieces ? nb[t] : kP2PMaxPieces;
-        P = P < 1 ? 1 : (P > cap ? (cap > 0 ? cap : 1) : P);
-        np[t] = P;
-        const unsigned w32 = l ? (unsigned)(((unsigned long long)l + P - 1) / P) : 0u;
-        keys[t] = ((uint64_t)(255u - qlen8(w32)) << 32) | (unsigned)t;
+// the warp's sum of v, and *before = the sum over the lanes below
+__device__ inline unsigned long long warp_total(unsigned long long v, unsigned long long* before) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
     }
+    *before = x - v;
+    return __shfl_sync(0xffffffffu, x, 31);
 }
 
-// per position q of the sorted order: items nit[q] (pieces x items per piece; 0 for a leaf
-// without active particles) and pieces npc[q]; tot[1] += items, tot[3] += pieces, tot[4] += the
-// partial sums of split leaves (pieces x sinks), tot[5] += split leaves
+// per position q of the sorted order: its leaf index order[q], items nit[q] (pieces x items per
+// piece; 0 for a leaf without active particles) and pieces npc[q]; a split leaf (more than one
+// piece) takes the first of its partial-sum slots pbase[q] (pieces x sinks of them; -1: not split)
+// and an entry (leaf index, first slot) of the split list.  tot[1] items, tot[3] pieces, tot[4]
+// slots, tot[5] split leaves; one atomic per warp and counter (a thread each took 60 us for 43,000
+// leaves).
+template <class PL>
 __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __restrict__ leaves, int nleaves, Cells c,
                              const int* __restrict__ np, int* __restrict__ order, int* __restrict__ nit,
-                             int* __restrict__ npc, unsigned long long* __restrict__ tot) {
-    unsigned long long my = 0, mp = 0, mpart = 0, msplit = 0;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nleaves; q += gridDim.x * blockDim.x) {
-        const int t = (int)(keys[q] & 0xffffffffu);
-        order[q] = t;
-        const int leaf = leaves[t];
-        int k = 0, R, S, P = 0;
-        if (cell_active(c, leaf)) {
-            p2p_chunking(c.count[leaf], k, R, S);
-            P = np[t];
+                             int* __restrict__ npc, int* __restrict__ pbase, int2* __restrict__ split,
+                             unsigned long long* __restrict__ tot) {
+    const int lane = threadIdx.x & 31;
+    for (int q0 = blockIdx.x * blockDim.x; q0 < nleaves; q0 += gridDim.x * blockDim.x) {
+        const int q = q0 + threadIdx.x;
+        int t = 0, k = 0, P = 0, count = 0;
+        if (q < nleaves) {
+            t = (int)(keys[q] & 0xffffffffu);
+            order[q] = t;
+            const int leaf = leaves[t];
+            count = c.count[leaf];
+            if (cell_active(c, leaf)) {
+                k = PL::chunk(count).k;
+                P = np[t];
+            }
+            nit[q] = k * P;
+            npc[q] = P;
         }
-        nit[q] = k * P;
-        npc[q] = P;
-        my += (unsigned long long)(k * P);
-        mp += (unsigned long long)P;
-        if (P > 1) {
-            mpart += (unsigned long long)P * (unsigned long long)c.count[leaf];
-            ++msplit;
+        const bool sp = P > 1;
+        const unsigned long long slots = sp ? (unsigned long long)P * (unsigned long long)count : 0ull;
+        unsigned long long ex, sbefore, lbefore;
+        const unsigned long long ti = warp_total((unsigned long long)k * P, &ex), tp = warp_total(P, &ex);
+        const unsigned long long ts = warp_total(slots, &sbefore), tl = warp_total(sp ? 1 : 0, &lbefore);
+        unsigned long long sb = 0, lb = 0;
+        if (lane == 0) {
+            if (ti) atomicAdd(&tot[1], ti);
+            if (tp) atomicAdd(&tot[3], tp);
+            if (tl) {
+                sb = atomicAdd(&tot[4], ts);
+                lb = atomicAdd(&tot[5], tl);
+            }
+        }
+        sb = __shfl_sync(0xffffffffu, sb, 0) + sbefore;
+        lb = __shfl_sync(0xffffffffu, lb, 0) + lbefore;
+        if (q < nleaves) {
+            pbase[q] = sp ? (int)sb : -1;
+            if (sp) split[lb] = make_int2(t, (int)sb);
         }
     }
-    if (my) atomicAdd(&tot[1], my);
-    if (mp) atomicAdd(&tot[3], mp);
-    if (mpart) atomicAdd(&tot[4], mpart);
-    if (msplit) atomicAdd(&tot[5], msplit);
 }
 
 // per piece v: its leaf index, its region of ranges [r0, r1) (near ranges from the front, far
@@ -291,132 +350,140 @@ struct Pieces {
     int *leaf, *r0, *r1, *nnear, *nfar, *part;
 };
 
-// ranges of the pieces of leaf index t (sorted position q); items (piece, chunk).  One warp per
-// position.  Piece j takes the source cells j e / P .. (j + 1) e / P - 1 of the leaf's stream
-// (its own segment, then each ancestor's; e cells in all) and owns that part of the leaf's region
-// [roff[t], roff[t] + e).  Within a piece the sources are merged per class in stream order: an
+// ranges and items of piece v, one warp per piece (the pieces of a long leaf side by side: with one
+// warp per leaf the longest leaf set the kernel's time).  Piece j of a leaf (sorted position q, the
+// last with voff[q] <= v; j = v - voff[q]) takes the source cells j e / P .. (j + 1) e / P - 1 of
+// the leaf's stream (its own segment, then each ancestor's; e cells in all) and owns that part of
+// the leaf's region [roff[t], roff[t] + e).  Within a piece the sources are merged per class in
+// stream order: an
 // entry joins the open range of its class when its particles follow that range's directly.  The
 // lanes take up to 32 entries at a time; each finds its class predecessor (the closest lower
 // lane of its class, else the open range carried from the earlier entries), the entries that do
 // not join start a run, a run's count and guard flag are summed in shared memory, and every run
 // but the last of its class is written out; the last stays open until the piece ends.  This is
-// the result of the sequential pass.  A split leaf takes its partial-sum slots (P x sinks) and
-// an entry of the split list (t, first slot) from the counters tot[6], tot[7].
+// the result of the sequential pass.
 constexpr int kEmitWarps = 4;
 __global__ void __launch_bounds__(kEmitWarps * 32)
     k_p2p_emit(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int mode,
                const int* __restrict__ order, const int* __restrict__ roff, const int* __restrict__ nb,
                const int* __restrict__ ioff, const int* __restrict__ nit, const int* __restrict__ voff,
-               const int* __restrict__ npc, Pieces pc, int2* __restrict__ ranges, int2* __restrict__ items,
-               int2* __restrict__ split, unsigned long long* __restrict__ tot) {
+               const int* __restrict__ npc, const int* __restrict__ pbase, int npieces, Pieces pc,
+               int2* __restrict__ ranges, int2* __restrict__ items) {
     __shared__ int rsum_all[kEmitWarps][33], rg_all[kEmitWarps][33];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int* rsum = rsum_all[wid];  // [0]: the open range carried in; [1 + L]: the run starting at lane L
     int* rg = rg_all[wid];
     const unsigned below = (1u << lane) - 1u, upto = below | (1u << lane);
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < nleaves; q += nw) {
-        const int P = npc[q];
-        if (P == 0) continue;  // no active particle: no items, no ranges
-        const int t = order[q];
+    for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < npieces; v += nw) {
+        int q = 0;
+        for (int hi = nleaves - 1; q < hi;) {
+            const int mid = (q + hi + 1) >> 1;
+            if (voff[mid] <= v) q = mid;
+            else hi = mid - 1;
+        }
+        const int P = npc[q], pj = v - voff[q], t = order[q];
         const int kper = nit[q] / P;  // items per piece
         const int leaf = leaves[t];
         const int count = c.count[leaf];
-        int pbase = -1;
-        if (P > 1 && lane == 0) {
-            pbase = (int)atomicAdd(&tot[6], (unsigned long long)P * (unsigned long long)count);
-            const int si = (int)atomicAdd(&tot[7], 1ull);
-            split[si] = make_int2(t, pbase);
-        }
-        pbase = __shfl_sync(0xffffffffu, pbase, 0);
-        for (int j = lane; j < nit[q]; j += 32) items[ioff[q] + j] = make_int2(voff[q] + j / kper, j % kper);
+        for (int j = lane; j < kper; j += 32) items[ioff[q] + pj * kper + j] = make_int2(v, j);
         const d4 sb = c.sr[leaf];
         const long long b0 = c.first[leaf], b1 = b0 + count;
         const long long e = nb[t];
+        const long long f0 = e * pj / P, f1 = e * (pj + 1) / P;
+        const int r0 = roff[t] + (int)f0, r1 = roff[t] + (int)f1;
         // the cursor over the leaf's stream of source cells: cell, its list segment, position
         int cell = leaf, s1 = seg_end[leaf], at = seg_start[leaf];
-        for (int pj = 0; pj < P; ++pj) {
-            const int v = voff[q] + pj;
-            const long long f0 = e * pj / P, f1 = e * (pj + 1) / P;
-            const int r0 = roff[t] + (int)f0, r1 = roff[t] + (int)f1;
-            int cf[2] = {0, 0}, cn[2] = {0, 0}, cnt[2] = {0, 0};  // open range and records written per class
-            bool cg[2] = {false, false};
-            auto put = [&](int k, int idx, int f, int n, bool g) {
-                ranges[k ? r0 + idx : r1 - 1 - idx] =
-                    make_int2(f, n | (k << 30) | ((g ? 1 : 0) << kRangeCountBits));
-            };
-            for (long long fi = f0; fi < f1;) {
-                while (at >= s1) {  // on to the next ancestor's segment
-                    cell = c.parent[cell];
-                    at = seg_start[cell];
-                    s1 = seg_end[cell];
-                }
-                const int m = (int)min((long long)min(32, s1 - at), f1 - fi);
-                int f = 0, n = 0, kk = -1;
-                if (lane < m) {
-                    const int A = list[at + lane].x;
-                    f = c.first[A];
-                    n = c.count[A];
-                    kk = mode == 1 ? (p2p_near(c.sr[A], sb) ? 1 : 0) : (mode == 3 ? 1 : 0);
-                    if (n <= 0) kk = -1;
-                }
-                at += m;
-                fi += m;
-                const bool g = kk >= 0 && f < b1 && b0 < (long long)f + n;
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const unsigned M = __ballot_sync(0xffffffffu, kk == k);
-                    if (!M) continue;
-                    const unsigned pm = M & below;
-                    const int pl = pm ? 31 - __clz(pm) : lane;
-                    const int pf = __shfl_sync(0xffffffffu, f, pl), pn = __shfl_sync(0xffffffffu, n, pl);
-                    const long long pe = pm ? (long long)pf + pn : (cn[k] > 0 ? (long long)cf[k] + cn[k] : -1);
-                    const bool mine = kk == k;
-                    const unsigned S = __ballot_sync(0xffffffffu, mine && pe != f);
-                    const unsigned sm = S & upto;
-                    const int rs = sm ? 31 - __clz(sm) : -1;  // the run this lane belongs to
-                    rsum[lane] = 0;
-                    rg[lane] = 0;
-                    if (lane == 0) rsum[32] = rg[32] = 0;
-                    __syncwarp();
-                    if (mine) {
-                        atomicAdd(&rsum[rs + 1], n);
-                        if (g) atomicOr(&rg[rs + 1], 1);
-                    }
-                    __syncwarp();
-                    if (!S) {  // every entry joins the open range
-                        cn[k] += rsum[0];
-                        cg[k] = cg[k] || rg[0];
-                    } else {
-                        int base = cnt[k];
-                        if (cn[k] > 0) {  // the open range closes at the first start
-                            if (lane == 0) put(k, base, cf[k], cn[k] + rsum[0], cg[k] || rg[0]);
-                            ++base;
-                        }
-                        const int last = 31 - __clz(S);
-                        if (((S >> lane) & 1) && lane != last)
-                            put(k, base + __popc(S & below), f, rsum[lane + 1], rg[lane + 1] != 0);
-                        cnt[k] = base + __popc(S) - 1;
-                        cf[k] = __shfl_sync(0xffffffffu, f, last);
-                        cn[k] = rsum[last + 1];
-                        cg[k] = rg[last + 1] != 0;
-                    }
-                    __syncwarp();
-                }
+        for (long long skip = f0; skip > 0;) {
+            const long long len = s1 - at;
+            if (len > skip) {
+                at += (int)skip;
+                break;
             }
-            if (lane == 0) {
-                for (int k = 1; k >= 0; --k)
-                    if (cn[k] > 0) put(k, cnt[k]++, cf[k], cn[k], cg[k]);
-                pc.leaf[v] = t;
-                pc.r0[v] = r0;
-                pc.r1[v] = r1;
-                pc.nnear[v] = cnt[1];
-                pc.nfar[v] = cnt[0];
-                pc.part[v] = P > 1 ? pbase + pj * count : -1;
+            skip -= len;
+            at = s1;
+            if (skip > 0) {
+                cell = c.parent[cell];
+                at = seg_start[cell];
+                s1 = seg_end[cell];
             }
-            __syncwarp();
         }
+        int cf[2] = {0, 0}, cn[2] = {0, 0}, cnt[2] = {0, 0};  // open range and records written per class
+        bool cg[2] = {false, false};
+        auto put = [&](int k, int idx, int f, int n, bool g) {
+            ranges[k ? r0 + idx : r1 - 1 - idx] = make_int2(f, n | (k << 30) | ((g ? 1 : 0) << kRangeCountBits));
+        };
+        for (long long fi = f0; fi < f1;) {
+            while (at >= s1) {  // on to the next ancestor's segment
+                cell = c.parent[cell];
+                at = seg_start[cell];
+                s1 = seg_end[cell];
+            }
+            const int m = (int)min((long long)min(32, s1 - at), f1 - fi);
+            int f = 0, n = 0, kk = -1;
+            if (lane < m) {
+                const int A = list[at + lane].x;
+                f = c.first[A];
+                n = c.count[A];
+                kk = mode == 1 ? (p2p_near(c.sr[A], sb) ? 1 : 0) : (mode == 3 ? 1 : 0);
+                if (n <= 0) kk = -1;
+            }
+            at += m;
+            fi += m;
+            const bool g = kk >= 0 && f < b1 && b0 < (long long)f + n;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const unsigned M = __ballot_sync(0xffffffffu, kk == k);
+                if (!M) continue;
+                const unsigned pm = M & below;
+                const int pl = pm ? 31 - __clz(pm) : lane;
+                const int pf = __shfl_sync(0xffffffffu, f, pl), pn = __shfl_sync(0xffffffffu, n, pl);
+                const long long pe = pm ? (long long)pf + pn : (cn[k] > 0 ? (long long)cf[k] + cn[k] : -1);
+                const bool mine = kk == k;
+                const unsigned S = __ballot_sync(0xffffffffu, mine && pe != f);
+                const unsigned sm = S & upto;
+                const int rs = sm ? 31 - __clz(sm) : -1;  // the run this lane belongs to
+                rsum[lane] = 0;
+                rg[lane] = 0;
+                if (lane == 0) rsum[32] = rg[32] = 0;
+                __syncwarp();
+                if (mine) {
+                    atomicAdd(&rsum[rs + 1], n);
+                    if (g) atomicOr(&rg[rs + 1], 1);
+                }
+                __syncwarp();
+                if (!S) {  // every entry joins the open range
+                    cn[k] += rsum[0];
+                    cg[k] = cg[k] || rg[0];
+                } else {
+                    int base = cnt[k];
+                    if (cn[k] > 0) {  // the open range closes at the first start
+                        if (lane == 0) put(k, base, cf[k], cn[k] + rsum[0], cg[k] || rg[0]);
+                        ++base;
+                    }
+                    const int last = 31 - __clz(S);
+                    if (((S >> lane) & 1) && lane != last)
+                        put(k, base + __popc(S & below), f, rsum[lane + 1], rg[lane + 1] != 0);
+                    cnt[k] = base + __popc(S) - 1;
+                    cf[k] = __shfl_sync(0xffffffffu, f, last);
+                    cn[k] = rsum[last + 1];
+                    cg[k] = rg[last + 1] != 0;
+                }
+                __syncwarp();
+            }
+        }
+        if (lane == 0) {
+            for (int k = 1; k >= 0; --k)
+                if (cn[k] > 0) put(k, cnt[k]++, cf[k], cn[k], cg[k]);
+            pc.leaf[v] = t;
+            pc.r0[v] = r0;
+            pc.r1[v] = r1;
+            pc.nnear[v] = cnt[1];
+            pc.nfar[v] = cnt[0];
+            pc.part[v] = P > 1 ? pbase[q] + pj * count : -1;
+        }
+        __syncwarp();
     }
 }
 
@@ -544,8 +611,8 @@ __global__ void __launch_bounds__(kP2PWarpsM * 32, 4)
         const int2 it = items[w];
         const int v = it.x, t = pc.leaf[v], leaf = leaves[t];
         const int first = c.first[leaf], count = c.count[leaf];
-        int k, R, S;
-        p2p_chunking(count, k, R, S);
+        const Chunk ch = PlanMixed::chunk(count);
+        const int R = ch.R, S = ch.S;
         const int s0 = it.y * 2 * S, chunk = min(2 * S, count - s0);
         // lanes past S * R repeat replica 0's work; their sums are not used.  The lane's sinks
         // are s0 + slot and s0 + S + slot; a missing one repeats the item's first sink
@@ -695,14 +762,137 @@ __global__ void __launch_bounds__(kP2PWarpsM * 32, 4)
     }
 }
 
+// FP64: one warp per item, sinks and replicas as the plan lays them out (PlanF64), the item's ranges
+// as tiles of up to 64 FP64 records in shared memory.  WANT_F: only sum mu / r^2 (the estimate of
+// f, eq. 6), in place of psi.
+constexpr int kP2PWarpsD = 4;
+constexpr int kP2PTileD = 64;
+
+// r2 > 0 by its bits (r2 is no NaN: positions are finite; a comparison of doubles takes the FP64 pipe)
+__device__ __forceinline__ bool positive_bits(double r2) { return __double_as_longlong(r2) > 0; }
+
+template <int Q, bool WANT_F>
+__device__ __forceinline__ void tile_f64(const d4* __restrict__ tile, int nt, int rep, int R, const double (&b)[4][3],
+                                         double (&v)[4][4]) {
+    for (int j = rep; j < nt; j += R) {
+        const d4 a = tile[j];
+#pragma unroll
+        for (int u = 0; u < Q; ++u) {
+            const double dx = a.x - b[u][0], dy = a.y - b[u][1], dz = a.z - b[u][2];
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            if (positive_bits(r2)) {
+                const double rinv = rsqrt(r2);
+                const double r2i = rinv * rinv;
+                if (WANT_F) {
+                    v[u][0] = fma(a.w, r2i, v[u][0]);
+                } else {
+                    const double qm = a.w * rinv, q3 = qm * r2i;
+                    v[u][0] += qm;
+                    v[u][1] = fma(q3, dx, v[u][1]);
+                    v[u][2] = fma(q3, dy, v[u][2]);
+                    v[u][3] = fma(q3, dz, v[u][3]);
+                }
+            }
+        }
+    }
+}
+
+template <bool WANT_F>
+__global__ void __launch_bounds__(kP2PWarpsD * 32)
+    k_p2p_f64(const d4* __restrict__ xm, Cells c, const int* __restrict__ leaves, const int2* __restrict__ ranges,
+              const Pieces pc, const int2* __restrict__ items, int nitems, unsigned* __restrict__ counter,
+              double* __restrict__ psi, double* __restrict__ acc, double* __restrict__ part) {
+    constexpr int NV = WANT_F ? 1 : 4;
+    __shared__ __align__(32) d4 tiles[kP2PWarpsD][kP2PTileD];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    d4* tile = tiles[wid];
+    for (;;) {
+        unsigned w = 0;
+        if (lane == 0) w = atomicAdd(counter, 1u);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= (unsigned)nitems) break;
+        const int2 it = items[w];
+        const int pv = it.x, leaf = leaves[pc.leaf[pv]];
+        const int first = c.first[leaf], count = c.count[leaf];
+        const Chunk ch = PlanF64::chunk(count);
+        const int R = ch.R, S = ch.S, Q = ch.Q;
+        const int s0 = it.y * Q * S, chunk = min(Q * S, count - s0);
+        // lanes past S * R repeat replica 0's work; their sums are not used.  A missing sink repeats
+        // the item's first one
+        const int slot = lane % S, rep = lane / S < R ? lane / S : 0;
+        double b[4][3], v[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = u * S + slot;
+            const d4 xb = xm[first + s0 + (u < Q && k < chunk ? k : 0)];
+            b[u][0] = xb.x;
+            b[u][1] = xb.y;
+            b[u][2] = xb.z;
+#pragma unroll
+            for (int d = 0; d < 4; ++d) v[u][d] = 0.0;
+        }
+        RangeStream cur;
+        {
+            const int r0 = pc.r0[pv], r1 = pc.r1[pv];
+            cur.start(ranges, lane, r0, r0 + pc.nnear[pv], r1 - pc.nfar[pv], r1);
+        }
+        const int T = R * (kP2PTileD / R);  // sources per tile, shared by the replicas
+        for (;;) {
+            bool near, guard;
+            __syncwarp();  // every lane is done with the previous tile
+            const int nt = cur.fill<true>(ranges, (const float4*)xm, lane, T, (float4*)tile, near, guard);
+            if (nt == 0) break;
+            cp_async_commit();
+            cp_async_wait0();
+            __syncwarp();
+            switch (Q) {
+                case 1: tile_f64<1, WANT_F>(tile, nt, rep, R, b, v); break;
+                case 2: tile_f64<2, WANT_F>(tile, nt, rep, R, b, v); break;
+                case 3: tile_f64<3, WANT_F>(tile, nt, rep, R, b, v); break;
+                default: tile_f64<4, WANT_F>(tile, nt, rep, R, b, v); break;
+            }
+        }
+        // the replicas' sums into the lanes of replica 0, in the order of a tree
+        for (int h = 1; h < R; h *= 2) {
+            const int src = min(lane + h * S, 31);
+            const bool take = rep % (2 * h) == 0 && rep + h < R && lane < S * R;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int d = 0; d < NV; ++d) {
+                    const double o = __shfl_sync(0xffffffffu, v[u][d], src);
+                    if (take) v[u][d] += o;
+                }
+        }
+        const int pslot = pc.part[pv];
+        if (lane < S) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = u * S + slot;
+                if (u >= Q || k >= chunk) continue;
+                if (pslot >= 0) {
+                    double* o = part + 4 * ((size_t)pslot + (size_t)(s0 + k));
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) o[d] = v[u][d];
+                } else {
+                    const size_t i = (size_t)first + s0 + k;
+                    psi[i] = v[u][0];
+#pragma unroll
+                    for (int d = 1; d < NV; ++d) acc[3 * i + d - 1] = v[u][d];
+                }
+            }
+        }
+    }
+}
+
 namespace {
 // layout of the fixed part of the scratch (depends on the number of leaves only)
 struct PlanLayout {
     uint64_t *k0, *k1;
-    unsigned* len;
-    int *order, *nb, *roff, *np, *npc, *voff, *nit, *ioff, *stmp, *rtmp;
+    int *order, *nb, *roff, *np, *npc, *voff, *nit, *ioff, *pbase, *stmp, *rtmp;
+    int2* split;
     unsigned long long* tot;  // [0] ranges, [1] items, [3] pieces, [4] partial slots, [5] split
-                              // leaves, [6] [7] allocators of the emit ([2] unused)
+                              // leaves ([2] unused)
     unsigned* counter;
     size_t bytes;
 };
@@ -719,7 +909,6 @@ PlanLayout plan_layout(void* base, int nleaves) {
     };
     L.k0 = (uint64_t*)take(nl * 8);
     L.k1 = (uint64_t*)take(nl * 8);
-    L.len = (unsigned*)take(nl * 4);
     L.order = (int*)take(nl * 4);
     L.nb = (int*)take(nl * 4);
     L.roff = (int*)take((nl + 1) * 4);
@@ -728,6 +917,8 @@ PlanLayout plan_layout(void* base, int nleaves) {
     L.voff = (int*)take((nl + 1) * 4);
     L.nit = (int*)take(nl * 4);
     L.ioff = (int*)take((nl + 1) * 4);
+    L.pbase = (int*)take(nl * 4);
+    L.split = (int2*)take(nl * 8);
     L.stmp = (int*)take(scan_tmp_ints((long long)nl + 1) * 4);
     L.rtmp = (int*)take(radix_tmp_ints((long long)nl) * 4);
     L.tot = (unsigned long long*)take(8 * 8);
@@ -735,36 +926,28 @@ PlanLayout plan_layout(void* base, int nleaves) {
     L.bytes = (off + 255) & ~(size_t)255;
     return L;
 }
-}  // namespace
 
-size_t p2p_plan_fixed_bytes(int nleaves) { return plan_layout(nullptr, nleaves).bytes; }
-
-size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
-                        const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, int mode,
-                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+// the work plan of PL over the segments of list, then run(ranges, pieces, items, nitems, counter,
+// part) and the sum of the split leaves' pieces into psi and acc; the return value as
+// launch_p2p_mixed's
+template <class PL, class RUN>
+size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, const int* seg_end, const int* leaves,
+                    int nleaves, double* psi, double* acc, int mode, void* tmp, size_t tmp_bytes,
+                    unsigned long long* h_tot, cudaStream_t s, RUN run) {
     if (nleaves <= 0) return 0;
     if (n > kRangeMax) return ~(size_t)0;  // no range is ever cut: a leaf's region holds its source cells
     PlanLayout L = plan_layout(tmp, nleaves);
     if (tmp_bytes < L.bytes) return L.bytes;
-    int bps = 1;
-    auto kern_of = [&]() {
-        return mode == 1 ? k_p2p_mixed<1> : mode == 2 ? k_p2p_mixed<2> : mode == 3 ? k_p2p_mixed<3> : k_p2p_mixed<0>;
-    };
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern_of(), kP2PWarpsM * 32, 0);
-    if (bps < 1) bps = 1;
-    const int nblocks = sm_count() * bps;
     cudaMemsetAsync(L.tot, 0, 8 * sizeof(unsigned long long), s);
     cudaMemsetAsync(L.counter, 0, 4 * sizeof(unsigned), s);
-    k_p2p_count<<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(c, list, seg_start, seg_end, leaves,
-                                                                           nleaves, L.nb, L.len, L.tot);
+    k_p2p_count<PL><<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(c, list, seg_start, seg_end, leaves,
+                                                                               nleaves, L.nb, L.np, L.k0, L.tot);
     note_launch();
     scan_exclusive_i32(L.nb, L.roff, nleaves, L.roff + nleaves, L.stmp, s);
-    k_p2p_pieces<<<grid_for(nleaves, 256), 256, 0, s>>>(L.len, L.nb, nleaves, L.np, L.k0);
-    note_launch();
     // the low 32 bits are the leaf index, already in order: sort the 8 length bits only
     const int flip = radix_sort_pairs_bits(L.k0, nullptr, L.k1, nullptr, nleaves, L.rtmp, 32, 40, s);
-    k_p2p_nitems<<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.order,
-                                                         L.nit, L.npc, L.tot);
+    k_p2p_nitems<PL><<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.order,
+                                                            L.nit, L.npc, L.pbase, L.split, L.tot);
     note_launch();
     scan_exclusive_i32(L.nit, L.ioff, nleaves, L.ioff + nleaves, L.stmp, s);
     scan_exclusive_i32(L.npc, L.voff, nleaves, L.voff + nleaves, L.stmp, s);
@@ -777,8 +960,8 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
         return ~(size_t)0;
     auto a256 = [](unsigned long long b) { return (size_t)((b + 255) & ~255ull); };
     const size_t o_ranges = L.bytes, o_items = o_ranges + a256(nranges * sizeof(int2)),
-                 o_pieces = o_items + a256(nitems * sizeof(int2)), o_split = o_pieces + a256(npieces * 6 * sizeof(int)),
-                 o_part = o_split + a256(nsplit * sizeof(int2)), need = o_part + a256(nslots * 4 * sizeof(double)) + 256;
+                 o_pieces = o_items + a256(nitems * sizeof(int2)), o_part = o_pieces + a256(npieces * 6 * sizeof(int)),
+                 need = o_part + a256(nslots * 4 * sizeof(double)) + 256;
     if (tmp_bytes < need) return need;
     unsigned char* b = (unsigned char*)tmp;
     int2* ranges = (int2*)(b + o_ranges);
@@ -786,30 +969,68 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
     int* pv = (int*)(b + o_pieces);
     const size_t npv = (size_t)npieces;
     const Pieces pc{pv, pv + npv, pv + 2 * npv, pv + 3 * npv, pv + 4 * npv, pv + 5 * npv};
-    int2* split = (int2*)(b + o_split);
     double* part = (double*)(b + o_part);
-    const unsigned g = grid_for((long long)nleaves * 32, kEmitWarps * 32, 16);  // one warp per leaf
-    k_p2p_emit<<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
-                                             L.nb, L.ioff, L.nit, L.voff, L.npc, pc, ranges, items, split, L.tot);
-    note_launch();
     if (nitems == 0) return need;
-    auto go = [&](auto kern) {
-        kern<<<nblocks, kP2PWarpsM * 32, 0, s>>>(xp, c, leaves, ranges, pc, items, (int)nitems, L.counter, psi, acc,
-                                                 part);
-    };
-    mark_begin(s);
-    if (mode == 1) go(k_p2p_mixed<1>);
-    else if (mode == 2) go(k_p2p_mixed<2>);
-    else if (mode == 3) go(k_p2p_mixed<3>);
-    else go(k_p2p_mixed<0>);
-    mark_end(s);
+    const unsigned g = grid_for((long long)npieces * 32, kEmitWarps * 32, 16);  // one warp per piece
+    k_p2p_emit<<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
+                                             L.nb, L.ioff, L.nit, L.voff, L.npc, L.pbase, (int)npieces, pc, ranges,
+                                             items);
     note_launch();
+    run(ranges, pc, items, (int)nitems, L.counter, part);
     if (nsplit > 0) {
-        k_p2p_reduce<<<grid_for((long long)nsplit * 32, 128, 16), 128, 0, s>>>(c, leaves, L.np, split, (int)nsplit,
+        k_p2p_reduce<<<grid_for((long long)nsplit * 32, 128, 16), 128, 0, s>>>(c, leaves, L.np, L.split, (int)nsplit,
                                                                               part, psi, acc);
         note_launch();
     }
     return need;
+}
+// persistent blocks of a kernel: as many as are resident on the device at once
+template <class K>
+int resident_blocks(K kern, int threads) {
+    int bps = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads, 0);
+    return sm_count() * (bps < 1 ? 1 : bps);
+}
+}  // namespace
+
+size_t p2p_plan_fixed_bytes(int nleaves) { return plan_layout(nullptr, nleaves).bytes; }
+
+size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
+                        const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, int mode,
+                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+    auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
+                   double* part) {
+        auto go = [&](auto kern) {
+            const int nblocks = resident_blocks(kern, kP2PWarpsM * 32);
+            mark_begin(s);
+            kern<<<nblocks, kP2PWarpsM * 32, 0, s>>>(xp, c, leaves, ranges, pc, items, nitems, counter, psi, acc, part);
+            mark_end(s);
+        };
+        if (mode == 1) go(k_p2p_mixed<1>);
+        else if (mode == 2) go(k_p2p_mixed<2>);
+        else if (mode == 3) go(k_p2p_mixed<3>);
+        else go(k_p2p_mixed<0>);
+        note_launch();
+    };
+    return plan_and_run<PlanMixed>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, mode, tmp, tmp_bytes,
+                                   h_tot, s, run);
+}
+
+size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,
+                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, void* tmp,
+                           size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+    auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
+                   double* part) {
+        auto go = [&](auto kern) {
+            const int nblocks = resident_blocks(kern, kP2PWarpsD * 32);
+            kern<<<nblocks, kP2PWarpsD * 32, 0, s>>>(xm, c, leaves, ranges, pc, items, nitems, counter, psi, acc, part);
+        };
+        if (want_f) go(k_p2p_f64<true>);
+        else go(k_p2p_f64<false>);
+        note_launch();
+    };
+    return plan_and_run<PlanF64>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, 0, tmp, tmp_bytes, h_tot,
+                                 s, run);
 }
 
 }  // namespace gb3

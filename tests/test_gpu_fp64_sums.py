@@ -1,5 +1,5 @@
-"""The FP64 direct sum at the edges of its work split (sinks per block, slices of the sources) against
-plain FP64 sums."""
+"""The FP64 direct sum and the FP64 P2P at the edges of their work splits (sinks per block, slices
+of the sources, slots and replicas of a leaf, pieces of a long item) against plain FP64 sums."""
 import numpy as np
 import pytest
 
@@ -67,3 +67,18 @@ def test_direct_splits(g, n, ns, want_f):
         assert np.max(np.abs(out[2].cpu().numpy() - ref[2]) / np.maximum(ref[2], 1e-300)) < TOL
     ctx.close()
 
+
+@pytest.mark.parametrize("n,leaf", [(2, 1), (33, 1), (500, 3), (777, 17), (1500, 33), (2000, 65), (5001, 64),
+                                    (4000, 130), (3000, 1000), (700, 4096)])
+@pytest.mark.parametrize("mac", [0, 1])
+def test_fp64_p2p_splits(g, n, leaf, mac):
+    """With eps near 0 every pair is summed directly, so the evaluation is the direct sum: leaves of
+    1 to 4096 sinks, items with and without pieces, a coincident pair."""
+    x, mu = inputs.plummer(n, 950 + n)
+    if n > 300:
+        x[20] = x[21]
+    ctx = g.Context(p=3, eps=1e-30, leaf_size=leaf, p2p_c=1.0, mac=mac, precision=g.FMM_PREC_FP64)
+    psi, acc, st = ctx.fmm_evaluate(_dev(x), _dev(mu), stats=True)
+    assert st["n_m2l"] == 0
+    _check(psi.cpu().numpy(), acc.cpu().numpy(), _sums(x, mu, np.arange(n)))
+    ctx.close()
