@@ -103,65 +103,61 @@ void launch_p2m(const d4* xm, Cells c, const d4* cen, const int* leaves, int nle
 }
 
 // ---------------------------------------------------------------- M2M
-// M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z), one warp per
-// parent; daughters one after another through shared memory.
-__global__ void k_m2m(Cells c, const d4* __restrict__ cen, int lev_begin, int lev_end, int p,
-                      double* __restrict__ M, LaneSched sched) {
+// M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z): one block per parent and one
+// warp per daughter (a level is a chain of one daughter's FP64 work: with the daughters one after
+// another in one warp, 13 levels of a 6e4 cusp at p = 14 took 8.1 ms, so 1.9 ms); the daughters'
+// contributions are then added in daughter order.
+constexpr int kM2MWarps64 = 8;
+__global__ void __launch_bounds__(kM2MWarps64 * 32) k_m2m(Cells c, const d4* __restrict__ cen, int lev_begin,
+                                                          int p, double* __restrict__ M, LaneSched sched) {
     extern __shared__ cd csm[];
-    const int wpb = blockDim.x >> 5;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
+    const int nco = ncoef(p), nout = (p + 1) * (p + 2) / 2;
     cd* Yw = csm + (size_t)wid * 2 * nco;
     cd* Mw = Yw + nco;
-    int cell = lev_begin + blockIdx.x * wpb + wid;
-    if (cell >= lev_end) return;
-    int nch = c.nchild[cell];
+    cd* res = csm + (size_t)kM2MWarps64 * 2 * nco;  // [kM2MWarps64][nout]
+    const int cell = lev_begin + blockIdx.x;
+    const int nch = c.nchild[cell];
     if (nch == 0) return;
-    const d4 zp = cen[cell];
-    cd acc[kMaxPerLane];
-    const int cnt = sched.cnt[lane];
-#pragma unroll
-    for (int k = 0; k < kMaxPerLane; ++k) acc[k] = mkc(0.0, 0.0);
-    for (int j = 0; j < nch; ++j) {
-        int d = c.child[cell] + j;
+    if (wid < nch) {
+        const d4 zp = cen[cell];
+        const int d = c.child[cell] + wid, cnt = sched.cnt[lane];
         const d4 z = cen[d];
         if (lane <= p) upsilon_column(p, lane, z.x - zp.x, z.y - zp.y, z.z - zp.z, Yw, false);
         expand_real(p, M + (size_t)d * nco, Mw, false, lane, 32);
         __syncwarp();
-#pragma unroll
-        for (int q = 0; q < kMaxPerLane; ++q) {
-            if (q < cnt) {
-                int n = sched.n[lane][q], m = sched.m[lane][q];
-                cd s = mkc(0.0, 0.0);
-                for (int k = 0; k <= n; ++k) {
-                    int nn = n - k;
-                    int lmin = max(-k, m - nn), lmax = min(k, m + nn);
-                    for (int l = lmin; l <= lmax; ++l) cmac(s, Yw[cix(k, l)], Mw[cix(nn, m - l)]);
-                }
-                acc[q] = acc[q] + s;
+        for (int q = 0; q < cnt; ++q) {
+            const int n = sched.n[lane][q], m = sched.m[lane][q];
+            cd s = mkc(0.0, 0.0);
+            for (int k = 0; k <= n; ++k) {
+                const int nn = n - k;
+                const int lmin = max(-k, m - nn), lmax = min(k, m + nn);
+                for (int l = lmin; l <= lmax; ++l) cmac(s, Yw[cix(k, l)], Mw[cix(nn, m - l)]);
             }
+            res[wid * nout + n * (n + 1) / 2 + m] = s;
         }
-        __syncwarp();
     }
+    __syncthreads();
     double* out = M + (size_t)cell * nco;
-#pragma unroll
-    for (int q = 0; q < kMaxPerLane; ++q) {
-        if (q < cnt) {
-            int n = sched.n[lane][q], m = sched.m[lane][q];
-            out[cix(n, m)] = acc[q].re;
-            if (m) out[cix(n, -m)] = acc[q].im;
-        }
+    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
+        int n = 0;
+        while ((n + 1) * (n + 2) / 2 <= o) ++n;
+        const int m = o - n * (n + 1) / 2;
+        cd v = mkc(0.0, 0.0);
+        for (int j = 0; j < nch; ++j) v = v + res[j * nout + o];
+        out[cix(n, m)] = v.re;
+        if (m) out[cix(n, -m)] = v.im;
     }
 }
 
 void launch_m2m_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M, cudaStream_t s) {
     int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
-    const int wpb = 4;
-    size_t sm = (size_t)wpb * 2 * ncoef(p) * sizeof(cd);
+    const size_t sm = (size_t)kM2MWarps64 * (2 * ncoef(p) + (p + 1) * (p + 2) / 2) * sizeof(cd);
     LaneSched sched = make_lane_sched(p, kSchedUp);
     init_rec_tables();
-    k_m2m<<<(ncl + wpb - 1) / wpb, wpb * 32, sm, s>>>(c, cen, lev_begin, lev_end, p, M, sched); note_launch();
+    cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_m2m<<<ncl, kM2MWarps64 * 32, sm, s>>>(c, cen, lev_begin, p, M, sched); note_launch();
 }
 
 // ---------------------------------------------------------------- power
