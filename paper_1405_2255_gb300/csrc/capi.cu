@@ -750,15 +750,16 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
     // A9: M2L
     CU(cudaMemsetAsync(ctx->F.p, 0, sizeof(double) * nco * (size_t)nc, s));
     if (split) {
-        TRY(ensure(ctx->m2l_tmp, m2l_split_tmp_bytes(nc, prm.p, ctx->n_m2l)));
+        TRY(ensure(ctx->m2l_tmp, std::max(m2l_split_tmp_bytes(nc, prm.p, ctx->n_m2l),
+                                          m2l_f64_tmp_bytes(nc, prm.p, ctx->n_m2l))));  // p <= 2 takes the latter
         kernel_marks(timing ? &ctx->ev[EV_M2LK0] : nullptr);
         launch_m2l_split(P<int2>(ctx->m2l), P<int>(ctx->m2l_seg_start), P<int>(ctx->m2l_seg_end), ctx->m2l_tmp.p, nc,
                          c.sr, P<double>(ctx->M), prm.p, P<double>(ctx->F), prm.m2l_rot != 0, s, wp.adaptive != 0,
                          ctx->n_m2l);
     } else {
-        TRY(ensure(ctx->m2l_tmp, m2l_tmp_bytes(nc, prm.p)));
-        launch_m2l(P<int2>(ctx->m2l), P<int>(ctx->m2l_seg_start), P<int>(ctx->m2l_seg_end), ctx->m2l_tmp.p, nc, c.sr,
-                   P<double>(ctx->M), prm.p, P<double>(ctx->F), s);
+        TRY(ensure(ctx->m2l_tmp, m2l_f64_tmp_bytes(nc, prm.p, ctx->n_m2l)));
+        launch_m2l_f64(P<int2>(ctx->m2l), P<int>(ctx->m2l_seg_start), P<int>(ctx->m2l_seg_end), ctx->m2l_tmp.p, nc,
+                       c.sr, P<double>(ctx->M), prm.p, P<double>(ctx->F), ctx->n_m2l, s);
     }
     ctx->marked_m2l = marks_recorded();
     kernel_marks(nullptr);

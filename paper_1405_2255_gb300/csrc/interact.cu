@@ -1,97 +1,12 @@
-// interact.cu -- A9-A12 of the path: M2L (eq. 3b), L2L (eq. 5), L2P (eqs. 3a, 7),
-// P2P (eq. 1) in FP64 and in mixed precision, the p = 0 kernels of the low-order
+// interact.cu -- A9-A12 of the path: M2L (eq. 3b, the mixed mode's direct form), L2L (eq. 5), L2P
+// (eqs. 3a, 7), P2P (eq. 1) in FP64 without a work plan, the p = 0 kernels of the low-order
 // f estimate (Sec. 5.3.2), and the final scatter to the caller's order.
 #include "harmonics.cuh"
 #include "kernels.cuh"
 
 namespace gb3 {
 
-// ---------------------------------------------------------------- M2L
-// conj(M_A) of every cell as a full complex array (all m), once per evaluation, so
-// that M2L reads it instead of re-expanding the real storage for every pair
-__global__ void k_expand_conj(const double* __restrict__ M, int ncells, int p, cd* __restrict__ Mc) {
-    const int nco = ncoef(p);
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)ncells * nco;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int cell = (int)(t / nco), i = (int)(t % nco);
-        int n = (int)sqrtf((float)i);
-        while (n * n > i) --n;
-        while ((n + 1) * (n + 1) <= i) ++n;
-        const cd v = load_real_storage(M + (size_t)cell * nco, n, i - n * n - n);
-        Mc[t] = conjc(v);
-    }
-}
-
-// One warp per sink cell B.  Its sources (a segment of the sorted M2L list) are
-// taken NB at a time: the warp copies conj(M_A) of the NB sources to shared
-// memory and builds Theta(s_B - z_A) for all NB pairs at once (32/NB lanes per
-// pair, each lane a few m-columns), so that the serial recurrences of one pair
-// do not leave the other lanes idle; then each lane accumulates its scheduled
-// outputs F_n^m(s_B) over the NB pairs in registers.  Warps take sinks from an
-// atomic counter over the sinks ordered by decreasing list length.
-template <int MAXQ, int NB>
-__global__ void __launch_bounds__(64) k_m2l(const int2* __restrict__ list, const int* __restrict__ seg_start,
-                                            const int* __restrict__ seg_end, const int* __restrict__ order,
-                                            int nsinks, unsigned* __restrict__ work, const d4* __restrict__ cen,
-                                            const cd* __restrict__ Mc, int p, double* __restrict__ F,
-                                            LaneSched sched) {
-    extern __shared__ cd csm[];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
-    cd* T = csm + (size_t)wid * 2 * NB * nco;  // [NB][nco]
-    cd* Mb = T + NB * nco;                     // [NB][nco]
-    constexpr int LPP = 32 / NB;               // lanes per pair while building Theta
-    const int cnt = sched.cnt[lane];
-    for (;;) {
-        unsigned w = 0;
-        if (lane == 0) w = atomicAdd(work, 1u);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= (unsigned)nsinks) break;
-        const int B = order[w];
-        const int e0 = seg_start[B], e1 = seg_end[B];
-        if (e1 <= e0) continue;
-        const d4 sB = cen[B];
-        cd acc[MAXQ];
-#pragma unroll
-        for (int q = 0; q < MAXQ; ++q) acc[q] = mkc(0.0, 0.0);
-        for (int eb = e0; eb < e1; eb += NB) {
-            const int nb = min(NB, e1 - eb);
-            // conj(M) of the batch
-            for (int b = 0; b < nb; ++b) {
-                const cd* src = Mc + (size_t)m2l_src(list[eb + b].x) * nco;
-                for (int i = lane; i < nco; i += 32) Mb[b * nco + i] = src[i];
-            }
-            // Theta of the batch
-            {
-                const int b = lane / LPP, sub = lane % LPP;
-                if (b < nb) {
-                    const d4 zA = cen[m2l_src(list[eb + b].x)];
-                    const double x = sB.x - zA.x, y = sB.y - zA.y, z = sB.z - zA.z;
-                    for (int m = sub; m <= p; m += LPP) theta_column(p, m, x, y, z, T + b * nco);
-                }
-            }
-            __syncwarp();
-            for (int b = 0; b < nb; ++b) {
-                const int pb = m2l_order(list[eb + b].x, p);  // the pair's order (adaptive walk) or p
-#pragma unroll
-                for (int q = 0; q < MAXQ; ++q)
-                    if (q < cnt && sched.n[lane][q] <= pb)
-                        acc[q] = acc[q] + contract(pb, sched.n[lane][q], sched.m[lane][q], Mb + b * nco, T + b * nco);
-            }
-            __syncwarp();
-        }
-        double* out = F + (size_t)B * nco;
-#pragma unroll
-        for (int q = 0; q < MAXQ; ++q) {
-            if (q < cnt) {
-                int n = sched.n[lane][q], m = sched.m[lane][q];
-                out[cix(n, m)] = acc[q].re;
-                if (m) out[cix(n, -m)] = acc[q].im;
-            }
-        }
-    }
-}
-
+// ---------------------------------------------------------------- M2L, mixed mode: order of the sinks
 // sinks with a non-empty M2L segment, ordered by decreasing segment length (eight steps per
 // octave, qlen8)
 __global__ void k_sink_keys(const int* __restrict__ seg_start, const int* __restrict__ seg_end, int ncells,
@@ -112,61 +27,9 @@ __global__ void k_sink_order(const uint64_t* __restrict__ keys, int ncells, int*
     }
 }
 
-size_t m2l_tmp_bytes(int ncells, int p) {
+static size_t m2l_order_bytes(int ncells) {
     size_t n = (size_t)(ncells > 0 ? ncells : 1);
-    return n * (2 * sizeof(uint64_t) + 3 * sizeof(int)) + radix_tmp_ints(n) * sizeof(int) + 256 +
-           n * (size_t)ncoef(p) * sizeof(cd);
-}
-
-template <int MAXQ, int NB>
-static void m2l_launch(const int2* list, const int* seg_start, const int* seg_end, const int* order, int ncells,
-                       unsigned* work, const d4* cen, const cd* Mc, int p, double* F, const LaneSched& sched,
-                       cudaStream_t s) {
-    const int wpb = 2;
-    size_t sm = (size_t)wpb * 2 * NB * ncoef(p) * sizeof(cd);
-    cudaFuncSetAttribute(k_m2l<MAXQ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int dev = 0, nsm = 152, bps = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_m2l<MAXQ, NB>, wpb * 32, sm);
-    unsigned g = (unsigned)(nsm * (bps > 0 ? bps : 1));
-    k_m2l<MAXQ, NB><<<g, wpb * 32, sm, s>>>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched);
-    note_launch();
-}
-
-void launch_m2l(const int2* list, const int* seg_start, const int* seg_end, void* tmp, int ncells, const d4* cen,
-                const double* M, int p, double* F, cudaStream_t s) {
-    if (ncells <= 0) return;
-    init_rec_tables();
-    // order the sinks by decreasing work
-    uint64_t* k0 = (uint64_t*)tmp;
-    uint64_t* k1 = k0 + ncells;
-    int* v0 = (int*)(k1 + ncells);
-    int* v1 = v0 + ncells;
-    int* order = v1 + ncells;
-    unsigned* work = (unsigned*)(order + ncells);  // [0] counter, [1] number of sinks
-    int* rtmp = (int*)(work + 4);
-    cd* Mc = (cd*)(((uintptr_t)(rtmp + radix_tmp_ints(ncells)) + 255) & ~(uintptr_t)255);
-    cudaMemsetAsync(work, 0, 4 * sizeof(unsigned), s);
-    k_sink_keys<<<grid_for(ncells, 256), 256, 0, s>>>(seg_start, seg_end, ncells, k0, v0); note_launch();
-    // the low 32 bits are the sink's index, already in order: the stable pass over the 8
-    // length bits alone keeps ties in index order
-    int flip = radix_sort_pairs_bits(k0, v0, k1, v1, ncells, rtmp, 32, 40, s);
-    k_sink_order<<<grid_for(ncells, 256), 256, 0, s>>>(flip ? k1 : k0, ncells, order, work + 1); note_launch();
-    k_expand_conj<<<grid_for((long long)ncells * ncoef(p), 256), 256, 0, s>>>(M, ncells, p, Mc); note_launch();
-    LaneSched sched = make_lane_sched(p, kSchedDown);
-    int maxq = 0;
-    for (int l = 0; l < 32; ++l) maxq = sched.cnt[l] > maxq ? sched.cnt[l] : maxq;
-    // every cell is visited (empty segments cost one counter step); the order puts them last
-    if (p <= 12) {
-        if (maxq <= 4) m2l_launch<4, 8>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched, s);
-        else m2l_launch<8, 8>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched, s);
-    } else if (p <= 16) {
-        if (maxq <= 8) m2l_launch<8, 4>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched, s);
-        else m2l_launch<12, 4>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched, s);
-    } else {
-        m2l_launch<24, 2>(list, seg_start, seg_end, order, ncells, work, cen, Mc, p, F, sched, s);
-    }
+    return n * (2 * sizeof(uint64_t) + 3 * sizeof(int)) + radix_tmp_ints(n) * sizeof(int) + 256;
 }
 
 // ---------------------------------------------------------------- M2L, precision-split (mixed mode)
@@ -548,7 +411,7 @@ static void m2l_rounds_launch(const int2* list, const int* seg_start, const int*
 size_t m2l_split_tmp_bytes(int ncells, int p, long long npairs) {
     size_t n = (size_t)(ncells > 0 ? ncells : 1);
     size_t items = (size_t)(npairs / kChunk) + n + 1;
-    return m2l_tmp_bytes(ncells, p) + n * (size_t)ncoef(p) * sizeof(float2) + n * kN64 * sizeof(cd) +
+    return m2l_order_bytes(ncells) + n * (size_t)ncoef(p) * sizeof(float2) + n * kN64 * sizeof(cd) +
            2 * n * sizeof(int) + scan_tmp_ints(n) * sizeof(int) + items * (size_t)ncoef(p) * sizeof(double) +
            m2l_rot_group_bytes((long long)items) + 4096;
 }
@@ -591,7 +454,7 @@ void launch_m2l_split(const int2* list, const int* seg_start, const int* seg_end
                       const double* M, int p, double* F, bool rot, cudaStream_t s, bool adaptive, long long npairs) {
     if (ncells <= 0) return;
     if (p <= kJ64) {  // nothing to split
-        launch_m2l(list, seg_start, seg_end, tmp, ncells, cen, M, p, F, s);
+        launch_m2l_f64(list, seg_start, seg_end, tmp, ncells, cen, M, p, F, npairs, s);
         return;
     }
     init_split_tables();

@@ -169,9 +169,11 @@ void launch_segments(const int2* list, long long npairs, int ncells, int* seg_st
                      cudaStream_t s);
 
 // ---------------------------------------------------------------- interactions (interact.cu)
-size_t m2l_tmp_bytes(int ncells, int p);
-void launch_m2l(const int2* list, const int* seg_start, const int* seg_end, void* tmp, int ncells,
-                const d4* cen, const double* M, int p, double* F, cudaStream_t s);
+// FP64 M2L through rotations (m2l_f64.cu) of the npairs pairs of list into F (zero beforehand); tmp:
+// m2l_f64_tmp_bytes
+size_t m2l_f64_tmp_bytes(int ncells, int p, long long npairs);
+void launch_m2l_f64(const int2* list, const int* seg_start, const int* seg_end, void* tmp, int ncells,
+                    const d4* cen, const double* M, int p, double* F, long long npairs, cudaStream_t s);
 // mixed mode: orders <= 2 of Theta in FP64, the rest in FP32 on scaled harmonics, either
 // directly (eq. 3b) or, when rot is set and m2l_rot_supported(p), through rotations into
 // the interaction's z frame (App. A.5, m2l_rot.cu)

@@ -18,6 +18,7 @@
 // everything that must start at zero is cleared here; two calls whose work
 // overlaps on the GPU (different streams, or different host threads) race on it
 // and give wrong results: serialise them.
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <stdio.h>
@@ -292,7 +293,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     double* F1 = A.take<double>(4 * (size_t)nc);
     double* Ff = A.take<double>(nc);
     float4* walkf = A.take<float4>((size_t)(2 + walk_fstride(p) / 4) * nc);
-    void* m2l_tmp = A.take<unsigned char>(m2l_split_tmp_bytes(nc, p > 1 ? p : 1, kListCap));
+    void* m2l_tmp = A.take<unsigned char>(std::max(m2l_split_tmp_bytes(nc, p, kListCap), m2l_f64_tmp_bytes(nc, p, kListCap)));
     if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the expansions and lists");
     // the rest of the array serves the list sorts and, once a list is sorted, the mixed P2P's
     // work plan (the two never overlap on the stream)
@@ -390,7 +391,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     if (split)
         launch_m2l_split(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, M, p, F, prm.m2l_rot != 0, s, false, nm);
     else
-        launch_m2l(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, M, p, F, s);
+        launch_m2l_f64(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, M, p, F, nm, s);
     sort_pairs_by_sink(p2p, np, nc, r.sort_tmp, s);
     launch_segments(p2p, np, nc, seg_start, seg_end, s);
     if (prm.precision == FMM_PREC_MIXED) {

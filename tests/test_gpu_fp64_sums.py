@@ -1,4 +1,4 @@
-"""The FP64 direct sum and the FP64 P2P at the edges of their work splits (sinks per block, slices
+"""The FP64 direct sum, the FP64 P2P and the FP64 M2L and M2M at the edges of their work splits (sinks per block, slices
 of the sources, slots and replicas of a leaf, pieces of a long item) against plain FP64 sums."""
 import numpy as np
 import pytest
@@ -82,3 +82,28 @@ def test_fp64_p2p_splits(g, n, leaf, mac):
     assert st["n_m2l"] == 0
     _check(psi.cpu().numpy(), acc.cpu().numpy(), _sums(x, mu, np.arange(n)))
     ctx.close()
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 9, 16, 17, 18])
+@pytest.mark.parametrize("shape", ["plummer", "z axis", "x axis", "plane"])
+def test_fp64_m2l_orders_and_directions(g, orc, p, shape):
+    """Every order class of the rotated M2L, with interaction directions along the axes (where the
+    rotation angle about z is undefined) among them: tree, lists and forces equal the oracle's
+    to 1e-10 of the sum of the magnitudes of a sink's terms (f of eq. 6; on a line neighbours on both
+    sides cancel).  The geometric criterion gives lists of all lengths."""
+    x, mu = inputs.plummer(3000, inputs.BASE_SEED + 31)
+    if shape == "z axis":
+        x[:, :2] = 0.0
+    elif shape == "x axis":
+        x[:, 1:] = 0.0
+    elif shape == "plane":
+        x[:, 2] = 0.0
+    prm = dict(p=p, mac=2, theta_crit=0.6, leaf_size=12, p2p_c=0.0)
+    ctx = g.Context(precision=g.FMM_PREC_FP64, **prm)
+    psi, acc, st = ctx.fmm_evaluate(_dev(x), _dev(mu), stats=True)
+    ctx.close()
+    run = orc.fmm(x, mu, **prm)
+    assert st["n_m2l"] == run.stats["n_m2l"] > 1000
+    f = orc.direct(x, mu)[2]
+    assert np.max(np.linalg.norm(acc.cpu().numpy() - run.acc, axis=1) / f) <= 1e-10
+    assert np.max(np.abs(psi.cpu().numpy() - run.psi) / run.psi) <= 1e-10
