@@ -470,6 +470,25 @@ static int p2p_fp64(fmm_ctx* ctx, const int2* list, cudaStream_t s) {
     return 0;
 }
 
+// the near tidal tensor: in mixed mode with a work plan where there is room for one
+static int run_p2p_tidal(fmm_ctx* ctx, cudaStream_t s) {
+    Cells c = cells_of(ctx);
+    const bool mixed = ctx->prm.precision == FMM_PREC_MIXED;
+    size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
+    for (int attempt = 0; mixed && attempt < 2; ++attempt) {
+        if (ensure(ctx->p2p_tmp, need)) break;
+        need = launch_p2p_tidal_plan(P<float4>(ctx->xp), ctx->n, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
+                                     P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves,
+                                     P<double>(ctx->tid_near), ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
+                                     ctx->h_counters + 8, s);
+        if (need <= ctx->p2p_tmp.bytes) return 0;
+        if (need == ~(size_t)0) break;
+    }
+    launch_p2p_tidal(P<d4>(ctx->xm), P<float4>(ctx->xp), ctx->n, mixed, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
+                     P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->tid_near), s);
+    return 0;
+}
+
 // ------------------------------------------------------------------ the low-order scale (A7)
 static int estimate_scale(fmm_ctx* ctx, cudaStream_t s) {
     const int nc = ctx->ncells;
@@ -794,9 +813,7 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
                       ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
     if (tidal) {  // Sec. 7.4: the near part over the same sources as the P2P
         TRY(ensure(ctx->tid_near, sizeof(double) * 6 * (size_t)n));
-        launch_p2p_tidal(P<d4>(ctx->xm), P<float4>(ctx->xp), n, prm.precision == FMM_PREC_MIXED,
-                         c, P<int2>(ctx->p2p), P<int>(ctx->seg_start), P<int>(ctx->seg_end), P<int>(ctx->leaves),
-                         ctx->nleaves, P<double>(ctx->tid_near), s);
+        TRY(run_p2p_tidal(ctx, s));
     }
     if (timing) CU(cudaEventRecord(ctx->ev[EV_P2P], s));
     CU(cudaEventRecord(ctx->ev_join_est, s));

@@ -283,6 +283,11 @@ void launch_l2p_tidal(const d4* xm, Cells c, const d4* cen, const int* leaves, i
 void launch_p2p_tidal(const d4* xm, const float4* xp, int n, bool fp32, Cells c, const int2* list,
                       const int* seg_start, const int* seg_end, const int* leaves, int nleaves, double* T,
                       cudaStream_t s);
+// the near part in mixed precision with a work plan as launch_p2p_mixed's (same scratch, return value
+// and host read)
+size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
+                             const int* seg_end, const int* leaves, int nleaves, double* T, void* tmp,
+                             size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
 void launch_finish_tidal(const double* Tf, const double* Tn, const int* perm, int n, double G,
                          const unsigned char* pact, double* T, cudaStream_t s, const int* e = nullptr);
 // individual accuracy parameters (Sec. 7, opening): scale_sorted[i] *= eps_b[perm[i]] / eps

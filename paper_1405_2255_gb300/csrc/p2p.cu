@@ -182,6 +182,8 @@ struct Chunk {
 struct PlanMixed {
     static constexpr unsigned piece_steps = 8192;
     static constexpr int max_pieces = 64;
+    static constexpr bool merge = true;
+    static constexpr int nv = 4;  // sums per sink
     __device__ static inline Chunk chunk(int c) {
         Chunk r{1, 1, 1, 2};
         if (c <= 0) return r;
@@ -209,6 +211,8 @@ struct PlanMixed {
 struct PlanF64 {
     static constexpr unsigned piece_steps = 256;
     static constexpr int max_pieces = 1024;
+    static constexpr bool merge = true;
+    static constexpr int nv = 4;
     __device__ static inline Chunk chunk(int c) {
         Chunk r{1, 1, 1, 1};
         if (c <= 0) return r;
@@ -222,6 +226,30 @@ struct PlanF64 {
                     best = cost;
                     r = Chunk{k, R, S, Q};
                 }
+            }
+        }
+        return r;
+    }
+};
+
+// The mixed tidal P2P: a slot holds two sinks as the halves of packed operations, and the R groups of
+// S lanes take shares of the source cells of their own: the fewest items k / R per source.
+struct PlanTidal {
+    static constexpr unsigned piece_steps = 1024;
+    static constexpr int max_pieces = 256;
+    static constexpr bool merge = false;
+    static constexpr int nv = 6;
+    __device__ static inline Chunk chunk(int c) {
+        Chunk r{1, 1, 1, 2};
+        if (c <= 0) return r;
+        const int slots = (c + 1) / 2, kmin = (slots + 31) / 32;
+        float best = 3.0e38f;
+        for (int k = kmin; k < kmin + 6; ++k) {
+            const int S = (slots + k - 1) / k, R = min(32 / S, 4);
+            const float cost = (float)k / (float)R * (1.0f + 0.05f * (float)R);
+            if (cost < best) {
+                best = cost;
+                r = Chunk{(slots + S - 1) / S, R, S, 2};
             }
         }
         return r;
@@ -362,7 +390,9 @@ struct Pieces {
 // not join start a run, a run's count and guard flag are summed in shared memory, and every run
 // but the last of its class is written out; the last stays open until the piece ends.  This is
 // the result of the sequential pass.
+// MERGE false: one far record per source cell, in stream order from the front (the tidal P2P).
 constexpr int kEmitWarps = 4;
+template <bool MERGE>
 __global__ void __launch_bounds__(kEmitWarps * 32)
     k_p2p_emit(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int mode,
@@ -426,11 +456,13 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
                 const int A = list[at + lane].x;
                 f = c.first[A];
                 n = c.count[A];
-                kk = mode == 1 ? (p2p_near(c.sr[A], sb) ? 1 : 0) : (mode == 3 ? 1 : 0);
+                if (MERGE) kk = mode == 1 ? (p2p_near(c.sr[A], sb) ? 1 : 0) : (mode == 3 ? 1 : 0);
+                else ranges[r0 + (int)(fi - f0) + lane] = make_int2(f, n);
                 if (n <= 0) kk = -1;
             }
             at += m;
             fi += m;
+            if (!MERGE) continue;
             const bool g = kk >= 0 && f < b1 && b0 < (long long)f + n;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -487,8 +519,10 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
     }
 }
 
-// the FP64 partial sums of the split leaves added in piece order into psi and acc: one warp per
-// entry (t, first slot) of the split list, lanes over the leaf's sinks
+// the FP64 partial sums of the split leaves added in piece order into psi and acc (NV = 4) or into
+// the NV values per sink of acc: one warp per entry (t, first slot) of the split list, lanes over
+// the leaf's sinks
+template <int NV>
 __global__ void k_p2p_reduce(Cells c, const int* __restrict__ leaves, const int* __restrict__ np,
                              const int2* __restrict__ split, int nsplit, const double* __restrict__ part,
                              double* __restrict__ psi, double* __restrict__ acc) {
@@ -499,17 +533,24 @@ __global__ void k_p2p_reduce(Cells c, const int* __restrict__ leaves, const int*
         const int leaf = leaves[sp.x], P = np[sp.x];
         const int first = c.first[leaf], count = c.count[leaf];
         for (int sk = lane; sk < count; sk += 32) {
-            double v[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int j = 0; j < P; ++j) {
-                const double* pp = part + 4 * ((size_t)sp.y + (size_t)j * count + sk);
+            double v[NV];
 #pragma unroll
-                for (int d = 0; d < 4; ++d) v[d] += pp[d];
+            for (int d = 0; d < NV; ++d) v[d] = 0.0;
+            for (int j = 0; j < P; ++j) {
+                const double* pp = part + NV * ((size_t)sp.y + (size_t)j * count + sk);
+#pragma unroll
+                for (int d = 0; d < NV; ++d) v[d] += pp[d];
             }
             const size_t i = (size_t)first + sk;
-            psi[i] = v[0];
-            acc[3 * i] = v[1];
-            acc[3 * i + 1] = v[2];
-            acc[3 * i + 2] = v[3];
+            if (NV == 4) {
+                psi[i] = v[0];
+                acc[3 * i] = v[1];
+                acc[3 * i + 1] = v[2];
+                acc[3 * i + 2] = v[3];
+            } else {
+#pragma unroll
+                for (int d = 0; d < NV; ++d) acc[NV * i + d] = v[d];
+            }
         }
     }
 }
@@ -885,6 +926,183 @@ __global__ void __launch_bounds__(kP2PWarpsD * 32)
     }
 }
 
+// The near tidal tensor in mixed precision (Sec. 7.4): dx from the two-float positions, FP32 pair terms
+// summed over a tile (at most 32 sources of one source cell, in order), the tiles added as two-float
+// sums.  30 packed FP32 operations and two rsqrt for the two pairs of a slot: bound by the FMA pipe.
+// The R groups of S lanes take tiles of their own, all in step: the source cells are cut into tiles 32
+// records at a time, the tiles ordered by length and dealt to the groups, so that the tiles of a round
+// are about equally long (the shorter ones are filled up with massless sources).  150,001 particles,
+// 1.16e9 pairs: 19.0 ms with one warp per leaf and one sink per lane (the longest leaf ran on alone),
+// 3.3 ms with groups that run through their tiles on their own (they diverge), 2.2 ms so.
+constexpr int kTidWarps = 4;
+constexpr int kTidTile = 32;
+constexpr int kTidGroups = 4;  // PlanTidal's largest R
+constexpr int kTidBatch = 64;  // tiles ordered together
+
+struct TidAcc {
+    f2 p[6];
+};
+// one source (h: high parts and mass, l: low parts) against the slot's two sinks
+__device__ __forceinline__ void tid_pair(const float4& h, const float4& l, const f2 (&bh)[3], const f2 (&bl)[3],
+                                         TidAcc& a) {
+    const f2 dx = f2_add(f2_sub(bh[0], f2_pack(h.x, h.x)), f2_sub(bl[0], f2_pack(l.x, l.x)));
+    const f2 dy = f2_add(f2_sub(bh[1], f2_pack(h.y, h.y)), f2_sub(bl[1], f2_pack(l.y, l.y)));
+    const f2 dz = f2_add(f2_sub(bh[2], f2_pack(h.z, h.z)), f2_sub(bl[2], f2_pack(l.z, l.z)));
+    const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
+    float ra, rb;
+    f2_unpack(r2, ra, rb);
+    float ia = rsqrt_ftz(ra), ib = rsqrt_ftz(rb);
+    if (fminf(ra, rb) < 0x1p-126f) {  // coincident (skipped) or subnormal
+        if (ra < 0x1p-126f) ia = ra > 0.f ? rsqrtf(ra) : 0.f;
+        if (rb < 0x1p-126f) ib = rb > 0.f ? rsqrtf(rb) : 0.f;
+    }
+    const f2 ri = f2_pack(ia, ib), ri2 = f2_mul(ri, ri);
+    const f2 q5 = f2_mul(f2_mul(f2_mul(f2_pack(h.w, h.w), ri), ri2), ri2);
+    const f2 q3 = f2_mul(f2_pack(3.f, 3.f), q5);
+    const f2 nq5 = q5 ^ 0x8000000080000000ull;  // -q5
+    const f2 qx = f2_mul(q3, dx), qy = f2_mul(q3, dy), qz = f2_mul(q3, dz);
+    a.p[0] = f2_fma(qx, dx, f2_fma(nq5, r2, a.p[0]));
+    a.p[1] = f2_fma(qx, dy, a.p[1]);
+    a.p[2] = f2_fma(qx, dz, a.p[2]);
+    a.p[3] = f2_fma(qy, dy, f2_fma(nq5, r2, a.p[3]));
+    a.p[4] = f2_fma(qy, dz, a.p[4]);
+    a.p[5] = f2_fma(qz, dz, f2_fma(nq5, r2, a.p[5]));
+}
+// sum += the tile's value (TwoSum, both halves)
+__device__ __forceinline__ void tid_fold(f2& hi, f2& lo, f2 v) {
+    const f2 s = f2_add(hi, v), bb = f2_sub(s, hi);
+    const f2 e = f2_add(f2_sub(hi, f2_sub(s, bb)), f2_sub(v, bb));
+    hi = s;
+    lo = f2_add(lo, e);
+}
+
+__global__ void __launch_bounds__(kTidWarps * 32)
+    k_p2p_tidal_mixed(const float4* __restrict__ xp, Cells c, const int* __restrict__ leaves,
+                      const int2* __restrict__ ranges, const Pieces pc, const int2* __restrict__ items, int nitems,
+                      unsigned* __restrict__ counter, double* __restrict__ T, double* __restrict__ part) {
+    __shared__ __align__(16) float4 bufs[kTidWarps][2][kTidGroups][2 * kTidTile];
+    __shared__ int2 tiles_all[kTidWarps][kTidBatch], sorted_all[kTidWarps][kTidBatch];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const f2 zero = f2_pack(0.f, 0.f);
+    for (;;) {
+        unsigned w = 0;
+        if (lane == 0) w = atomicAdd(counter, 1u);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= (unsigned)nitems) break;
+        const int2 it = items[w];
+        const int pv = it.x, leaf = leaves[pc.leaf[pv]];
+        const int first = c.first[leaf], count = c.count[leaf];
+        const Chunk ch = PlanTidal::chunk(count);
+        const int R = ch.R, S = ch.S;
+        const int s0 = it.y * 2 * S, chunk = min(2 * S, count - s0);
+        const int slot = lane % S, g = lane / S;
+        const bool in = g < R;
+        const int kA = slot < chunk ? slot : 0, kB = S + slot < chunk ? S + slot : 0;
+        f2 bh[3], bl[3], sh[6], sl[6];
+        {
+            const size_t iA = (size_t)(first + s0 + kA), iB = (size_t)(first + s0 + kB);
+            const float4 ah = xp[2 * iA], al = xp[2 * iA + 1], dh = xp[2 * iB], dl = xp[2 * iB + 1];
+            bh[0] = f2_pack(ah.x, dh.x);
+            bh[1] = f2_pack(ah.y, dh.y);
+            bh[2] = f2_pack(ah.z, dh.z);
+            bl[0] = f2_pack(al.x, dl.x);
+            bl[1] = f2_pack(al.y, dl.y);
+            bl[2] = f2_pack(al.z, dl.z);
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sh[q] = sl[q] = zero;
+        int2 *tiles = tiles_all[wid], *sorted = sorted_all[wid];
+        const int end = pc.r1[pv];
+        int at = pc.r0[pv], off = 0;  // the next record and the tiles of it that are done
+        while (at < end) {
+            // the next records' tiles, as many as the batch holds
+            const int2 rec = at + lane < end ? ranges[at + lane] : make_int2(0, 0);
+            const int o = lane == 0 ? off : 0, nt = (rec.y + kTidTile - 1) / kTidTile - o;
+            int incl = nt;
+#pragma unroll
+            for (int h = 1; h < 32; h <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, h);
+                if (lane >= h) incl += y;
+            }
+            const unsigned fit = __ballot_sync(0xffffffffu, incl <= kTidBatch);
+            const int nrec = fit ? __popc(fit & ~(fit + 1u)) : 0;  // records taken whole (a prefix)
+            const int ntl = nrec ? __shfl_sync(0xffffffffu, incl, nrec - 1) : kTidBatch;
+            const int take = nrec ? (lane < nrec ? nt : 0) : (lane == 0 ? kTidBatch : 0);
+            for (int k = 0; k < take; ++k) {
+                const int d = (o + k) * kTidTile;
+                tiles[incl - nt + k] = make_int2(rec.x + d, min(kTidTile, rec.y - d));
+            }
+            if (nrec) {
+                at += min(nrec, end - at);
+                off = 0;
+            } else {
+                off += kTidBatch;
+            }
+            __syncwarp();
+            // ordered by decreasing length
+            for (int k = lane; k < ntl; k += 32) {
+                const int2 mine = tiles[k];
+                int r = 0;
+                for (int j = 0; j < ntl; ++j) {
+                    const int y = tiles[j].y;
+                    r += y > mine.y || (y == mine.y && j < k);
+                }
+                sorted[r] = mine;
+            }
+            __syncwarp();
+            // copy the tiles of round i (one per group), filled up to the longest of them
+            auto fetch = [&](int i, int b) {
+                if (i * R >= ntl || !in) return;
+                const int nmax = sorted[i * R].y, k = i * R + g;
+                const int2 t = k < ntl ? sorted[k] : make_int2(0, 0);
+                float4* buf = bufs[wid][b][g];
+                const float4* src = xp + 2 * (size_t)t.x;
+                for (int j = slot; j < 2 * t.y; j += S) cp_async16(buf + j, src + j);
+                for (int j = 2 * t.y + slot; j < 2 * nmax; j += S) buf[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            fetch(0, 0);
+            cp_async_commit();
+            for (int i = 0; i * R < ntl; ++i) {
+                cp_async_wait0();
+                __syncwarp();  // the round's tiles have arrived, and the other buffer is no longer read
+                fetch(i + 1, (i + 1) & 1);
+                cp_async_commit();
+                const int n = sorted[i * R].y;
+                const float4* t = bufs[wid][i & 1][in ? g : 0];
+                TidAcc a;
+#pragma unroll
+                for (int q = 0; q < 6; ++q) a.p[q] = zero;
+#pragma unroll 2
+                for (int j = 0; j < n; ++j) tid_pair(t[2 * j], t[2 * j + 1], bh, bl, a);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) tid_fold(sh[q], sl[q], a.p[q]);
+            }
+            cp_async_wait0();
+            __syncwarp();
+        }
+        __syncwarp();
+        // the groups' sums, in group order, as FP64
+        const int pslot = pc.part[pv];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            float hA, hB, lA, lB;
+            f2_unpack(sh[q], hA, hB);
+            f2_unpack(sl[q], lA, lB);
+            double vA = (double)hA + (double)lA, vB = (double)hB + (double)lB;
+            double tA = vA, tB = vB;
+            for (int r = 1; r < R; ++r) {
+                tA += __shfl_sync(0xffffffffu, vA, min(slot + r * S, 31));
+                tB += __shfl_sync(0xffffffffu, vB, min(slot + r * S, 31));
+            }
+            if (lane < S) {
+                double* o = pslot >= 0 ? part + 6 * ((size_t)pslot + (size_t)s0) : T + 6 * ((size_t)first + s0);
+                if (slot < chunk) o[6 * (size_t)slot + q] = tA;
+                if (S + slot < chunk) o[6 * (size_t)(S + slot) + q] = tB;
+            }
+        }
+    }
+}
+
 namespace {
 // layout of the fixed part of the scratch (depends on the number of leaves only)
 struct PlanLayout {
@@ -961,7 +1179,7 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     auto a256 = [](unsigned long long b) { return (size_t)((b + 255) & ~255ull); };
     const size_t o_ranges = L.bytes, o_items = o_ranges + a256(nranges * sizeof(int2)),
                  o_pieces = o_items + a256(nitems * sizeof(int2)), o_part = o_pieces + a256(npieces * 6 * sizeof(int)),
-                 need = o_part + a256(nslots * 4 * sizeof(double)) + 256;
+                 need = o_part + a256(nslots * PL::nv * sizeof(double)) + 256;
     if (tmp_bytes < need) return need;
     unsigned char* b = (unsigned char*)tmp;
     int2* ranges = (int2*)(b + o_ranges);
@@ -972,14 +1190,14 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     double* part = (double*)(b + o_part);
     if (nitems == 0) return need;
     const unsigned g = grid_for((long long)npieces * 32, kEmitWarps * 32, 16);  // one warp per piece
-    k_p2p_emit<<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
+    k_p2p_emit<PL::merge><<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
                                              L.nb, L.ioff, L.nit, L.voff, L.npc, L.pbase, (int)npieces, pc, ranges,
                                              items);
     note_launch();
     run(ranges, pc, items, (int)nitems, L.counter, part);
     if (nsplit > 0) {
-        k_p2p_reduce<<<grid_for((long long)nsplit * 32, 128, 16), 128, 0, s>>>(c, leaves, L.np, L.split, (int)nsplit,
-                                                                              part, psi, acc);
+        k_p2p_reduce<PL::nv><<<grid_for((long long)nsplit * 32, 128, 16), 128, 0, s>>>(
+            c, leaves, L.np, L.split, (int)nsplit, part, psi, acc);
         note_launch();
     }
     return need;
@@ -1031,6 +1249,19 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
     };
     return plan_and_run<PlanF64>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, 0, tmp, tmp_bytes, h_tot,
                                  s, run);
+}
+
+size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
+                             const int* seg_end, const int* leaves, int nleaves, double* T, void* tmp,
+                             size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+    auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
+                   double* part) {
+        k_p2p_tidal_mixed<<<resident_blocks(k_p2p_tidal_mixed, kTidWarps * 32), kTidWarps * 32, 0, s>>>(
+            xp, c, leaves, ranges, pc, items, nitems, counter, T, part);
+        note_launch();
+    };
+    return plan_and_run<PlanTidal>(n, c, list, seg_start, seg_end, leaves, nleaves, nullptr, T, 0, tmp, tmp_bytes,
+                                   h_tot, s, run);
 }
 
 }  // namespace gb3

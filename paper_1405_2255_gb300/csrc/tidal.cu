@@ -9,80 +9,158 @@
 
 namespace gb3 {
 
-// far part: one block per leaf, F in shared memory (complex), one thread per particle
-// streaming the columns of Upsilon(s - x) by their recurrences
-constexpr int kTidThreads = 64;
+// far part (FP64).  Psi_2^m = sum_{k,l} conj(Upsilon_k^l) F_{k+2}^{m+l}, m = 0, 1, 2, at s - x.  With
+// X_k^{-l} = (-1)^l conj(X_k^l) the terms of l and -l combine: for a coefficient pair A = F_{k+2}^{m+l},
+// B = (-1)^l F_{k+2}^{m-l},
+//   conj(Y) A + Y B = Y.re (A + B) + Y.im (i (B - A)),  Y = Upsilon_k^l,
+// and for m = 0 the imaginary part cancels: ten multiply-adds per (k, l) with the combinations formed
+// once per leaf.  The recurrence (k^2 - l^2) Y_k = (2k - 1) z Y_{k-1} - r^2 Y_{k-2} is run on W_k = Y_k /
+// sigma_k with sigma_k = (2k - 1) / (k^2 - l^2) sigma_{k-1}, sigma_l = 1, so that z W_{k-1} needs no
+// factor; sigma is folded into the combinations.
+// What bounds it: the FP64 pipe, whose instructions cost the same however many lanes are active.  A
+// block takes the particles of kTidLeaves leaves together, so that its warps are full.  150,001
+// particles, p = 14: 2.00 ms with a block per leaf, eq. 7 term by term and a division per (k, l);
+// 0.62 ms so.
+constexpr int kTidThreads = 128;
+constexpr int kTidLeaves = 8;
+
+struct TidTab {
+    double beta[kMaxP + 1][kMaxP + 1];   // 1 / (k^2 - l^2) sigma_{k-2} / sigma_k at [l][k]
+    double sigma[kMaxP + 1][kMaxP + 1];  // [l][k]
+    double inv2l[kMaxP + 1];
+};
+static __constant__ TidTab c_tid;
+static void init_tid_tab() {
+    static DeviceOnce once;
+    once_per_device(once, [] {
+        TidTab t;
+        memset(&t, 0, sizeof t);
+        for (int l = 0; l <= kMaxP; ++l) {
+            t.sigma[l][l] = 1.0;
+            for (int k = l + 1; k <= kMaxP; ++k) {
+                const double inv = 1.0 / (double)(k * k - l * l);
+                t.sigma[l][k] = (2.0 * k - 1.0) * inv * t.sigma[l][k - 1];
+                t.beta[l][k] = k >= l + 2 ? inv * t.sigma[l][k - 2] / t.sigma[l][k] : 0.0;
+            }
+            t.inv2l[l] = l ? 1.0 / (2.0 * l) : 0.0;
+        }
+        cudaMemcpyToSymbol(c_tid, &t, sizeof t);
+    });
+}
+
+// combinations of one (k, l), sigma_k folded in: m = 0: Y.re and Y.im weights of Psi_2^0; m = 1, 2:
+// the complex weights of Y.re and Y.im
+struct TidComb {
+    double r0, i0, ar[2], ai[2], br[2], bi[2];
+};
+
 __global__ void __launch_bounds__(kTidThreads) k_l2p_tidal(const d4* __restrict__ xm, Cells c,
                                                            const d4* __restrict__ cen,
                                                            const int* __restrict__ leaves, int nleaves, int p,
                                                            const double* __restrict__ F, double* __restrict__ T) {
-    extern __shared__ cd Fc[];
-    const int nco = ncoef(p);
-    for (int t = blockIdx.x; t < nleaves; t += gridDim.x) {
-        const int cell = leaves[t];
-        if (!cell_active(c, cell)) continue;  // block-uniform
+    extern __shared__ __align__(16) unsigned char tsm[];
+    TidComb* comb_all = (TidComb*)tsm;  // [kTidLeaves][npair]
+    __shared__ int s_cell[kTidLeaves], s_end[kTidLeaves];
+    const int nco = ncoef(p), q = p - 2, npair = (q + 1) * (q + 2) / 2;
+    for (int t0 = blockIdx.x * kTidLeaves; t0 < nleaves; t0 += gridDim.x * kTidLeaves) {
         __syncthreads();
-        expand_real(p, F + (size_t)cell * nco, Fc, false, threadIdx.x, blockDim.x);
+        if (threadIdx.x == 0) {
+            int sum = 0;
+            for (int u = 0; u < kTidLeaves; ++u) {
+                const int cell = t0 + u < nleaves ? leaves[t0 + u] : -1;
+                const bool on = cell >= 0 && cell_active(c, cell);
+                sum += on ? c.count[cell] : 0;
+                s_cell[u] = cell;
+                s_end[u] = sum;  // particles of the leaves up to this one
+            }
+        }
         __syncthreads();
-        const d4 s = cen[cell];
-        const int first = c.first[cell], count = c.count[cell];
-        for (int j = threadIdx.x; j < count; j += blockDim.x) {
-            const d4 xb = xm[first + j];
-            const double x = s.x - xb.x, y = s.y - xb.y, z = s.z - xb.z;
-            const double r2 = x * x + y * y + z * z;
-            cd p20 = mkc(0.0, 0.0), p21 = p20, p22 = p20;
-            cd d = mkc(1.0, 0.0);
-            for (int l = 0; l <= p - 2; ++l) {
-                if (l > 0) {
-                    const double sc = 1.0 / (2.0 * l);
-                    d = cd{sc * (x * d.re - y * d.im), sc * (x * d.im + y * d.re)};
-                }
-                const double sg = (l & 1) ? -1.0 : 1.0;
-                cd prev2 = mkc(0.0, 0.0), prev = d;
-                for (int k = l; k <= p - 2; ++k) {
-                    cd Y;
-                    if (k == l) Y = d;
-                    else {
-                        const double inv = 1.0 / (double)(k * k - l * l);
-                        const double a = (2.0 * k - 1.0) * z;
-                        Y = cd{(a * prev.re - r2 * prev2.re) * inv, (a * prev.im - r2 * prev2.im) * inv};
-                        prev2 = prev;
-                        prev = Y;
-                    }
-                    const cd Xp = conjc(Y);                 // conj(Upsilon_k^l)
-                    const cd Xn = cd{sg * Y.re, sg * Y.im};  // conj(Upsilon_k^{-l}) = (-1)^l Upsilon_k^l
-                    const cd* Fk = Fc + (k + 2) * (k + 2) + (k + 2);  // F_{k+2}^{.}
-                    cmac(p20, Xp, Fk[l]);
-                    cmac(p21, Xp, Fk[1 + l]);
-                    cmac(p22, Xp, Fk[2 + l]);
-                    if (l > 0) {
-                        cmac(p20, Xn, Fk[-l]);
-                        cmac(p21, Xn, Fk[1 - l]);
-                        cmac(p22, Xn, Fk[2 - l]);
-                    }
+        for (int i = threadIdx.x; i < kTidLeaves * npair; i += blockDim.x) {
+            const int u = i / npair, r = i % npair;
+            if (s_end[u] == (u ? s_end[u - 1] : 0)) continue;
+            // r counts (l, k) with l <= k <= q, columns l one after another
+            int l = 0, b = 0;
+            while (r >= b + q + 1 - l) b += q + 1 - l++;
+            const int k = l + r - b;
+            const double* Fr = F + (size_t)s_cell[u] * nco;
+            const double sg = (l & 1) ? -1.0 : 1.0, sc = c_tid.sigma[l][k];
+            TidComb cb;
+#pragma unroll
+            for (int m = 0; m <= 2; ++m) {
+                const cd A = load_real_storage(Fr, k + 2, m + l);
+                cd Bq = mkc(0.0, 0.0);
+                if (l) Bq = load_real_storage(Fr, k + 2, m - l);
+                const cd B = mkc(sg * Bq.re, sg * Bq.im);
+                const cd a = mkc(sc * (A.re + B.re), sc * (A.im + B.im));  // of Y.re
+                const cd d = mkc(sc * (A.im - B.im), sc * (B.re - A.re));  // of Y.im: i (B - A)
+                if (m == 0) {
+                    cb.r0 = a.re;
+                    cb.i0 = d.re;
+                } else {
+                    cb.ar[m - 1] = a.re;
+                    cb.ai[m - 1] = a.im;
+                    cb.br[m - 1] = d.re;
+                    cb.bi[m - 1] = d.im;
                 }
             }
-            double* o = T + 6 * (size_t)(first + j);
-            o[0] = -0.5 * p20.re + 0.5 * p22.re;
-            o[1] = 0.5 * p22.im;
-            o[2] = p21.re;
-            o[3] = -0.5 * p20.re - 0.5 * p22.re;
-            o[4] = p21.im;
-            o[5] = p20.re;
+            comb_all[i] = cb;
+        }
+        __syncthreads();
+        const int total = s_end[kTidLeaves - 1];
+        for (int j = threadIdx.x; j < total; j += blockDim.x) {
+            int u = 0;
+            while (j >= s_end[u]) ++u;
+            const int cell = s_cell[u], at = c.first[cell] + j - (u ? s_end[u - 1] : 0);
+            const d4 s = cen[cell], xb = xm[at];
+            const double x = s.x - xb.x, y = s.y - xb.y, z = s.z - xb.z;
+            const double r2 = x * x + y * y + z * z;
+            double p20 = 0.0, r21 = 0.0, i21 = 0.0, r22 = 0.0, i22 = 0.0;
+            cd d = mkc(1.0, 0.0);
+            const TidComb* cb = comb_all + u * npair;
+            for (int l = 0; l <= q; ++l) {
+                if (l > 0) {
+                    const double sc = c_tid.inv2l[l], sx = sc * x, sy = sc * y;
+                    d = cd{sx * d.re - sy * d.im, sx * d.im + sy * d.re};
+                }
+                cd prev2 = mkc(0.0, 0.0), Y = d;
+                for (int k = l; k <= q; ++k, ++cb) {
+                    if (k > l) {
+                        const double b = r2 * c_tid.beta[l][k];
+                        const cd nx = cd{z * Y.re - b * prev2.re, z * Y.im - b * prev2.im};
+                        prev2 = Y;
+                        Y = nx;
+                    }
+                    p20 = fma(Y.re, cb->r0, fma(Y.im, cb->i0, p20));
+                    r21 = fma(Y.re, cb->ar[0], fma(Y.im, cb->br[0], r21));
+                    i21 = fma(Y.re, cb->ai[0], fma(Y.im, cb->bi[0], i21));
+                    r22 = fma(Y.re, cb->ar[1], fma(Y.im, cb->br[1], r22));
+                    i22 = fma(Y.re, cb->ai[1], fma(Y.im, cb->bi[1], i22));
+                }
+            }
+            double* o = T + 6 * (size_t)at;
+            o[0] = -0.5 * p20 + 0.5 * r22;
+            o[1] = 0.5 * i22;
+            o[2] = r21;
+            o[3] = -0.5 * p20 - 0.5 * r22;
+            o[4] = i21;
+            o[5] = p20;
         }
     }
 }
 
 void launch_l2p_tidal(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, const double* F,
                       double* T, cudaStream_t s) {
-    if (nleaves <= 0) return;  // (p < 2: the loops are empty and T_far = 0)
-    const size_t sm = sizeof(cd) * (size_t)ncoef(p);
-    const unsigned g = (unsigned)std::min<long long>(nleaves, (long long)sm_count() * 16);
+    if (nleaves <= 0) return;  // (p < 2: no terms and T_far = 0)
+    init_tid_tab();
+    const size_t sm = sizeof(TidComb) * (size_t)kTidLeaves * (p >= 2 ? (p - 1) * p / 2 : 0);
+    cudaFuncSetAttribute(k_l2p_tidal, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const unsigned g = grid_for(((long long)nleaves + kTidLeaves - 1) / kTidLeaves * kTidThreads, kTidThreads, 16);
     k_l2p_tidal<<<g, kTidThreads, sm, s>>>(xm, c, cen, leaves, nleaves, p, F, T);
     note_launch();
 }
 
-// near part: one warp per sink leaf, lane = sink (chunks of 32), the sources of the leaf's
+// near part without a work plan (FP64 mode; mixed mode where the planned form of p2p.cu has no room
+// for its scratch): one warp per sink leaf, lane = sink (chunks of 32), the sources of the leaf's
 // own P2P segment and of its ancestors' segments through shared-memory tiles of 32.
 // FP32 = true: dx from the two-float position records (hi + lo), FP32 pair terms, two-float sums
 // folded per tile; false: FP64 throughout.
