@@ -247,107 +247,7 @@ int sort_by_system(const uint64_t* keys, const int* idx, int n, const int* off, 
     return 0;
 }
 
-// ------------------------------------------------------------------ A2 radix sort
-// Stable LSD radix sort of (key, index) pairs, 8 bits per pass, 8 passes over the
-// 63 key bits (index arrays nullptr: the keys alone).  Per pass: a digit histogram per tile, a device-wide exclusive scan
-// in digit-major order, and a stable scatter that ranks equal digits inside the
-// tile in item order with warp match masks.
-constexpr int kRsThreads = 256;
-constexpr int kRsRounds = 16;
-constexpr int kRsTile = kRsThreads * kRsRounds;
-
-__global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint64_t* __restrict__ keys, int n, int shift,
-                                                        int* __restrict__ hist, int nblocks) {
-    __shared__ int h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    long long base = (long long)blockIdx.x * kRsTile;
-    for (int r = 0; r < kRsRounds; ++r) {
-        long long i = base + r * kRsThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255], 1);
-    }
-    __syncthreads();
-    hist[threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint64_t* __restrict__ kin,
-                                                           const int* __restrict__ vin,
-                                                           uint64_t* __restrict__ kout, int* __restrict__ vout,
-                                                           int n, int shift, const int* __restrict__ offs,
-                                                           int nblocks) {
-    __shared__ int running[256];
-    __shared__ int wc[kRsThreads / 32][256];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    running[threadIdx.x] = offs[threadIdx.x * nblocks + blockIdx.x];
-    long long base = (long long)blockIdx.x * kRsTile;
-    for (int r = 0; r < kRsRounds; ++r) {
-#pragma unroll
-        for (int k = 0; k < kRsThreads / 32; ++k) wc[k][threadIdx.x] = 0;
-        __syncthreads();
-        long long i = base + r * kRsThreads + threadIdx.x;
-        bool valid = i < n;
-        uint64_t key = valid ? kin[i] : 0;
-        int val = (valid && vin) ? vin[i] : 0;
-        int d = valid ? (int)((key >> shift) & 255) : 256;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        int rank = __popc(peers & ((1u << lane) - 1));
-        int leader = __ffs(peers) - 1;
-        if (valid && lane == leader) wc[w][d] = __popc(peers);
-        __syncthreads();
-        {   // per digit: exclusive prefix over the warps of this round
-            int dg = threadIdx.x;
-            int b = running[dg];
-#pragma unroll
-            for (int k = 0; k < kRsThreads / 32; ++k) {
-                int c = wc[k][dg];
-                wc[k][dg] = b;
-                b += c;
-            }
-            running[dg] = b;
-        }
-        __syncthreads();
-        if (valid) {
-            int dst = wc[w][d] + rank;
-            kout[dst] = key;
-            if (vout) vout[dst] = val;
-        }
-        __syncthreads();
-    }
-}
-
-size_t radix_tmp_ints(long long n) {
-    long long nb = (n + kRsTile - 1) / kRsTile;
-    if (nb < 1) nb = 1;
-    return (size_t)(2 * 256 * nb) + scan_tmp_ints(256 * nb) + 8;
-}
-
-int radix_sort_pairs_bits(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx_alt, long long n, int* tmp,
-                          int begin_bit, int end_bit, cudaStream_t s) {
-    if (n <= 1) return 0;
-    int nb = (int)((n + kRsTile - 1) / kRsTile);
-    int* hist = tmp;
-    int* offs = tmp + 256 * nb;
-    int* stmp = tmp + 2 * 256 * nb;
-    uint64_t *ka = keys, *kb = keys_alt;
-    int *va = idx, *vb = idx_alt;
-    int flips = 0;
-    for (int shift = begin_bit; shift < end_bit; shift += 8) {
-        k_rs_hist<<<nb, kRsThreads, 0, s>>>(ka, (int)n, shift, hist, nb); note_launch();
-        scan_exclusive_i32(hist, offs, 256LL * nb, nullptr, stmp, s);
-        k_rs_scatter<<<nb, kRsThreads, 0, s>>>(ka, va, kb, vb, (int)n, shift, offs, nb); note_launch();
-        uint64_t* tk = ka; ka = kb; kb = tk;
-        int* tv = va; va = vb; vb = tv;
-        flips ^= 1;
-    }
-    return flips;
-}
-
-void radix_sort_pairs(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx_alt, int n, int* tmp,
-                      cudaStream_t s) {
-    // 8 passes over the 63 key bits: the result is back in (keys, idx)
-    radix_sort_pairs_bits(keys, idx, keys_alt, idx_alt, n, tmp, 0, 64, s);
-}
-
+// ------------------------------------------------------------------ A2 gather (the sort: sort.cu)
 // e (nullable): the working units, positions times 2^-e[0] and masses times 2^-e[1]
 __global__ void k_gather(const double* __restrict__ x, const double* __restrict__ mu, const int* __restrict__ idx,
                          int n, d4* __restrict__ xm, int* __restrict__ perm, const int* __restrict__ e) {
