@@ -69,11 +69,11 @@ struct fmm_ctx {
     // host-API staging
     Buf hx, hmu, hpsi, hacc;
     // particles and sort
-    Buf bounds, status, counters, coin, dtotal;
+    Buf bounds, status, counters, coin;
     Buf keys, keys_alt, idx, idx_alt, rtmp, xm, perm, xp;
     // cells
     Buf first, count, child, nchild, parent, level, sr, cr, mass, minscale;
-    Buf split_nchild, split_oct, split_offs, scan_tmp, leaves, leaf_flag, leaf_pos, rad_tmp, owner;
+    Buf tree_tmp, shape, leaves, rad_tmp, owner;
     // expansions
     Buf M, F, Pw, binom, pascal, M1, F1, Ff;
     // walk
@@ -112,10 +112,9 @@ struct fmm_ctx {
     // of tree_n particles that completed
     int tree_n = -1;
     std::vector<Buf*> bufs() {
-        return {&hx, &hmu, &hpsi, &hacc, &bounds, &status, &counters, &coin, &dtotal, &keys, &keys_alt, &idx,
+        return {&hx, &hmu, &hpsi, &hacc, &bounds, &status, &counters, &coin, &keys, &keys_alt, &idx,
                 &idx_alt, &rtmp, &xm, &perm, &xp, &first, &count, &child, &nchild, &parent, &level, &sr,
-                &cr, &mass, &minscale, &split_nchild, &split_oct, &split_offs, &scan_tmp, &leaves, &leaf_flag,
-                &leaf_pos, &rad_tmp, &M, &F, &Pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
+                &cr, &mass, &minscale, &tree_tmp, &shape, &leaves, &rad_tmp, &M, &F, &Pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
                 &sort_tmp, &sort_tmp2, &m2l_tmp, &p2p_tmp, &seg_start, &seg_end, &est_m2l, &est_p2p, &m2l_seg_start,
                 &m2l_seg_end, &psi_far, &acc_far, &psi_near, &acc_near, &scale_sorted, &sys_off, &sys_G,
                 &sys_roots, &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
@@ -185,48 +184,15 @@ static int check_params(const fmm_params* p) {
 }
 
 // ------------------------------------------------------------------ tree (A1-A4)
-__global__ void k_root(Cells c, int n) {
-    c.first[0] = 0;
-    c.count[0] = n;
-    c.level[0] = 0;
-    c.parent[0] = -1;
-    c.child[0] = -1;
-    c.nchild[0] = 0;
-}
-// one root per non-empty system of an ensemble (roots[r] = first, count)
-__global__ void k_roots(Cells c, const int2* __restrict__ roots, int nroots) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nroots; r += gridDim.x * blockDim.x) {
-        c.first[r] = roots[r].x;
-        c.count[r] = roots[r].y;
-        c.level[r] = 0;
-        c.parent[r] = -1;
-        c.child[r] = -1;
-        c.nchild[r] = 0;
-    }
-}
-__global__ void k_leaf_flags(const int* __restrict__ nchild, int nc, int* __restrict__ flag) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) flag[i] = nchild[i] == 0;
-}
-__global__ void k_leaf_compact(const int* __restrict__ flag, const int* __restrict__ pos, int nc, int* __restrict__ leaves) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x)
-        if (flag[i]) leaves[pos[i]] = i;
-}
-
-// the two-float records of the sorted positions and masses (the internal radii's
-// single-precision bounds, the mixed-mode kernels)
-static int split_positions(fmm_ctx* ctx, int n, cudaStream_t s) {
-    TRY(ensure(ctx->xp, 2 * sizeof(float4) * (size_t)n));
-    launch_split_positions(P<d4>(ctx->xm), n, P<float4>(ctx->xp), s);
-    return 0;
-}
-
 // Sec. 7.1's re-cycled tree: the previous evaluation's particle order, cells and centres
 // stay; positions and masses are gathered in that order and the radii, masses and
 // centres of mass are recomputed, so the MAC sees the true extent of every cell
 static int refresh_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, cudaStream_t s) {
     launch_bounds(x, mu, n, P<unsigned long long>(ctx->bounds), P<unsigned>(ctx->status), s);
     // the tree's centres are in the working units it was built in: keep them
-    launch_gather(x, mu, P<int>(ctx->perm), n, P<d4>(ctx->xm), P<int>(ctx->perm), s, P<int>(ctx->units));
+    TRY(ensure(ctx->xp, 2 * sizeof(float4) * (size_t)n));
+    launch_gather(x, mu, P<int>(ctx->perm), n, P<d4>(ctx->xm), P<int>(ctx->perm), s, P<int>(ctx->units),
+                  P<float4>(ctx->xp));
     unsigned st = 0;
     CU(cudaMemcpyAsync(&ctx->h_int[0], ctx->status.p, sizeof st, cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
@@ -234,7 +200,6 @@ static int refresh_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, 
     if (st & kStatInvalid) return fail(ctx, FMM_E_INVALID, "non-finite position or mass, or negative mass");
     Cells c = cells_of(ctx);
     const int nlev = (int)ctx->lev_start.size() - 1;
-    TRY(split_positions(ctx, n, s));
     TRY(ensure(ctx->owner, sizeof(int) * (size_t)n));
     launch_leaf_geometry(P<d4>(ctx->xm), c, P<int>(ctx->leaves), ctx->nleaves, P<unsigned>(ctx->status), s, true);
     launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
@@ -282,64 +247,41 @@ static int build_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, cu
     TRY(ensure(ctx->units, 2 * sizeof(int)));
     if (ctx->prm.precision == FMM_PREC_MIXED) launch_work_units(P<unsigned long long>(ctx->bounds), nsys, P<int>(ctx->units), s);
     else CU(cudaMemsetAsync(ctx->units.p, 0, 2 * sizeof(int), s));
-    launch_gather(x, mu, P<int>(ctx->idx), n, P<d4>(ctx->xm), P<int>(ctx->perm), s, P<int>(ctx->units));
+    TRY(ensure(ctx->xp, 2 * sizeof(float4) * (size_t)n));
+    launch_gather(x, mu, P<int>(ctx->idx), n, P<d4>(ctx->xm), P<int>(ctx->perm), s, P<int>(ctx->units),
+                  P<float4>(ctx->xp));
 
     // cell capacity: leaves <= n, internal cells hold > leaf particles, <= 21 levels
     const int nroots = ctx->nroots;
-    long long cap = (long long)n + 21LL * (n / (leaf + 1)) + nroots + 64;
+    const long long cap = std::min<long long>((long long)n + 21LL * (n / (leaf + 1)) + nroots + 64, 0x7fffffffLL);
     Buf* ib[] = {&ctx->first, &ctx->count, &ctx->child, &ctx->nchild, &ctx->parent, &ctx->level};
     for (Buf* b : ib) TRY(ensure(*b, sizeof(int) * cap));
     TRY(ensure(ctx->sr, sizeof(d4) * cap));
     TRY(ensure(ctx->cr, sizeof(d4) * cap));
     TRY(ensure(ctx->mass, sizeof(double) * cap));
     TRY(ensure(ctx->minscale, sizeof(double) * cap));
+    TRY(ensure(ctx->leaves, sizeof(int) * (size_t)n));
+    TRY(ensure(ctx->tree_tmp, sizeof(int) * tree_tmp_ints(n)));
     Cells c = cells_of(ctx);
-    if (nsys == 0) {
-        k_root<<<1, 1, 0, s>>>(c, n); note_launch();
-    } else {
-        k_roots<<<grid_for(nroots, 256), 256, 0, s>>>(c, P<int2>(ctx->sys_roots), nroots); note_launch();
-    }
-    ctx->lev_start.assign({0, nroots});
-    for (int L = 0;; ++L) {
-        int b = ctx->lev_start[L], e = ctx->lev_start[L + 1];
-        int ncl = e - b;
-        if (ncl <= 0) break;
-        TRY(ensure(ctx->split_nchild, sizeof(int) * ncl));
-        TRY(ensure(ctx->split_oct, sizeof(int) * 9 * (size_t)ncl));
-        TRY(ensure(ctx->split_offs, sizeof(int) * ncl));
-        TRY(ensure(ctx->scan_tmp, sizeof(int) * scan_tmp_ints(std::max<long long>(ncl, cap))));
-        launch_split_level(P<uint64_t>(ctx->keys), c, b, e, L, leaf, P<int>(ctx->split_nchild), P<int>(ctx->split_oct),
-                           P<int>(ctx->split_offs), P<int>(ctx->scan_tmp), P<int>(ctx->dtotal), s);
-        CU(cudaMemcpyAsync(ctx->h_int, ctx->dtotal.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CU(cudaStreamSynchronize(s));
-        int tot = ctx->h_int[0];
-        if (tot <= 0) break;
-        if ((long long)e + tot > cap) return fail(ctx, FMM_E_OVERFLOW, "cell capacity exceeded");
-        ctx->lev_start.push_back(e + tot);
-    }
-    int nc = ctx->lev_start.back();
-    ctx->ncells = nc;
-    // leaves
-    TRY(ensure(ctx->leaf_flag, sizeof(int) * nc));
-    TRY(ensure(ctx->leaf_pos, sizeof(int) * nc));
-    TRY(ensure(ctx->leaves, sizeof(int) * nc));
-    TRY(ensure(ctx->scan_tmp, sizeof(int) * scan_tmp_ints(nc)));
-    k_leaf_flags<<<grid_for(nc, 256), 256, 0, s>>>(c.nchild, nc, P<int>(ctx->leaf_flag)); note_launch();
-    scan_exclusive_i32(P<int>(ctx->leaf_flag), P<int>(ctx->leaf_pos), nc, P<int>(ctx->dtotal), P<int>(ctx->scan_tmp), s);
-    k_leaf_compact<<<grid_for(nc, 256), 256, 0, s>>>(P<int>(ctx->leaf_flag), P<int>(ctx->leaf_pos), nc, P<int>(ctx->leaves)); note_launch();
-    CU(cudaMemcpyAsync(ctx->h_int, ctx->dtotal.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    launch_tree(P<uint64_t>(ctx->keys), c, n, leaf, (int)cap, nsys ? P<int>(ctx->sys_off) : nullptr, nsys,
+                P<int>(ctx->leaves), P<int>(ctx->tree_tmp), P<int>(ctx->shape), s);
+    CU(cudaMemcpyAsync(ctx->h_int, ctx->shape.p, sizeof(int) * kTreeShapeInts, cudaMemcpyDeviceToHost, s));
+    CU(cudaMemcpyAsync(ctx->h_int + kTreeShapeInts, ctx->status.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    ctx->nleaves = ctx->h_int[0];
-    unsigned st = 0;
-    CU(cudaMemcpy(&st, ctx->status.p, sizeof st, cudaMemcpyDeviceToHost));
-    if (st & kStatInvalid) return fail(ctx, FMM_E_INVALID, "non-finite position or mass, or negative mass");
+    if ((unsigned)ctx->h_int[kTreeShapeInts] & kStatInvalid)
+        return fail(ctx, FMM_E_INVALID, "non-finite position or mass, or negative mass");
+    const int nc = ctx->h_int[kMaxLevel + 1];
+    if (nc > cap) return fail(ctx, FMM_E_OVERFLOW, "cell capacity exceeded");
+    ctx->lev_start.assign(1, 0);
+    for (int L = 1; L <= kMaxLevel + 1 && ctx->lev_start.back() < nc; ++L) ctx->lev_start.push_back(ctx->h_int[L]);
+    ctx->ncells = nc;
+    ctx->nleaves = ctx->h_int[23];
 
     // geometry: leaves, then internal cells bottom-up
     int nlev = (int)ctx->lev_start.size() - 1;
     int maxlev_cells = 0;
     for (int L = 0; L < nlev; ++L) maxlev_cells = std::max(maxlev_cells, ctx->lev_start[L + 1] - ctx->lev_start[L]);
     TRY(ensure(ctx->rad_tmp, sizeof(unsigned long long) * rad_tmp_u64_per_cell() * (size_t)maxlev_cells));
-    TRY(split_positions(ctx, n, s));
     TRY(ensure(ctx->owner, sizeof(int) * (size_t)n));
     launch_leaf_geometry(P<d4>(ctx->xm), c, P<int>(ctx->leaves), ctx->nleaves, P<unsigned>(ctx->status), s);
     launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
@@ -904,9 +846,9 @@ int fmm_create(fmm_ctx** out, const fmm_params* params, int device) {
     if (!rc) rc = ensure(ctx->status, 16);
     if (!rc) rc = ensure(ctx->counters, 8 * sizeof(unsigned long long));
     if (!rc) rc = ensure(ctx->coin, 16);
-    if (!rc) rc = ensure(ctx->dtotal, 16);
+    if (!rc) rc = ensure(ctx->shape, kTreeShapeInts * sizeof(int));
     if (!rc && cudaMallocHost((void**)&ctx->h_counters, 16 * sizeof(unsigned long long)) != cudaSuccess) rc = FMM_E_OOM;
-    if (!rc && cudaMallocHost((void**)&ctx->h_int, 16 * sizeof(int)) != cudaSuccess) rc = FMM_E_OOM;
+    if (!rc && cudaMallocHost((void**)&ctx->h_int, (kTreeShapeInts + 1) * sizeof(int)) != cudaSuccess) rc = FMM_E_OOM;
     if (!rc) {
         ctx->ev_ok = true;
         for (int i = 0; i < EV_N; ++i)

@@ -689,26 +689,7 @@ void launch_p2p_fp64(const d4* xm, Cells c, const int2* list, const int* seg_sta
     note_launch();
 }
 
-// ---------------------------------------------------------------- P2P, mixed
-// Positions as two floats (hi + lo, exact to 2^-48 relative), so that
-// dx = (hi_a - hi_b) + (lo_a - lo_b) keeps its relative accuracy even for close
-// pairs.  Pair terms are FP32; the FP32 sums of every ~32 pairs are added to
-// two-float accumulators (TwoSum), so the sum over tiles is compensated.
-// Layout: one 32-byte record per particle, xp[2i] = (high parts of the position, mass as
-// FP32), xp[2i + 1] = (low parts, 0), so that a range of particles is one contiguous block.
-__global__ void k_split_positions(const d4* __restrict__ xm, int n, float4* __restrict__ xp) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        d4 v = xm[i];
-        const float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
-        xp[2 * (size_t)i] = make_float4(hx, hy, hz, (float)v.w);
-        xp[2 * (size_t)i + 1] =
-            make_float4((float)(v.x - (double)hx), (float)(v.y - (double)hy), (float)(v.z - (double)hz), 0.f);
-    }
-}
-void launch_split_positions(const d4* xm, int n, float4* xp, cudaStream_t s) {
-    if (n > 0) k_split_positions<<<grid_for(n, 256), 256, 0, s>>>(xm, n, xp); note_launch();
-}
-
+// ---------------------------------------------------------------- coincident pairs
 // number of ordered pairs (a != b) at distance 0: equal positions have equal keys,
 // so they sit next to each other in key order inside one leaf
 __global__ void k_coincident(const d4* __restrict__ xm, const uint64_t* __restrict__ keys, int n,

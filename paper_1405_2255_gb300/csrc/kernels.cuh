@@ -47,8 +47,10 @@ int radix_sort_pairs_bits(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx
 void radix_sort_pairs(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx_alt, int n, int* tmp,
                       cudaStream_t s);
 // e (nullable, device): positions enter scaled by 2^-e[0], masses by 2^-e[1] (launch_work_units)
+// xp: their two-float records, 32 bytes per particle: xp[2i] = (hi x, hi y, hi z, mass), xp[2i + 1] =
+// (lo x, lo y, lo z, 0) with hi = fl32(x) and lo = fl32(x - hi)
 void launch_gather(const double* x, const double* mu, const int* idx, int n, d4* xm, int* perm,
-                   cudaStream_t s, const int* e = nullptr);
+                   cudaStream_t s, const int* e, float4* xp);
 // working units of the mixed-precision path: e[0] = floor(log2 extent), e[1] = floor(log2 max mass)
 // from the bounds of launch_bounds (nsys = 0; the largest mass in bounds[6]) or
 // launch_bounds_sys (the largest mass in bounds[6 nsys])
@@ -64,12 +66,14 @@ void launch_keys_sys(const double* x, int n, const int* off, int nsys, const uns
 int sort_by_system(const uint64_t* keys, const int* idx, int n, const int* off, int nsys, uint64_t* skey,
                    uint64_t* skey_alt, int* pos, int* pos_alt, int* tmp, uint64_t* keys_out, int* idx_out,
                    cudaStream_t s);
-// A3: one level of the top-down build.  Cells [lev_begin, lev_end) are split;
-// nchild_tmp/oct_tmp are scratch of the level's size.  Daughters are appended at
-// lev_end; *d_total receives their number.
-void launch_split_level(const uint64_t* keys, Cells c, int lev_begin, int lev_end, int level, int leaf_size,
-                        int* nchild_tmp, int* oct_tmp, int* offs_tmp, int* scan_tmp, int* d_total,
-                        cudaStream_t s);
+// A3: the oct-tree of the sorted keys (off, nsys: the systems of an ensemble, else nullptr, 0): first,
+// count, child, nchild, parent and level of at most cap cells, leaves (the leaf cells in cell order;
+// at most n), tmp: tree_tmp_ints(n) ints.  shape (device, kTreeShapeInts ints): [0 .. 22] the first cell
+// of every level and the number of cells, [23] the number of leaves, [24 + l] the largest cell of level l
+constexpr int kTreeShapeInts = 24 + kMaxLevel + 1;
+size_t tree_tmp_ints(int n);
+void launch_tree(const uint64_t* keys, Cells c, int n, int leaf_size, int cap, const int* off, int nsys, int* leaves,
+                 int* tmp, int* shape, cudaStream_t s);
 // A4: geometry.  Leaves: smallest enclosing ball of the particles, rho, mass,
 // centre of mass.  Internal cells of one level: smallest ball of the daughter balls,
 // mass and centre of mass from the daughters, then the exact radii over particles.
@@ -77,7 +81,7 @@ void launch_split_level(const uint64_t* keys, Cells c, int lev_begin, int lev_en
 // radii, masses and centres of mass for the particles' new positions
 void launch_leaf_geometry(const d4* xm, Cells c, const int* leaves, int nleaves, unsigned* status,
                           cudaStream_t s, bool keep_centre = false);
-// xp: the two-float position records (launch_split_positions); owner: per particle, set by
+// xp: the two-float position records (launch_gather); owner: per particle, set by
 // launch_leaf_owner before the deepest level and moved up as the levels are processed
 // bottom-up; rad_tmp: rad_tmp_u64_per_cell() words per cell of the largest level
 void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_begin, int lev_end,
@@ -245,9 +249,6 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
 // an ensemble (off != nullptr) only pairs inside one system count
 void launch_coincident(const d4* xm, const uint64_t* keys, int n, unsigned long long* coincident, cudaStream_t s,
                        const int* off = nullptr, int nsys = 0);
-// two-float position records, 32 bytes per particle: xp[2i] = (hi x, hi y, hi z, mass),
-// xp[2i + 1] = (lo x, lo y, lo z, 0) with hi = fl32(x) and lo = fl32(x - hi)
-void launch_split_positions(const d4* xm, int n, float4* xp, cudaStream_t s);
 // low-order f estimate (p = 0, 1/r^2 kernel): M2L, pass-down, P2P, evaluation
 void launch_f_m2l(const int2* list, const int* seg_start, const int* seg_end, int ncells, Cells c, double* Ff,
                   cudaStream_t s);

@@ -81,23 +81,6 @@ int scratch_for_current_device(void** out) {
     return 0;
 }
 
-__global__ void k_root_na(Cells c, int n) {
-    c.first[0] = 0;
-    c.count[0] = n;
-    c.level[0] = 0;
-    c.parent[0] = -1;
-    c.child[0] = -1;
-    c.nchild[0] = 0;
-}
-__global__ void k_leaf_flags_na(const int* __restrict__ nchild, int nc, int* __restrict__ flag) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) flag[i] = nchild[i] == 0;
-}
-__global__ void k_leaf_compact_na(const int* __restrict__ flag, const int* __restrict__ pos, int nc,
-                                  int* __restrict__ leaves) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x)
-        if (flag[i]) leaves[pos[i]] = i;
-}
-
 struct Run {
     Arena a;
     cudaStream_t s;
@@ -111,7 +94,6 @@ struct Run {
     int* leaves = nullptr;
     unsigned long long* counters = nullptr;
     unsigned* status = nullptr;
-    int* dtotal = nullptr;
     int2 *front0 = nullptr, *front1 = nullptr;
     void* sort_tmp = nullptr;
     void* p2p_tmp = nullptr;
@@ -198,7 +180,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     unsigned long long* bounds = A.take<unsigned long long>(8);
     r.status = A.take<unsigned>(4);
     r.counters = A.take<unsigned long long>(8);
-    r.dtotal = A.take<int>(4);
+    int* shape = A.take<int>(kTreeShapeInts);
     const long long cap = (long long)n + 21LL * (n / (prm.leaf_size + 1)) + 64;
     int* ib[6];
     for (int k = 0; k < 6; ++k) ib[k] = A.take<int>(cap);
@@ -207,10 +189,9 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     r.c.cr = A.take<d4>(cap);
     r.c.mass = A.take<double>(cap);
     r.c.minscale = A.take<double>(cap);
-    int* split_nchild = A.take<int>(cap);
-    int* split_oct = A.take<int>(9 * cap);
-    int* split_offs = A.take<int>(cap);
-    int* scan_tmp = A.take<int>(scan_tmp_ints(cap));
+    r.leaves = A.take<int>(n);
+    int* tree_tmp = A.take<int>(tree_tmp_ints(n));
+    float4* xp = A.take<float4>(2 * (size_t)n);  // two records per particle: hi and mass, lo
     if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the particle arrays");
     NA_CU(cudaMemsetAsync(r.status, 0, sizeof(unsigned), s));
     // working units of the mixed path (positions and masses scaled by powers of two)
@@ -221,49 +202,28 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     else NA_CU(cudaMemsetAsync(units, 0, 2 * sizeof(int), s));
     launch_keys(x, n, bounds, r.keys, idx, s);
     radix_sort_pairs(r.keys, idx, keys_alt, idx_alt, n, rtmp, s);
-    launch_gather(x, mu, idx, n, r.xm, r.perm, s, units);
-    k_root_na<<<1, 1, 0, s>>>(r.c, n);
-    note_launch();
-    // top-down levels
-    r.lev[0] = 0;
-    r.lev[1] = 1;
-    int nl = 1;
-    for (int L = 0;; ++L) {
-        int b = r.lev[L], e = r.lev[L + 1];
-        if (e - b <= 0) break;
-        launch_split_level(r.keys, r.c, b, e, L, prm.leaf_size, split_nchild, split_oct, split_offs, scan_tmp,
-                           r.dtotal, s);
-        int tot = 0;
-        NA_CU(cudaMemcpyAsync(&tot, r.dtotal, sizeof tot, cudaMemcpyDeviceToHost, s));
-        NA_CU(cudaStreamSynchronize(s));
-        if (tot <= 0) break;
-        if ((long long)e + tot > cap || nl + 1 > kMaxLevels) return fail_na(r, FMM_E_OVERFLOW, "cell capacity exceeded");
-        r.lev[++nl] = e + tot;
-    }
-    r.nlev = nl;
-    r.nc = r.lev[nl];
-    const int nc = r.nc;
-    int* leaf_flag = A.take<int>(nc);
-    int* leaf_pos = A.take<int>(nc);
-    r.leaves = A.take<int>(nc);
-    unsigned long long* rad_tmp = A.take<unsigned long long>(rad_tmp_u64_per_cell() * (size_t)nc);
-    if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the tree");
-    k_leaf_flags_na<<<grid_for(nc, 256), 256, 0, s>>>(r.c.nchild, nc, leaf_flag);
-    note_launch();
-    scan_exclusive_i32(leaf_flag, leaf_pos, nc, r.dtotal, scan_tmp, s);
-    k_leaf_compact_na<<<grid_for(nc, 256), 256, 0, s>>>(leaf_flag, leaf_pos, nc, r.leaves);
-    note_launch();
+    launch_gather(x, mu, idx, n, r.xm, r.perm, s, units, xp);
+    launch_tree(r.keys, r.c, n, prm.leaf_size, (int)cap, nullptr, 0, r.leaves, tree_tmp, shape, s);
+    int h_shape[kTreeShapeInts];
     unsigned st = 0;
-    NA_CU(cudaMemcpyAsync(&r.nleaves, r.dtotal, sizeof(int), cudaMemcpyDeviceToHost, s));
+    NA_CU(cudaMemcpyAsync(h_shape, shape, sizeof h_shape, cudaMemcpyDeviceToHost, s));
     NA_CU(cudaMemcpyAsync(&st, r.status, sizeof st, cudaMemcpyDeviceToHost, s));
     NA_CU(cudaStreamSynchronize(s));
     if (st & kStatInvalid) return fail_na(r, FMM_E_INVALID, "non-finite position or mass, or negative mass");
-    // two-float positions: the internal radii's single-precision bounds and the mixed P2P
-    float4* xp = A.take<float4>(2 * (size_t)n);  // two records per particle: hi and mass, lo
+    const int nc = r.nc = h_shape[kMaxLevel + 1];
+    if (nc > cap) return fail_na(r, FMM_E_OVERFLOW, "cell capacity exceeded");
+    r.nleaves = h_shape[23];
+    r.lev[0] = 0;
+    int nl = 0;
+    while (r.lev[nl] < nc) {
+        ++nl;
+        r.lev[nl] = h_shape[nl];
+    }
+    r.nlev = nl;
+    unsigned long long* rad_tmp = A.take<unsigned long long>(rad_tmp_u64_per_cell() * (size_t)nc);
     if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the tree");
     int* owner = A.take<int>(n);
     if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the tree");
-    launch_split_positions(r.xm, n, xp, s);
     launch_leaf_geometry(r.xm, r.c, r.leaves, r.nleaves, r.status, s);
     launch_leaf_owner(r.c, r.leaves, r.nleaves, owner, s);
     for (int L = nl - 1; L >= 0; --L)

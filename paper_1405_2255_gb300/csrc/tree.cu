@@ -248,20 +248,28 @@ int sort_by_system(const uint64_t* keys, const int* idx, int n, const int* off, 
 }
 
 // ------------------------------------------------------------------ A2 gather (the sort: sort.cu)
-// e (nullable): the working units, positions times 2^-e[0] and masses times 2^-e[1]
+// e (nullable): the working units, positions times 2^-e[0] and masses times 2^-e[1]; with the sorted
+// positions their two-float records (hi + lo = x to 2^-48, the mass as FP32), one 32-byte block per
+// particle, so that a range of particles is contiguous
 __global__ void k_gather(const double* __restrict__ x, const double* __restrict__ mu, const int* __restrict__ idx,
-                         int n, d4* __restrict__ xm, int* __restrict__ perm, const int* __restrict__ e) {
+                         int n, d4* __restrict__ xm, int* __restrict__ perm, const int* __restrict__ e,
+                         float4* __restrict__ xp) {
     const double fx = e ? pow2i(-e[0]) : 1.0, fm = e ? pow2i(-e[1]) : 1.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         int j = idx[i];
-        xm[i] = mk4(x[3 * (long long)j] * fx, x[3 * (long long)j + 1] * fx, x[3 * (long long)j + 2] * fx, mu[j] * fm);
+        const d4 v = mk4(x[3 * (long long)j] * fx, x[3 * (long long)j + 1] * fx, x[3 * (long long)j + 2] * fx, mu[j] * fm);
+        xm[i] = v;
         perm[i] = j;
+        const float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
+        xp[2 * (size_t)i] = make_float4(hx, hy, hz, (float)v.w);
+        xp[2 * (size_t)i + 1] =
+            make_float4((float)(v.x - (double)hx), (float)(v.y - (double)hy), (float)(v.z - (double)hz), 0.f);
     }
 }
 
 void launch_gather(const double* x, const double* mu, const int* idx, int n, d4* xm, int* perm,
-                   cudaStream_t s, const int* e) {
-    if (n > 0) k_gather<<<grid_for(n, 256), 256, 0, s>>>(x, mu, idx, n, xm, perm, e); note_launch();
+                   cudaStream_t s, const int* e, float4* xp) {
+    if (n > 0) k_gather<<<grid_for(n, 256), 256, 0, s>>>(x, mu, idx, n, xm, perm, e, xp); note_launch();
 }
 
 // The mixed-precision path works in units in which the system's extent and its largest mass
@@ -289,69 +297,208 @@ void launch_work_units(const unsigned long long* bounds, int nsys, int* e, cudaS
 }
 
 // ------------------------------------------------------------------ A3 oct-tree
-// A cell of level L holding more than leaf_size particles (and L < 21) is split
-// into its non-empty octants, in key order.  One warp per cell; lane o < 8 finds
-// the first particle whose level-(L+1) digit is >= o by binary search.
-__global__ void k_split(const uint64_t* __restrict__ keys, Cells c, int lev_begin, int lev_end, int level,
-                        int leaf_size, int* __restrict__ nchild_tmp, int* __restrict__ oct_tmp) {
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    int cell = lev_begin + warp;
-    if (cell >= lev_end) return;
-    int first = c.first[cell], count = c.count[cell];
-    bool split = count > leaf_size && level < kMaxLevel;
-    int b = first + count;
-    if (split && lane < 8) {
-        int shift = 3 * (kMaxLevel - (level + 1));
-        int lo = first, hi = first + count;
-        while (lo < hi) {
-            int mid = (lo + hi) >> 1;
-            int dg = (int)((keys[mid] >> shift) & 7);
-            if (dg < lane) lo = mid + 1;
-            else hi = mid;
-        }
-        b = lo;
-    }
-    int bnext = __shfl_down_sync(0xffffffffu, b, 1);
-    int size = (lane < 8) ? ((lane == 7 ? first + count : bnext) - b) : 0;
-    unsigned nonempty = __ballot_sync(0xffffffffu, split && lane < 8 && size > 0);
-    if (lane < 8) oct_tmp[9 * (long long)warp + lane] = b;
-    if (lane == 8) oct_tmp[9 * (long long)warp + 8] = first + count;
-    if (lane == 0) nchild_tmp[warp] = split ? __popc(nonempty) : 0;
+// A cell of level L holding more than leaf_size particles (and L < 21) is split into its non-empty
+// octants, in key order; cells are numbered level by level, each level in key order.  The sorted keys
+// give all levels at once: with c(f) the number of leading octal digits that particle f shares with
+// f - 1 (-1 at the start of its system), f is the first particle of a group of every level l > c(f), and
+// that group is a cell iff the group of level l - 1 around f holds more than leaf_size particles.  For
+// l > c(f) + 1 that group starts at f too, so it does iff f and f + leaf_size share l - 1 digits; only
+// l = c(f) + 1 needs the group around f.  Hence the cells that start at f are those of the levels
+// c(f) + 1 .. top(f), and the one of level top(f) is a leaf.
+// Three kernels and a scan whatever the depth, and one read by the host (a launch chain and a host
+// read per level took 0.30 ms of the 10 levels of a 1e4 Plummer sphere's tree).
+constexpr int kTreeThreads = 256;
+constexpr int kTreeTile = 1024;  // particles per block
+constexpr int kTreeLevels = kMaxLevel + 1;
+
+__device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b) {
+    const uint64_t d = a ^ b;
+    return d ? (__clzll((long long)d) - 1) / 3 : kMaxLevel;
 }
 
-__global__ void k_write_children(Cells c, int lev_begin, int lev_end, int level, const int* __restrict__ nchild_tmp,
-                                 const int* __restrict__ oct_tmp, const int* __restrict__ offs) {
-    int w = blockIdx.x * blockDim.x + threadIdx.x;
-    int cell = lev_begin + w;
-    if (cell >= lev_end) return;
-    int nc = nchild_tmp[w];
-    int base = lev_end + offs[w];
-    c.nchild[cell] = nc;
-    c.child[cell] = nc ? base : -1;
-    if (!nc) return;
-    int k = 0;
-    for (int o = 0; o < 8; ++o) {
-        int b0 = oct_tmp[9 * (long long)w + o], b1 = oct_tmp[9 * (long long)w + o + 1];
-        if (b1 > b0) {
-            int d = base + k++;
-            c.first[d] = b0;
-            c.count[d] = b1 - b0;
-            c.level[d] = level + 1;
-            c.parent[d] = cell;
-            c.nchild[d] = 0;
-            c.child[d] = -1;
+// levels lo .. hi of the cells that start at particle f (none: lo > hi), [sb, se) its system
+__device__ inline void cell_levels(const uint64_t* __restrict__ keys, int f, int sb, int se, int leaf, int& lo, int& hi) {
+    const uint64_t k = keys[f];
+    const int c = f > sb ? shared_digits(keys[f - 1], k) : -1;
+    const int S = f + leaf < se ? shared_digits(k, keys[f + leaf]) : -1;
+    lo = c + 1;
+    if (lo > kMaxLevel) {  // a copy of the particle before it
+        hi = lo - 1;
+        return;
+    }
+    if (c < 0 || S >= lo) {
+        hi = min(S + 1, kMaxLevel);
+        return;
+    }
+    // one cell at most, of level c + 1: is the group of level c around f larger than leaf?
+    bool big = f - leaf >= sb && shared_digits(keys[f - leaf], k) >= c;
+    if (!big) {
+        int a = max(sb, f - leaf), b = f - 1;  // first particle of the group: b shares c digits
+        while (a < b) {
+            const int m = (a + b) >> 1;
+            if (shared_digits(keys[m], k) >= c) b = m;
+            else a = m + 1;
+        }
+        big = a + leaf < se && shared_digits(keys[a + leaf], k) >= c;
+    }
+    hi = big ? lo : lo - 1;
+}
+__device__ inline void system_range(const int* __restrict__ off, int nsys, int n, int i, int& sb, int& se) {
+    sb = 0;
+    se = n;
+    if (off) {
+        const int k = system_of(off, nsys, i);
+        sb = off[k];
+        se = off[k + 1];
+    }
+}
+
+// cnt[l * nb + block]: the block's cells of level l; cnt[(22 + l) * nb + block]: its leaves of level l
+__global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __restrict__ keys, int n, int leaf,
+                                                             const int* __restrict__ off, int nsys, int nb,
+                                                             int* __restrict__ cnt) {
+    __shared__ int h[2 * kTreeLevels];
+    if (threadIdx.x < 2 * kTreeLevels) h[threadIdx.x] = 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < kTreeTile; j += kTreeThreads) {
+        const long long f = (long long)blockIdx.x * kTreeTile + j;
+        if (f >= n) break;
+        int sb, se, lo, hi;
+        system_range(off, nsys, n, (int)f, sb, se);
+        cell_levels(keys, (int)f, sb, se, leaf, lo, hi);
+        for (int l = lo; l <= hi; ++l) atomicAdd(&h[l], 1);
+        if (hi >= lo) atomicAdd(&h[kTreeLevels + hi], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * kTreeLevels) cnt[(size_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
+}
+
+// first, level and leaves from the scanned counts (at[0]: cells, at[22 nb]: the number of cells, from
+// which the leaves' positions count on)
+__global__ void __launch_bounds__(kTreeThreads) k_tree_cells(const uint64_t* __restrict__ keys, int n, int leaf,
+                                                             const int* __restrict__ off, int nsys, int nb,
+                                                             const int* __restrict__ at, int cap, Cells c,
+                                                             int* __restrict__ leaves) {
+    __shared__ int base[2 * kTreeLevels], wcnt[kTreeThreads / 32][2 * kTreeLevels];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ncells = at[(size_t)kTreeLevels * nb];
+    if (threadIdx.x < 2 * kTreeLevels)
+        base[threadIdx.x] = at[(size_t)threadIdx.x * nb + blockIdx.x] - (threadIdx.x >= kTreeLevels ? ncells : 0);
+    for (int j0 = 0; j0 < kTreeTile; j0 += kTreeThreads) {
+        const long long f = (long long)blockIdx.x * kTreeTile + j0 + threadIdx.x;
+        int sb, se, lo = 1, hi = 0;
+        if (f < n) {
+            system_range(off, nsys, n, (int)f, sb, se);
+            cell_levels(keys, (int)f, sb, se, leaf, lo, hi);
+        }
+        const bool any = hi >= lo;
+        unsigned present = any ? (2u << hi) - (1u << lo) : 0u;  // bit l: a cell of level l starts here
+        unsigned wall = present;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wall |= __shfl_xor_sync(0xffffffffu, wall, o);
+        // the lanes' ranks per level, then the warps'
+        for (int i = lane; i < 2 * kTreeLevels; i += 32) wcnt[w][i] = 0;
+        __syncwarp();
+        for (unsigned m = wall; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const unsigned bc = __ballot_sync(0xffffffffu, (present >> l) & 1);
+            const unsigned bl = __ballot_sync(0xffffffffu, any && hi == l);
+            if (lane == 0) {
+                wcnt[w][l] = __popc(bc);
+                wcnt[w][kTreeLevels + l] = __popc(bl);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < 2 * kTreeLevels) {
+            int run = base[threadIdx.x];
+            for (int k = 0; k < kTreeThreads / 32; ++k) {
+                const int v = wcnt[k][threadIdx.x];
+                wcnt[k][threadIdx.x] = run;
+                run += v;
+            }
+            base[threadIdx.x] = run;
+        }
+        __syncthreads();
+        for (unsigned m = wall; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const unsigned bc = __ballot_sync(0xffffffffu, (present >> l) & 1);
+            const unsigned bl = __ballot_sync(0xffffffffu, any && hi == l);
+            const unsigned below = (1u << lane) - 1u;
+            if ((present >> l) & 1) {
+                const int i = wcnt[w][l] + __popc(bc & below);
+                if (i < cap) {
+                    c.first[i] = (int)f;
+                    c.level[i] = l;
+                    if (hi == l) leaves[wcnt[w][kTreeLevels + l] + __popc(bl & below)] = i;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// counts, parents and daughters; shape[0 .. 22]: the first cell of every level and the number of cells,
+// [23]: the number of leaves, [24 .. 45]: the largest cell of every level (zero beforehand)
+__global__ void k_tree_link(const uint64_t* __restrict__ keys, int n, int leaf, const int* __restrict__ off, int nsys,
+                            int nb, const int* __restrict__ at, const int* __restrict__ total, int cap, Cells c,
+                            int* __restrict__ shape) {
+    const int ncells = min(at[(size_t)kTreeLevels * nb], cap);
+    if (blockIdx.x == 0 && threadIdx.x <= kTreeLevels + 1)
+        shape[threadIdx.x] = threadIdx.x <= kTreeLevels ? at[(size_t)threadIdx.x * nb] : *total - at[(size_t)kTreeLevels * nb];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += gridDim.x * blockDim.x) {
+        const int f = c.first[i], l = c.level[i];
+        int sb, se;
+        system_range(off, nsys, n, f, sb, se);
+        const uint64_t k = keys[f];
+        int a = f, b = se;  // the last particle of the group: a shares l digits, b does not
+        while (b - a > 1) {
+            const int m = a + ((b - a) >> 1);
+            if (shared_digits(keys[m], k) >= l) a = m;
+            else b = m;
+        }
+        const int count = b - f;
+        c.count[i] = count;
+        atomicMax(&shape[24 + l], count);
+        // among the cells of one level, in order of their first particles: the first one at or past v
+        auto lower = [&](int lev, int v) {
+            int lo = at[(size_t)lev * nb], hi = min(at[(size_t)(lev + 1) * nb], cap);
+            while (lo < hi) {
+                const int m = (lo + hi) >> 1;
+                if (c.first[m] < v) lo = m + 1;
+                else hi = m;
+            }
+            return lo;
+        };
+        c.parent[i] = l > 0 ? lower(l - 1, f + 1) - 1 : -1;
+        if (count > leaf && l < kMaxLevel) {
+            const int ch = lower(l + 1, f);
+            c.child[i] = ch;
+            c.nchild[i] = lower(l + 1, f + count) - ch;
+        } else {
+            c.child[i] = -1;
+            c.nchild[i] = 0;
         }
     }
 }
 
-void launch_split_level(const uint64_t* keys, Cells c, int lev_begin, int lev_end, int level, int leaf_size,
-                        int* nchild_tmp, int* oct_tmp, int* offs_tmp, int* scan_tmp, int* d_total,
-                        cudaStream_t s) {
-    int ncl = lev_end - lev_begin;
-    k_split<<<(unsigned)(((long long)ncl * 32 + 255) / 256), 256, 0, s>>>(keys, c, lev_begin, lev_end, level,
-                                                                         leaf_size, nchild_tmp, oct_tmp); note_launch();
-    scan_exclusive_i32(nchild_tmp, offs_tmp, ncl, d_total, scan_tmp, s);
-    k_write_children<<<(ncl + 255) / 256, 256, 0, s>>>(c, lev_begin, lev_end, level, nchild_tmp, oct_tmp, offs_tmp); note_launch();
+size_t tree_tmp_ints(int n) {
+    const size_t nb = ((size_t)n + kTreeTile - 1) / kTreeTile, m = 2 * kTreeLevels * nb;
+    return 2 * m + 1 + scan_tmp_ints((long long)m);
+}
+
+void launch_tree(const uint64_t* keys, Cells c, int n, int leaf_size, int cap, const int* off, int nsys, int* leaves,
+                 int* tmp, int* shape, cudaStream_t s) {
+    if (n <= 0) return;
+    const int nb = (int)(((long long)n + kTreeTile - 1) / kTreeTile);
+    const long long m = 2LL * kTreeLevels * nb;
+    int *cnt = tmp, *at = cnt + m, *total = at + m, *stmp = total + 1;
+    cudaMemsetAsync(shape, 0, kTreeShapeInts * sizeof(int), s);
+    k_tree_count<<<nb, kTreeThreads, 0, s>>>(keys, n, leaf_size, off, nsys, nb, cnt); note_launch();
+    scan_exclusive_i32(cnt, at, m, total, stmp, s);
+    k_tree_cells<<<nb, kTreeThreads, 0, s>>>(keys, n, leaf_size, off, nsys, nb, at, cap, c, leaves); note_launch();
+    // (the number of cells is on the device; about one per leaf_size / 4 particles)
+    k_tree_link<<<grid_for(4LL * n / leaf_size + 64, 256, 16), 256, 0, s>>>(keys, n, leaf_size, off, nsys, nb, at,
+                                                                           total, cap, c, shape); note_launch();
 }
 
 // ------------------------------------------------------------------ A4 geometry
