@@ -75,7 +75,7 @@ struct fmm_ctx {
     Buf first, count, child, nchild, parent, level, sr, cr, mass, minscale;
     Buf tree_tmp, shape, leaves, rad_tmp, owner;
     // expansions
-    Buf M, F, Pw, binom, pascal, M1, F1, Ff;
+    Buf M, F, Pw, pw, binom, pascal, M1, F1, Ff;
     // walk
     Buf walkf;  // single-precision view of the cells for the walk's acceptance test
     Buf units;  // int[2]: the working units of the tree in use (launch_work_units)
@@ -114,7 +114,7 @@ struct fmm_ctx {
     std::vector<Buf*> bufs() {
         return {&hx, &hmu, &hpsi, &hacc, &bounds, &status, &counters, &coin, &keys, &keys_alt, &idx,
                 &idx_alt, &rtmp, &xm, &perm, &xp, &first, &count, &child, &nchild, &parent, &level, &sr,
-                &cr, &mass, &minscale, &tree_tmp, &shape, &leaves, &rad_tmp, &M, &F, &Pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
+                &cr, &mass, &minscale, &tree_tmp, &shape, &leaves, &rad_tmp, &M, &F, &Pw, &pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
                 &sort_tmp, &sort_tmp2, &m2l_tmp, &p2p_tmp, &seg_start, &seg_end, &est_m2l, &est_p2p, &m2l_seg_start,
                 &m2l_seg_end, &psi_far, &acc_far, &psi_near, &acc_near, &scale_sorted, &sys_off, &sys_G,
                 &sys_roots, &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
@@ -597,6 +597,7 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
     TRY(ensure(ctx->M, sizeof(double) * nco * (size_t)nc));
     TRY(ensure(ctx->F, sizeof(double) * nco * (size_t)nc));
     TRY(ensure(ctx->Pw, sizeof(double) * (prm.p + 1) * (size_t)nc));
+    TRY(ensure(ctx->pw, sizeof(double) * 2 * (prm.p + 1) * (size_t)nc));
     TRY(ensure(ctx->binom, sizeof(double) * (kMaxP + 1)));
     {
         double bn[kMaxP + 1];
@@ -609,10 +610,11 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
         cudaStream_t u = ctx->s2;
         CU(cudaEventRecord(ctx->ev_fork, s));
         CU(cudaStreamWaitEvent(u, ctx->ev_fork, 0));
-        if (split) launch_p2m_split(P<d4>(ctx->xm), c, c.sr, P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->M), u);
+        if (split) launch_pow_tables(c.sr, nc, prm.p, P<double>(ctx->pw), u);
+        if (split) launch_p2m_split(P<d4>(ctx->xm), c, c.sr, P<double>(ctx->pw), P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->M), u);
         else launch_p2m(P<d4>(ctx->xm), c, c.sr, P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->M), u);
         for (int L = nlev - 1; L >= 0; --L) {
-            if (split) launch_m2m_split(c, c.sr, ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->M), u);
+            if (split) launch_m2m_split(c, c.sr, P<double>(ctx->pw), ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->M), u);
             else launch_m2m_level(c, c.sr, ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->M), u);
         }
         launch_power(P<double>(ctx->M), nc, prm.p, P<double>(ctx->Pw), u);
@@ -715,7 +717,7 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
                                           m2l_f64_tmp_bytes(nc, prm.p, ctx->n_m2l))));  // p <= 2 takes the latter
         kernel_marks(timing ? &ctx->ev[EV_M2LK0] : nullptr);
         launch_m2l_split(P<int2>(ctx->m2l), P<int>(ctx->m2l_seg_start), P<int>(ctx->m2l_seg_end), ctx->m2l_tmp.p, nc,
-                         c.sr, P<double>(ctx->M), prm.p, P<double>(ctx->F), prm.m2l_rot != 0, s, wp.adaptive != 0,
+                         c.sr, P<double>(ctx->pw), P<double>(ctx->M), prm.p, P<double>(ctx->F), prm.m2l_rot != 0, s, wp.adaptive != 0,
                          ctx->n_m2l);
     } else {
         TRY(ensure(ctx->m2l_tmp, m2l_f64_tmp_bytes(nc, prm.p, ctx->n_m2l)));
@@ -727,11 +729,11 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
     if (timing) CU(cudaEventRecord(ctx->ev[EV_M2L], s));
     // A11-A12: L2L, L2P
     for (int L = 1; L < nlev; ++L) {
-        if (split) launch_l2l_split(c, c.sr, ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->F), s);
+        if (split) launch_l2l_split(c, c.sr, P<double>(ctx->pw), ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->F), s);
         else launch_l2l_level(c, c.sr, ctx->lev_start[L], ctx->lev_start[L + 1], prm.p, P<double>(ctx->F), s);
     }
     if (split)
-        launch_l2p_split(P<d4>(ctx->xm), c, c.sr, P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->F),
+        launch_l2p_split(P<d4>(ctx->xm), c, c.sr, P<double>(ctx->pw), P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->F),
                          P<double>(ctx->psi_far), P<double>(ctx->acc_far), s);
     else
         launch_l2p(P<d4>(ctx->xm), c, c.sr, P<int>(ctx->leaves), ctx->nleaves, prm.p, P<double>(ctx->F),

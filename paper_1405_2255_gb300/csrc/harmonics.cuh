@@ -90,6 +90,21 @@ __device__ inline void theta_column(int p, int m, double x, double y, double z, 
     }
 }
 
+// the nine real-storage coefficients of Upsilon_n^m(d), n <= 2 (App. A.3.1 in closed form):
+// U0 = 1, U1^0 = z, U1^1 = (x+iy)/2, U2^0 = (3z^2-r^2)/4, U2^1 = z(x+iy)/2, U2^2 = (x+iy)^2/8
+__device__ inline void upsilon_low(double x, double y, double z, double u[9]) {
+    const double r2 = x * x + y * y + z * z;
+    u[cix(0, 0)] = 1.0;
+    u[cix(1, -1)] = 0.5 * y;
+    u[cix(1, 0)] = z;
+    u[cix(1, 1)] = 0.5 * x;
+    u[cix(2, -2)] = 0.25 * x * y;
+    u[cix(2, -1)] = 0.5 * z * y;
+    u[cix(2, 0)] = 0.25 * (3.0 * z * z - r2);
+    u[cix(2, 1)] = 0.5 * z * x;
+    u[cix(2, 2)] = 0.125 * (x * x - y * y);
+}
+
 // complex FP32 multiply-accumulate: acc += a * b
 __device__ inline void cmacf(float2& acc, float2 a, float2 b) {
     acc.x = fmaf(a.x, b.x, acc.x);

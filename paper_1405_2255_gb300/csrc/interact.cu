@@ -451,7 +451,7 @@ __global__ void k_m2l_reduce(const int* __restrict__ order, const int* __restric
 }
 
 void launch_m2l_split(const int2* list, const int* seg_start, const int* seg_end, void* tmp, int ncells, const d4* cen,
-                      const double* M, int p, double* F, bool rot, cudaStream_t s, bool adaptive, long long npairs) {
+                      const double* pw, const double* M, int p, double* F, bool rot, cudaStream_t s, bool adaptive, long long npairs) {
     if (ncells <= 0) return;
     if (p <= kJ64) {  // nothing to split
         launch_m2l_f64(list, seg_start, seg_end, tmp, ncells, cen, M, p, F, npairs, s);
@@ -486,7 +486,7 @@ void launch_m2l_split(const int2* list, const int* seg_start, const int* seg_end
     k_item_counts<<<grid_for(ncells, 256), 256, 0, s>>>(order, seg_start, seg_end, ncells, cnt); note_launch();
     scan_exclusive_i32(cnt, item_start, ncells, (int*)(work + 2), stmp, s);
     if (rot && m2l_rot_supported(p)) {
-        item_q = launch_m2l_rot(list, seg_start, seg_end, order, item_start, cnt, work, cen, M, ncells, p, (float*)Mf,
+        item_q = launch_m2l_rot(list, seg_start, seg_end, order, item_start, cnt, work, cen, pw, M, ncells, p, (float*)Mf,
                                 M64, part, F, adaptive, gtmp, items_cap, s);
         single = true;
         if (!adaptive) return;  // every sink's F was written once by the kernel

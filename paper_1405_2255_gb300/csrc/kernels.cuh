@@ -182,11 +182,12 @@ void launch_m2l_f64(const int2* list, const int* seg_start, const int* seg_end, 
 // directly (eq. 3b) or, when rot is set and m2l_rot_supported(p), through rotations into
 // the interaction's z frame (App. A.5, m2l_rot.cu)
 size_t m2l_split_tmp_bytes(int ncells, int p, long long npairs);
-// adaptive: the list comes from an adaptive-order walk (pairs carry their orders);
+// pw: the powers of the radii (launch_pow_tables); adaptive: the list comes from an adaptive-order walk
+// (pairs carry their orders);
 // npairs: the list's length (bounds the work items)
 void launch_m2l_split(const int2* list, const int* seg_start, const int* seg_end, void* tmp, int ncells,
-                      const d4* cen, const double* M, int p, double* F, bool rot, cudaStream_t s,
-                      bool adaptive = false, long long npairs = 0);
+                      const d4* cen, const double* pw, const double* M, int p, double* F, bool rot,
+                      cudaStream_t s, bool adaptive = false, long long npairs = 0);
 // M2L pairs per work item of the mixed-mode M2L: each sink's list is cut into chunks of
 // this many pairs from its start, summed separately and then added in chunk order
 constexpr int kM2LChunk = 32;
@@ -208,8 +209,8 @@ bool m2l_rot_supported(int p);
 // that a sink whose list is a single item has its expansion written to F (zeroed beforehand)
 // directly; returns the per-item orders (device) for the reduction
 const int* launch_m2l_rot(const int2* list, const int* seg_start, const int* seg_end, const int* order,
-                          const int* item_start, const int* cnt, unsigned* work, const d4* cen, const double* M,
-                          int ncells, int p, float* Mt, cd* M64, double* part, double* F, bool adaptive, void* gtmp,
+                          const int* item_start, const int* cnt, unsigned* work, const d4* cen, const double* pw,
+                          const double* M, int ncells, int p, float* Mt, cd* M64, double* part, double* F, bool adaptive, void* gtmp,
                           long long items_cap, cudaStream_t s);
 size_t m2l_rot_group_bytes(long long items_cap);
 void launch_l2l_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* F,
@@ -218,12 +219,14 @@ void launch_l2l_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p,
 void launch_l2p(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p,
                 const double* F, double* psi, double* acc, cudaStream_t s);
 // mixed mode: P2M and L2P with orders <= 2 in FP64 and higher orders in FP32 (split.cu)
-void launch_p2m_split(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, double* M,
+// pw: the powers of every cell's radius (launch_pow_tables, 2 (p + 1) doubles per cell)
+void launch_pow_tables(const d4* cen, int ncells, int p, double* pw, cudaStream_t s);
+void launch_p2m_split(const d4* xm, Cells c, const d4* cen, const double* pw, const int* leaves, int nleaves, int p, double* M,
                       cudaStream_t s);
-void launch_l2p_split(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, const double* F,
+void launch_l2p_split(const d4* xm, Cells c, const d4* cen, const double* pw, const int* leaves, int nleaves, int p, const double* F,
                       double* psi, double* acc, cudaStream_t s);
-void launch_m2m_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M, cudaStream_t s);
-void launch_l2l_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* F, cudaStream_t s);
+void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* M, cudaStream_t s);
+void launch_l2l_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* F, cudaStream_t s);
 // P2P (eq. 1) into psi_near/acc_near (sorted order): every leaf takes the sources of
 // its own P2P segment and those of its ancestors' segments.  This form needs no scratch; where
 // there is room for a work plan, launch_p2p_f64_plan is several times faster.

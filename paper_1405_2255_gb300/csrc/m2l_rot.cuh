@@ -309,7 +309,7 @@ constexpr RotNorm make_rot_norm() {
         for (int m = -n; m <= n; ++m) t.v[n * n + n + m] = norm_nm(n, m);
     return t;
 }
-static __constant__ RotNorm c_rot_norm = make_rot_norm();
+static __device__ const RotNorm c_rot_norm = make_rot_norm();  // (read at consecutive places by the lanes)
 
 // 4-byte asynchronous global -> shared copy; nbytes = 0 writes a zero
 __device__ __forceinline__ void rot_cp_async4(float* smem, const float* gmem, unsigned nbytes) {

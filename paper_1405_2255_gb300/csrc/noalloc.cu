@@ -249,6 +249,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     double* M = A.take<double>((size_t)nco * nc);
     double* F = A.take<double>((size_t)nco * nc);
     double* Pw = A.take<double>((size_t)(p + 1) * nc);
+    double* pw = A.take<double>(2 * (size_t)(p + 1) * nc);  // the radii's powers
     double* binom = A.take<double>(kMaxP + 1);
     double* F1 = A.take<double>(4 * (size_t)nc);
     double* Ff = A.take<double>(nc);
@@ -312,10 +313,11 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     for (int k = 1; k <= p; ++k) bn[k] = bn[k - 1] * (p - k + 1) / k;
     NA_CU(cudaMemcpyAsync(binom, bn, sizeof(double) * (p + 1), cudaMemcpyHostToDevice, s));
     const bool split = prm.precision == FMM_PREC_MIXED && prm.m2l_split;
-    if (split) launch_p2m_split(r.xm, r.c, r.c.sr, r.leaves, r.nleaves, p, M, s);
+    if (split) launch_pow_tables(r.c.sr, nc, p, pw, s);
+    if (split) launch_p2m_split(r.xm, r.c, r.c.sr, pw, r.leaves, r.nleaves, p, M, s);
     else launch_p2m(r.xm, r.c, r.c.sr, r.leaves, r.nleaves, p, M, s);
     for (int L = nl - 1; L >= 0; --L) {
-        if (split) launch_m2m_split(r.c, r.c.sr, r.lev[L], r.lev[L + 1], p, M, s);
+        if (split) launch_m2m_split(r.c, r.c.sr, pw, r.lev[L], r.lev[L + 1], p, M, s);
         else launch_m2m_level(r.c, r.c.sr, r.lev[L], r.lev[L + 1], p, M, s);
     }
     launch_power(M, nc, p, Pw, s);
@@ -349,7 +351,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     // A9-A12
     NA_CU(cudaMemsetAsync(F, 0, sizeof(double) * nco * (size_t)nc, s));
     if (split)
-        launch_m2l_split(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, M, p, F, prm.m2l_rot != 0, s, false, nm);
+        launch_m2l_split(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, pw, M, p, F, prm.m2l_rot != 0, s, false, nm);
     else
         launch_m2l_f64(m2l, m2l_seg_start, m2l_seg_end, m2l_tmp, nc, r.c.sr, M, p, F, nm, s);
     sort_pairs_by_sink(p2p, np, nc, r.sort_tmp, s);
@@ -360,10 +362,10 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     } else if (!p2p_f64_na(r, p2p, seg_start, seg_end, psi_near, acc_near, false))
         launch_p2p_fp64(r.xm, r.c, p2p, seg_start, seg_end, r.leaves, r.nleaves, psi_near, acc_near, s);
     for (int L = 1; L < nl; ++L) {
-        if (split) launch_l2l_split(r.c, r.c.sr, r.lev[L], r.lev[L + 1], p, F, s);
+        if (split) launch_l2l_split(r.c, r.c.sr, pw, r.lev[L], r.lev[L + 1], p, F, s);
         else launch_l2l_level(r.c, r.c.sr, r.lev[L], r.lev[L + 1], p, F, s);
     }
-    if (split) launch_l2p_split(r.xm, r.c, r.c.sr, r.leaves, r.nleaves, p, F, psi_far, acc_far, s);
+    if (split) launch_l2p_split(r.xm, r.c, r.c.sr, pw, r.leaves, r.nleaves, p, F, psi_far, acc_far, s);
     else launch_l2p(r.xm, r.c, r.c.sr, r.leaves, r.nleaves, p, F, psi_far, acc_far, s);
     launch_finish(psi_far, acc_far, psi_near, acc_near, r.perm, n, G, psi, acc, s, nullptr, nullptr, 0, nullptr,
                   units);

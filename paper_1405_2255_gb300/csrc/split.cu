@@ -1,4 +1,4 @@
-// split.cu -- mixed-mode P2M (eq. 3c) and L2P (eqs. 3a, 7) with the same order
+// split.cu -- mixed-mode M2M (eq. 4), L2L (eq. 5) and L2P (eqs. 3a, 7; P2M: p2m_split.cu) with the same order
 // split as the M2L: the expansion orders n <= 2 are formed in FP64, the higher
 // orders in FP32 on quantities scaled by the cell radius (Upsilon evaluated at
 // (x - z)/rho, whose values are bounded by 1/n!), then rescaled in FP64.  The
@@ -28,139 +28,80 @@ static void init_split_up_tables() {
     });
 }
 
-__device__ inline float warp_sumf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// What bounds these kernels: the FP64 pipe (2 lanes a cycle and SM, an instruction costs the same
+// however many lanes are active, and so does a conversion between FP64 and FP32).  So the powers of the
+// radii are formed once per cell, every real coefficient is converted once (the entries of order -m are
+// sign changes of those of order m), and the low orders are taken as real linear forms.
+
+// pw[cell][k] = rho^k, pw[cell][p + 1 + k] = rho^-k (0 for k > 0 of a cell of radius 0), by repeated
+// products; one thread per cell
+__global__ void k_pow_tables(const d4* __restrict__ cen, int ncells, int p, double* __restrict__ pw) {
+    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= ncells) return;
+    const double rho = cen[cell].w, inv = rho > 0 ? 1.0 / rho : 0.0;
+    double* t = pw + (size_t)cell * 2 * (p + 1);
+    double v = 1.0, u = 1.0;
+    for (int k = 0; k <= p; ++k) {
+        t[k] = v;
+        t[p + 1 + k] = u;
+        v *= rho;
+        u *= inv;
+    }
+}
+void launch_pow_tables(const d4* cen, int ncells, int p, double* pw, cudaStream_t s) {
+    if (ncells > 0) {
+        k_pow_tables<<<(ncells + 127) / 128, 128, 0, s>>>(cen, ncells, p, pw);
+        note_launch();
+    }
 }
 
-// the nine real-storage coefficients of Upsilon_n^m(d), n <= 2 (App. A.3.1 in closed form):
-// U0 = 1, U1^0 = z, U1^1 = (x+iy)/2, U2^0 = (3z^2-r^2)/4, U2^1 = z(x+iy)/2, U2^2 = (x+iy)^2/8
-__device__ inline void upsilon_low(double x, double y, double z, double u[9]) {
-    const double r2 = x * x + y * y + z * z;
-    u[cix(0, 0)] = 1.0;
-    u[cix(1, -1)] = 0.5 * y;
-    u[cix(1, 0)] = z;
-    u[cix(1, 1)] = 0.5 * x;
-    u[cix(2, -2)] = 0.25 * x * y;
-    u[cix(2, -1)] = 0.5 * z * y;
-    u[cix(2, 0)] = 0.25 * (3.0 * z * z - r2);
-    u[cix(2, 1)] = 0.5 * z * x;
-    u[cix(2, 2)] = 0.125 * (x * x - y * y);
+__device__ inline int n_of(int i) {
+    int n = (int)sqrtf((float)i);
+    while (n * n > i) --n;
+    while ((n + 1) * (n + 1) <= i) ++n;
+    return n;
+}
+// out (full complex, FP32) = R (real storage) times sc[n] for the (p+1)^2 coefficients, one warp
+__device__ __forceinline__ void expand_scaled(const double* __restrict__ R, const double* __restrict__ sc, int nco,
+                                              int lane, float2* out) {
+    for (int i = lane; i < nco; i += 32) {
+        const int n = n_of(i), c0 = n * n + n, m = i - c0, am = m < 0 ? -m : m;
+        const float v = (float)(R[i] * sc[n]);
+        const float w = (am & 1) ? -v : v;
+        if (m >= 0) {
+            out[c0 + am].x = v;
+            out[c0 - am].x = w;
+            if (m == 0) out[c0].y = 0.f;
+        } else {
+            out[c0 + am].y = v;
+            out[c0 - am].y = -w;
+        }
+    }
 }
 
-// ---------------------------------------------------------------- P2M
 constexpr int kSplitWarps = 4;
-
-__global__ void __launch_bounds__(kSplitWarps * 32) k_p2m_split(const d4* __restrict__ xm, Cells c,
-                                                                const d4* __restrict__ cen,
-                                                                const int* __restrict__ leaves, int nleaves, int p,
-                                                                double* __restrict__ M) {
-    extern __shared__ float fsm[];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
-    float* acc = fsm + (size_t)wid * nco;
-    const int t = blockIdx.x * kSplitWarps + wid;
-    if (t >= nleaves) return;
-    const int cell = leaves[t];
-    for (int i = lane; i < nco; i += 32) acc[i] = 0.f;
-    __syncwarp();
-    const d4 z = cen[cell];
-    const double rho = z.w, rinv = rho > 0 ? 1.0 / rho : 0.0;
-    const int first = c.first[cell], count = c.count[cell];
-    double lo[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) lo[i] = 0.0;
-    for (int b = 0; b < count; b += 32) {
-        const int i = b + lane;
-        double dx = 0, dy = 0, dz = 0, mu = 0;
-        if (i < count) {
-            const d4 q = xm[first + i];
-            dx = q.x - z.x; dy = q.y - z.y; dz = q.z - z.z; mu = q.w;
-        }
-        double u[9];
-        upsilon_low(dx, dy, dz, u);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) lo[k] = fma(mu, u[k], lo[k]);
-        if (rho > 0 && p > 2) {
-            // mu * Upsilon_n^m((x - z)/rho) in FP32, n >= 3 kept
-            const float x = (float)(dx * rinv), y = (float)(dy * rinv), zz = (float)(dz * rinv), w = (float)mu;
-            const float r2 = x * x + y * y + zz * zz;
-            float2 d = make_float2(w, 0.f);
-            for (int m = 0; m <= p; ++m) {
-                if (m > 0) {
-                    const float s = c_inv2jf[m];
-                    d = make_float2(s * (x * d.x - y * d.y), s * (x * d.y + y * d.x));
-                }
-                float2 prev2 = make_float2(0.f, 0.f), prev = d;
-                for (int n = m; n <= p; ++n) {
-                    float2 v;
-                    if (n == m) v = d;
-                    else {
-                        const float a = c_twf2[n] * zz, iv = c_inv_upf[n][m];
-                        v = make_float2((a * prev.x - r2 * prev2.x) * iv, (a * prev.y - r2 * prev2.y) * iv);
-                        prev2 = prev;
-                        prev = v;
-                    }
-                    if (n >= 3) {
-                        const float sr = warp_sumf(v.x), si = warp_sumf(v.y);
-                        if (lane == 0) {
-                            acc[cix(n, m)] += sr;
-                            if (m) acc[cix(n, -m)] += si;
-                        }
-                    }
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) lo[k] = warp_sum(lo[k]);
-    __syncwarp();
-    double* out = M + (size_t)cell * nco;
-    __shared__ double pw_all[kSplitWarps][kMaxP + 1];
-    double* pw = pw_all[wid];
-    warp_pow_table(rho, p, lane, pw);
-    __syncwarp();
-    if (lane == 0)
-        for (int k = 0; k < 9 && k < nco; ++k) out[k] = lo[k];
-    for (int i = 9 + lane; i < nco; i += 32) {
-        int n = (int)sqrtf((float)i);
-        while (n * n > i) --n;
-        while ((n + 1) * (n + 1) <= i) ++n;
-        out[i] = (double)acc[i] * pw[n];
-    }
-}
-
-void launch_p2m_split(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, double* M,
-                      cudaStream_t s) {
-    if (nleaves <= 0) return;
-    if (p < 2) {
-        launch_p2m(xm, c, cen, leaves, nleaves, p, M, s);
-        return;
-    }
-    init_split_up_tables();
-    size_t sm = (size_t)kSplitWarps * ncoef(p) * sizeof(float);
-    k_p2m_split<<<(nleaves + kSplitWarps - 1) / kSplitWarps, kSplitWarps * 32, sm, s>>>(xm, c, cen, leaves, nleaves,
-                                                                                          p, M);
-    note_launch();
-}
 
 // ---------------------------------------------------------------- L2P
 // Psi_0^0 = sum_{k,l} Upsilon_k^{l*} F_k^l and Psi_1^m = sum_{k,l} Upsilon_k^{l*} F_{k+1}^{m+l}
 // (Upsilon at s_B - x_b): terms with k <= 2 in FP64; terms with k >= 3 in FP32 as
 // Uhat_k^{l*} Fhat_k^l and Uhat_k^{l*} Fhat_{k+1}^{m+l} / rho with Uhat_k = Upsilon_k((s - x)/rho),
 // Fhat_n = F_n rho^n.  One warp per leaf, lane = particle.
+// The terms k <= 2 are linear in the nine real entries u of Upsilon (upsilon_low): with l and -l taken
+// together (F^{-l} = (-1)^l conj(F^l)), psi and az take 2 Re and 2 Im of F_k^l and F_{k+1}^l, and ax, ay
+// the parts of A + B (of Re Y) and i (B - A) (of Im Y), A = F_{k+1}^{1+l}, B = (-1)^l F_{k+1}^{1-l}:
+// 36 multiply-adds per particle (some 90 when every complex term was taken by itself).
 __global__ void __launch_bounds__(kSplitWarps * 32) k_l2p_split(const d4* __restrict__ xm, Cells c,
                                                                 const d4* __restrict__ cen,
+                                                                const double* __restrict__ pw,
                                                                 const int* __restrict__ leaves, int nleaves, int p,
                                                                 const double* __restrict__ F, double* __restrict__ psi,
                                                                 double* __restrict__ acc) {
-    extern __shared__ unsigned char sraw[];
+    extern __shared__ __align__(16) unsigned char sraw[];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nco = ncoef(p);
-    const size_t per_warp = ((size_t)nco * sizeof(float2) + 16 * sizeof(cd) + 15) & ~(size_t)15;
-    float2* Fh = (float2*)(sraw + wid * per_warp);  // [nco] F_n rho^n
-    cd* F64 = (cd*)(Fh + nco);                      // [16] F_n, n <= 3
+    const size_t per_warp = ((size_t)nco * sizeof(float2) + 36 * sizeof(double) + 15) & ~(size_t)15;
+    double* C = (double*)(sraw + wid * per_warp);  // [9][4]: weights of u in psi, p10, Re p11, Im p11
+    float2* Fh = (float2*)(C + 36);                // [nco] F_n rho^n
     const int t = blockIdx.x * kSplitWarps + wid;
     if (t >= nleaves) return;
     const int cell = leaves[t];
@@ -168,50 +109,45 @@ __global__ void __launch_bounds__(kSplitWarps * 32) k_l2p_split(const d4* __rest
     const d4 s = cen[cell];
     const double rho = s.w;
     const double* Fr = F + (size_t)cell * nco;
-    __shared__ double pw_all[kSplitWarps][kMaxP + 1];
-    double* pw = pw_all[wid];
-    warp_pow_table(rho, p, lane, pw);
-    __syncwarp();
-    for (int i = lane; i < nco; i += 32) {
-        int n = (int)sqrtf((float)i);
-        while (n * n > i) --n;
-        while ((n + 1) * (n + 1) <= i) ++n;
-        const cd v = load_real_storage(Fr, n, i - n * n - n);
-        const double sc = pw[n];
-        Fh[i] = make_float2((float)(v.re * sc), (float)(v.im * sc));
-        if (i < 16) F64[i] = v;
+    const double* pc = pw + (size_t)cell * 2 * (p + 1);
+    expand_scaled(Fr, pc, nco, lane, Fh);
+    if (lane < 9) {
+        const int k = lane < 1 ? 0 : (lane < 4 ? 1 : 2), m = lane - k * k - k, l = m < 0 ? -m : m;
+        const cd f0 = load_real_storage(Fr, k, l), f1 = load_real_storage(Fr, k + 1, l);
+        const cd A = load_real_storage(Fr, k + 1, 1 + l);
+        cd B = mkc(0.0, 0.0);
+        if (l) B = load_real_storage(Fr, k + 1, 1 - l);
+        if (l & 1) B = mkc(-B.re, -B.im);
+        double* w = C + 4 * lane;
+        if (m >= 0) {
+            w[0] = l ? f0.re + f0.re : f0.re;
+            w[1] = l ? f1.re + f1.re : f1.re;
+            w[2] = A.re + B.re;
+            w[3] = A.im + B.im;
+        } else {
+            w[0] = f0.im + f0.im;
+            w[1] = f1.im + f1.im;
+            w[2] = A.im - B.im;
+            w[3] = B.re - A.re;
+        }
     }
     __syncwarp();
-    const double rinv = rho > 0 ? 1.0 / rho : 0.0;
+    const double rinv = pc[p + 2];
     const int first = c.first[cell], count = c.count[cell];
     for (int j = lane; j < count; j += 32) {
         const d4 xb = xm[first + j];
         const double vx = s.x - xb.x, vy = s.y - xb.y, vz = s.z - xb.z;
         // k <= 2 in FP64
-        double u[9];
+        double u[9], q[4] = {0.0, 0.0, 0.0, 0.0};
         upsilon_low(vx, vy, vz, u);
-        double p00 = 0;
-        cd p10 = mkc(0, 0), p11 = mkc(0, 0);
-        for (int k = 0; k <= 2 && k <= p; ++k) {
-            for (int l = 0; l <= k; ++l) {
-                const cd Y = mkc(u[cix(k, l)], l ? u[cix(k, -l)] : 0.0);  // Upsilon_k^l
-                const cd Xp = conjc(Y);
-                const double sg = (l & 1) ? -1.0 : 1.0;
-                const cd Xn = mkc(sg * Y.re, sg * Y.im);                 // conj(Upsilon_k^{-l})
-                const cd* Fk = F64 + k * k + k;
-                if (l == 0) p00 += Xp.re * Fk[0].re - Xp.im * Fk[0].im;
-                else p00 += 2.0 * (Xp.re * Fk[l].re - Xp.im * Fk[l].im);
-                if (k + 1 <= p) {
-                    const cd* Fk1 = F64 + (k + 1) * (k + 1) + (k + 1);
-                    cmac(p10, Xp, Fk1[l]);
-                    cmac(p11, Xp, Fk1[1 + l]);
-                    if (l > 0) {
-                        cmac(p10, Xn, Fk1[-l]);
-                        cmac(p11, Xn, Fk1[1 - l]);
-                    }
-                }
-            }
-        }
+        // the weights are read from shared memory here: kept in registers across the loop (127 of them)
+        // they cost more warps than the reads (0.68 ms for the 43,413 leaves of a Plummer sphere of 1e6)
+        const double* Cj = C;
+        asm volatile("" : "+l"(Cj));
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+#pragma unroll
+            for (int d = 0; d < 4; ++d) q[d] = fma(u[i], Cj[4 * i + d], q[d]);
         // k >= 3 in FP32 on the scaled offset
         float h00 = 0.f;
         float2 h10 = make_float2(0.f, 0.f), h11 = make_float2(0.f, 0.f);
@@ -254,24 +190,24 @@ __global__ void __launch_bounds__(kSplitWarps * 32) k_l2p_split(const d4* __rest
             }
         }
         const int i = first + j;
-        psi[i] = p00 + (double)h00;
-        acc[3 * (size_t)i] = -(p11.re + (double)h11.x * rinv);
-        acc[3 * (size_t)i + 1] = -(p11.im + (double)h11.y * rinv);
-        acc[3 * (size_t)i + 2] = -(p10.re + (double)h10.x * rinv);
+        psi[i] = q[0] + (double)h00;
+        acc[3 * (size_t)i] = -(q[2] + (double)h11.x * rinv);
+        acc[3 * (size_t)i + 1] = -(q[3] + (double)h11.y * rinv);
+        acc[3 * (size_t)i + 2] = -(q[1] + (double)h10.x * rinv);
     }
 }
 
-void launch_l2p_split(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, const double* F,
-                      double* psi, double* acc, cudaStream_t s) {
+void launch_l2p_split(const d4* xm, Cells c, const d4* cen, const double* pw, const int* leaves, int nleaves, int p,
+                      const double* F, double* psi, double* acc, cudaStream_t s) {
     if (nleaves <= 0) return;
     if (p < 3) {
         launch_l2p(xm, c, cen, leaves, nleaves, p, F, psi, acc, s);
         return;
     }
     init_split_up_tables();
-    const size_t per_warp = ((size_t)ncoef(p) * sizeof(float2) + 16 * sizeof(cd) + 15) & ~(size_t)15;
+    const size_t per_warp = ((size_t)ncoef(p) * sizeof(float2) + 36 * sizeof(double) + 15) & ~(size_t)15;
     k_l2p_split<<<(nleaves + kSplitWarps - 1) / kSplitWarps, kSplitWarps * 32, kSplitWarps * per_warp, s>>>(
-        xm, c, cen, leaves, nleaves, p, F, psi, acc);
+        xm, c, cen, pw, leaves, nleaves, p, F, psi, acc);
     note_launch();
 }
 
@@ -285,9 +221,8 @@ __device__ inline void upsilon_low_full(double x, double y, double z, cd out[9],
             if (conj_out) v = conjc(v);
             out[cix(k, l)] = v;
             if (l) {
-                const double sg = (l & 1) ? -1.0 : 1.0;
                 // X^{-l} = (-1)^l conj(X^l) for both Upsilon and its conjugate
-                out[cix(k, -l)] = mkc(sg * v.re, -sg * v.im);
+                out[cix(k, -l)] = (l & 1) ? mkc(-v.re, v.im) : mkc(v.re, -v.im);
             }
         }
 }
@@ -317,13 +252,6 @@ __device__ inline void upsilon_column_f(int p, int m, float x, float y, float z,
     }
 }
 
-__device__ inline int n_of(int i) {
-    int n = (int)sqrtf((float)i);
-    while (n * n > i) --n;
-    while ((n + 1) * (n + 1) <= i) ++n;
-    return n;
-}
-
 // ---------------------------------------------------------------- M2M
 // M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z): outputs n <= 2 in FP64,
 // outputs n >= 3 in FP32 as Mhat_n = M_n / rho'^n = sum Uhat_k Mt_{n-k} with
@@ -338,7 +266,8 @@ __host__ __device__ inline size_t m2m_smem_bytes(int p) {
     return kM2MWarps * m2m_warp_bytes(p) + kM2MWarps * nout * sizeof(float2) + kM2MWarps * 6 * sizeof(cd);
 }
 template <int MAXQ>
-__global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4* __restrict__ cen, int lev_begin,
+__global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4* __restrict__ cen,
+                                                               const double* __restrict__ pw, int lev_begin,
                                                                int lev_end, int p, double* __restrict__ M,
                                                                LaneSched sched) {
     extern __shared__ __align__(16) unsigned char sraw[];
@@ -351,16 +280,13 @@ __global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4*
     cd* M64 = Y64 + 9;
     float2* r32 = (float2*)(sraw + kM2MWarps * per_warp);  // [kM2MWarps][nout]
     cd* r64 = (cd*)(r32 + kM2MWarps * nout);                // [kM2MWarps][6]
-    __shared__ double pwi[kMaxP + 1], pwr[kMaxP + 1];        // rho^-n, rho^n
     const int cell = lev_begin + blockIdx.x;
     if (cell >= lev_end) return;
     const int nch = c.nchild[cell];
     if (nch == 0) return;  // leaves
     const d4 zp = cen[cell];
-    const double rho = zp.w, inv = rho > 0 ? 1.0 / rho : 0.0;
-    if (wid == 0) warp_pow_table(inv, p, lane, pwi);
-    if (wid == 1) warp_pow_table(rho, p, lane, pwr);
-    __syncthreads();
+    const double *pwr = pw + (size_t)cell * 2 * (p + 1), *pwi = pwr + p + 1;  // rho^n, rho^-n
+    const double rho = zp.w, inv = pwi[1];
     if (wid < nch) {
         const int cnt = sched.cnt[lane];
         const int d = c.child[cell] + wid;
@@ -368,12 +294,10 @@ __global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4*
         const double vx = z.x - zp.x, vy = z.y - zp.y, vz = z.z - zp.z;
         if (lane <= p) upsilon_column_f(p, lane, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, false);
         const double* Md = M + (size_t)d * nco;
-        for (int i = lane; i < nco; i += 32) {
-            const int n = n_of(i);
-            const cd v = load_real_storage(Md, n, i - n * n - n);
-            const double sc = pwi[n];
-            Mt[i] = make_float2((float)(v.re * sc), (float)(v.im * sc));
-            if (i < 9) M64[i] = v;
+        expand_scaled(Md, pwi, nco, lane, Mt);
+        if (lane < 9) {
+            const int n = n_of(lane);
+            M64[lane] = load_real_storage(Md, n, lane - n * n - n);
         }
         if (lane == 0) upsilon_low_full(vx, vy, vz, Y64, false);
         __syncwarp();
@@ -428,7 +352,7 @@ __global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4*
     }
 }
 
-void launch_m2m_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M, cudaStream_t s) {
+void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* M, cudaStream_t s) {
     const int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
     if (p < 3) {
@@ -443,13 +367,13 @@ void launch_m2m_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p,
     const unsigned g = (unsigned)ncl;  // one block per cell of the level (leaves return at once)
     if (maxq <= 4) {
         cudaFuncSetAttribute(k_m2m_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<4><<<g, kM2MWarps * 32, sm, s>>>(c, cen, lev_begin, lev_end, p, M, sched);
+        k_m2m_split<4><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
     } else if (maxq <= 8) {
         cudaFuncSetAttribute(k_m2m_split<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<8><<<g, kM2MWarps * 32, sm, s>>>(c, cen, lev_begin, lev_end, p, M, sched);
+        k_m2m_split<8><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
     } else {
         cudaFuncSetAttribute(k_m2m_split<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<24><<<g, kM2MWarps * 32, sm, s>>>(c, cen, lev_begin, lev_end, p, M, sched);
+        k_m2m_split<24><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
     }
     note_launch();
 }
@@ -458,17 +382,30 @@ void launch_m2m_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p,
 // F_n^m(s') += sum_{k<=p-n} sum_l Upsilon_k^{l*}(s - s') F_{n+k}^{m+l}(s): terms with n+k <= 2
 // in FP64, the others in FP32 as rho^-n sum Uhat_k^{l*} Fhat_{n+k}^{m+l} with
 // Uhat_k = Upsilon_k((s - s')/rho), Fhat_j = F_j(s) rho^j (rho: the parent's radius).
-template <int MAXQ>
-__global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict__ cen, int lev_begin, int lev_end,
+// One warp per cell.  The FP64 terms of the six outputs n <= 2 are 20 products, one per lane.
+struct L2LTerm {
+    signed char n, m, k, l;
+};
+__device__ constexpr L2LTerm kL2LTerm[20] = {
+    {0, 0, 0, 0},  {0, 0, 1, -1}, {0, 0, 1, 0}, {0, 0, 1, 1},  {0, 0, 2, -2}, {0, 0, 2, -1}, {0, 0, 2, 0},
+    {0, 0, 2, 1},  {0, 0, 2, 2},  {1, 0, 0, 0}, {1, 0, 1, -1}, {1, 0, 1, 0},  {1, 0, 1, 1},  {1, 1, 0, 0},
+    {1, 1, 1, -1}, {1, 1, 1, 0},  {1, 1, 1, 1}, {2, 0, 0, 0},  {2, 1, 0, 0},  {2, 2, 0, 0}};
+__device__ constexpr int kL2LStart[7] = {0, 9, 13, 17, 18, 19, 20};  // first product of output n (n + 1) / 2 + m
+__host__ __device__ inline size_t l2l_warp_bytes(int p) {
+    return ((size_t)2 * ncoef(p) * sizeof(float2) + (9 + 9 + 20 + 6) * sizeof(cd) + 15) & ~(size_t)15;
+}
+__global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict__ cen,
+                                                   const double* __restrict__ pw, int lev_begin, int lev_end,
                                                    int p, double* __restrict__ F, LaneSched sched) {
-    extern __shared__ unsigned char sraw[];
+    extern __shared__ __align__(16) unsigned char sraw[];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nco = ncoef(p);
-    const size_t per_warp = ((size_t)2 * nco * sizeof(float2) + 18 * sizeof(cd) + 15) & ~(size_t)15;
-    float2* Yh = (float2*)(sraw + wid * per_warp);
-    float2* Fh = Yh + nco;
-    cd* Y64 = (cd*)(Fh + nco);
+    cd* Y64 = (cd*)(sraw + wid * l2l_warp_bytes(p));
     cd* F64 = Y64 + 9;
+    cd* prod = F64 + 9;
+    cd* low = prod + 20;
+    float2* Yh = (float2*)(low + 6);
+    float2* Fh = Yh + nco;
     const int cell = lev_begin + blockIdx.x * 4 + wid;
     if (cell >= lev_end || !cell_active(c, cell)) return;
     const int par = c.parent[cell];
@@ -480,29 +417,31 @@ __global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict
         for (int i = lane; i < nco; i += 32) out[i] += Fp[i];
         return;
     }
-    const double inv = 1.0 / rho;
-    __shared__ double pwi_all[4][kMaxP + 1], pwr_all[4][kMaxP + 1];
-    double *pwi = pwi_all[wid], *pwr = pwr_all[wid];  // rho^-n, rho^n
-    warp_pow_table(inv, p, lane, pwi);
-    warp_pow_table(rho, p, lane, pwr);
-    __syncwarp();
+    const double *pwr = pw + (size_t)par * 2 * (p + 1), *pwi = pwr + p + 1;  // rho^n, rho^-n
+    const double inv = pwi[1];
     const double vx = s.x - sp.x, vy = s.y - sp.y, vz = s.z - sp.z;
     if (lane <= p) upsilon_column_f(p, lane, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, true);
-    for (int i = lane; i < nco; i += 32) {
-        const int n = n_of(i);
-        const cd v = load_real_storage(Fp, n, i - n * n - n);
-        const double sc = pwr[n];
-        Fh[i] = make_float2((float)(v.re * sc), (float)(v.im * sc));
-        if (i < 9) F64[i] = v;
+    expand_scaled(Fp, pwr, nco, lane, Fh);
+    if (lane < 9) {
+        const int n = n_of(lane);
+        F64[lane] = load_real_storage(Fp, n, lane - n * n - n);
     }
     if (lane == 0) upsilon_low_full(vx, vy, vz, Y64, true);
+    __syncwarp();
+    if (lane < 20) {
+        const L2LTerm t = kL2LTerm[lane];
+        prod[lane] = Y64[cix(t.k, t.l)] * F64[cix(t.n + t.k, t.m + t.l)];
+    }
+    __syncwarp();
+    if (lane < 6) {
+        cd v = mkc(0.0, 0.0);
+        for (int i = kL2LStart[lane]; i < kL2LStart[lane + 1]; ++i) v = v + prod[i];
+        low[lane] = v;
+    }
     __syncwarp();
     const int cnt = sched.cnt[lane];
     for (int q = 0; q < cnt; ++q) {
         const int n = sched.n[lane][q], m = sched.m[lane][q];
-        cd v64 = mkc(0.0, 0.0);
-        for (int k = 0; k + n <= 2 && k <= p - n; ++k)
-            for (int l = -k; l <= k; ++l) cmac(v64, Y64[cix(k, l)], F64[cix(n + k, m + l)]);
         float2 v32 = make_float2(0.f, 0.f);
         for (int k = max(0, 3 - n); k <= p - n; ++k) {
             const float2* xk = Yh + k * k + k;
@@ -510,12 +449,18 @@ __global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict
             for (int l = -k; l <= k; ++l) cmacf(v32, xk[l], yk[l]);
         }
         const double sc = pwi[n];
-        out[cix(n, m)] += v64.re + (double)v32.x * sc;
-        if (m) out[cix(n, -m)] += v64.im + (double)v32.y * sc;
+        double re = out[cix(n, m)], im = m ? out[cix(n, -m)] : 0.0;
+        if (n <= 2) {
+            const cd v = low[n * (n + 1) / 2 + m];
+            re += v.re;
+            im += v.im;
+        }
+        out[cix(n, m)] = fma((double)v32.x, sc, re);
+        if (m) out[cix(n, -m)] = fma((double)v32.y, sc, im);
     }
 }
 
-void launch_l2l_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* F, cudaStream_t s) {
+void launch_l2l_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* F, cudaStream_t s) {
     const int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
     if (p < 3) {
@@ -524,8 +469,9 @@ void launch_l2l_split(Cells c, const d4* cen, int lev_begin, int lev_end, int p,
     }
     init_split_up_tables();
     LaneSched sched = make_lane_sched(p, kSchedDown);
-    const size_t per_warp = ((size_t)2 * ncoef(p) * sizeof(float2) + 18 * sizeof(cd) + 15) & ~(size_t)15;
-    k_l2l_split<4><<<(unsigned)((ncl + 3) / 4), 128, 4 * per_warp, s>>>(c, cen, lev_begin, lev_end, p, F, sched);
+    const size_t sm = 4 * l2l_warp_bytes(p);
+    cudaFuncSetAttribute(k_l2l_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_l2l_split<<<(unsigned)((ncl + 3) / 4), 128, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, F, sched);
     note_launch();
 }
 
