@@ -143,7 +143,7 @@ const int* launch_m2l_rot(const int2* list, const int* seg_start, const int* seg
     const int nco = ncoef(p);
 #define GB3_ROT(PP)                                                                                      \
     case PP:                                                                                             \
-        rot_launch<PP>(RotArgs{list, seg_start, seg_end, order, item_start, work, cen, Mt, M64, part, F, il,  \
+        rot_launch<PP>(RotArgs{list, seg_start, seg_end, order, item_start, work, cen, pw, p, Mt, M64, part, F, il,  \
                                go, gq, ctr, nco, adapt, by_sink ? cnt : nullptr, by_sink ? work + 3 : nullptr,  \
                                units, work + 4},                                                         \
                        s);                                                                               \

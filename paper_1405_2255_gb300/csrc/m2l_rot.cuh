@@ -54,6 +54,8 @@ struct RotArgs {
     const int* item_start;
     unsigned* work;
     const d4* cen;
+    const double* pw;  // powers of the radii, 2 (p + 1) doubles per cell
+    int p;
     const float* Mt;
     const cd* M64;
     double* part;
@@ -329,6 +331,27 @@ __device__ inline cd theta_low_rot(int j, int m, double x, double y, double z, d
     return mkc(3.0 * (x * x - y * y) * r5, 6.0 * x * y * r5);
 }
 
+// The six FP64 sums over the warp (butterfly order: xor 16, 8, 4, 2, 1), a lane passing on at each step
+// the values that it will not keep: 8 additions in place of 30
+static_assert(kRotLow == 3, "sum6 takes three complex values");
+__device__ inline double sum6(const cd (&lo)[kRotLow], int lane) {
+    const double v[6] = {lo[0].re, lo[0].im, lo[1].re, lo[1].im, lo[2].re, lo[2].im};
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    double a[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double keep = h16 ? v[i + 3] : v[i], send = h16 ? v[i] : v[i + 3];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+    const double k0 = h8 ? a[1] : a[0], s0 = h8 ? a[0] : a[1];
+    const double b0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 8);
+    const double b1 = a[2] + __shfl_xor_sync(0xffffffffu, a[2], 8);
+    const double k1 = h4 ? b1 : b0, s1 = h4 ? b0 : b1;
+    double c = k1 + __shfl_xor_sync(0xffffffffu, s1, 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+
 // Shared memory of one warp: the per-lane vectors S[NCO][kPad] (floats), sigma^-n and
 // the FP64 low-order outputs; then the sink's accumulated expansion (NCO doubles, by-sink mode).
 template <int P>
@@ -529,14 +552,11 @@ __global__ void __launch_bounds__(32 * rot_warps<P>(), 1) k_m2l_rot(const RotArg
 #pragma unroll
                         for (int l = -k; l <= k; ++l) cmac(lo[n * (n + 1) / 2 + m], Mx[cix(k, l)], T[cix(n + k, m + l)]);
         }
-#pragma unroll
-        for (int i = 0; i < kRotLow; ++i) {
-            lo[i].re = warp_sum(lo[i].re);
-            lo[i].im = warp_sum(lo[i].im);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < kRotLow; ++i) lowF[i] = lo[i];
+        {
+            const double low = sum6(lo, lane);
+            // value v ends in the lanes with bits 16 (v >= 3), 4 (v = 2, 5) or else 8 (v = 1, 4)
+            const int v = ((lane & 16) ? 3 : 0) + ((lane & 4) ? 2 : ((lane & 8) ? 1 : 0));
+            if (!(lane & 3) && !((lane & 4) && (lane & 8))) ((double*)lowF)[v] = low;
         }
         rot_cp_async_wait_all();
         __syncthreads();
@@ -546,7 +566,14 @@ __global__ void __launch_bounds__(32 * rot_warps<P>(), 1) k_m2l_rot(const RotArg
         else zm2l_all<P, false>(Sl, P, upto<P / 2>{});
         __syncthreads();
         bwd_all<P>(Sl, cw, cu, tB, upto<P>{});
-        warp_pow_table(1.0 / sigma, P + 1, lane, pws);
+        // sigma^-n: the radius's powers, or those of the distance that stands in for a radius of 0
+        if (has && sB.w > 0) {
+            const double* pi = args.pw + (size_t)B * 2 * (args.p + 1) + args.p + 1;
+            if (lane <= P) pws[lane] = pi[lane];
+            if (lane == 0) pws[P + 1] = pi[P] * pi[1];
+        } else {
+            warp_pow_table(1.0 / sigma, P + 1, lane, pws);
+        }
         __syncwarp();
         if (has) {
             double* out = by_sink ? accF
