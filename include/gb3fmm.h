@@ -333,8 +333,8 @@ int fmm_swap_probe(int npairs, int reps, double* ms, double* maxdiff);
  * any stream capture.  All calls share the array and it keeps the last call's
  * contents (what must start at zero is cleared on every call); calls whose work
  * overlaps on the GPU race on it and give wrong results, so serialise them.  The
- * call waits for its stream several times (the tree's level sizes and the walk's
- * frontier lengths are read on the host).
+ * call waits for its stream several times (the tree's shape and the lists' lengths
+ * are read on the host).
  *   n       0 <= n <= 8192, else FMM_E_INVALID
  *   x, mu   device, [n][3] and [n] FP64 (as fmm_evaluate)
  *   params  host; p <= 10, 24 <= leaf_size <= 4096, scale_src = FMM_SCALE_ESTIMATE

@@ -84,7 +84,7 @@ struct fmm_ctx {
     long long front_cap = 0, m2l_cap = 0, p2p_cap = 0, est_m2l_cap = 0, est_p2p_cap = 0;
     // per particle results (sorted order)
     Buf psi_far, acc_far, psi_near, acc_near, scale_sorted;
-    unsigned long long* h_counters = nullptr;  // pinned, 16 words: the walk [0, 8), the P2P plan [8, 14)
+    unsigned long long* h_counters = nullptr;  // pinned: the walk [0, kWalkCounters), then the P2P plan's 6
     int* h_int = nullptr;                      // pinned
     cudaEvent_t ev[EV_N];
     bool ev_ok = false;
@@ -316,38 +316,22 @@ static int run_walk(fmm_ctx* ctx, WalkParams wp, Buf& m2l, long long& m2l_cap, B
         wb.p2p = P<int2>(p2p);
         wb.p2p_cap = p2p_cap;
         wb.counters = P<unsigned long long>(ctx->counters);
-        // counters: [0], [4] the frontier lengths (ping-pong), [1] M2L, [2] P2P, [3] overflow,
-        // [5] the largest frontier demand.  Every step of a pair descends one cell level on
-        // at least one side, so 2 * levels steps end the walk; the steps read their frontier
-        // lengths on the device and the host waits once, after the last one.
-        CU(cudaMemsetAsync(wb.counters, 0, 8 * sizeof(unsigned long long), s));
-        launch_walk_roots(wb.front[0], ctx->nroots, s, wb.counters);
-        const int nlev = (int)ctx->lev_start.size() - 1;
-        const int steps = 2 * nlev + 1;
-        int cur = 0;
-        for (int k = 0; k < steps; ++k) {
-            unsigned long long* in_cnt = wb.counters + (k & 1 ? 4 : 0);
-            unsigned long long* out_cnt = wb.counters + (k & 1 ? 0 : 4);
-            CU(cudaMemsetAsync(out_cnt, 0, sizeof(unsigned long long), s));
-            launch_walk_step_dev(c, wp, wb.front[cur], in_cnt, wb.front[cur ^ 1], wb, out_cnt, s);
-            cur ^= 1;
-        }
-        CU(cudaMemcpyAsync(ctx->h_counters, wb.counters, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        const int steps = walk_steps((int)ctx->lev_start.size() - 1);
+        launch_walk(c, wp, wb, ctx->nroots, nc, steps, s);
+        CU(cudaMemcpyAsync(ctx->h_counters, wb.counters, kWalkCounters * sizeof(unsigned long long),
+                           cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
-        const long long left = (long long)ctx->h_counters[(steps - 1) & 1 ? 0 : 4];
-        const long long need_front = std::max<long long>((long long)ctx->h_counters[5], left);
-        const bool overflow = ctx->h_counters[3] != 0;
-        if (!overflow && left != 0) return fail(ctx, FMM_E_CUDA, "the tree walk did not end within 2 x levels steps");
-        if (!overflow) {
-            *n_m2l = (long long)ctx->h_counters[1];
-            *n_p2p = (long long)ctx->h_counters[2];
+        const WalkResult r = walk_result(ctx->h_counters, steps);
+        if (!r.overflow && r.left != 0) return fail(ctx, FMM_E_CUDA, "the tree walk did not end within 2 x levels steps");
+        if (!r.overflow) {
+            *n_m2l = r.n_m2l;
+            *n_p2p = r.n_p2p;
             return 0;
         }
         // grow what overflowed (the counters hold at least the demand seen so far) and redo the walk
-        if (need_front > ctx->front_cap)
-            ctx->front_cap = std::max<long long>(2 * ctx->front_cap, 2 * need_front);
-        if ((long long)ctx->h_counters[1] > m2l_cap) m2l_cap = std::max<long long>(2 * m2l_cap, 2 * (long long)ctx->h_counters[1]);
-        if ((long long)ctx->h_counters[2] > p2p_cap) p2p_cap = std::max<long long>(2 * p2p_cap, 2 * (long long)ctx->h_counters[2]);
+        if (r.need_front > ctx->front_cap) ctx->front_cap = std::max<long long>(2 * ctx->front_cap, 2 * r.need_front);
+        if (r.n_m2l > m2l_cap) m2l_cap = std::max<long long>(2 * m2l_cap, 2 * r.n_m2l);
+        if (r.n_p2p > p2p_cap) p2p_cap = std::max<long long>(2 * p2p_cap, 2 * r.n_p2p);
     }
     char msg[200];
     snprintf(msg, sizeof msg, "walk lists could not be grown enough (caps: front %lld, m2l %lld, p2p %lld)",
@@ -375,7 +359,7 @@ static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t 
         const size_t need = launch_p2p_mixed(P<float4>(ctx->xp), ctx->n, c, list,
                                              P<int>(ctx->seg_start), P<int>(ctx->seg_end), P<int>(ctx->leaves),
                                              ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), mode,
-                                             ctx->p2p_tmp.p, ctx->p2p_tmp.bytes, ctx->h_counters + 8, s);
+                                             ctx->p2p_tmp.p, ctx->p2p_tmp.bytes, ctx->h_counters + kWalkCounters, s);
         if (need == ~(size_t)0) return fail(ctx, FMM_E_OVERFLOW, "P2P plan beyond 2^31 source ranges or n >= 2^29");
         if (need <= ctx->p2p_tmp.bytes) return 0;
         TRY(ensure(ctx->p2p_tmp, need));
@@ -394,7 +378,7 @@ static int run_p2p_fp64(fmm_ctx* ctx, const int2* list, bool want_f, bool* plann
         need = launch_p2p_f64_plan(P<d4>(ctx->xm), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
                                    P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near),
                                    P<double>(ctx->acc_near), want_f, ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
-                                   ctx->h_counters + 8, s);
+                                   ctx->h_counters + kWalkCounters, s);
         if (need == ~(size_t)0) return 0;
         if (need <= ctx->p2p_tmp.bytes) {
             *planned = true;
@@ -422,7 +406,7 @@ static int run_p2p_tidal(fmm_ctx* ctx, cudaStream_t s) {
         need = launch_p2p_tidal_plan(P<float4>(ctx->xp), ctx->n, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
                                      P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves,
                                      P<double>(ctx->tid_near), ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
-                                     ctx->h_counters + 8, s);
+                                     ctx->h_counters + kWalkCounters, s);
         if (need <= ctx->p2p_tmp.bytes) return 0;
         if (need == ~(size_t)0) break;
     }
@@ -846,10 +830,10 @@ int fmm_create(fmm_ctx** out, const fmm_params* params, int device) {
     int rc = 0;
     if (!rc) rc = ensure(ctx->bounds, 8 * sizeof(unsigned long long));
     if (!rc) rc = ensure(ctx->status, 16);
-    if (!rc) rc = ensure(ctx->counters, 8 * sizeof(unsigned long long));
+    if (!rc) rc = ensure(ctx->counters, kWalkCounters * sizeof(unsigned long long));
     if (!rc) rc = ensure(ctx->coin, 16);
     if (!rc) rc = ensure(ctx->shape, kTreeShapeInts * sizeof(int));
-    if (!rc && cudaMallocHost((void**)&ctx->h_counters, 16 * sizeof(unsigned long long)) != cudaSuccess) rc = FMM_E_OOM;
+    if (!rc && cudaMallocHost((void**)&ctx->h_counters, (kWalkCounters + 8) * sizeof(unsigned long long)) != cudaSuccess) rc = FMM_E_OOM;
     if (!rc && cudaMallocHost((void**)&ctx->h_int, (kTreeShapeInts + 1) * sizeof(int)) != cudaSuccess) rc = FMM_E_OOM;
     if (!rc) {
         ctx->ev_ok = true;

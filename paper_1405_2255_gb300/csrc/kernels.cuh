@@ -143,27 +143,36 @@ __host__ __device__ inline int m2l_order(int x, int p) {
 }
 constexpr int kMacEstimate = 3;  // theta < 1 only (low-order estimate, Sec. 5.3.2)
 
+// device counters of a walk: [1] M2L pairs, [2] P2P pairs, [3] overflow flag, [kWalkFronts + k] the
+// frontier of step k (kWalkStopped set: a list or frontier overflowed in the step before)
+constexpr int kWalkFronts = 8, kWalkCounters = 64;
+constexpr unsigned long long kWalkStopped = 1ull << 62;
 struct WalkBuffers {
-    int2* front[2];
+    int2* front[2];  // step k reads front[k & 1]
     long long front_cap;
     int2* m2l;
     long long m2l_cap;
     int2* p2p;
     long long p2p_cap;
-    unsigned long long* counters;  // [0] next frontier, [1] m2l, [2] p2p, [3] overflow flag
+    unsigned long long* counters;  // kWalkCounters words
 };
-// the first frontier: (r, r) for the roots r = 0 .. nroots-1
-// count (nullable): receives nroots, the first frontier's length on the device
-void launch_walk_roots(int2* front, int nroots, cudaStream_t s, unsigned long long* count = nullptr);
-// one breadth-first step over a frontier of nfront pairs (host value); the next frontier is
-// counted in wb.counters[0]
-void launch_walk_step(Cells c, WalkParams wp, const int2* front_in, long long nfront, int2* front_out,
-                      WalkBuffers wb, cudaStream_t s);
-// the same with the frontier's length read on the device from *nfront_dev (no host round
-// trip between steps); the next frontier is counted in *out_cnt and wb.counters[5] keeps
-// the largest frontier demand seen
-void launch_walk_step_dev(Cells c, WalkParams wp, const int2* front_in, const unsigned long long* nfront_dev,
-                          int2* front_out, WalkBuffers wb, unsigned long long* out_cnt, cudaStream_t s);
+// the whole walk from the pairs (r, r) of the roots r = 0 .. nroots - 1: every step of a pair descends
+// one cell level on at least one side, so steps = 2 * levels + 1 end it (and stay below the counters).
+// A tree of few cells takes one kernel, a larger one a launch per step; nothing is read by the host.
+// The line lies where a cluster's 16 SMs take as long as all SMs and the launches (main walk with its
+// list sort, launches against one kernel: 1,027 cells 0.213 and 0.164 ms, 2,997 cells 0.319 and 0.338,
+// 6,474 cells 0.342 and 0.591; the estimate's walk visits fewer pairs: the estimate of 6,474 cells took
+// 0.576 and 0.542 ms, of 9,115 cells 0.620 and 0.590).
+constexpr int kWalkClusterCells = 2048, kWalkClusterCellsEst = 8192;
+inline int walk_steps(int nlev) { return 2 * nlev + 1; }
+void launch_walk(Cells c, WalkParams wp, WalkBuffers wb, int nroots, int ncells, int steps, cudaStream_t s);
+// the counters of a finished walk (host copy): the lists' lengths, whether one overflowed, the pairs left
+// after the last step and the largest frontier
+struct WalkResult {
+    long long n_m2l, n_p2p, left, need_front;
+    bool overflow;
+};
+WalkResult walk_result(const unsigned long long* h, int steps);
 // sort a pair list by (sink, first entry) -- the first entry taken as unsigned, so an adaptive
 // walk's M2L entries (wide: order bits above the source index) sort by (sink, order, source) --
 // then mark per-sink segments [seg_start, seg_end); tmp: list_sort_tmp_bytes(npairs, ncells)

@@ -5,8 +5,8 @@
 // Some callers cannot allocate device memory: simulation codes whose memory is
 // owned by their own pool allocator, and plugins that are not allowed to grow the
 // process's device footprint.  This entry point lets them evaluate systems of up
-// to kNoAllocMaxN particles.  It waits for its stream several times (level sizes
-// and frontier lengths are read on the host), like fmm_evaluate.
+// to kNoAllocMaxN particles.  It waits for its stream several times (the tree's
+// shape and the lists' lengths are read on the host), like fmm_evaluate.
 //
 // The scratch array is a file-scope __device__ variable: every GPU that loads
 // the library holds it (kNoAllocBytes) until the process exits.  Host code cannot
@@ -126,23 +126,16 @@ int walk_na(Run& r, WalkParams wp, int2* m2l, long long m2l_cap, int2* p2p, long
     wb.p2p = p2p;
     wb.p2p_cap = p2p_cap;
     wb.counters = r.counters;
-    int2 root = make_int2(0, 0);
-    NA_CU(cudaMemcpyAsync(wb.front[0], &root, sizeof root, cudaMemcpyHostToDevice, r.s));
-    NA_CU(cudaMemsetAsync(wb.counters, 0, 4 * sizeof(unsigned long long), r.s));
-    long long nfront = 1;
-    int cur = 0;
-    unsigned long long h[4];
-    while (nfront > 0) {
-        NA_CU(cudaMemsetAsync(wb.counters, 0, sizeof(unsigned long long), r.s));
-        launch_walk_step(r.c, wp, wb.front[cur], nfront, wb.front[cur ^ 1], wb, r.s);
-        NA_CU(cudaMemcpyAsync(h, wb.counters, sizeof h, cudaMemcpyDeviceToHost, r.s));
-        NA_CU(cudaStreamSynchronize(r.s));
-        if (h[3]) return fail_na(r, FMM_E_OVERFLOW, "interaction lists exceed the static scratch capacity");
-        nfront = (long long)h[0];
-        cur ^= 1;
-    }
-    *nm = (long long)h[1];
-    *np = (long long)h[2];
+    const int steps = walk_steps(r.nlev);
+    launch_walk(r.c, wp, wb, 1, r.nc, steps, r.s);
+    unsigned long long h[kWalkCounters];
+    NA_CU(cudaMemcpyAsync(h, wb.counters, sizeof h, cudaMemcpyDeviceToHost, r.s));
+    NA_CU(cudaStreamSynchronize(r.s));
+    const WalkResult w = walk_result(h, steps);
+    if (w.overflow) return fail_na(r, FMM_E_OVERFLOW, "interaction lists exceed the static scratch capacity");
+    if (w.left) return fail_na(r, FMM_E_CUDA, "the tree walk did not end within 2 x levels steps");
+    *nm = w.n_m2l;
+    *np = w.n_p2p;
     return 0;
 }
 
@@ -179,7 +172,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     r.perm = A.take<int>(n);
     unsigned long long* bounds = A.take<unsigned long long>(8);
     r.status = A.take<unsigned>(4);
-    r.counters = A.take<unsigned long long>(8);
+    r.counters = A.take<unsigned long long>(kWalkCounters);
     int* shape = A.take<int>(kTreeShapeInts);
     const long long cap = (long long)n + 21LL * (n / (prm.leaf_size + 1)) + 64;
     int* ib[6];

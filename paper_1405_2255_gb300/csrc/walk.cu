@@ -3,6 +3,8 @@
 // the current frontier of cell pairs and writes M2L pairs, P2P pairs and the next
 // frontier.  Afterwards the lists are sorted by (sink, source), which fixes the
 // order in which every sink accumulates its interactions.
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 namespace gb3 {
@@ -20,16 +22,20 @@ __device__ inline unsigned warp_excl(unsigned v, unsigned* tot) {
     return x - v;
 }
 
-// reserve `mine` slots in a list for each lane; returns the lane's first slot or -1 on overflow
+// reserve `mine` slots in a list for each lane; returns the lane's first slot or -1 on overflow (then
+// the overflow flag and the top bit of the next frontier's counter are set: the walk ends there)
 __device__ inline long long warp_reserve(unsigned mine, unsigned long long* counter, long long cap,
-                                         unsigned long long* overflow) {
+                                         unsigned long long* overflow, unsigned long long* next) {
     unsigned tot;
     unsigned ex = warp_excl(mine, &tot);
     unsigned long long base = 0;
     if ((threadIdx.x & 31) == 31 && tot) base = atomicAdd(counter, (unsigned long long)tot);
     base = __shfl_sync(0xffffffffu, base, 31);
     if (tot && (long long)(base + tot) > cap) {
-        if ((threadIdx.x & 31) == 31) atomicOr(overflow, 1ull);
+        if ((threadIdx.x & 31) == 31) {
+            atomicOr(overflow, 1ull);
+            atomicOr(next, kWalkStopped);
+        }
         return -1;
     }
     return (long long)(base + ex);
@@ -159,30 +165,21 @@ void launch_walk_prep(Cells c, const d4* cen, const double* P, int p, double eps
     note_launch();
 }
 
-// nfront_dev (nullable): the frontier's length on the device (read here, capped at the
-// buffer's capacity), else nfront; the next frontier is counted in *out_cnt
-// 32 registers (a few spills) so that the launch of 8 blocks per SM is one wave: the steps are
-// bound by the latency of the cell gathers
-__global__ void __launch_bounds__(256, 8) k_walk(Cells c, WalkParams wp, const int2* __restrict__ front_in, long long nfront,
-                       const unsigned long long* __restrict__ nfront_dev, int2* __restrict__ front_out, WalkBuffers wb,
-                       unsigned long long* __restrict__ out_cnt) {
-    if (nfront_dev) {
-        const unsigned long long nd = *nfront_dev;
-        if (blockIdx.x == 0 && threadIdx.x == 0 && nd) atomicMax(&wb.counters[5], nd);  // demand seen
-        // after an overflow the frontier may have holes: no further steps (the walk is redone)
-        if (*(volatile const unsigned long long*)&wb.counters[3]) return;
-        nfront = (long long)nd < wb.front_cap ? (long long)nd : wb.front_cap;
-    }
+// one step: pairs first, first + stride, ... of a frontier of nfront pairs (whole warps, so that the
+// lanes stay together); CG: the frontier was written by other blocks of this kernel (read through L2)
+template <bool CG>
+__device__ __forceinline__ void walk_step(const Cells& c, const WalkParams& wp, const int2* front_in,
+                                          long long nfront, int2* front_out, const WalkBuffers& wb,
+                                          unsigned long long* out_cnt, long long first, long long stride) {
     // cnt_A cnt_B < p2p_thresh as integers: the product of two counts is exact in FP64
     // below 2^53 and far above any threshold beyond it
     const double tc = ceil(wp.p2p_thresh);
     const long long thr = tc <= 0.0 ? 0LL : (tc >= 0x1p62 ? (1LL << 62) : (long long)tc);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < nfront; base += stride) {
-        long long i = base + threadIdx.x;
+    for (long long i = first; i - (threadIdx.x & 31) < nfront; i += stride) {
         int act = kActNone, A = -1, B = -1, nchA = 0, nchB = 0, chA = 0, chB = 0;
-        if (i < nfront && cell_active(c, front_in[i].y)) {  // a sink without active particles has no work
-            int2 pr = front_in[i];
+        int2 pr = make_int2(0, 0);
+        if (i < nfront) pr = CG ? __ldcg(front_in + i) : front_in[i];
+        if (i < nfront && cell_active(c, pr.y)) {  // a sink without active particles has no work
             A = pr.x;
             B = pr.y;
             const long long cntA = c.count[A], cntB = c.count[B];
@@ -254,9 +251,9 @@ __global__ void __launch_bounds__(256, 8) k_walk(Cells c, WalkParams wp, const i
         }
         unsigned nm = act == kActM2L, np = act == kActP2P;
         unsigned nf = act == kActSelf ? nchA * nchA : act == kActSplitA ? nchA : act == kActSplitB ? nchB : 0;
-        long long om = warp_reserve(nm, &wb.counters[1], wb.m2l_cap, &wb.counters[3]);
-        long long op = warp_reserve(np, &wb.counters[2], wb.p2p_cap, &wb.counters[3]);
-        long long of = warp_reserve(nf, out_cnt, wb.front_cap, &wb.counters[3]);
+        long long om = warp_reserve(nm, &wb.counters[1], wb.m2l_cap, &wb.counters[3], out_cnt);
+        long long op = warp_reserve(np, &wb.counters[2], wb.p2p_cap, &wb.counters[3], out_cnt);
+        long long of = warp_reserve(nf, out_cnt, wb.front_cap, &wb.counters[3], out_cnt);
         if (nm && om >= 0) wb.m2l[om] = make_int2(A, B);
         if (np && op >= 0) wb.p2p[op] = make_int2(A, B);
         if (nf && of >= 0) {
@@ -272,25 +269,92 @@ __global__ void __launch_bounds__(256, 8) k_walk(Cells c, WalkParams wp, const i
     }
 }
 
-__global__ void k_walk_roots(int2* front, int nroots, unsigned long long* count) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nroots; r += gridDim.x * blockDim.x) front[r] = make_int2(r, r);
-    if (count && blockIdx.x == 0 && threadIdx.x == 0) *count = (unsigned long long)nroots;
-}
-void launch_walk_roots(int2* front, int nroots, cudaStream_t s, unsigned long long* count) {
-    if (nroots > 0) k_walk_roots<<<grid_for(nroots, 256), 256, 0, s>>>(front, nroots, count); note_launch();
+// Step k reads the frontier's length from counters[kWalkFronts + k] and counts the next frontier in the
+// word after it.  32 registers (a few spills) so that the launch of 8 blocks per SM is one wave: the
+// steps are bound by the latency of the cell gathers
+__global__ void __launch_bounds__(256, 8) k_walk(const __grid_constant__ Cells c, const __grid_constant__ WalkParams wp,
+                                              const __grid_constant__ WalkBuffers wb, int k) {
+    unsigned long long* cnt = wb.counters + kWalkFronts + k;
+    const unsigned long long n = *cnt;
+    if (n == 0) return;
+    if (n & kWalkStopped) {  // after an overflow the frontier may have holes: no further steps
+        if (blockIdx.x == 0 && threadIdx.x == 0) cnt[1] = kWalkStopped;
+        return;
+    }
+    walk_step<false>(c, wp, wb.front[k & 1], (long long)n, wb.front[(k & 1) ^ 1], wb, cnt + 1,
+                     (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
-void launch_walk_step(Cells c, WalkParams wp, const int2* front_in, long long nfront, int2* front_out,
-                      WalkBuffers wb, cudaStream_t s) {
-    if (nfront <= 0) return;
-    k_walk<<<grid_for(nfront, 256, 16), 256, 0, s>>>(c, wp, front_in, nfront, nullptr, front_out, wb,
-                                                             &wb.counters[0]);
-    note_launch();
+// All steps of a small tree in one kernel of one cluster, whose blocks meet at the cluster's barrier
+// between the steps: a launch per step costs 4 to 8 us however short its frontier is.
+constexpr int kWalkClusterThreads = 1024;
+__global__ void __launch_bounds__(kWalkClusterThreads) k_walk_all(const __grid_constant__ Cells c,
+                                                                  const __grid_constant__ WalkParams wp,
+                                                                  const __grid_constant__ WalkBuffers wb, int nroots,
+                                                                  int steps) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    for (long long r = t; r < nroots; r += nt) wb.front[0][r] = make_int2((int)r, (int)r);
+    if (t == 0) wb.counters[kWalkFronts] = (unsigned long long)nroots;
+    for (int k = 0; k < steps; ++k) {
+        cl.sync();
+        unsigned long long* cnt = wb.counters + kWalkFronts + k;
+        // (written in the step before only, so every block reads the same)
+        const unsigned long long n = *(volatile unsigned long long*)cnt;
+        if (n == 0 || (n & kWalkStopped)) break;
+        walk_step<true>(c, wp, wb.front[k & 1], (long long)n, wb.front[(k & 1) ^ 1], wb, cnt + 1, t, nt);
+    }
+    cl.sync();
 }
-void launch_walk_step_dev(Cells c, WalkParams wp, const int2* front_in, const unsigned long long* nfront_dev,
-                          int2* front_out, WalkBuffers wb, unsigned long long* out_cnt, cudaStream_t s) {
-    k_walk<<<sm_count() * 8, 256, 0, s>>>(c, wp, front_in, 0, nfront_dev, front_out, wb, out_cnt);
+
+__global__ void k_walk_roots(int2* front, int nroots, unsigned long long* count) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nroots; r += gridDim.x * blockDim.x) front[r] = make_int2(r, r);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *count = (unsigned long long)nroots;
+}
+
+void launch_walk(Cells c, WalkParams wp, WalkBuffers wb, int nroots, int ncells, int steps, cudaStream_t s) {
+    cudaMemsetAsync(wb.counters, 0, kWalkCounters * sizeof(unsigned long long), s);
+    if (ncells <= (wp.mac == kMacEstimate ? kWalkClusterCellsEst : kWalkClusterCells)) {
+        static DeviceOnce once;
+        once_per_device(once, [] {
+            cudaFuncSetAttribute(k_walk_all, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        });
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.blockDim = dim3(kWalkClusterThreads);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        for (unsigned size = 16; size >= 8; size /= 2) {  // 8 blocks where the device has no room for 16
+            at.val.clusterDim.x = size;
+            cfg.gridDim = dim3(size);
+            if (cudaLaunchKernelEx(&cfg, k_walk_all, c, wp, wb, nroots, steps) == cudaSuccess) {
+                note_launch();
+                return;
+            }
+            cudaGetLastError();
+        }
+    }
+    k_walk_roots<<<grid_for(nroots, 256), 256, 0, s>>>(wb.front[0], nroots, wb.counters + kWalkFronts);
     note_launch();
+    for (int k = 0; k < steps; ++k) {
+        k_walk<<<sm_count() * 8, 256, 0, s>>>(c, wp, wb, k);
+        note_launch();
+    }
+}
+
+WalkResult walk_result(const unsigned long long* h, int steps) {
+    WalkResult r;
+    r.n_m2l = (long long)h[1];
+    r.n_p2p = (long long)h[2];
+    r.overflow = h[3] != 0;
+    r.left = (long long)(h[kWalkFronts + steps] & ~kWalkStopped);
+    r.need_front = 0;
+    for (int k = 0; k <= steps; ++k) r.need_front = std::max(r.need_front, (long long)(h[kWalkFronts + k] & ~kWalkStopped));
+    return r;
 }
 
 // ---------------------------------------------------------------- segments (the list sort: sort.cu)
