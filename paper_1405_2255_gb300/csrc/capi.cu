@@ -103,7 +103,7 @@ struct fmm_ctx {
     // ensemble of the current evaluation (nsys = 0: one system): system offsets and G
     // on the device, roots (first, count) of the non-empty systems
     Buf sys_off, sys_G, sys_roots, skey, skey_alt, spos, spos_alt;
-    int nsys = 0, nroots = 1;
+    int nsys = 0, nroots = 1, smallest = 0;  // (the smallest non-empty system's particles)
     // force evaluation for a subset (Sec. 7.1): per sorted particle and per cell activity
     Buf pact, act, act_i, act_scan;
     bool active_mode = false;
@@ -359,7 +359,9 @@ static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t 
         const size_t need = launch_p2p_mixed(P<float4>(ctx->xp), ctx->n, c, list,
                                              P<int>(ctx->seg_start), P<int>(ctx->seg_end), P<int>(ctx->leaves),
                                              ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), mode,
-                                             ctx->p2p_tmp.p, ctx->p2p_tmp.bytes, ctx->h_counters + kWalkCounters, s);
+                                             ctx->p2p_tmp.p, ctx->p2p_tmp.bytes, ctx->h_counters + kWalkCounters, s,
+                                             p2p_shares(ctx->nsys ? ctx->smallest : ctx->n),
+                                             ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
         if (need == ~(size_t)0) return fail(ctx, FMM_E_OVERFLOW, "P2P plan beyond 2^31 source ranges or n >= 2^29");
         if (need <= ctx->p2p_tmp.bytes) return 0;
         TRY(ensure(ctx->p2p_tmp, need));
@@ -965,6 +967,8 @@ int fmm_evaluate_batch(fmm_ctx* ctx, int nsys, const int64_t* offsets, const dou
     // the host arrays above are pageable and local: wait for the copies before returning
     ctx->nsys = nsys;
     ctx->nroots = (int)roots.size();
+    ctx->smallest = n;
+    for (const int2& r : roots) ctx->smallest = std::min(ctx->smallest, r.y);
     int rc = evaluate_device(ctx, n, x, mu, 1.0, nullptr, psi, acc, s, stats);
     cudaError_t e = cudaStreamSynchronize(s);
     ctx->nsys = 0;

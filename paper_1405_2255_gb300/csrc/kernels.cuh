@@ -31,6 +31,16 @@ struct Cells {
     const unsigned char* act = nullptr;
     const unsigned char* pact = nullptr;
 };
+// the system of particle i of an ensemble: the last k with off[k] <= i
+__device__ inline int system_of(const int* __restrict__ off, int nsys, int i) {
+    int lo = 0, hi = nsys - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= i) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
 __device__ __forceinline__ bool cell_active(const Cells& c, int cell) { return !c.act || c.act[cell]; }
 
 // ---------------------------------------------------------------- tree (tree.cu)
@@ -246,12 +256,16 @@ void launch_p2p_fp64(const d4* xm, Cells c, const int2* list, const int* seg_sta
 // leaf's centre for the others, 2 offsets for all, 3 two-float for all.  tmp holds the work
 // plan: at least p2p_plan_fixed_bytes(nleaves); the call plans, reads the plan's size on the
 // host (h_tot: 6 host words; the stream is synchronised once) and runs the P2P if tmp_bytes
-// holds it.  Returns the bytes the call needs: a value above tmp_bytes means nothing was
+// holds it.  shares: the pieces of small systems are shared by several warps (off, nsys: the systems
+// of an ensemble); it takes more scratch.  Returns the bytes the call needs: a value above tmp_bytes means nothing was
 // computed (call again with that much), ~0 a plan beyond 2^31 ranges or items or n >= 2^29.
 size_t p2p_plan_fixed_bytes(int nleaves);
 size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
                         const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, int mode,
-                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
+                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s,
+                        bool shares = false, const int* off = nullptr, int nsys = 0);
+// whether a forest whose smallest system has this many particles has pieces to be shared
+bool p2p_shares(int smallest_system);
 // FP64 P2P with a work plan as launch_p2p_mixed's (the same scratch, return value and host read);
 // want_f: psi receives sum mu / r^2 instead (eq. 6; acc is scratch)
 size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,

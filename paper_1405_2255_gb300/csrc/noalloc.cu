@@ -144,8 +144,11 @@ int p2p_na(Run& r, const float4* xp, const int2* list, const int* seg_start, con
            double* psi, double* acc, int mode) {
     unsigned long long h_tot[6] = {0, 0, 0, 0, 0, 0};
     const size_t have = r.p2p_tmp_bytes;
-    const size_t need = launch_p2p_mixed(xp, r.n, r.c, list, seg_start, seg_end, r.leaves, r.nleaves, psi, acc,
-                                         mode, r.p2p_tmp, have, h_tot, r.s);
+    size_t need = launch_p2p_mixed(xp, r.n, r.c, list, seg_start, seg_end, r.leaves, r.nleaves, psi, acc,
+                                   mode, r.p2p_tmp, have, h_tot, r.s, p2p_shares(r.n));
+    if (need > have)  // whole pieces take less scratch
+        need = launch_p2p_mixed(xp, r.n, r.c, list, seg_start, seg_end, r.leaves, r.nleaves, psi, acc, mode, r.p2p_tmp,
+                                have, h_tot, r.s);
     if (need > have) return fail_na(r, FMM_E_OVERFLOW, "the P2P work plan exceeds the static scratch capacity");
     return 0;
 }

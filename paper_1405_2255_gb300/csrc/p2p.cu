@@ -180,7 +180,8 @@ struct Chunk {
 // pair), then k = ceil(c / (2 S)) so that no item is empty.  Items longer than piece_steps steps
 // are split (see below).
 struct PlanMixed {
-    static constexpr unsigned piece_steps = 8192;
+    static constexpr unsigned piece_steps = 8192, sub_steps = 1024;
+    static constexpr int sub_n = 16384;  // particles of the largest system whose pieces are shared
     static constexpr int max_pieces = 64;
     static constexpr bool merge = true;
     static constexpr int nv = 4;  // sums per sink
@@ -209,7 +210,8 @@ struct PlanMixed {
 // Q <= 4 sinks per slot.  Short pieces (a step of 18 FP64 instructions holds a quarter of an SM for
 // 1152 cycles, so 256 steps are 0.14 ms) keep every SM busy to the end.
 struct PlanF64 {
-    static constexpr unsigned piece_steps = 256;
+    static constexpr unsigned piece_steps = 256, sub_steps = 0;
+    static constexpr int sub_n = 0;
     static constexpr int max_pieces = 1024;
     static constexpr bool merge = true;
     static constexpr int nv = 4;
@@ -235,7 +237,8 @@ struct PlanF64 {
 // The mixed tidal P2P: a slot holds two sinks as the halves of packed operations, and the R groups of
 // S lanes take shares of the source cells of their own: the fewest items k / R per source.
 struct PlanTidal {
-    static constexpr unsigned piece_steps = 1024;
+    static constexpr unsigned piece_steps = 1024, sub_steps = 0;
+    static constexpr int sub_n = 0;
     static constexpr int max_pieces = 256;
     static constexpr bool merge = false;
     static constexpr int nv = 6;
@@ -268,16 +271,24 @@ __device__ inline bool p2p_near(const d4& a, const d4& b) {
 // max_pieces pieces of about equal numbers of source cells, each with its own ranges, items
 // and FP64 partial sums, which k_p2p_reduce adds in piece order.  The split depends on the leaf
 // alone, so a system gives the same result in an ensemble as alone.
+// A piece of the mixed P2P of a small system is shared by U = its steps / sub_steps warps: its stream of
+// sources is cut at tile boundaries into U parts with ranges, items and partial sums of their own, so
+// the tiles and their FP32 sums are those of the whole piece.  With few leaves the longest item sets
+// the kernel's time: 1e4 particles (892 leaves) 0.37 ms with whole pieces, 0.18 ms with parts of 1024
+// steps; with enough leaves the parts only cost (their starts and sums; 1e5: 1.71 and 1.89 ms, 1e6: 4.74
+// and 5.03 ms), so systems of more than sub_n particles have none (counted is the leaf's own system: the
+// same alone and in an ensemble).
 
 // per leaf index t (one warp each): the number of its source cells nb[t] (the ranges it can need
-// at most: its own and its ancestors' segment lengths), its pieces np[t] and its sort key,
+// at most: its own and its ancestors' segment lengths), its pieces P and their parts U as np[t] =
+// P | U << 16 and its sort key,
 // descending in the length of a piece's items (a lane's steps, Q source particles / R; 0 for a leaf
 // without active particles); tot[0] += nb
 template <class PL>
 __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
-                            const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves,
-                            int* __restrict__ nb, int* __restrict__ np, uint64_t* __restrict__ keys,
-                            unsigned long long* __restrict__ tot) {
+                            const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int sub_n,
+                            int n, const int* __restrict__ off, int nsys, int* __restrict__ nb, int* __restrict__ np,
+                            uint64_t* __restrict__ keys, unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long my = 0;
@@ -300,9 +311,18 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
             int P = (int)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
             const int cap = e < PL::max_pieces ? (int)e : PL::max_pieces;
             P = P < 1 ? 1 : (P > cap ? (cap > 0 ? cap : 1) : P);
-            np[t] = P;
             const unsigned w32 = len ? (unsigned)(((unsigned long long)len + P - 1) / P) : 0u;
-            keys[t] = ((uint64_t)(255u - qlen8(w32)) << 32) | (unsigned)t;
+            unsigned U = 1;
+            if constexpr (PL::sub_steps > 0) {
+                int size = n;
+                if (off) {
+                    const int k = system_of(off, nsys, c.first[leaf]);
+                    size = off[k + 1] - off[k];
+                }
+                if (size <= sub_n) U = min(max(min(w32 / PL::sub_steps, (unsigned)(e / P)), 1u), 255u);
+            }
+            np[t] = P | (int)(U << 16);
+            keys[t] = ((uint64_t)(255u - qlen8((w32 + U - 1) / U)) << 32) | (unsigned)t;
         }
     }
     if (lane == 0 && my) atomicAdd(&tot[0], my);
@@ -321,8 +341,8 @@ __device__ inline unsigned long long warp_total(unsigned long long v, unsigned l
     return __shfl_sync(0xffffffffu, x, 31);
 }
 
-// per position q of the sorted order: its leaf index order[q], items nit[q] (pieces x items per
-// piece; 0 for a leaf without active particles) and pieces npc[q]; a split leaf (more than one
+// per position q of the sorted order: its leaf index order[q], pieces npc[q] (their parts counted) and
+// items nit[q] (pieces x items per piece; 0 for a leaf without active particles); a split leaf (more than one
 // piece) takes the first of its partial-sum slots pbase[q] (pieces x sinks of them; -1: not split)
 // and an entry (leaf index, first slot) of the split list.  tot[1] items, tot[3] pieces, tot[4]
 // slots, tot[5] split leaves; one atomic per warp and counter (a thread each took 60 us for 43,000
@@ -343,7 +363,7 @@ __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __res
             count = c.count[leaf];
             if (cell_active(c, leaf)) {
                 k = PL::chunk(count).k;
-                P = np[t];
+                P = (np[t] & 0xffff) * (np[t] >> 16);
             }
             nit[q] = k * P;
             npc[q] = P;
@@ -379,8 +399,9 @@ struct Pieces {
 };
 
 // ranges and items of piece v, one warp per piece (the pieces of a long leaf side by side: with one
-// warp per leaf the longest leaf set the kernel's time).  Piece j of a leaf (sorted position q, the
-// last with voff[q] <= v; j = v - voff[q]) takes the source cells j e / P .. (j + 1) e / P - 1 of
+// warp per leaf the longest leaf set the kernel's time); with parts, one warp per piece and its parts
+// (v the first of them).  Piece j of a leaf (sorted position q, the last with voff[q] <= v; j = (v -
+// voff[q]) / U) takes the source cells j e / P .. (j + 1) e / P - 1 of
 // the leaf's stream (its own segment, then each ancestor's; e cells in all) and owns that part of
 // the leaf's region [roff[t], roff[t] + e).  Within a piece the sources are merged per class in
 // stream order: an
@@ -390,16 +411,17 @@ struct Pieces {
 // not join start a run, a run's count and guard flag are summed in shared memory, and every run
 // but the last of its class is written out; the last stays open until the piece ends.  This is
 // the result of the sequential pass.
-// MERGE false: one far record per source cell, in stream order from the front (the tidal P2P).
+// Without PL::merge: one far record per source cell, in stream order from the front (the tidal P2P).
 constexpr int kEmitWarps = 4;
-template <bool MERGE>
+template <class PL>
 __global__ void __launch_bounds__(kEmitWarps * 32)
     k_p2p_emit(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int mode,
                const int* __restrict__ order, const int* __restrict__ roff, const int* __restrict__ nb,
                const int* __restrict__ ioff, const int* __restrict__ nit, const int* __restrict__ voff,
-               const int* __restrict__ npc, const int* __restrict__ pbase, int npieces, Pieces pc,
-               int2* __restrict__ ranges, int2* __restrict__ items) {
+               const int* __restrict__ npc, const int* __restrict__ np, const int* __restrict__ pbase, int npieces,
+               Pieces pc, int2* __restrict__ ranges, int2* __restrict__ cuts, int2* __restrict__ items) {
+    constexpr bool MERGE = PL::merge;
     __shared__ int rsum_all[kEmitWarps][33], rg_all[kEmitWarps][33];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int* rsum = rsum_all[wid];  // [0]: the open range carried in; [1 + L]: the run starting at lane L
@@ -413,11 +435,14 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
             if (voff[mid] <= v) q = mid;
             else hi = mid - 1;
         }
-        const int P = npc[q], pj = v - voff[q], t = order[q];
-        const int kper = nit[q] / P;  // items per piece
+        const int t = order[q], P = np[t] & 0xffff, U = np[t] >> 16;
+        if ((v - voff[q]) % U) continue;  // a later part of a piece: its first part's warp makes it
+        const int pj = (v - voff[q]) / U;
+        const int kper = nit[q] / (P * U);  // items per piece or part
         const int leaf = leaves[t];
         const int count = c.count[leaf];
-        for (int j = lane; j < kper; j += 32) items[ioff[q] + pj * kper + j] = make_int2(v, j);
+        for (int j = lane; j < kper * U; j += 32)
+            items[ioff[q] + pj * kper * U + j] = make_int2(v + j / kper, j % kper);
         const d4 sb = c.sr[leaf];
         const long long b0 = c.first[leaf], b1 = b0 + count;
         const long long e = nb[t];
@@ -513,7 +538,68 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
             pc.r1[v] = r1;
             pc.nnear[v] = cnt[1];
             pc.nfar[v] = cnt[0];
-            pc.part[v] = P > 1 ? pbase[q] + pj * count : -1;
+            pc.part[v] = P * U > 1 ? pbase[q] + pj * U * count : -1;
+        }
+        __syncwarp();
+        if (U == 1) continue;
+        // The parts: the piece's tiles are cut (tiles of T sources of the near records, then of the far
+        // ones); part u has the tiles u K .. (u + 1) K - 1, the last part the rest.  The records of a
+        // class that overlap its interval of sources are copied, clipped, behind those of the part
+        // before it (a record cut in two is in both, hence one place more per part; U is at most the
+        // number of the piece's source cells, so three times its region hold them).
+        const int nr[2] = {__shfl_sync(0xffffffffu, cnt[1], 0), __shfl_sync(0xffffffffu, cnt[0], 0)};  // near, far
+        const int rb[2] = {r0, r1 - nr[1]};
+        int2* cut = cuts + 3 * (size_t)r0;
+        const int T = p2p_tile(PL::chunk(count).R), K = max(1, (int)PL::sub_steps * PL::chunk(count).R / (2 * T));
+        long long total[2] = {0, 0};
+        for (int k = 0; k < 2; ++k) {
+            for (int i = lane; i < nr[k]; i += 32) total[k] += ranges[rb[k] + i].y & kRangeMax;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) total[k] += __shfl_xor_sync(0xffffffffu, total[k], o);
+        }
+        const long long ntl = (total[0] + T - 1) / T;  // near tiles
+        for (int u = 0; u < U; ++u) {
+            const long long t0 = (long long)u * K, t1 = u + 1 < U ? t0 + K : LLONG_MAX / T;
+            int at2[2], num[2];
+            for (int k = 0; k < 2; ++k) {
+                // the part's interval [a, b) of the class's sources
+                const long long s0 = k ? max(t0 - ntl, 0ll) : min(t0, ntl), s1 = k ? max(t1 - ntl, 0ll) : min(t1, ntl);
+                const long long a = min(s0 * T, total[k]), b = s1 > total[k] / T ? total[k] : s1 * T;
+                int2* dst = cut + (k ? nr[0] + U : 0);
+                long long before = 0;
+                int n = 0, firstrec = -1;
+                for (int i0 = 0; i0 < nr[k] && a < b; i0 += 32) {
+                    const int i = i0 + lane;
+                    const int2 rec = i < nr[k] ? ranges[rb[k] + i] : make_int2(0, 0);
+                    const int m = rec.y & kRangeMax;
+                    int x = m;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += y;
+                    }
+                    const long long p0 = before + x - m;  // sources before this record
+                    const long long lo = max(p0, a), hi = min(p0 + m, b);
+                    const unsigned on = __ballot_sync(0xffffffffu, lo < hi);
+                    if (on && firstrec < 0) firstrec = i0 + __ffs(on) - 1;
+                    if (lo < hi)
+                        dst[firstrec + u + n + __popc(on & below)] =
+                            make_int2(rec.x + (int)(lo - p0), (int)(hi - lo) | (rec.y & ~kRangeMax));
+                    n += __popc(on);
+                    before += __shfl_sync(0xffffffffu, x, 31);
+                    if (before >= b) break;
+                }
+                at2[k] = (int)(dst - ranges) + (firstrec < 0 ? 0 : firstrec + u);
+                num[k] = n;
+            }
+            if (lane == 0) {
+                pc.leaf[v + u] = t;
+                pc.r0[v + u] = at2[0];
+                pc.nnear[v + u] = num[0];
+                pc.r1[v + u] = at2[1] + num[1];
+                pc.nfar[v + u] = num[1];
+                pc.part[v + u] = pbase[q] + (pj * U + u) * count;
+            }
         }
         __syncwarp();
     }
@@ -530,7 +616,7 @@ __global__ void k_p2p_reduce(Cells c, const int* __restrict__ leaves, const int*
     const int nw = (gridDim.x * blockDim.x) >> 5;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nsplit; w += nw) {
         const int2 sp = split[w];
-        const int leaf = leaves[sp.x], P = np[sp.x];
+        const int leaf = leaves[sp.x], P = (np[sp.x] & 0xffff) * (np[sp.x] >> 16);
         const int first = c.first[leaf], count = c.count[leaf];
         for (int sk = lane; sk < count; sk += 32) {
             double v[NV];
@@ -1151,15 +1237,15 @@ PlanLayout plan_layout(void* base, int nleaves) {
 template <class PL, class RUN>
 size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, const int* seg_end, const int* leaves,
                     int nleaves, double* psi, double* acc, int mode, void* tmp, size_t tmp_bytes,
-                    unsigned long long* h_tot, cudaStream_t s, RUN run) {
+                    unsigned long long* h_tot, bool shares, const int* off, int nsys, cudaStream_t s, RUN run) {
     if (nleaves <= 0) return 0;
     if (n > kRangeMax) return ~(size_t)0;  // no range is ever cut: a leaf's region holds its source cells
     PlanLayout L = plan_layout(tmp, nleaves);
     if (tmp_bytes < L.bytes) return L.bytes;
     cudaMemsetAsync(L.tot, 0, 8 * sizeof(unsigned long long), s);
     cudaMemsetAsync(L.counter, 0, 4 * sizeof(unsigned), s);
-    k_p2p_count<PL><<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(c, list, seg_start, seg_end, leaves,
-                                                                               nleaves, L.nb, L.np, L.k0, L.tot);
+    k_p2p_count<PL><<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(
+        c, list, seg_start, seg_end, leaves, nleaves, shares ? PL::sub_n : 0, n, off, nsys, L.nb, L.np, L.k0, L.tot);
     note_launch();
     scan_exclusive_i32(L.nb, L.roff, nleaves, L.roff + nleaves, L.stmp, s);
     // the low 32 bits are the leaf index, already in order: sort the 8 length bits only
@@ -1174,11 +1260,13 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     const unsigned long long nranges = h_tot[0], nitems = h_tot[1], npieces = h_tot[3], nslots = h_tot[4],
                              nsplit = h_tot[5];
     if (nranges > (unsigned long long)INT_MAX || nitems > (unsigned long long)INT_MAX ||
-        nslots > (unsigned long long)INT_MAX)
+        nslots > (unsigned long long)INT_MAX || (shares && 4 * (nranges + nitems + npieces) > (unsigned long long)INT_MAX))
         return ~(size_t)0;
     auto a256 = [](unsigned long long b) { return (size_t)((b + 255) & ~255ull); };
     const size_t o_ranges = L.bytes, o_items = o_ranges + a256(nranges * sizeof(int2)),
-                 o_pieces = o_items + a256(nitems * sizeof(int2)), o_part = o_pieces + a256(npieces * 6 * sizeof(int)),
+                 o_pieces = o_items + a256(nitems * sizeof(int2)),
+                 o_cuts = o_pieces + a256(npieces * 6 * sizeof(int)),
+                 o_part = o_cuts + (shares ? a256(3 * nranges * sizeof(int2)) : 0),
                  need = o_part + a256(nslots * PL::nv * sizeof(double)) + 256;
     if (tmp_bytes < need) return need;
     unsigned char* b = (unsigned char*)tmp;
@@ -1190,9 +1278,9 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     double* part = (double*)(b + o_part);
     if (nitems == 0) return need;
     const unsigned g = grid_for((long long)npieces * 32, kEmitWarps * 32, 16);  // one warp per piece
-    k_p2p_emit<PL::merge><<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
-                                             L.nb, L.ioff, L.nit, L.voff, L.npc, L.pbase, (int)npieces, pc, ranges,
-                                             items);
+    k_p2p_emit<PL><<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
+                                             L.nb, L.ioff, L.nit, L.voff, L.npc, L.np, L.pbase, (int)npieces, pc, ranges,
+                                             (int2*)(b + o_cuts), items);
     note_launch();
     run(ranges, pc, items, (int)nitems, L.counter, part);
     if (nsplit > 0) {
@@ -1211,11 +1299,14 @@ int resident_blocks(K kern, int threads) {
 }
 }  // namespace
 
+bool p2p_shares(int smallest_system) { return smallest_system <= PlanMixed::sub_n; }
+
 size_t p2p_plan_fixed_bytes(int nleaves) { return plan_layout(nullptr, nleaves).bytes; }
 
 size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
                         const int* seg_end, const int* leaves, int nleaves, double* psi, double* acc, int mode,
-                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+                        void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s, bool shares,
+                        const int* off, int nsys) {
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
         auto go = [&](auto kern) {
@@ -1231,7 +1322,7 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
         note_launch();
     };
     return plan_and_run<PlanMixed>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, mode, tmp, tmp_bytes,
-                                   h_tot, s, run);
+                                   h_tot, shares, off, nsys, s, run);
 }
 
 size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,
@@ -1248,7 +1339,7 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
         note_launch();
     };
     return plan_and_run<PlanF64>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, 0, tmp, tmp_bytes, h_tot,
-                                 s, run);
+                                 false, nullptr, 0, s, run);
 }
 
 size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
@@ -1261,7 +1352,7 @@ size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list,
         note_launch();
     };
     return plan_and_run<PlanTidal>(n, c, list, seg_start, seg_end, leaves, nleaves, nullptr, T, 0, tmp, tmp_bytes,
-                                   h_tot, s, run);
+                                   h_tot, false, nullptr, 0, s, run);
 }
 
 }  // namespace gb3

@@ -139,16 +139,6 @@ void launch_keys(const double* x, int n, const unsigned long long* bounds, uint6
 // of the caller's arrays) is built as a forest: every system gets the bounding box,
 // root cube and keys it would get alone, and its particles stay in their own block
 // after sorting, so each tree is exactly the tree of the system alone.
-__device__ inline int system_of(const int* __restrict__ off, int nsys, int i) {
-    int lo = 0, hi = nsys - 1;  // last k with off[k] <= i
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= i) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 __global__ void k_bounds_init_sys(unsigned long long* b, int nsys) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= 6 * nsys; i += gridDim.x * blockDim.x)
         b[i] = (i < 6 * nsys && (i % 6) < 3) ? ~0ull : 0ull;  // [6 nsys]: the largest mass
