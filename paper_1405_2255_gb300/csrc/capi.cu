@@ -120,7 +120,7 @@ struct fmm_ctx {
                 &sys_roots, &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
     }
     // tree shape of the last evaluation
-    std::vector<int> lev_start;
+    std::vector<int> lev_start, lev_largest;  // first cell and largest cell's particles of every level
     int n = 0, ncells = 0, nleaves = 0;
     long long n_m2l = 0, n_p2p = 0, n_est_m2l = 0, n_est_p2p = 0;
 };
@@ -202,10 +202,11 @@ static int refresh_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, 
     const int nlev = (int)ctx->lev_start.size() - 1;
     TRY(ensure(ctx->owner, sizeof(int) * (size_t)n));
     launch_leaf_geometry(P<d4>(ctx->xm), c, P<int>(ctx->leaves), ctx->nleaves, P<unsigned>(ctx->status), s, true);
-    launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
+    if (geometry_needs_owner(n, ctx->ncells))
+        launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
     for (int L = nlev - 1; L >= 0; --L)
         launch_internal_geometry(P<d4>(ctx->xm), P<float4>(ctx->xp), c, ctx->lev_start[L],
-                                 ctx->lev_start[L + 1], n, P<int>(ctx->owner), P<unsigned long long>(ctx->rad_tmp),
+                                 ctx->lev_start[L + 1], ctx->lev_largest[L], n, P<int>(ctx->owner), P<unsigned long long>(ctx->rad_tmp),
                                  P<unsigned>(ctx->status), s, true);
     return 0;
 }
@@ -274,6 +275,7 @@ static int build_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, cu
     if (nc > cap) return fail(ctx, FMM_E_OVERFLOW, "cell capacity exceeded");
     ctx->lev_start.assign(1, 0);
     for (int L = 1; L <= kMaxLevel + 1 && ctx->lev_start.back() < nc; ++L) ctx->lev_start.push_back(ctx->h_int[L]);
+    ctx->lev_largest.assign(ctx->h_int + 24, ctx->h_int + 24 + ctx->lev_start.size() - 1);
     ctx->ncells = nc;
     ctx->nleaves = ctx->h_int[23];
 
@@ -284,10 +286,11 @@ static int build_tree(fmm_ctx* ctx, int n, const double* x, const double* mu, cu
     TRY(ensure(ctx->rad_tmp, sizeof(unsigned long long) * rad_tmp_u64_per_cell() * (size_t)maxlev_cells));
     TRY(ensure(ctx->owner, sizeof(int) * (size_t)n));
     launch_leaf_geometry(P<d4>(ctx->xm), c, P<int>(ctx->leaves), ctx->nleaves, P<unsigned>(ctx->status), s);
-    launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
+    if (geometry_needs_owner(n, ctx->ncells))
+        launch_leaf_owner(c, P<int>(ctx->leaves), ctx->nleaves, P<int>(ctx->owner), s);
     for (int L = nlev - 1; L >= 0; --L)
         launch_internal_geometry(P<d4>(ctx->xm), P<float4>(ctx->xp), c, ctx->lev_start[L],
-                                 ctx->lev_start[L + 1], n, P<int>(ctx->owner), P<unsigned long long>(ctx->rad_tmp),
+                                 ctx->lev_start[L + 1], ctx->lev_largest[L], n, P<int>(ctx->owner), P<unsigned long long>(ctx->rad_tmp),
                                  P<unsigned>(ctx->status), s);
     return 0;
 }
@@ -640,8 +643,8 @@ static int evaluate_device(fmm_ctx* ctx, int n, const double* x, const double* m
             memcpy(&st, &ctx->h_int[0], sizeof st);
             if (st & kStatInvalid) return fail(ctx, FMM_E_INVALID, "eps_b must be positive and finite");
         }
-        launch_minscale_leaves(P<double>(ctx->scale_sorted), c, P<int>(ctx->leaves), ctx->nleaves, s);
-        for (int L = nlev - 1; L >= 0; --L) launch_minscale_level(c, ctx->lev_start[L], ctx->lev_start[L + 1], s);
+        launch_minscale(P<double>(ctx->scale_sorted), c, P<int>(ctx->leaves), ctx->nleaves, ctx->lev_start.data(),
+                        nlev, s);
     }
     if (timing) CU(cudaEventRecord(ctx->ev[EV_EST], s));
     CU(cudaEventRecord(ctx->ev_join_est, s));

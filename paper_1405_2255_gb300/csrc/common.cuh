@@ -160,6 +160,23 @@ __device__ inline double warp_min(double v) {
     return v;
 }
 
+// the sums over the warp of four values in the order of a butterfly (xor 16, 8, 4, 2, 1), a lane passing
+// on the values it will not keep: value k ends in the lanes with (lane >> 3) & 3 = k
+__device__ inline double warp_sum4(const double (&v)[4], int lane) {
+    const bool h16 = lane & 16, h8 = lane & 8;
+    double a[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double keep = h16 ? v[i + 2] : v[i], send = h16 ? v[i] : v[i + 2];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+    const double keep = h8 ? a[1] : a[0], send = h8 ? a[0] : a[1];
+    double t = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    return t + __shfl_xor_sync(0xffffffffu, t, 1);
+}
+
 // ---------------------------------------------------------------- two-float sums
 // (hi, lo) with hi + lo the sum to about 2^-48 relative: TwoSum (Knuth) of the running sum
 // and each FP32 partial, in explicit round-to-nearest operations

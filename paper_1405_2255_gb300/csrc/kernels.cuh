@@ -91,10 +91,12 @@ void launch_tree(const uint64_t* keys, Cells c, int n, int leaf_size, int cap, c
 // radii, masses and centres of mass for the particles' new positions
 void launch_leaf_geometry(const d4* xm, Cells c, const int* leaves, int nleaves, unsigned* status,
                           cudaStream_t s, bool keep_centre = false);
-// xp: the two-float position records (launch_gather); owner: per particle, set by
-// launch_leaf_owner before the deepest level and moved up as the levels are processed
-// bottom-up; rad_tmp: rad_tmp_u64_per_cell() words per cell of the largest level
-void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_begin, int lev_end,
+// xp: the two-float position records (launch_gather); largest: the particles of the level's largest
+// cell; owner: per particle, set by launch_leaf_owner before the deepest level and moved up as the levels
+// are processed bottom-up (read only where geometry_needs_owner); rad_tmp:
+// rad_tmp_u64_per_cell() words per cell of the largest level
+bool geometry_needs_owner(int n, int ncells);
+void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_begin, int lev_end, int largest,
                               int n, int* owner, unsigned long long* rad_tmp, unsigned* status, cudaStream_t s,
                               bool keep_centre = false);
 void launch_leaf_owner(Cells c, const int* leaves, int nleaves, int* owner, cudaStream_t s);
@@ -108,10 +110,10 @@ void launch_p2m(const d4* xm, Cells c, const d4* cen, const int* leaves, int nle
 void launch_m2m_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M,
                       cudaStream_t s);
 void launch_power(const double* M, int ncells, int p, double* P, cudaStream_t s);
-// minimum of a per-particle scale over leaves, then over the daughters of one level
-void launch_minscale_leaves(const double* scale_sorted, Cells c, const int* leaves, int nleaves,
-                            cudaStream_t s);
-void launch_minscale_level(Cells c, int lev_begin, int lev_end, cudaStream_t s);
+// minimum of a per-particle scale over the (active) particles of every cell; lev_start (host): the first
+// cell of every level and the number of cells, nlev + 1 of them
+void launch_minscale(const double* scale_sorted, Cells c, const int* leaves, int nleaves, const int* lev_start, int nlev,
+                     cudaStream_t s);
 void launch_scale_from_caller(const double* scale, const int* perm, int n, double* scale_sorted,
                               cudaStream_t s, const int* e = nullptr);
 

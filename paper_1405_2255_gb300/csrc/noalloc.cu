@@ -221,9 +221,9 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     int* owner = A.take<int>(n);
     if (!A.ok) return fail_na(r, FMM_E_OVERFLOW, "static scratch too small for the tree");
     launch_leaf_geometry(r.xm, r.c, r.leaves, r.nleaves, r.status, s);
-    launch_leaf_owner(r.c, r.leaves, r.nleaves, owner, s);
+    if (geometry_needs_owner(n, nc)) launch_leaf_owner(r.c, r.leaves, r.nleaves, owner, s);
     for (int L = nl - 1; L >= 0; --L)
-        launch_internal_geometry(r.xm, xp, r.c, r.lev[L], r.lev[L + 1], n, owner, rad_tmp, r.status, s);
+        launch_internal_geometry(r.xm, xp, r.c, r.lev[L], r.lev[L + 1], h_shape[24 + L], n, owner, rad_tmp, r.status, s);
 
     // per-particle results and lists
     double* psi_far = A.take<double>(n);
@@ -299,8 +299,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
                 launch_p2p_fp64(r.xm, r.c, est_p2p, seg_start, seg_end, r.leaves, r.nleaves, psi_near, acc_near, s);
             launch_est_scale(r.c, r.leaves, r.nleaves, F1, acc_near, scale, s);
         }
-        launch_minscale_leaves(scale, r.c, r.leaves, r.nleaves, s);
-        for (int L = nl - 1; L >= 0; --L) launch_minscale_level(r.c, r.lev[L], r.lev[L + 1], s);
+        launch_minscale(scale, r.c, r.leaves, r.nleaves, r.lev, nl, s);
     }
 
     // A5-A6: upward pass

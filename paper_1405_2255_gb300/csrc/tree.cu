@@ -872,8 +872,20 @@ __device__ void meb_points_mtf_warp(float (*L)[3], int n, float c[3], float& rad
     rad = r0 < 0 ? 0 : r0;
 }
 
-// one warp per leaf: smallest enclosing ball, exact radius, mass, centre of mass
-constexpr int kGeoWarps = 4;
+// maxima of non-negative doubles by their bits (a comparison of doubles takes the FP64 pipe)
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+__device__ inline double warp_max_nonneg(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_nonneg(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+// one warp per leaf: smallest enclosing ball, exact radius, mass, centre of mass.  A block is one warp:
+// the leaves' solves differ by several times in length, and a block of four held its registers until the
+// longest was done (43,413 leaves of a Plummer sphere of 1e6: 1.15 ms).  The FP64 sums, square roots and
+// divisions are spread over the lanes (an instruction holds the FP64 pipe as long for one lane as for 32).
+constexpr int kGeoWarps = 1;
 __global__ void __maxnreg__(128) k_leaf_geometry(const d4* __restrict__ xm, Cells c,
                                                                  const int* __restrict__ leaves, int nleaves,
                                                                  unsigned* status, bool keep_centre) {
@@ -930,36 +942,37 @@ __global__ void __maxnreg__(128) k_leaf_geometry(const d4* __restrict__ xm, Cell
     }
     // radii as the square root of the largest squared distance (sqrt is monotonic and
     // correctly rounded, so this equals the largest distance)
-    double r2max = 0, m = 0, mx[3] = {0, 0, 0};
+    double r2max = 0, v[4] = {0, 0, 0, 0};  // v: mass and mass times position
     for (int i = lane; i < count; i += 32) {
-        double p[3];
-        ld3(X, i, p);
-        const double dx = p[0] - s[0], dy = p[1] - s[1], dz = p[2] - s[2];
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 > r2max) r2max = r2;
-        double w = X[i].w;
-        m += w;
-        for (int k = 0; k < 3; ++k) mx[k] += w * p[k];
+        const d4 q = X[i];
+        const double dx = q.x - s[0], dy = q.y - s[1], dz = q.z - s[2];
+        r2max = max_nonneg(r2max, dx * dx + dy * dy + dz * dz);
+        v[0] += q.w;
+        v[1] += q.w * q.x;
+        v[2] += q.w * q.y;
+        v[3] += q.w * q.z;
     }
-    const double rmax = sqrt(warp_max(r2max));
-    m = warp_sum(m);
-    for (int k = 0; k < 3; ++k) mx[k] = warp_sum(mx[k]);
+    r2max = warp_max_nonneg(r2max);
+    const double sum = warp_sum4(v, lane);  // the sum of value (lane >> 3) & 3
+    const double m = __shfl_sync(0xffffffffu, sum, 0);
+    const int k = (lane >> 3) & 3;
+    const double cm = k == 0 ? 0.0 : (m > 0 ? sum / m : (k == 1 ? s[0] : k == 2 ? s[1] : s[2]));
     double com[3];
-    for (int k = 0; k < 3; ++k) com[k] = (m > 0) ? mx[k] / m : s[k];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) com[d] = __shfl_sync(0xffffffffu, cm, 8 * (d + 1));
     double rc2 = 0;
     for (int i = lane; i < count; i += 32) {
-        double p[3];
-        ld3(X, i, p);
-        const double dx = p[0] - com[0], dy = p[1] - com[1], dz = p[2] - com[2];
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 > rc2) rc2 = r2;
+        const d4 q = X[i];
+        const double dx = q.x - com[0], dy = q.y - com[1], dz = q.z - com[2];
+        rc2 = max_nonneg(rc2, dx * dx + dy * dy + dz * dz);
     }
-    const double rc = sqrt(warp_max(rc2));
+    rc2 = warp_max_nonneg(rc2);
+    const double root = sqrt(lane == 1 ? rc2 : r2max);
     if (lane == 0) {
-        c.sr[cell] = mk4(s[0], s[1], s[2], rmax);
-        c.cr[cell] = mk4(com[0], com[1], com[2], rc);
+        c.sr[cell] = mk4(s[0], s[1], s[2], root);
         c.mass[cell] = m;
     }
+    if (lane == 1) c.cr[cell] = mk4(com[0], com[1], com[2], root);
 }
 
 void launch_leaf_geometry(const d4* xm, Cells c, const int* leaves, int nleaves, unsigned* status,
@@ -982,16 +995,25 @@ struct RadTmp {
 };
 size_t rad_tmp_u64_per_cell() { return 9; }
 
-__device__ inline void write_cen_f(const RadTmp& R, int k, const double s[3], const double m[3]) {
-    float* q = R.cen + 12 * (size_t)k;
+// FP32 bounds of the distance of particle i from a two-float centre q (hi[3], lo[3])
+__device__ inline void dist_bounds_f(const float4* __restrict__ xp, int i, const float* q, float& lb, float& ub) {
+    const float4 h = xp[2 * (size_t)i], l = xp[2 * (size_t)i + 1];
+    const float xhs[3] = {h.x, h.y, h.z}, xls[3] = {l.x, l.y, l.z};
+    float d2 = 0.f, mag = 0.f;
     for (int d = 0; d < 3; ++d) {
-        const float h = (float)s[d];
-        q[d] = h;
-        q[3 + d] = (float)(s[d] - (double)h);
-        const float hm = (float)m[d];
-        q[6 + d] = hm;
-        q[9 + d] = (float)(m[d] - (double)hm);
+        const float xh = xhs[d];
+        const float dd = __fadd_rn(__fsub_rn(xh, q[d]), __fsub_rn(xls[d], q[3 + d]));
+        d2 = __fmaf_rn(dd, dd, d2);
+        mag = __fadd_rn(mag, __fadd_rn(fabsf(xh), fabsf(q[d])));
     }
+    if (!(mag >= 0x1p-18f && mag <= 0x1p60f)) {
+        lb = 0.f;
+        ub = __int_as_float(0x7f800000);
+        return;
+    }
+    const float df = sqrtf(d2), E = mag * 0x1p-44f;
+    lb = fmaxf(0.f, df * (1.0f - 0x1p-20f) - E);
+    ub = df * (1.0f + 0x1p-20f) + E;
 }
 
 // Internal cells of one level: smallest ball enclosing the daughter balls (s_d, rho_d),
@@ -1001,9 +1023,23 @@ __device__ inline void write_cen_f(const RadTmp& R, int k, const double s[3], co
 // one block of kMebWarps warps per internal cell; warp w tries the support sets with
 // bit masks 1 + 32 w + lane (at most 4 daughters), and the block keeps the smallest
 // valid ball (ties: the smaller mask)
+// Then the cell's mass and centre of mass, and, for a cell of at most `small` particles, its exact
+// radii by the block (below); the radii of a larger cell are taken by all blocks over its level's
+// particles, k_internal_radii_lb and k_internal_radii.  With at most kLevelCells cells in the level, small
+// is kLevelRadii if no cell is larger (a launch in place of five: tree of 1e4 particles 0.54 -> 0.45 ms, of
+// 4096 0.52 -> 0.41) and else kCellRadii (the level's kernels run anyway, and a block takes 15 us for a cell
+// of 8192: tree of 1e5 0.733 ms with 2048, 0.748 with 4096, 0.804 with 8192); with more cells 0 (a block
+// per cell has too little to do: block step of 1e6 1.1 % slower).
+// keep_centre: a reused tree keeps its centres (one warp per block where the block takes no radii).
 constexpr int kMebWarps = 8;
-__global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(Cells c, int lev_begin, int lev_end,
-                                                                 unsigned* status, unsigned long long* tmp) {
+constexpr int kLevelRadii = 16384, kCellRadii = 2048, kLevelCells = 2048;
+__device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, const Cells& c, int cell,
+                           const float* q, const double (&s)[3], const double (&com)[3]);
+__global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __restrict__ xm,
+                                                                 const float4* __restrict__ xp, Cells c,
+                                                                 int lev_begin, int lev_end, unsigned* status,
+                                                                 unsigned long long* tmp, bool keep_centre,
+                                                                 int small) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int cell = lev_begin + blockIdx.x;
     if (cell >= lev_end) return;
@@ -1016,7 +1052,7 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(Cells c, int le
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         cen[i][0] = cen[i][1] = cen[i][2] = rad[i] = 0.f;
-        if (i < nch) {
+        if (i < nch && !keep_centre) {
             const d4 v = c.sr[ch + i];
             cen[i][0] = (float)(v.x - o.x);
             cen[i][1] = (float)(v.y - o.y);
@@ -1027,7 +1063,7 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(Cells c, int le
     float best = -1, bc[3] = {0, 0, 0};
     int bmask = 1 << 30;
     const int mask = 1 + lane + 32 * wid;
-    if (mask < (1 << nch) && __popc(mask) <= 4) {
+    if (!keep_centre && mask < (1 << nch) && __popc(mask) <= 4) {
         // the k-th daughter of the mask into slot k of the support set
         float sc[4][3] = {}, sr[4] = {};
         int k = 0;
@@ -1082,34 +1118,72 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(Cells c, int le
         wmask[wid] = bmask;
         wbc[wid][0] = bc[0]; wbc[wid][1] = bc[1]; wbc[wid][2] = bc[2];
     }
+    __shared__ double s_cen[6];
+    __shared__ float s_q[12];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kMebWarps; ++w) {
-            const float ob = wbest[w];
-            const int om = wmask[w];
-            if ((ob >= 0) && (best < 0 || ob < best || (ob == best && om < bmask))) {
-                best = ob; bmask = om;
-                bc[0] = wbc[w][0]; bc[1] = wbc[w][1]; bc[2] = wbc[w][2];
+    if (wid == 0) {
+        for (int w = 1; w < kMebWarps && !keep_centre; ++w) {
+            const float ob = wbest[w], b0 = wbest[0];
+            const int om = wmask[w], b1 = wmask[0];
+            const bool take = (ob >= 0) && (b0 < 0 || ob < b0 || (ob == b0 && om < b1));
+            __syncwarp();
+            if (take && lane == 0) {
+                wbest[0] = ob;
+                wmask[0] = om;
+                wbc[0][0] = wbc[w][0]; wbc[0][1] = wbc[w][1]; wbc[0][2] = wbc[w][2];
             }
+            __syncwarp();
         }
+        best = wbest[0];
+        bc[0] = wbc[0][0]; bc[1] = wbc[0][1]; bc[2] = wbc[0][2];
         if (best < 0) {  // no valid support set: the first daughter's centre
-            atomicOr(status, kStatMeb);
+            if (lane == 0 && !keep_centre) atomicOr(status, kStatMeb);
             bc[0] = bc[1] = bc[2] = 0.f;
         }
-        double m = 0, mx[3] = {0, 0, 0};
+        // lane 0 the mass, lanes 1 .. 3 the coordinates of the centre of mass
+        double m = 0, mx = 0;
         for (int i = 0; i < nch; ++i) {
             const double md = c.mass[ch + i];
             const d4 cm = c.cr[ch + i];
             m += md;
-            mx[0] += md * cm.x; mx[1] += md * cm.y; mx[2] += md * cm.z;
+            mx += md * (lane == 1 ? cm.x : lane == 2 ? cm.y : cm.z);
         }
         double s[3] = {o.x + (double)bc[0], o.y + (double)bc[1], o.z + (double)bc[2]};
-        double com[3];
-        for (int k = 0; k < 3; ++k) com[k] = (m > 0) ? mx[k] / m : s[k];
-        c.sr[cell] = mk4(s[0], s[1], s[2], 0.0);
-        c.cr[cell] = mk4(com[0], com[1], com[2], 0.0);
-        c.mass[cell] = m;
-        write_cen_f(RadTmp(tmp, lev_end - lev_begin), cell - lev_begin, s, com);
+        if (keep_centre) {
+            const d4 v = c.sr[cell];
+            s[0] = v.x; s[1] = v.y; s[2] = v.z;
+        }
+        if (lane >= 1 && lane <= 3) {
+            const double sl = lane == 1 ? s[0] : lane == 2 ? s[1] : s[2];
+            s_cen[lane - 1] = sl;
+            s_cen[lane + 2] = (m > 0) ? mx / m : sl;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            c.sr[cell] = mk4(s_cen[0], s_cen[1], s_cen[2], 0.0);
+            c.cr[cell] = mk4(s_cen[3], s_cen[4], s_cen[5], 0.0);
+            c.mass[cell] = m;
+        }
+        if (lane < 6) {  // two-float centres: s hi, s lo, com hi, com lo
+            const double v = s_cen[lane];
+            const float h = (float)v;
+            const int d = lane < 3 ? lane : lane + 3;
+            s_q[d] = h;
+            s_q[d + 3] = (float)(v - (double)h);
+        }
+    }
+    __syncthreads();
+    const double s[3] = {s_cen[0], s_cen[1], s_cen[2]}, com[3] = {s_cen[3], s_cen[4], s_cen[5]};
+    if (c.count[cell] <= small) {
+        cell_radii(xm, xp, c, cell, s_q, s, com);
+    } else if (threadIdx.x < 12) {  // for the level's radii kernels; bounds and keys start at 0
+        const RadTmp R(tmp, lev_end - lev_begin);
+        const int k = cell - lev_begin;
+        R.cen[12 * (size_t)k + threadIdx.x] = s_q[threadIdx.x];
+        if (threadIdx.x < 2) {
+            R.key[2 * k + threadIdx.x] = 0ull;
+            R.lb[2 * k + threadIdx.x] = 0.f;
+        }
     }
 }
 
@@ -1125,9 +1199,70 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(Cells c, int le
 // at most the largest distance, so the particle attaining it has an upper bound >= LB;
 // the second pass takes the FP64 distance of every particle whose upper bound reaches LB,
 // and the maximum over those is the maximum over all, bit for bit.
-// owner[i]: the particle's ancestor at the level processed last (its leaf to begin with).
-// The levels are processed bottom-up, so at level L the owner moves up one cell when it
-// lies below L; the particle belongs to an internal cell of level L iff its owner is one.
+// One block, its own cell (the centres in shared memory):
+__device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, const Cells& c, int cell,
+                           const float* q, const double (&s)[3], const double (&com)[3]) {
+    __shared__ int s_lb[2];
+    __shared__ unsigned long long s_key[2];
+    const int first = c.first[cell], end = first + c.count[cell], lane = threadIdx.x & 31;
+    if (threadIdx.x < 2) {
+        s_lb[threadIdx.x] = 0;
+        s_key[threadIdx.x] = 0ull;
+    }
+    __syncthreads();
+    float l0 = 0.f, l1 = 0.f;
+    for (int i = first + threadIdx.x; i < end; i += blockDim.x) {
+        float a, b, u;
+        dist_bounds_f(xp, i, q, a, u);
+        dist_bounds_f(xp, i, q + 6, b, u);
+        l0 = fmaxf(l0, a);
+        l1 = fmaxf(l1, b);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        l0 = fmaxf(l0, __shfl_xor_sync(0xffffffffu, l0, o));
+        l1 = fmaxf(l1, __shfl_xor_sync(0xffffffffu, l1, o));
+    }
+    if (lane == 0) {  // non-negative floats order as their bit patterns
+        atomicMax(&s_lb[0], __float_as_int(l0));
+        atomicMax(&s_lb[1], __float_as_int(l1));
+    }
+    __syncthreads();
+    l0 = __int_as_float(s_lb[0]);
+    l1 = __int_as_float(s_lb[1]);
+    double d2 = 0, e2 = 0;
+    for (int i = first + threadIdx.x; i < end; i += blockDim.x) {
+        float l, u0, u1;
+        dist_bounds_f(xp, i, q, l, u0);
+        dist_bounds_f(xp, i, q + 6, l, u1);
+        const bool want0 = u0 >= l0, want1 = u1 >= l1;
+        if (!want0 && !want1) continue;
+        const d4 p = xm[i];
+        if (want0) {
+            const double dx = p.x - s[0], dy = p.y - s[1], dz = p.z - s[2];
+            d2 = max_nonneg(d2, dx * dx + dy * dy + dz * dz);
+        }
+        if (want1) {
+            const double ex = p.x - com[0], ey = p.y - com[1], ez = p.z - com[2];
+            e2 = max_nonneg(e2, ex * ex + ey * ey + ez * ez);
+        }
+    }
+    d2 = warp_max_nonneg(d2);
+    e2 = warp_max_nonneg(e2);
+    if (lane == 0) {
+        atomicMax(&s_key[0], (unsigned long long)__double_as_longlong(d2));
+        atomicMax(&s_key[1], (unsigned long long)__double_as_longlong(e2));
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        const double r = sqrt(__longlong_as_double((long long)s_key[threadIdx.x]));
+        if (threadIdx.x == 0) c.sr[cell].w = r;
+        else c.cr[cell].w = r;
+    }
+}
+// All blocks, the cells of more than `small` particles of a level.
+// owner[i]: an ancestor of the particle at or below the level processed last (its leaf to begin with).
+// The levels are processed bottom-up, so at level L the owner moves up to the ancestor at or above L;
+// the particle belongs to such a cell of level L iff its owner is one.
 __global__ void k_leaf_owner(Cells c, const int* __restrict__ leaves, int nleaves, int* __restrict__ owner) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nleaves; t += gridDim.x * blockDim.x) {
         const int leaf = leaves[t];
@@ -1140,43 +1275,23 @@ void launch_leaf_owner(Cells c, const int* leaves, int nleaves, int* owner, cuda
         note_launch();
     }
 }
-__device__ inline int level_cell_up(const Cells& c, int L, int* __restrict__ owner, int i) {
+__device__ inline int level_cell_up(const Cells& c, int L, int small, int* __restrict__ owner, int i) {
     int a = owner[i];
     if (c.level[a] > L) {
-        a = c.parent[a];
+        do a = c.parent[a];
+        while (c.level[a] > L);
         owner[i] = a;
     }
-    return (c.level[a] == L && c.nchild[a] > 0) ? a : -1;
+    return (c.level[a] == L && c.count[a] > small && c.nchild[a] > 0) ? a : -1;
 }
-__device__ inline int level_cell_now(const Cells& c, int L, const int* __restrict__ owner, int i) {
+__device__ inline int level_cell_now(const Cells& c, int L, int small, const int* __restrict__ owner, int i) {
     const int a = owner[i];
-    return (c.level[a] == L && c.nchild[a] > 0) ? a : -1;
-}
-
-// FP32 bounds of the distance of particle i from a two-float centre q (hi[3], lo[3])
-__device__ inline void dist_bounds_f(const float4* __restrict__ xp, int i, const float* q, float& lb, float& ub) {
-    const float4 h = xp[2 * (size_t)i], l = xp[2 * (size_t)i + 1];
-    const float xhs[3] = {h.x, h.y, h.z}, xls[3] = {l.x, l.y, l.z};
-    float d2 = 0.f, mag = 0.f;
-    for (int d = 0; d < 3; ++d) {
-        const float xh = xhs[d];
-        const float dd = __fadd_rn(__fsub_rn(xh, q[d]), __fsub_rn(xls[d], q[3 + d]));
-        d2 = __fmaf_rn(dd, dd, d2);
-        mag = __fadd_rn(mag, __fadd_rn(fabsf(xh), fabsf(q[d])));
-    }
-    if (!(mag >= 0x1p-18f && mag <= 0x1p60f)) {
-        lb = 0.f;
-        ub = __int_as_float(0x7f800000);
-        return;
-    }
-    const float df = sqrtf(d2), E = mag * 0x1p-44f;
-    lb = fmaxf(0.f, df * (1.0f - 0x1p-20f) - E);
-    ub = df * (1.0f + 0x1p-20f) + E;
+    return (c.level[a] == L && c.count[a] > small && c.nchild[a] > 0) ? a : -1;
 }
 
 constexpr int kRadThreads = 256;
 __global__ void __launch_bounds__(kRadThreads) k_internal_radii_lb(const float4* __restrict__ xp, int n, Cells c,
-                                    int lev_begin, int lev_end, int* __restrict__ owner,
+                                    int lev_begin, int lev_end, int small, int* __restrict__ owner,
                                     unsigned long long* __restrict__ tmp) {
     __shared__ int s_cell;
     __shared__ float s_l[kRadThreads / 32][2];
@@ -1189,7 +1304,7 @@ __global__ void __launch_bounds__(kRadThreads) k_internal_radii_lb(const float4*
         int cell = -1;
         float l0 = 0.f, l1 = 0.f;
         if (i < pend) {
-            cell = level_cell_up(c, L, owner, i);
+            cell = level_cell_up(c, L, small, owner, i);
             if (cell >= 0) {
                 const float* q = R.cen + 12 * (size_t)(cell - lev_begin);
                 float u;
@@ -1238,7 +1353,7 @@ __global__ void __launch_bounds__(kRadThreads) k_internal_radii_lb(const float4*
 }
 
 __global__ void k_internal_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, int n, Cells c,
-                                 int lev_begin, int lev_end,
+                                 int lev_begin, int lev_end, int small,
                                  const int* __restrict__ owner, unsigned long long* __restrict__ tmp) {
     const RadTmp R(tmp, lev_end - lev_begin);
     const int L = c.level[lev_begin];
@@ -1247,7 +1362,7 @@ __global__ void k_internal_radii(const d4* __restrict__ xm, const float4* __rest
     for (int i0 = blockIdx.x * blockDim.x; i0 < pend - pbeg; i0 += gridDim.x * blockDim.x) {
         const int i = pbeg + i0 + threadIdx.x;
         if (i >= pend) continue;
-        const int cell = level_cell_now(c, L, owner, i);
+        const int cell = level_cell_now(c, L, small, owner, i);
         if (cell < 0) continue;
         const int k = cell - lev_begin;
         const float* q = R.cen + 12 * (size_t)k;
@@ -1270,55 +1385,34 @@ __global__ void k_internal_radii(const d4* __restrict__ xm, const float4* __rest
     }
 }
 
-__global__ void k_internal_radii_finish(Cells c, int lev_begin, int lev_end,
+__global__ void k_internal_radii_finish(Cells c, int lev_begin, int lev_end, int small,
                                         const unsigned long long* __restrict__ rad_tmp) {
     int cell = lev_begin + blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= lev_end || c.nchild[cell] == 0) return;
+    if (cell >= lev_end || c.nchild[cell] == 0 || c.count[cell] <= small) return;
     double d2 = key_dbl(rad_tmp[2 * (cell - lev_begin)]);
     double e2 = key_dbl(rad_tmp[2 * (cell - lev_begin) + 1]);
     c.sr[cell].w = sqrt(d2);
     c.cr[cell].w = sqrt(e2);
 }
 
-// a reused tree: the centres stay, mass and centre of mass from the daughters
-__global__ void k_internal_keep(Cells c, int lev_begin, int lev_end, unsigned long long* tmp) {
-    const int cell = lev_begin + blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= lev_end) return;
-    const int nch = c.nchild[cell];
-    if (nch == 0) return;
-    const int ch = c.child[cell];
-    double m = 0, mx[3] = {0, 0, 0};
-    for (int i = 0; i < nch; ++i) {
-        const double md = c.mass[ch + i];
-        const d4 cm = c.cr[ch + i];
-        m += md;
-        mx[0] += md * cm.x; mx[1] += md * cm.y; mx[2] += md * cm.z;
-    }
-    const d4 s = c.sr[cell];
-    const double com[3] = {m > 0 ? mx[0] / m : s.x, m > 0 ? mx[1] / m : s.y, m > 0 ? mx[2] / m : s.z};
-    c.cr[cell] = mk4(com[0], com[1], com[2], 0.0);
-    c.mass[cell] = m;
-    const double sv[3] = {s.x, s.y, s.z};
-    write_cen_f(RadTmp(tmp, lev_end - lev_begin), cell - lev_begin, sv, com);
-}
-
-void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_begin, int lev_end,
+void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_begin, int lev_end, int largest,
                               int n, int* owner, unsigned long long* rad_tmp, unsigned* status, cudaStream_t s,
                               bool keep_centre) {
     int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
-    // bounds and keys start at 0 (every distance is >= 0)
-    cudaMemsetAsync(rad_tmp, 0, sizeof(unsigned long long) * 3 * (size_t)ncl, s);
-    if (keep_centre) k_internal_keep<<<(ncl + 127) / 128, 128, 0, s>>>(c, lev_begin, lev_end, rad_tmp);
-    else k_internal_meb<<<(unsigned)ncl, kMebWarps * 32, 0, s>>>(c, lev_begin, lev_end, status, rad_tmp);
+    const int small = ncl > kLevelCells ? 0 : largest <= kLevelRadii ? kLevelRadii : kCellRadii;
+    k_internal_meb<<<(unsigned)ncl, keep_centre && small == 0 ? 32 : kMebWarps * 32, 0, s>>>(
+        xm, xp, c, lev_begin, lev_end, status, rad_tmp, keep_centre, small);
     note_launch();
-    k_internal_radii_lb<<<grid_for(n, kRadThreads, 16), kRadThreads, 0, s>>>(xp, n, c, lev_begin, lev_end, owner,
-                                                                     rad_tmp);
+    if (largest <= small) return;
+    k_internal_radii_lb<<<grid_for(n, kRadThreads, 16), kRadThreads, 0, s>>>(xp, n, c, lev_begin, lev_end, small,
+                                                                             owner, rad_tmp);
     note_launch();
-    k_internal_radii<<<grid_for(n, 256, 16), 256, 0, s>>>(xm, xp, n, c, lev_begin, lev_end, owner,
-                                                                  rad_tmp);
+    k_internal_radii<<<grid_for(n, 256, 16), 256, 0, s>>>(xm, xp, n, c, lev_begin, lev_end, small, owner, rad_tmp);
     note_launch();
-    k_internal_radii_finish<<<(ncl + 255) / 256, 256, 0, s>>>(c, lev_begin, lev_end, rad_tmp); note_launch();
+    k_internal_radii_finish<<<(ncl + 255) / 256, 256, 0, s>>>(c, lev_begin, lev_end, small, rad_tmp);
+    note_launch();
 }
+bool geometry_needs_owner(int n, int ncells) { return n > kLevelRadii || ncells > kLevelCells; }
 
 }  // namespace gb3

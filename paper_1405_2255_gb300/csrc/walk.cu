@@ -358,19 +358,32 @@ WalkResult walk_result(const unsigned long long* h, int steps) {
 }
 
 // ---------------------------------------------------------------- segments (the list sort: sort.cu)
-__global__ void k_segments(const int2* __restrict__ list, long long n, int* __restrict__ seg_start,
+// [seg_start, seg_end) of every cell's pairs: two binary searches, side by side, per cell
+__global__ void k_segments(const int2* __restrict__ list, long long n, int ncells, int* __restrict__ seg_start,
                            int* __restrict__ seg_end) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        int b = list[i].y;
-        if (i == 0 || list[i - 1].y != b) seg_start[b] = (int)i;
-        if (i == n - 1 || list[i + 1].y != b) seg_end[b] = (int)(i + 1);
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= ncells) return;
+    long long a0 = 0, b0 = n, a1 = 0, b1 = n;  // first pairs with sink >= c and > c
+    while (a0 < b0 || a1 < b1) {
+        const long long m0 = (a0 + b0) >> 1, m1 = (a1 + b1) >> 1;
+        const int y0 = a0 < b0 ? list[m0].y : 0, y1 = a1 < b1 ? list[m1].y : 0;
+        if (a0 < b0) {
+            if (y0 < c) a0 = m0 + 1;
+            else b0 = m0;
+        }
+        if (a1 < b1) {
+            if (y1 <= c) a1 = m1 + 1;
+            else b1 = m1;
+        }
     }
+    seg_start[c] = (int)a0;
+    seg_end[c] = (int)a1;
 }
 
 void launch_segments(const int2* list, long long npairs, int ncells, int* seg_start, int* seg_end, cudaStream_t s) {
-    cudaMemsetAsync(seg_start, 0, sizeof(int) * (size_t)ncells, s);
-    cudaMemsetAsync(seg_end, 0, sizeof(int) * (size_t)ncells, s);
-    if (npairs > 0) k_segments<<<grid_for(npairs, 256), 256, 0, s>>>(list, npairs, seg_start, seg_end); note_launch();
+    if (ncells <= 0) return;
+    k_segments<<<(ncells + 127) / 128, 128, 0, s>>>(list, npairs, ncells, seg_start, seg_end);
+    note_launch();
 }
 
 }  // namespace gb3
