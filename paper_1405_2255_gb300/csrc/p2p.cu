@@ -28,6 +28,7 @@
 // raw tile while the previous tile is computed, then converted into the structure-of-arrays
 // tile the pairs read (offsets from the leaf centre for far tiles); a tile holds one class.
 // Items run in decreasing order of their length (source particles / R) from an atomic counter.
+#include <algorithm>
 #include <climits>
 
 #include "kernels.cuh"
@@ -215,21 +216,29 @@ struct PlanF64 {
     static constexpr int max_pieces = 1024;
     static constexpr bool merge = true;
     static constexpr int nv = 4;
+    // (all lanes of a warp together: lane S - 1 looks at S slots; the least cost, of equal ones the most
+    // slots.  One lane through all 128 pairs took 20 us a call)
     __device__ static inline Chunk chunk(int c) {
-        Chunk r{1, 1, 1, 1};
-        if (c <= 0) return r;
+        const int S = (int)(threadIdx.x & 31) + 1, R = min(32 / S, 16);
         float best = 3.0e38f;
-        for (int S = min(c, 32); S >= 1; --S) {
-            const int R = min(32 / S, 16);
+        int bq = 1;
+        if (S <= c)
             for (int Q = 1; Q <= 4; ++Q) {
                 const int k = (c + Q * S - 1) / (Q * S);
                 const float cost = (float)(k * Q) / (float)R + 0.02f * (float)k;
                 if (cost < best) {
                     best = cost;
-                    r = Chunk{k, R, S, Q};
+                    bq = Q;
                 }
             }
-        }
+        const int least = __reduce_min_sync(0xffffffffu, __float_as_int(best));  // positive: ordered as integers
+        const int l = 31 - __clz(__ballot_sync(0xffffffffu, __float_as_int(best) == least));
+        if (c <= 0) return Chunk{1, 1, 1, 1};
+        Chunk r;
+        r.S = l + 1;
+        r.Q = __shfl_sync(0xffffffffu, bq, l);
+        r.R = min(32 / r.S, 16);
+        r.k = (c + r.Q * r.S - 1) / (r.Q * r.S);
         return r;
     }
 };
@@ -281,14 +290,14 @@ __device__ inline bool p2p_near(const d4& a, const d4& b) {
 
 // per leaf index t (one warp each): the number of its source cells nb[t] (the ranges it can need
 // at most: its own and its ancestors' segment lengths), its pieces P and their parts U as np[t] =
-// P | U << 16 and its sort key,
+// P | U << 16, its items per piece kc[t] and its sort key,
 // descending in the length of a piece's items (a lane's steps, Q source particles / R; 0 for a leaf
 // without active particles); tot[0] += nb
 template <class PL>
 __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                             const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int sub_n,
                             int n, const int* __restrict__ off, int nsys, int* __restrict__ nb, int* __restrict__ np,
-                            uint64_t* __restrict__ keys, unsigned long long* __restrict__ tot) {
+                            int* __restrict__ kc, uint64_t* __restrict__ keys, unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long my = 0;
@@ -302,10 +311,11 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) src += __shfl_xor_sync(0xffffffffu, src, o);
+        const Chunk ch = PL::chunk(c.count[leaf]);  // (by the whole warp)
         if (lane == 0) {
             nb[t] = (int)e;
             my += (unsigned long long)e;
-            const Chunk ch = PL::chunk(c.count[leaf]);
+            kc[t] = ch.k;
             const unsigned long long l = (unsigned long long)ch.Q * (unsigned long long)src / (unsigned long long)ch.R + 1;
             const unsigned len = !cell_active(c, leaf) ? 0u : (l > 0xfffffffeull ? 0xfffffffeu : (unsigned)l);
             int P = (int)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
@@ -347,9 +357,8 @@ __device__ inline unsigned long long warp_total(unsigned long long v, unsigned l
 // and an entry (leaf index, first slot) of the split list.  tot[1] items, tot[3] pieces, tot[4]
 // slots, tot[5] split leaves; one atomic per warp and counter (a thread each took 60 us for 43,000
 // leaves).
-template <class PL>
 __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __restrict__ leaves, int nleaves, Cells c,
-                             const int* __restrict__ np, int* __restrict__ order, int* __restrict__ nit,
+                             const int* __restrict__ np, const int* __restrict__ kc, int* __restrict__ order, int* __restrict__ nit,
                              int* __restrict__ npc, int* __restrict__ pbase, int2* __restrict__ split,
                              unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
@@ -362,7 +371,7 @@ __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __res
             const int leaf = leaves[t];
             count = c.count[leaf];
             if (cell_active(c, leaf)) {
-                k = PL::chunk(count).k;
+                k = kc[t];
                 P = (np[t] & 0xffff) * (np[t] >> 16);
             }
             nit[q] = k * P;
@@ -1193,7 +1202,7 @@ namespace {
 // layout of the fixed part of the scratch (depends on the number of leaves only)
 struct PlanLayout {
     uint64_t *k0, *k1;
-    int *order, *nb, *roff, *np, *npc, *voff, *nit, *ioff, *pbase, *stmp, *rtmp;
+    int *order, *nb, *roff, *np, *kc, *npc, *voff, *nit, *ioff, *pbase, *stmp, *rtmp;
     int2* split;
     unsigned long long* tot;  // [0] ranges, [1] items, [3] pieces, [4] partial slots, [5] split
                               // leaves ([2] unused)
@@ -1217,6 +1226,7 @@ PlanLayout plan_layout(void* base, int nleaves) {
     L.nb = (int*)take(nl * 4);
     L.roff = (int*)take((nl + 1) * 4);
     L.np = (int*)take(nl * 4);
+    L.kc = (int*)take(nl * 4);
     L.npc = (int*)take(nl * 4);
     L.voff = (int*)take((nl + 1) * 4);
     L.nit = (int*)take(nl * 4);
@@ -1245,12 +1255,12 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     cudaMemsetAsync(L.tot, 0, 8 * sizeof(unsigned long long), s);
     cudaMemsetAsync(L.counter, 0, 4 * sizeof(unsigned), s);
     k_p2p_count<PL><<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(
-        c, list, seg_start, seg_end, leaves, nleaves, shares ? PL::sub_n : 0, n, off, nsys, L.nb, L.np, L.k0, L.tot);
+        c, list, seg_start, seg_end, leaves, nleaves, shares ? PL::sub_n : 0, n, off, nsys, L.nb, L.np, L.kc, L.k0, L.tot);
     note_launch();
     scan_exclusive_i32(L.nb, L.roff, nleaves, L.roff + nleaves, L.stmp, s);
     // the low 32 bits are the leaf index, already in order: sort the 8 length bits only
     const int flip = radix_sort_pairs_bits(L.k0, nullptr, L.k1, nullptr, nleaves, L.rtmp, 32, 40, s);
-    k_p2p_nitems<PL><<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.order,
+    k_p2p_nitems<<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.kc, L.order,
                                                             L.nit, L.npc, L.pbase, L.split, L.tot);
     note_launch();
     scan_exclusive_i32(L.nit, L.ioff, nleaves, L.ioff + nleaves, L.stmp, s);
@@ -1290,12 +1300,16 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     }
     return need;
 }
-// persistent blocks of a kernel: as many as are resident on the device at once
+// persistent blocks of a kernel whose warps take the items: as many as are resident on the device at once
+// (at most per_sm per SM), but no more than the items need, so that a few items are spread over the SMs
+// (with every resident block some SMs' warps took several of the long items: the estimate of 4096
+// particles in FP64 0.65 ms)
 template <class K>
-int resident_blocks(K kern, int threads) {
+int item_blocks(K kern, int threads, int nitems, int per_sm = 32) {
     int bps = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads, 0);
-    return sm_count() * (bps < 1 ? 1 : bps);
+    const int w = threads / 32;
+    return std::min(sm_count() * std::min(bps < 1 ? 1 : bps, per_sm), (nitems + w - 1) / w);
 }
 }  // namespace
 
@@ -1310,7 +1324,7 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
         auto go = [&](auto kern) {
-            const int nblocks = resident_blocks(kern, kP2PWarpsM * 32);
+            const int nblocks = item_blocks(kern, kP2PWarpsM * 32, nitems);
             mark_begin(s);
             kern<<<nblocks, kP2PWarpsM * 32, 0, s>>>(xp, c, leaves, ranges, pc, items, nitems, counter, psi, acc, part);
             mark_end(s);
@@ -1331,7 +1345,8 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
         auto go = [&](auto kern) {
-            const int nblocks = resident_blocks(kern, kP2PWarpsD * 32);
+            // eight warps per SM keep the FP64 pipe busy; more only take items early
+            const int nblocks = item_blocks(kern, kP2PWarpsD * 32, nitems, 2);
             kern<<<nblocks, kP2PWarpsD * 32, 0, s>>>(xm, c, leaves, ranges, pc, items, nitems, counter, psi, acc, part);
         };
         if (want_f) go(k_p2p_f64<true>);
@@ -1347,7 +1362,7 @@ size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list,
                              size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
-        k_p2p_tidal_mixed<<<resident_blocks(k_p2p_tidal_mixed, kTidWarps * 32), kTidWarps * 32, 0, s>>>(
+        k_p2p_tidal_mixed<<<item_blocks(k_p2p_tidal_mixed, kTidWarps * 32, nitems), kTidWarps * 32, 0, s>>>(
             xp, c, leaves, ranges, pc, items, nitems, counter, T, part);
         note_launch();
     };
