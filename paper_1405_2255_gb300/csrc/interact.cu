@@ -501,106 +501,169 @@ void launch_m2l_split(const int2* list, const int* seg_start, const int* seg_end
 
 // ---------------------------------------------------------------- L2L
 // F_n^m(s') += sum_{k<=p-n} sum_l Upsilon_k^{l*}(s - s') F_{n+k}^{m+l}(s) for every
-// cell of one level (s = its parent's centre), one warp per cell.
-__global__ void __launch_bounds__(128) k_l2l(Cells c, const d4* __restrict__ cen, int lev_begin, int lev_end, int p,
-                                             double* __restrict__ F, LaneSched sched) {
+// cell of one level (s = its parent's centre).  One block of four warps per cell: a thread per output, the
+// outputs with the most terms in the first 32, and every warp a quarter of each output's terms.
+// What bounds it: the FP64 pipe, of which a warp has a quarter of an SM's, and whose instructions cost the
+// same however many lanes are active.  A level of few cells is as long as one cell: at p = 14 46 us with the
+// outputs dealt out to the warps, 30 us with their terms; 12 levels of a cusp of 6e4 0.94 ms with
+// all of a cell in one warp, 0.52 ms so.
+constexpr int kL2LWarps = 4;
+__global__ void __launch_bounds__(kL2LWarps * 32) k_l2l(Cells c, const d4* __restrict__ cen, int lev_begin, int p,
+                                                        double* __restrict__ F) {
     extern __shared__ cd csm[];
-    const int wpb = blockDim.x >> 5;
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
-    cd* X = csm + (size_t)wid * 2 * nco;
+    const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+    const int nco = ncoef(p), nout = out_count(p);
+    cd* X = csm;
     cd* Y = X + nco;
-    int cell = lev_begin + blockIdx.x * wpb + wid;
-    if (cell >= lev_end || !cell_active(c, cell)) return;
-    int par = c.parent[cell];
+    cd* part = Y + nco;  // [kL2LWarps][nout]
+    const int cell = lev_begin + blockIdx.x;
+    if (!cell_active(c, cell)) return;
+    const int par = c.parent[cell];
     const d4 s = cen[par], sp = cen[cell];
-    if (lane <= p) upsilon_column(p, lane, s.x - sp.x, s.y - sp.y, s.z - sp.z, X, true);
-    expand_real(p, F + (size_t)par * nco, Y, false, lane, 32);
-    __syncwarp();
+    const int t1 = (2 * (p + 1) + 31) & ~31;  // the warps after the columns' take F
+    if (t < t1) upsilon_columns2(p, t, s.x - sp.x, s.y - sp.y, s.z - sp.z, X, true);
+    else expand_real(p, F + (size_t)par * nco, Y, false, t - t1, kL2LWarps * 32 - t1);
+    __syncthreads();
+    for (int o = lane; o < nout; o += 32) {
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
+        // terms [i0, i1) of (p - n + 1)^2, term k^2 + k + l
+        const int all = (p - n + 1) * (p - n + 1), i0 = all * wid / kL2LWarps, i1 = all * (wid + 1) / kL2LWarps;
+        cd4 sum{0.0, 0.0, 0.0, 0.0};
+        int k = (int)sqrtf((float)i0);
+        while (k * k > i0) --k;
+        while ((k + 1) * (k + 1) <= i0) ++k;
+        for (; k * k < i1; ++k) {
+            const int c0 = k * k + k;
+            const cd *xk = X + c0, *yk = Y + (n + k) * (n + k) + (n + k) + m;
+            const int l1 = min(k, i1 - 1 - c0);
+#pragma unroll 4
+            for (int l = max(-k, i0 - c0); l <= l1; ++l) sum.add(xk[l], yk[l]);
+        }
+        part[wid * nout + o] = sum.sum();
+    }
+    __syncthreads();
     double* out = F + (size_t)cell * nco;
-    const int cnt = sched.cnt[lane];
-    for (int q = 0; q < cnt; ++q) {
-        int n = sched.n[lane][q], m = sched.m[lane][q];
-        cd v = contract(p, n, m, X, Y);
+    for (int o = t; o < nout; o += kL2LWarps * 32) {
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
+        cd v = part[o];
+#pragma unroll
+        for (int w = 1; w < kL2LWarps; ++w) v = v + part[w * nout + o];
         out[cix(n, m)] += v.re;
         if (m) out[cix(n, -m)] += v.im;
     }
 }
 
 void launch_l2l_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* F, cudaStream_t s) {
-    int ncl = lev_end - lev_begin;
-    if (ncl <= 0) return;
-    const int wpb = 4;
-    size_t sm = (size_t)wpb * 2 * ncoef(p) * sizeof(cd);
-    LaneSched sched = make_lane_sched(p, kSchedDown);
+    if (lev_end <= lev_begin) return;
     init_rec_tables();
-    k_l2l<<<(ncl + wpb - 1) / wpb, wpb * 32, sm, s>>>(c, cen, lev_begin, lev_end, p, F, sched); note_launch();
+    const size_t sm = (size_t)(2 * ncoef(p) + kL2LWarps * out_count(p)) * sizeof(cd);
+    k_l2l<<<lev_end - lev_begin, kL2LWarps * 32, sm, s>>>(c, cen, lev_begin, p, F);
+    note_launch();
 }
 
 // ---------------------------------------------------------------- L2P
 // Psi_n^m(x_b) = sum_{k<=p-n} sum_l Upsilon_k^{l*}(s_B - x_b) F_{n+k}^{m+l}(s_B) for
-// n = 0, 1; psi = Psi_0^0, a = -(Re Psi_1^1, Im Psi_1^1, Psi_1^0).  One block per
-// leaf, F in shared memory, one thread per particle streaming the Upsilon columns.
-constexpr int kL2PThreads = 64;
+// n = 0, 1; psi = Psi_0^0, a = -(Re Psi_1^1, Im Psi_1^1, Psi_1^0).  One thread per particle streams the
+// columns of Y = Upsilon(s_B - x_b).
+// The terms of one (k, |l|) are linear in Re Y and Im Y: with F^{-l} = (-1)^l conj(F^l), psi and Psi_1^0
+// take 2 Re and 2 Im of F_k^l and F_{k+1}^l, Psi_1^1 takes A + B of Re Y and i (B - A) of Im Y,
+// A = F_{k+1}^{1+l}, B = (-1)^l F_{k+1}^{1-l}.  These eight weights of a (k, l) are formed once per leaf;
+// a particle then has 8 multiply-adds and 5 operations of the recurrence per (k, l).
+// What bounds it: the FP64 pipe, so a block takes the particles of kL2PLeaves leaves together to fill its
+// warps.  1e5 particles, p = 10: 0.69 ms with a block per leaf, eq. 7 term by term and a division per
+// (k, l), 0.32 ms so.
+constexpr int kL2PThreads = 128;
+constexpr int kL2PLeaves = 8;
+struct L2PWeights {
+    double r[4], i[4];  // of Re Y and Im Y in psi, Psi_1^0, Re Psi_1^1, Im Psi_1^1
+};
 __global__ void __launch_bounds__(kL2PThreads) k_l2p(const d4* __restrict__ xm, Cells c, const d4* __restrict__ cen,
                                                      const int* __restrict__ leaves, int nleaves, int p,
                                                      const double* __restrict__ F, double* __restrict__ psi,
                                                      double* __restrict__ acc) {
-    extern __shared__ cd Fc[];
-    const int nco = ncoef(p);
-    for (int t = blockIdx.x; t < nleaves; t += gridDim.x) {
-        const int cell = leaves[t];
-        if (!cell_active(c, cell)) continue;  // block-uniform
+    extern __shared__ __align__(16) unsigned char l2psm[];
+    L2PWeights* wt = (L2PWeights*)l2psm;  // [kL2PLeaves][npair], (l, k) with l <= k, columns l one after another
+    __shared__ int s_cell[kL2PLeaves], s_end[kL2PLeaves];
+    const int nco = ncoef(p), npair = out_count(p);
+    for (int t0 = blockIdx.x * kL2PLeaves; t0 < nleaves; t0 += gridDim.x * kL2PLeaves) {
         __syncthreads();
-        expand_real(p, F + (size_t)cell * nco, Fc, false, threadIdx.x, blockDim.x);
+        if (threadIdx.x < 32) {
+            const int u = threadIdx.x;
+            const int cell = u < kL2PLeaves && t0 + u < nleaves ? leaves[t0 + u] : -1;
+            int sum = cell >= 0 && cell_active(c, cell) ? c.count[cell] : 0;
+#pragma unroll
+            for (int d = 1; d < kL2PLeaves; d *= 2) {
+                const int v = __shfl_up_sync(0xffffffffu, sum, d);
+                if (u >= d) sum += v;
+            }
+            if (u < kL2PLeaves) {
+                s_cell[u] = cell;
+                s_end[u] = sum;  // particles of the leaves up to this one
+            }
+        }
         __syncthreads();
-        const d4 s = cen[cell];
-        const int first = c.first[cell], count = c.count[cell];
-        for (int j = threadIdx.x; j < count; j += blockDim.x) {
-            const d4 xb = xm[first + j];
-            const double x = s.x - xb.x, y = s.y - xb.y, z = s.z - xb.z;
-            const double r2 = x * x + y * y + z * z;
-            double p00 = 0.0;
-            cd p10 = mkc(0.0, 0.0), p11 = mkc(0.0, 0.0);
-            cd d = mkc(1.0, 0.0);
-            for (int l = 0; l <= p; ++l) {
-                if (l > 0) {
-                    double sc = 1.0 / (2.0 * l);
-                    d = cd{sc * (x * d.re - y * d.im), sc * (x * d.im + y * d.re)};
-                }
-                const double sg = (l & 1) ? -1.0 : 1.0;
-                cd prev2 = mkc(0.0, 0.0), prev = d;
-                for (int k = l; k <= p; ++k) {
-                    cd Y;
-                    if (k == l) Y = d;
-                    else {
-                        double inv = 1.0 / (double)(k * k - l * l);
-                        double a = (2.0 * k - 1.0) * z;
-                        Y = cd{(a * prev.re - r2 * prev2.re) * inv, (a * prev.im - r2 * prev2.im) * inv};
-                        prev2 = prev;
-                        prev = Y;
-                    }
-                    const cd Xp = conjc(Y);                 // X_k^l
-                    const cd Xn = cd{sg * Y.re, sg * Y.im};  // X_k^{-l} = (-1)^l Upsilon_k^l
-                    const cd* Fk = Fc + k * k + k;
-                    if (l == 0) p00 += Xp.re * Fk[0].re - Xp.im * Fk[0].im;
-                    else p00 += 2.0 * (Xp.re * Fk[l].re - Xp.im * Fk[l].im);
-                    if (k < p) {
-                        const cd* Fk1 = Fc + (k + 1) * (k + 1) + (k + 1);
-                        cmac(p10, Xp, Fk1[l]);
-                        cmac(p11, Xp, Fk1[1 + l]);
-                        if (l > 0) {
-                            cmac(p10, Xn, Fk1[-l]);
-                            cmac(p11, Xn, Fk1[1 - l]);
-                        }
-                    }
+        const int total = s_end[kL2PLeaves - 1];
+        for (int i = threadIdx.x; i < kL2PLeaves * npair; i += blockDim.x) {
+            const int u = i / npair, r = i - u * npair;
+            if (s_end[u] == (u ? s_end[u - 1] : 0)) continue;
+            int l = 0, b = 0;
+            while (r >= b + p + 1 - l) b += p + 1 - l++;
+            const int k = l + r - b;
+            const double* Fr = F + (size_t)s_cell[u] * nco;
+            const cd f0 = load_real_storage(Fr, k, l);
+            cd f1 = mkc(0.0, 0.0), A = f1, B = f1;
+            if (k < p) {
+                f1 = load_real_storage(Fr, k + 1, l);
+                A = load_real_storage(Fr, k + 1, 1 + l);
+                if (l) {
+                    B = load_real_storage(Fr, k + 1, 1 - l);
+                    if (l & 1) B = mkc(-B.re, -B.im);
                 }
             }
-            const int i = first + j;
-            psi[i] = p00;
-            acc[3 * (size_t)i] = -p11.re;
-            acc[3 * (size_t)i + 1] = -p11.im;
-            acc[3 * (size_t)i + 2] = -p10.re;
+            const double e = l ? 2.0 : 1.0;
+            L2PWeights w;
+            w.r[0] = e * f0.re;
+            w.r[1] = e * f1.re;
+            w.r[2] = A.re + B.re;
+            w.r[3] = A.im + B.im;
+            w.i[0] = e * f0.im;
+            w.i[1] = e * f1.im;
+            w.i[2] = A.im - B.im;
+            w.i[3] = B.re - A.re;
+            wt[i] = w;
+        }
+        __syncthreads();
+        for (int j = threadIdx.x; j < total; j += blockDim.x) {
+            int u = 0;
+            while (j >= s_end[u]) ++u;
+            const int cell = s_cell[u], i = c.first[cell] + j - (u ? s_end[u - 1] : 0);
+            const d4 s = cen[cell], xb = xm[i];
+            const double x = s.x - xb.x, y = s.y - xb.y, z = s.z - xb.z;
+            const double r2 = x * x + y * y + z * z;
+            double q[4] = {0.0, 0.0, 0.0, 0.0};
+            cd d = mkc(1.0, 0.0);
+            const L2PWeights* w = wt + u * npair;
+            for (int l = 0; l <= p; ++l) {
+                if (l > 0) {
+                    const double sc = c_rec.inv_2j[l], sx = sc * x, sy = sc * y;
+                    d = cd{sx * d.re - sy * d.im, sx * d.im + sy * d.re};
+                }
+                cd prev2 = mkc(0.0, 0.0), Y = d;
+                for (int k = l; k <= p; ++k, ++w) {
+                    if (k > l) {
+                        const double a = c_rec.up_a[k][l] * z, b = c_rec.inv_up[k][l] * r2;
+                        const cd nx = cd{a * Y.re - b * prev2.re, a * Y.im - b * prev2.im};
+                        prev2 = Y;
+                        Y = nx;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) q[e] = fma(Y.re, w->r[e], fma(Y.im, w->i[e], q[e]));
+                }
+            }
+            psi[i] = q[0];
+            acc[3 * (size_t)i] = -q[2];
+            acc[3 * (size_t)i + 1] = -q[3];
+            acc[3 * (size_t)i + 2] = -q[1];
         }
     }
 }
@@ -608,9 +671,12 @@ __global__ void __launch_bounds__(kL2PThreads) k_l2p(const d4* __restrict__ xm, 
 void launch_l2p(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, const double* F,
                 double* psi, double* acc, cudaStream_t s) {
     if (nleaves <= 0) return;
-    size_t sm = (size_t)ncoef(p) * sizeof(cd);
-    unsigned g = (unsigned)std::min<long long>(nleaves, (long long)sm_count() * 64);
-    k_l2p<<<g, kL2PThreads, sm, s>>>(xm, c, cen, leaves, nleaves, p, F, psi, acc); note_launch();
+    init_rec_tables();
+    const size_t sm = sizeof(L2PWeights) * (size_t)kL2PLeaves * out_count(p);
+    cudaFuncSetAttribute(k_l2p, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const unsigned g = grid_for(((long long)nleaves + kL2PLeaves - 1) / kL2PLeaves * kL2PThreads, kL2PThreads, 16);
+    k_l2p<<<g, kL2PThreads, sm, s>>>(xm, c, cen, leaves, nleaves, p, F, psi, acc);
+    note_launch();
 }
 
 // ---------------------------------------------------------------- P2P, FP64

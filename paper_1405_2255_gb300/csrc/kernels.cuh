@@ -105,6 +105,22 @@ size_t rad_tmp_u64_per_cell();
 // ---------------------------------------------------------------- upward (upward.cu)
 // P2M (eq. 3c) at leaves about centre cen (sr or cr), M2M (eq. 4) for the internal
 // cells of one level, multipole power (eq. 14).
+// a kernel in clusters of eight blocks
+template <class K, class... A>
+inline void launch_cluster8(K kern, int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 8;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, args...);
+}
 void launch_p2m(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p,
                 double* M, cudaStream_t s);
 void launch_m2m_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M,

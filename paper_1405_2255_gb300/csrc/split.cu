@@ -4,6 +4,8 @@
 // (x - z)/rho, whose values are bounded by 1/n!), then rescaled in FP64.  The
 // higher orders carry a fraction ~ theta^n of an expansion's contribution, so
 // FP32 rounding there stays far below the targeted force error.
+#include <cooperative_groups.h>
+
 #include "harmonics.cuh"
 #include "kernels.cuh"
 
@@ -61,10 +63,10 @@ __device__ inline int n_of(int i) {
     while ((n + 1) * (n + 1) <= i) ++n;
     return n;
 }
-// out (full complex, FP32) = R (real storage) times sc[n] for the (p+1)^2 coefficients, one warp
+// out (full complex, FP32) = R (real storage) times sc[n] for the (p+1)^2 coefficients, by nt threads (t)
 __device__ __forceinline__ void expand_scaled(const double* __restrict__ R, const double* __restrict__ sc, int nco,
-                                              int lane, float2* out) {
-    for (int i = lane; i < nco; i += 32) {
+                                              int t, int nt, float2* out) {
+    for (int i = t; i < nco; i += nt) {
         const int n = n_of(i), c0 = n * n + n, m = i - c0, am = m < 0 ? -m : m;
         const float v = (float)(R[i] * sc[n]);
         const float w = (am & 1) ? -v : v;
@@ -110,7 +112,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32) k_l2p_split(const d4* __rest
     const double rho = s.w;
     const double* Fr = F + (size_t)cell * nco;
     const double* pc = pw + (size_t)cell * 2 * (p + 1);
-    expand_scaled(Fr, pc, nco, lane, Fh);
+    expand_scaled(Fr, pc, nco, lane, 32, Fh);
     if (lane < 9) {
         const int k = lane < 1 ? 0 : (lane < 4 ? 1 : 2), m = lane - k * k - k, l = m < 0 ? -m : m;
         const cd f0 = load_real_storage(Fr, k, l), f1 = load_real_storage(Fr, k + 1, l);
@@ -241,7 +243,7 @@ __device__ inline void upsilon_column_f(int p, int m, float x, float y, float z,
         float2 v;
         if (n == m) v = d;
         else {
-            const float a = c_twf2[n] * z, iv = c_inv_upf[n][m];
+            const float a = c_twf2[n] * z, iv = __frcp_rn((float)(n * n - m * m));
             v = make_float2((a * prev.x - r2 * prev2.x) * iv, (a * prev.y - r2 * prev2.y) * iv);
             prev2 = prev;
             prev = v;
@@ -255,94 +257,113 @@ __device__ inline void upsilon_column_f(int p, int m, float x, float y, float z,
 // ---------------------------------------------------------------- M2M
 // M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z): outputs n <= 2 in FP64,
 // outputs n >= 3 in FP32 as Mhat_n = M_n / rho'^n = sum Uhat_k Mt_{n-k} with
-// Uhat_k = Upsilon_k((z - z')/rho'), Mt_j = M_j(z) / rho'^j.  One block per parent and one
-// warp per daughter; the daughters' contributions are then summed in daughter order.
+// Uhat_k = Upsilon_k((z - z')/rho'), Mt_j = M_j(z) / rho'^j.  One block per parent, or a cluster of eight
+// with a block per daughter (kCluster).  The threads first prepare the daughters' arrays, then the warps take
+// (32 outputs, daughter) pairs, the outputs with the most terms first; the daughters' contributions are
+// summed in daughter order.
+// What bounds it: the chain of a level with few parents, which leaves the device idle (hence the clusters),
+// and on the large levels the instructions of the sums.  p = 14: 32 us a level of a sphere of 1e4 and
+// 0.68 ms for all levels of one of 1e6 with all outputs of a daughter in one warp, 13 us and
+// 0.53 ms so.
 constexpr int kM2MWarps = 8;
-__host__ __device__ inline size_t m2m_warp_bytes(int p) {
+__host__ __device__ inline size_t m2m_child_bytes(int p) {
     return ((size_t)2 * ncoef(p) * sizeof(float2) + 18 * sizeof(cd) + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t m2m_smem_bytes(int p) {
-    const size_t nout = (size_t)(p + 1) * (p + 2) / 2;
-    return kM2MWarps * m2m_warp_bytes(p) + kM2MWarps * nout * sizeof(float2) + kM2MWarps * 6 * sizeof(cd);
+__host__ __device__ inline size_t m2m_smem_bytes(int p) {  // per daughter of a block
+    return m2m_child_bytes(p) + out_count(p) * sizeof(float2) + 6 * sizeof(cd);
 }
-template <int MAXQ>
+template <bool kCluster>
 __global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4* __restrict__ cen,
                                                                const double* __restrict__ pw, int lev_begin,
-                                                               int lev_end, int p, double* __restrict__ M,
-                                                               LaneSched sched) {
+                                                               int p, double* __restrict__ M) {
     extern __shared__ __align__(16) unsigned char sraw[];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p), nout = (p + 1) * (p + 2) / 2;
-    const size_t per_warp = m2m_warp_bytes(p);
-    float2* Yh = (float2*)(sraw + wid * per_warp);
-    float2* Mt = Yh + nco;
-    cd* Y64 = (cd*)(Mt + nco);
-    cd* M64 = Y64 + 9;
-    float2* r32 = (float2*)(sraw + kM2MWarps * per_warp);  // [kM2MWarps][nout]
-    cd* r64 = (cd*)(r32 + kM2MWarps * nout);                // [kM2MWarps][6]
-    const int cell = lev_begin + blockIdx.x;
-    if (cell >= lev_end) return;
+    constexpr int S = kCluster ? 1 : 8;  // daughters of a block
+    const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+    const int nco = ncoef(p), nout = out_count(p);
+    const size_t per_child = m2m_child_bytes(p);
+    cd* r64 = (cd*)(sraw + S * per_child);  // [S][6]
+    float2* r32 = (float2*)(r64 + S * 6);    // [S][nout]
+    const int rank = kCluster ? (int)(blockIdx.x & 7) : 0;
+    const int cell = lev_begin + (kCluster ? blockIdx.x >> 3 : blockIdx.x);
     const int nch = c.nchild[cell];
-    if (nch == 0) return;  // leaves
+    if (nch == 0) return;  // leaves (the whole cluster)
+    const int mine = kCluster ? (rank < nch ? 1 : 0) : nch, first = c.child[cell] + rank;
     const d4 zp = cen[cell];
     const double *pwr = pw + (size_t)cell * 2 * (p + 1), *pwi = pwr + p + 1;  // rho^n, rho^-n
-    const double rho = zp.w, inv = pwi[1];
-    if (wid < nch) {
-        const int cnt = sched.cnt[lane];
-        const int d = c.child[cell] + wid;
-        const d4 z = cen[d];
-        const double vx = z.x - zp.x, vy = z.y - zp.y, vz = z.z - zp.z;
-        if (lane <= p) upsilon_column_f(p, lane, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, false);
-        const double* Md = M + (size_t)d * nco;
-        expand_scaled(Md, pwi, nco, lane, Mt);
-        if (lane < 9) {
-            const int n = n_of(lane);
-            M64[lane] = load_real_storage(Md, n, lane - n * n - n);
+    const double rho = zp.w;
+    const int t1 = (S * (p + 1) + 31) & ~31;  // the warps after the columns' take the moments
+    if (t < t1) {
+        const int d = t % S, m = t / S;
+        if (d < mine && m <= p) {
+            const double inv = pwi[1];
+            const d4 z = cen[first + d];
+            const double vx = z.x - zp.x, vy = z.y - zp.y, vz = z.z - zp.z;
+            float2* Yh = (float2*)((cd*)(sraw + d * per_child) + 18);
+            upsilon_column_f(p, m, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, false);
         }
-        if (lane == 0) upsilon_low_full(vx, vy, vz, Y64, false);
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < MAXQ; ++q) {
-            if (q < cnt) {
-                const int n = sched.n[lane][q], m = sched.m[lane][q];
-                const int o = n * (n + 1) / 2 + m;
-                if (n <= 2) {
-                    cd sum = mkc(0.0, 0.0);
-                    for (int k = 0; k <= n; ++k) {
-                        const int nn = n - k;
-                        for (int l = max(-k, m - nn); l <= min(k, m + nn); ++l)
-                            cmac(sum, Y64[cix(k, l)], M64[cix(nn, m - l)]);
-                    }
-                    r64[wid * 6 + o] = sum;
-                } else {
-                    float2 sum = make_float2(0.f, 0.f);
-                    if (rho > 0)
-                        for (int k = 0; k <= n; ++k) {
-                            const int nn = n - k;
-                            for (int l = max(-k, m - nn); l <= min(k, m + nn); ++l)
-                                cmacf(sum, Yh[cix(k, l)], Mt[cix(nn, m - l)]);
-                        }
-                    r32[wid * nout + o] = sum;
-                }
+    } else {
+        for (int d = 0; d < mine; ++d)
+            expand_scaled(M + (size_t)(first + d) * nco, pwi, nco, t - t1, kM2MWarps * 32 - t1,
+                          (float2*)((cd*)(sraw + d * per_child) + 18) + nco);
+        if (wid == kM2MWarps - 1) {
+            for (int i = lane; i < 9 * mine; i += 32) {
+                const int d = i / 9, e = i - 9 * d, n = n_of(e);
+                ((cd*)(sraw + d * per_child))[9 + e] = load_real_storage(M + (size_t)(first + d) * nco, n, e - n * n - n);
+            }
+            if (lane < mine) {
+                const d4 z = cen[first + lane];
+                upsilon_low_full(z.x - zp.x, z.y - zp.y, z.z - zp.z, (cd*)(sraw + lane * per_child), false);
             }
         }
     }
     __syncthreads();
+    const int units = mine * ((nout + 31) / 32);
+    for (int u = wid; u < units; u += kM2MWarps) {
+        const int w = u / mine, d = u - w * mine, o = nout - 1 - (w * 32 + lane);
+        if (o < 0) continue;
+        const cd* Y64 = (const cd*)(sraw + d * per_child);
+        const cd* M64 = Y64 + 9;
+        const float2* Yh = (const float2*)(M64 + 9);
+        const float2* Mt = Yh + nco;
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
+        if (n <= 2) {
+            cd sum = mkc(0.0, 0.0);
+            for (int k = 0; k <= n; ++k) {
+                const int nn = n - k;
+                for (int l = max(-k, m - nn); l <= min(k, m + nn); ++l)
+                    cmac(sum, Y64[cix(k, l)], M64[cix(nn, m - l)]);
+            }
+            r64[d * 6 + o] = sum;
+        } else {
+            float2 sum = make_float2(0.f, 0.f);
+            if (rho > 0)
+                for (int k = 0; k <= n; ++k) {
+                    const int nn = n - k, lmin = max(-k, m - nn), lmax = min(k, m + nn);
+                    const float2 *y = Yh + k * k + k, *x = Mt + nn * nn + nn + m;
+#pragma unroll 4
+                    for (int l = lmin; l <= lmax; ++l) cmacf(sum, y[l], x[-l]);
+                }
+            r32[d * nout + o] = sum;
+        }
+    }
+    if (kCluster) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
     // the parent's moments: the daughters' terms summed in daughter order
     double* out = M + (size_t)cell * nco;
-    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= o) ++n;
-        const int m = o - n * (n + 1) / 2;
+    for (int o = rank * (kM2MWarps * 32) + t; o < nout; o += S == 1 ? 8 * kM2MWarps * 32 : kM2MWarps * 32) {
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
         cd v;
         if (n <= 2) {
             v = mkc(0.0, 0.0);
-            for (int j = 0; j < nch; ++j) v = v + r64[j * 6 + o];
+            for (int j = 0; j < nch; ++j)
+                v = v + (kCluster ? *cooperative_groups::this_cluster().map_shared_rank(r64 + o, j) : r64[j * 6 + o]);
         } else {
             float2 a = make_float2(0.f, 0.f);
             for (int j = 0; j < nch; ++j) {
-                a.x += r32[j * nout + o].x;
-                a.y += r32[j * nout + o].y;
+                const float2 b = kCluster ? *cooperative_groups::this_cluster().map_shared_rank(r32 + o, j)
+                                          : r32[j * nout + o];
+                a.x += b.x;
+                a.y += b.y;
             }
             const double sc = pwr[n];
             v = mkc((double)a.x * sc, (double)a.y * sc);
@@ -350,6 +371,7 @@ __global__ void __launch_bounds__(kM2MWarps * 32) k_m2m_split(Cells c, const d4*
         out[cix(n, m)] = v.re;
         if (m) out[cix(n, -m)] = v.im;
     }
+    if (kCluster) cooperative_groups::this_cluster().sync();  // the sums are read before their block ends
 }
 
 void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* M, cudaStream_t s) {
@@ -360,20 +382,15 @@ void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, i
         return;
     }
     init_split_up_tables();
-    LaneSched sched = make_lane_sched(p, kSchedUp);
-    int maxq = 0;
-    for (int l = 0; l < 32; ++l) maxq = sched.cnt[l] > maxq ? sched.cnt[l] : maxq;
-    const size_t sm = m2m_smem_bytes(p);
-    const unsigned g = (unsigned)ncl;  // one block per cell of the level (leaves return at once)
-    if (maxq <= 4) {
-        cudaFuncSetAttribute(k_m2m_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<4><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
-    } else if (maxq <= 8) {
-        cudaFuncSetAttribute(k_m2m_split<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<8><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
+    const size_t per = m2m_smem_bytes(p);
+    // (leaves of the level return at once)
+    // a cluster per parent for up to six parents per SM: 944 parents at p = 14 take 43 us as blocks and 39 as
+    // clusters, 2016 parents 49 and 73
+    if (ncl <= 6 * sm_count()) {
+        launch_cluster8(k_m2m_split<true>, 8 * ncl, kM2MWarps * 32, per, s, c, cen, pw, lev_begin, p, M);
     } else {
-        cudaFuncSetAttribute(k_m2m_split<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_m2m_split<24><<<g, kM2MWarps * 32, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, M, sched);
+        cudaFuncSetAttribute(k_m2m_split<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * per));
+        k_m2m_split<false><<<(unsigned)ncl, kM2MWarps * 32, 8 * per, s>>>(c, cen, pw, lev_begin, p, M);
     }
     note_launch();
 }
@@ -382,7 +399,10 @@ void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, i
 // F_n^m(s') += sum_{k<=p-n} sum_l Upsilon_k^{l*}(s - s') F_{n+k}^{m+l}(s): terms with n+k <= 2
 // in FP64, the others in FP32 as rho^-n sum Uhat_k^{l*} Fhat_{n+k}^{m+l} with
 // Uhat_k = Upsilon_k((s - s')/rho), Fhat_j = F_j(s) rho^j (rho: the parent's radius).
-// One warp per cell.  The FP64 terms of the six outputs n <= 2 are 20 products, one per lane.
+// W warps per cell, a thread per output, the outputs with the most terms first.  The FP64 terms of the six
+// outputs n <= 2 are 20 products, one per lane of the last warp.
+// What bounds it: as for the M2M.  p = 14: 31 us a level of a sphere of 1e4 and 0.61 ms for all levels of
+// one of 1e6 with all outputs of a cell in one warp, 12.5 us and 0.585 ms so.
 struct L2LTerm {
     signed char n, m, k, l;
 };
@@ -391,67 +411,72 @@ __device__ constexpr L2LTerm kL2LTerm[20] = {
     {0, 0, 2, 1},  {0, 0, 2, 2},  {1, 0, 0, 0}, {1, 0, 1, -1}, {1, 0, 1, 0},  {1, 0, 1, 1},  {1, 1, 0, 0},
     {1, 1, 1, -1}, {1, 1, 1, 0},  {1, 1, 1, 1}, {2, 0, 0, 0},  {2, 1, 0, 0},  {2, 2, 0, 0}};
 __device__ constexpr int kL2LStart[7] = {0, 9, 13, 17, 18, 19, 20};  // first product of output n (n + 1) / 2 + m
-__host__ __device__ inline size_t l2l_warp_bytes(int p) {
+__host__ __device__ inline size_t l2l_cell_bytes(int p) {
     return ((size_t)2 * ncoef(p) * sizeof(float2) + (9 + 9 + 20 + 6) * sizeof(cd) + 15) & ~(size_t)15;
 }
-__global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict__ cen,
-                                                   const double* __restrict__ pw, int lev_begin, int lev_end,
-                                                   int p, double* __restrict__ F, LaneSched sched) {
+template <int W>
+__global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_l2l_split(Cells c, const d4* __restrict__ cen,
+                                                                     const double* __restrict__ pw, int lev_begin,
+                                                                     int lev_end, int p, double* __restrict__ F) {
     extern __shared__ __align__(16) unsigned char sraw[];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
-    cd* Y64 = (cd*)(sraw + wid * l2l_warp_bytes(p));
+    constexpr int kCells = W == 1 ? 4 : 1, T = W * 32;  // cells of a block, threads of a cell
+    const int g = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31;
+    const int nco = ncoef(p), nout = out_count(p);
+    cd* Y64 = (cd*)(sraw + g * l2l_cell_bytes(p));
     cd* F64 = Y64 + 9;
     cd* prod = F64 + 9;
     cd* low = prod + 20;
     float2* Yh = (float2*)(low + 6);
     float2* Fh = Yh + nco;
-    const int cell = lev_begin + blockIdx.x * 4 + wid;
-    if (cell >= lev_end || !cell_active(c, cell)) return;
+    const int cell = lev_begin + blockIdx.x * kCells + g;
+    if (cell >= lev_end || !cell_active(c, cell)) return;  // (the same for all threads of a cell)
     const int par = c.parent[cell];
     const d4 s = cen[par], sp = cen[cell];
     const double rho = s.w;
     double* out = F + (size_t)cell * nco;
     const double* Fp = F + (size_t)par * nco;
     if (!(rho > 0)) {  // all particles at the parent's centre: the shift is the identity
-        for (int i = lane; i < nco; i += 32) out[i] += Fp[i];
+        for (int i = t; i < nco; i += T) out[i] += Fp[i];
         return;
     }
     const double *pwr = pw + (size_t)par * 2 * (p + 1), *pwi = pwr + p + 1;  // rho^n, rho^-n
     const double inv = pwi[1];
     const double vx = s.x - sp.x, vy = s.y - sp.y, vz = s.z - sp.z;
-    if (lane <= p) upsilon_column_f(p, lane, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, true);
-    expand_scaled(Fp, pwr, nco, lane, Fh);
-    if (lane < 9) {
-        const int n = n_of(lane);
-        F64[lane] = load_real_storage(Fp, n, lane - n * n - n);
+    if (t <= p) upsilon_column_f(p, t, (float)(vx * inv), (float)(vy * inv), (float)(vz * inv), Yh, true);
+    if (W == 1 || t >= 32) expand_scaled(Fp, pwr, nco, W == 1 ? t : t - 32, W == 1 ? 32 : T - 32, Fh);
+    if (t >= T - 32) {
+        if (lane < 9) {
+            const int n = n_of(lane);
+            F64[lane] = load_real_storage(Fp, n, lane - n * n - n);
+        }
+        if (lane == 31) upsilon_low_full(vx, vy, vz, Y64, true);
+        __syncwarp();
+        if (lane < 20) {
+            const L2LTerm e = kL2LTerm[lane];
+            prod[lane] = Y64[cix(e.k, e.l)] * F64[cix(e.n + e.k, e.m + e.l)];
+        }
+        __syncwarp();
+        if (lane < 6) {
+            cd v = mkc(0.0, 0.0);
+            for (int i = kL2LStart[lane]; i < kL2LStart[lane + 1]; ++i) v = v + prod[i];
+            low[lane] = v;
+        }
     }
-    if (lane == 0) upsilon_low_full(vx, vy, vz, Y64, true);
-    __syncwarp();
-    if (lane < 20) {
-        const L2LTerm t = kL2LTerm[lane];
-        prod[lane] = Y64[cix(t.k, t.l)] * F64[cix(t.n + t.k, t.m + t.l)];
-    }
-    __syncwarp();
-    if (lane < 6) {
-        cd v = mkc(0.0, 0.0);
-        for (int i = kL2LStart[lane]; i < kL2LStart[lane + 1]; ++i) v = v + prod[i];
-        low[lane] = v;
-    }
-    __syncwarp();
-    const int cnt = sched.cnt[lane];
-    for (int q = 0; q < cnt; ++q) {
-        const int n = sched.n[lane][q], m = sched.m[lane][q];
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+    for (int o = t; o < nout; o += T) {
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
+        const double sc = pwi[n];
+        double re = out[cix(n, m)], im = m ? out[cix(n, -m)] : 0.0;
         float2 v32 = make_float2(0.f, 0.f);
         for (int k = max(0, 3 - n); k <= p - n; ++k) {
             const float2* xk = Yh + k * k + k;
             const float2* yk = Fh + (n + k) * (n + k) + (n + k) + m;
+#pragma unroll 4
             for (int l = -k; l <= k; ++l) cmacf(v32, xk[l], yk[l]);
         }
-        const double sc = pwi[n];
-        double re = out[cix(n, m)], im = m ? out[cix(n, -m)] : 0.0;
         if (n <= 2) {
-            const cd v = low[n * (n + 1) / 2 + m];
+            const cd v = low[o];
             re += v.re;
             im += v.im;
         }
@@ -460,19 +485,27 @@ __global__ void __launch_bounds__(128) k_l2l_split(Cells c, const d4* __restrict
     }
 }
 
+template <int W>
+static void go_l2l_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* F,
+                         cudaStream_t s) {
+    const int per = W == 1 ? 4 : 1;
+    k_l2l_split<W><<<(unsigned)((lev_end - lev_begin + per - 1) / per), per * W * 32, per * l2l_cell_bytes(p), s>>>(
+        c, cen, pw, lev_begin, lev_end, p, F);
+    note_launch();
+}
 void launch_l2l_split(Cells c, const d4* cen, const double* pw, int lev_begin, int lev_end, int p, double* F, cudaStream_t s) {
-    const int ncl = lev_end - lev_begin;
-    if (ncl <= 0) return;
+    if (lev_end <= lev_begin) return;
     if (p < 3) {
         launch_l2l_level(c, cen, lev_begin, lev_end, p, F, s);
         return;
     }
     init_split_up_tables();
-    LaneSched sched = make_lane_sched(p, kSchedDown);
-    const size_t sm = 4 * l2l_warp_bytes(p);
-    cudaFuncSetAttribute(k_l2l_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_l2l_split<<<(unsigned)((ncl + 3) / 4), 128, sm, s>>>(c, cen, pw, lev_begin, lev_end, p, F, sched);
-    note_launch();
+    switch ((out_count(p) + 31) / 32) {
+        case 1: go_l2l_split<1>(c, cen, pw, lev_begin, lev_end, p, F, s); break;
+        case 2: go_l2l_split<2>(c, cen, pw, lev_begin, lev_end, p, F, s); break;
+        case 3: go_l2l_split<3>(c, cen, pw, lev_begin, lev_end, p, F, s); break;
+        default: go_l2l_split<4>(c, cen, pw, lev_begin, lev_end, p, F, s); break;
+    }
 }
 
 }  // namespace gb3

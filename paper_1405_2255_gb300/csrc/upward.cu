@@ -1,4 +1,4 @@
-// upward.cu -- A5-A6 of the path (P2M eq. 3c, M2M eq. 4, multipole power eq. 14)
+// upward.cu -- A5-A6 of the path (M2M eq. 4, multipole power eq. 14; P2M eq. 3c: p2m_split.cu)
 // and the per-cell minimum of the acceleration scale used by eqs. (18a,b).
 #include <cooperative_groups.h>
 
@@ -10,156 +10,81 @@
 
 namespace gb3 {
 
-LaneSched make_lane_sched(int p, SchedKind kind) {
-    LaneSched s;
-    memset(&s, 0, sizeof s);
-    std::vector<std::pair<int, int>> outs;
-    for (int n = 0; n <= p; ++n)
-        for (int m = 0; m <= n; ++m) outs.push_back({n, m});
-    auto cost = [p, kind](int n) -> long long {
-        long long t = kind == kSchedDown ? (p - n + 1) : (n + 1);
-        return t * t;
-    };
-    std::stable_sort(outs.begin(), outs.end(), [&](const std::pair<int, int>& a, const std::pair<int, int>& b) {
-        return cost(a.first) > cost(b.first);
-    });
-    long long load[32] = {0};
-    for (auto& o : outs) {
-        int best = 0;
-        for (int l = 1; l < 32; ++l)
-            if (load[l] < load[best] || (load[l] == load[best] && s.cnt[l] < s.cnt[best])) best = l;
-        if (s.cnt[best] >= kMaxPerLane) {  // fall back to the lane with the fewest outputs
-            for (int l = 0; l < 32; ++l)
-                if (s.cnt[l] < s.cnt[best]) best = l;
-        }
-        int k = s.cnt[best]++;
-        s.n[best][k] = (unsigned char)o.first;
-        s.m[best][k] = (unsigned char)o.second;
-        load[best] += cost(o.first);
-    }
-    return s;
-}
-
-// ---------------------------------------------------------------- P2M
-// One warp per leaf; lane j takes particles j, j+32, ...; for each m-column the
-// Upsilon_n^m(x - z) values of the 32 particles are summed over the warp.
-__global__ void k_p2m(const d4* __restrict__ xm, Cells c, const d4* __restrict__ cen, const int* __restrict__ leaves,
-                      int nleaves, int p, double* __restrict__ M) {
-    extern __shared__ double smem[];
-    const int wpb = blockDim.x >> 5;
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p);
-    double* acc = smem + (size_t)wid * nco;
-    int t = blockIdx.x * wpb + wid;
-    if (t >= nleaves) return;
-    int cell = leaves[t];
-    for (int i = lane; i < nco; i += 32) acc[i] = 0.0;
-    __syncwarp();
-    const d4 z = cen[cell];
-    const int first = c.first[cell], count = c.count[cell];
-    for (int b = 0; b < count; b += 32) {
-        int i = b + lane;
-        double x = 0, y = 0, zz = 0, mu = 0;
-        if (i < count) {
-            d4 q = xm[first + i];
-            x = q.x - z.x; y = q.y - z.y; zz = q.z - z.z; mu = q.w;
-        }
-        const double r2 = x * x + y * y + zz * zz;
-        cd d = mkc(mu, 0.0);  // mu * Upsilon_m^m
-        for (int m = 0; m <= p; ++m) {
-            if (m > 0) {
-                double s = 1.0 / (2.0 * m);
-                d = cd{s * (x * d.re - y * d.im), s * (x * d.im + y * d.re)};
-            }
-            cd prev2 = mkc(0.0, 0.0), prev = d;
-            for (int n = m; n <= p; ++n) {
-                cd v;
-                if (n == m) v = d;
-                else {
-                    double inv = 1.0 / (double)(n * n - m * m);
-                    double a = (2.0 * n - 1.0) * zz;
-                    v = cd{(a * prev.re - r2 * prev2.re) * inv, (a * prev.im - r2 * prev2.im) * inv};
-                    prev2 = prev;
-                    prev = v;
-                }
-                double sr = warp_sum(v.re);
-                double si = warp_sum(v.im);
-                if (lane == 0) {
-                    acc[cix(n, m)] += sr;
-                    if (m) acc[cix(n, -m)] += si;
-                }
-            }
-        }
-    }
-    __syncwarp();
-    double* out = M + (size_t)cell * nco;
-    for (int i = lane; i < nco; i += 32) out[i] = acc[i];
-}
-
-void launch_p2m(const d4* xm, Cells c, const d4* cen, const int* leaves, int nleaves, int p, double* M,
-                cudaStream_t s) {
-    if (nleaves <= 0) return;
-    const int wpb = 4;
-    size_t sm = (size_t)wpb * ncoef(p) * sizeof(double);
-    k_p2m<<<(nleaves + wpb - 1) / wpb, wpb * 32, sm, s>>>(xm, c, cen, leaves, nleaves, p, M); note_launch();
-}
+namespace cg = cooperative_groups;
 
 // ---------------------------------------------------------------- M2M
-// M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z): one block per parent and one
-// warp per daughter (a level is a chain of one daughter's FP64 work: with the daughters one after
-// another in one warp, 13 levels of a 6e4 cusp at p = 14 took 8.1 ms, so 1.9 ms); the daughters'
-// contributions are then added in daughter order.
+// M_n^m(z') = sum_{k<=n} sum_l Upsilon_k^l(z - z') M_{n-k}^{m-l}(z): a cluster of eight blocks per parent, a
+// block per daughter: a thread per output, the outputs with the most terms in the first warps, the terms of
+// an output dealt out to four warps.  The daughters' contributions are added in daughter order.
+// What bounds it: the FP64 pipe, of which a warp has a quarter of an SM's, and whose instructions cost the
+// same however many lanes are active; at p = 14 a parent with eight daughters has some 70 us of it on one SM.
+// A level with few parents is as long as one parent, hence the cluster.  13 levels of a cusp of 6e4 at p = 14:
+// 8.1 ms with the daughters one after another in one warp, 1.9 ms with a warp per daughter, 0.61 ms so.
+// (On levels that fill the device the empty blocks of missing daughters cost less than the even shares give:
+// 2072 parents at p = 10 128 us with a block per parent, 88 us so.)
 constexpr int kM2MWarps64 = 8;
+constexpr int kM2MParts = 4;
 __global__ void __launch_bounds__(kM2MWarps64 * 32) k_m2m(Cells c, const d4* __restrict__ cen, int lev_begin,
-                                                          int p, double* __restrict__ M, LaneSched sched) {
+                                                          int p, double* __restrict__ M) {
     extern __shared__ cd csm[];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nco = ncoef(p), nout = (p + 1) * (p + 2) / 2;
-    cd* Yw = csm + (size_t)wid * 2 * nco;
+    constexpr int T = kM2MWarps64 * 32;
+    const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+    const int nco = ncoef(p), nout = out_count(p);
+    cd* Yw = csm;
     cd* Mw = Yw + nco;
-    cd* res = csm + (size_t)kM2MWarps64 * 2 * nco;  // [kM2MWarps64][nout]
-    const int cell = lev_begin + blockIdx.x;
+    cd* res = Mw + nco;  // [kM2MParts][nout]
+    const cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)(blockIdx.x & 7), cell = lev_begin + (int)(blockIdx.x >> 3);
     const int nch = c.nchild[cell];
-    if (nch == 0) return;
-    if (wid < nch) {
-        const d4 zp = cen[cell];
-        const int d = c.child[cell] + wid, cnt = sched.cnt[lane];
-        const d4 z = cen[d];
-        if (lane <= p) upsilon_column(p, lane, z.x - zp.x, z.y - zp.y, z.z - zp.z, Yw, false);
-        expand_real(p, M + (size_t)d * nco, Mw, false, lane, 32);
-        __syncwarp();
-        for (int q = 0; q < cnt; ++q) {
-            const int n = sched.n[lane][q], m = sched.m[lane][q];
-            cd s = mkc(0.0, 0.0);
-            for (int k = 0; k <= n; ++k) {
+    if (nch == 0) return;  // (the whole cluster)
+    if (rank < nch) {
+        const int d = c.child[cell] + rank;
+        const int t1 = (2 * (p + 1) + 31) & ~31;  // the warps after the columns' take the moments
+        if (t < t1) {
+            const d4 zp = cen[cell], z = cen[d];
+            upsilon_columns2(p, t, z.x - zp.x, z.y - zp.y, z.z - zp.z, Yw, false);
+        } else {
+            expand_real(p, M + (size_t)d * nco, Mw, false, t - t1, T - t1);
+        }
+        __syncthreads();
+        // (warp w takes part w % 4, so that the four parts of the SM's pipe have the same)
+        for (int u = wid; u < kM2MParts * ((nout + 31) / 32); u += kM2MWarps64) {
+            const int q = u % kM2MParts, o = nout - 1 - (u / kM2MParts * 32 + lane);
+            if (o < 0) continue;
+            const int n = out_order(o), m = o - n * (n + 1) / 2;
+            cd4 s{0.0, 0.0, 0.0, 0.0};
+            for (int k = q; k <= n; k += kM2MParts) {
                 const int nn = n - k;
                 const int lmin = max(-k, m - nn), lmax = min(k, m + nn);
-                for (int l = lmin; l <= lmax; ++l) cmac(s, Yw[cix(k, l)], Mw[cix(nn, m - l)]);
+                const cd *y = Yw + k * k + k, *x = Mw + nn * nn + nn + m;
+#pragma unroll 4
+                for (int l = lmin; l <= lmax; ++l) s.add(y[l], x[-l]);
             }
-            res[wid * nout + n * (n + 1) / 2 + m] = s;
+            res[q * nout + o] = s.sum();
         }
+        __syncthreads();
+        for (int o = t; o < nout; o += T)
+            res[o] = ((res[o] + res[nout + o]) + res[2 * nout + o]) + res[3 * nout + o];
     }
-    __syncthreads();
+    cl.sync();
     double* out = M + (size_t)cell * nco;
-    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= o) ++n;
-        const int m = o - n * (n + 1) / 2;
+    for (int o = rank * T + t; o < nout; o += 8 * T) {
+        const int n = out_order(o), m = o - n * (n + 1) / 2;
         cd v = mkc(0.0, 0.0);
-        for (int j = 0; j < nch; ++j) v = v + res[j * nout + o];
+        for (int j = 0; j < nch; ++j) v = v + *cl.map_shared_rank(res + o, j);
         out[cix(n, m)] = v.re;
         if (m) out[cix(n, -m)] = v.im;
     }
+    cl.sync();  // the sums are read before their block ends
 }
 
 void launch_m2m_level(Cells c, const d4* cen, int lev_begin, int lev_end, int p, double* M, cudaStream_t s) {
     int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
-    const size_t sm = (size_t)kM2MWarps64 * (2 * ncoef(p) + (p + 1) * (p + 2) / 2) * sizeof(cd);
-    LaneSched sched = make_lane_sched(p, kSchedUp);
     init_rec_tables();
-    cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_m2m<<<ncl, kM2MWarps64 * 32, sm, s>>>(c, cen, lev_begin, p, M, sched); note_launch();
+    const size_t sm = (size_t)(2 * ncoef(p) + kM2MParts * out_count(p)) * sizeof(cd);
+    launch_cluster8(k_m2m, 8 * ncl, kM2MWarps64 * 32, sm, s, c, cen, lev_begin, p, M);
+    note_launch();
 }
 
 // ---------------------------------------------------------------- power
@@ -236,8 +161,7 @@ struct Levels {
 constexpr int kMinThreads = 1024;
 __global__ void __launch_bounds__(kMinThreads) k_minscale_levels(const __grid_constant__ Cells c,
                                                                  const __grid_constant__ Levels lv) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
+        cg::cluster_group cl = cg::this_cluster();
     for (int L = lv.n - 1; L >= 0; --L) {
         for (int cell = lv.start[L] + blockIdx.x * blockDim.x + threadIdx.x; cell < lv.start[L + 1];
              cell += gridDim.x * blockDim.x) {
