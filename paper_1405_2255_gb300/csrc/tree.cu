@@ -5,9 +5,13 @@
 // Compiled with --fmad=false: the decision quantities (keys, centres, radii) are
 // plain IEEE FP64 sums and products, so that the tree and the acceptance tests do
 // not depend on how a compiler contracts them.
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 namespace gb3 {
+
+namespace cg = cooperative_groups;
 
 // ------------------------------------------------------------------ A1 bounds
 __global__ void k_bounds_init(unsigned long long* b) {
@@ -1016,13 +1020,104 @@ __device__ inline void dist_bounds_f(const float4* __restrict__ xp, int i, const
     ub = df * (1.0f + 0x1p-20f) + E;
 }
 
+// Exact radii of the internal cells of one level: max over their particles of |x - s|
+// and |x - com| (Sec. 4), taken in FP64, but only for the particles that can attain the
+// maximum.  A first pass bounds every distance in FP32 from the two-float positions and
+// the two-float centres: the difference of two-float values carries at most 2^-23 |d| +
+// 2^-46 (|x| + |s|) per coordinate, so with d_f the FP32 distance
+//   d_f (1 - 2^-20) - E <= d <= d_f (1 + 2^-20) + E,  E = 2^-44 sum_c (|x_c| + |s_c|)
+// (the FP32 square and square root stay inside the relative margin; below the coordinate
+// range 2^-18 an underflowed square would escape E and above 2^60 it would overflow, so
+// there every particle is a candidate).  The per-cell maximum LB of the lower bounds is
+// at most the largest distance, so the particle attaining it has an upper bound >= LB;
+// the second pass takes the FP64 distance of every particle whose upper bound reaches LB,
+// and the maximum over those is the maximum over all, bit for bit.
+// One block, its own cell (the centres in shared memory), or the eight blocks of a cluster (kShared):
+template <bool kShared>
+__device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, const Cells& c, int cell,
+                           const float* q, const double (&s)[3], const double (&com)[3]) {
+    __shared__ int s_lb[2];
+    __shared__ unsigned long long s_key[2];
+    const int rank = kShared ? blockIdx.x & 7 : 0, step = (kShared ? 8 : 1) * blockDim.x;
+    const int first = c.first[cell], end = first + c.count[cell], lane = threadIdx.x & 31;
+    const int begin = first + rank * blockDim.x + threadIdx.x;
+    if (threadIdx.x < 2) {
+        s_lb[threadIdx.x] = 0;
+        s_key[threadIdx.x] = 0ull;
+    }
+    __syncthreads();
+    float l0 = 0.f, l1 = 0.f;
+#pragma unroll 4
+    for (int i = begin; i < end; i += step) {
+        float a, b, u;
+        dist_bounds_f(xp, i, q, a, u);
+        dist_bounds_f(xp, i, q + 6, b, u);
+        l0 = fmaxf(l0, a);
+        l1 = fmaxf(l1, b);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        l0 = fmaxf(l0, __shfl_xor_sync(0xffffffffu, l0, o));
+        l1 = fmaxf(l1, __shfl_xor_sync(0xffffffffu, l1, o));
+    }
+    if (lane == 0) {  // non-negative floats order as their bit patterns
+        atomicMax(&s_lb[0], __float_as_int(l0));
+        atomicMax(&s_lb[1], __float_as_int(l1));
+    }
+    if (kShared) {
+        cg::this_cluster().sync();
+        int v = *cg::this_cluster().map_shared_rank(s_lb + (lane & 1), (lane >> 1) & 7);
+        for (int o = 2; o < 16; o <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+        l0 = __int_as_float(__shfl_sync(0xffffffffu, v, 0));
+        l1 = __int_as_float(__shfl_sync(0xffffffffu, v, 1));
+    } else {
+        __syncthreads();
+        l0 = __int_as_float(s_lb[0]);
+        l1 = __int_as_float(s_lb[1]);
+    }
+    double d2 = 0, e2 = 0;
+#pragma unroll 2
+    for (int i = begin; i < end; i += step) {
+        float l, u0, u1;
+        dist_bounds_f(xp, i, q, l, u0);
+        dist_bounds_f(xp, i, q + 6, l, u1);
+        const bool want0 = u0 >= l0, want1 = u1 >= l1;
+        if (!want0 && !want1) continue;
+        const d4 p = xm[i];
+        if (want0) {
+            const double dx = p.x - s[0], dy = p.y - s[1], dz = p.z - s[2];
+            d2 = max_nonneg(d2, dx * dx + dy * dy + dz * dz);
+        }
+        if (want1) {
+            const double ex = p.x - com[0], ey = p.y - com[1], ez = p.z - com[2];
+            e2 = max_nonneg(e2, ex * ex + ey * ey + ez * ez);
+        }
+    }
+    d2 = warp_max_nonneg(d2);
+    e2 = warp_max_nonneg(e2);
+    if (lane == 0) {
+        atomicMax(&s_key[0], (unsigned long long)__double_as_longlong(d2));
+        atomicMax(&s_key[1], (unsigned long long)__double_as_longlong(e2));
+    }
+    if (kShared) cg::this_cluster().sync();
+    else __syncthreads();
+    if (rank == 0 && threadIdx.x < 2) {
+        unsigned long long k = s_key[threadIdx.x];
+        if (kShared)
+            for (int b = 1; b < 8; ++b) k = max(k, *cg::this_cluster().map_shared_rank(s_key + threadIdx.x, b));
+        const double r = sqrt(__longlong_as_double((long long)k));
+        if (threadIdx.x == 0) c.sr[cell].w = r;
+        else c.cr[cell].w = r;
+    }
+    if (kShared) cg::this_cluster().sync();  // the maxima are read before their block ends
+}
+
 // Internal cells of one level: smallest ball enclosing the daughter balls (s_d, rho_d),
 // as the smallest support ball (over all subsets of 1..4 daughters, enumerated by
 // mask) that contains every daughter ball; single precision relative to the first
 // daughter's centre.  One warp per cell, lanes take masks; ties go to the smaller mask.
-// one block of kMebWarps warps per internal cell; warp w tries the support sets with
-// bit masks 1 + 32 w + lane (at most 4 daughters), and the block keeps the smallest
-// valid ball (ties: the smaller mask)
+// one block of kMebWarps warps per internal cell; a thread tries one support set of at most 4
+// daughters, the sets of one size in the same warps, and the block keeps the smallest valid ball
+// (ties: the smaller mask)
 // Then the cell's mass and centre of mass, and, for a cell of at most `small` particles, its exact
 // radii by the block (below); the radii of a larger cell are taken by all blocks over its level's
 // particles, k_internal_radii_lb and k_internal_radii.  With at most kLevelCells cells in the level, small
@@ -1031,39 +1126,99 @@ __device__ inline void dist_bounds_f(const float4* __restrict__ xp, int i, const
 // of 8192: tree of 1e5 0.733 ms with 2048, 0.748 with 4096, 0.804 with 8192); with more cells 0 (a block
 // per cell has too little to do: block step of 1e6 1.1 % slower).
 // keep_centre: a reused tree keeps its centres (one warp per block where the block takes no radii).
+// kCluster, where a level of at most kWideCells cells has one of more than kWideRadii particles: eight blocks
+// share the radii of such a cell (the first one has its ball), of up to kWideLevel particles if no cell is
+// larger and else kWideCell.  A block took 25 us for a cell of 1000 to 2000 particles and 51 us for one of
+// 1e4, the cluster takes 17 and 22; levels of 100 to 560 cells of a cusp of 6e4 46 to 70 us as blocks, 18 to
+// 23 us so (the blocks that have nothing to do return at once).  From 32768 particles on all blocks are
+// faster (a cell of 6e4 in a cluster 43 us, by the level's kernels 28).
+// What bounds a level of few cells: the chain of one cell's loads, balls and FP64 operations (64 cycles
+// each in a warp that is alone): 1e4 particles 25 to 30 us a level with every warp converting all daughters,
+// masks of all sizes in a warp and the mass summed behind them, 12 us so (without the radii).
 constexpr int kMebWarps = 8;
+struct MebMasks {
+    unsigned char m[kMebWarps * 32];  // sets of 1 daughter in warp 0, of 2 in warp 1, of 3 in 2 and 3, of 4 in 4 to 6
+    constexpr MebMasks() : m{} {
+        const int start[5] = {0, 0, 32, 64, 128};
+        int n[5] = {0, 0, 0, 0, 0};
+        for (int k = 1; k < 256; ++k) {
+            int b = 0;
+            for (int i = 0; i < 8; ++i) b += (k >> i) & 1;
+            if (b <= 4) m[start[b] + n[b]++] = (unsigned char)k;
+        }
+    }
+};
+static __device__ const MebMasks g_meb_masks = MebMasks();
 constexpr int kLevelRadii = 16384, kCellRadii = 2048, kLevelCells = 2048;
-__device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, const Cells& c, int cell,
-                           const float* q, const double (&s)[3], const double (&com)[3]);
+constexpr int kWideCells = 912, kWideRadii = 1024, kWideLevel = 32768, kWideCell = 16384;
+template <bool kCluster>
 __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __restrict__ xm,
                                                                  const float4* __restrict__ xp, Cells c,
                                                                  int lev_begin, int lev_end, unsigned* status,
                                                                  unsigned long long* tmp, bool keep_centre,
                                                                  int small) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int cell = lev_begin + blockIdx.x;
+    const int cell = lev_begin + (kCluster ? blockIdx.x >> 3 : blockIdx.x), rank = kCluster ? blockIdx.x & 7 : 0;
     if (cell >= lev_end) return;
     const int nch = c.nchild[cell];
     if (nch == 0) return;  // leaves are done
-    const int ch = c.child[cell];
-    const d4 o = c.sr[ch];
-    // the daughters' balls relative to the first one (registers: loops over all 8 slots)
-    float cen[8][3], rad[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        cen[i][0] = cen[i][1] = cen[i][2] = rad[i] = 0.f;
-        if (i < nch && !keep_centre) {
-            const d4 v = c.sr[ch + i];
-            cen[i][0] = (float)(v.x - o.x);
-            cen[i][1] = (float)(v.y - o.y);
-            cen[i][2] = (float)(v.z - o.z);
-            rad[i] = (float)v.w;
-        }
+    const int count = c.count[cell];
+    __shared__ __align__(16) float s_ball[8][4];
+    __shared__ double s_cen[6], s_mass;
+    __shared__ float s_q[12];
+    const bool shared = kCluster && count > kWideRadii && count <= small;
+    if (kCluster && rank) {  // a block for the radii only
+        if (!shared) return;
+        cg::this_cluster().sync();  // the first block has the centres
+        if (threadIdx.x < 6) s_cen[threadIdx.x] = *cg::this_cluster().map_shared_rank(s_cen + threadIdx.x, 0);
+        if (threadIdx.x < 12) s_q[threadIdx.x] = *cg::this_cluster().map_shared_rank(s_q + threadIdx.x, 0);
+        __syncthreads();
+        const double s[3] = {s_cen[0], s_cen[1], s_cen[2]}, com[3] = {s_cen[3], s_cen[4], s_cen[5]};
+        cell_radii<true>(xm, xp, c, cell, s_q, s, com);
+        return;
     }
+    const int ch = c.child[cell];
+    // the daughters' balls relative to the first one
+    if (!keep_centre && threadIdx.x < 4 * nch) {
+        const double* sr = (const double*)(c.sr + ch);
+        const int e = threadIdx.x & 3;
+        const double v = sr[threadIdx.x], o = e < 3 ? sr[e] : 0.0;
+        s_ball[threadIdx.x >> 2][e] = (float)(v - o);
+    }
+    const int mask = keep_centre ? 0 : g_meb_masks.m[threadIdx.x];
+    const bool alone = blockDim.x == 32;
+    if (wid == kMebWarps - 1 || alone) {
+        // lane 0 the mass, lanes 1 .. 3 the coordinates of the centre of mass (this warp has no masks)
+        double md[8], cm[8];
+        const int e = lane >= 1 && lane <= 3 ? lane - 1 : 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            md[i] = i < nch ? c.mass[ch + i] : 0.0;
+            cm[i] = i < nch ? ((const double*)(c.cr + ch + i))[e] : 0.0;
+        }
+        double m = 0, mx = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < nch) {
+                m += md[i];
+                mx += md[i] * cm[i];
+            }
+        if (lane >= 1 && lane <= 3 && m > 0) s_cen[lane + 2] = mx / m;
+        if (lane == 0) s_mass = m;
+    }
+    __syncthreads();
     float best = -1, bc[3] = {0, 0, 0};
     int bmask = 1 << 30;
-    const int mask = 1 + lane + 32 * wid;
-    if (!keep_centre && mask < (1 << nch) && __popc(mask) <= 4) {
+    if (mask > 0 && mask < (1 << nch)) {
+        float cen[8][3], rad[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = i < nch ? *(const float4*)s_ball[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            cen[i][0] = v.x;
+            cen[i][1] = v.y;
+            cen[i][2] = v.z;
+            rad[i] = v.w;
+        }
         // the k-th daughter of the mask into slot k of the support set
         float sc[4][3] = {}, sr[4] = {};
         int k = 0;
@@ -1118,51 +1273,27 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __res
         wmask[wid] = bmask;
         wbc[wid][0] = bc[0]; wbc[wid][1] = bc[1]; wbc[wid][2] = bc[2];
     }
-    __shared__ double s_cen[6];
-    __shared__ float s_q[12];
     __syncthreads();
     if (wid == 0) {
-        for (int w = 1; w < kMebWarps && !keep_centre; ++w) {
-            const float ob = wbest[w], b0 = wbest[0];
-            const int om = wmask[w], b1 = wmask[0];
-            const bool take = (ob >= 0) && (b0 < 0 || ob < b0 || (ob == b0 && om < b1));
-            __syncwarp();
-            if (take && lane == 0) {
-                wbest[0] = ob;
-                wmask[0] = om;
-                wbc[0][0] = wbc[w][0]; wbc[0][1] = wbc[w][1]; wbc[0][2] = wbc[w][2];
-            }
-            __syncwarp();
+        int w = 0;  // the winning warp
+        for (int v = 1; v < kMebWarps && !keep_centre; ++v) {
+            const float ob = wbest[v], b0 = wbest[w];
+            if (ob >= 0 && (b0 < 0 || ob < b0 || (ob == b0 && wmask[v] < wmask[w]))) w = v;
         }
-        best = wbest[0];
-        bc[0] = wbc[0][0]; bc[1] = wbc[0][1]; bc[2] = wbc[0][2];
-        if (best < 0) {  // no valid support set: the first daughter's centre
-            if (lane == 0 && !keep_centre) atomicOr(status, kStatMeb);
-            bc[0] = bc[1] = bc[2] = 0.f;
-        }
-        // lane 0 the mass, lanes 1 .. 3 the coordinates of the centre of mass
-        double m = 0, mx = 0;
-        for (int i = 0; i < nch; ++i) {
-            const double md = c.mass[ch + i];
-            const d4 cm = c.cr[ch + i];
-            m += md;
-            mx += md * (lane == 1 ? cm.x : lane == 2 ? cm.y : cm.z);
-        }
-        double s[3] = {o.x + (double)bc[0], o.y + (double)bc[1], o.z + (double)bc[2]};
-        if (keep_centre) {
-            const d4 v = c.sr[cell];
-            s[0] = v.x; s[1] = v.y; s[2] = v.z;
-        }
+        const bool none = keep_centre || wbest[w] < 0;  // no valid support set: the first daughter's centre
+        if (none && lane == 0 && !keep_centre) atomicOr(status, kStatMeb);
         if (lane >= 1 && lane <= 3) {
-            const double sl = lane == 1 ? s[0] : lane == 2 ? s[1] : s[2];
-            s_cen[lane - 1] = sl;
-            s_cen[lane + 2] = (m > 0) ? mx / m : sl;
+            const int e = lane - 1;
+            const double sl = keep_centre ? ((const double*)(c.sr + cell))[e]
+                                          : ((const double*)(c.sr + ch))[e] + (double)(none ? 0.f : wbc[w][e]);
+            s_cen[e] = sl;
+            if (!(s_mass > 0)) s_cen[e + 3] = sl;
         }
         __syncwarp();
         if (lane == 0) {
             c.sr[cell] = mk4(s_cen[0], s_cen[1], s_cen[2], 0.0);
             c.cr[cell] = mk4(s_cen[3], s_cen[4], s_cen[5], 0.0);
-            c.mass[cell] = m;
+            c.mass[cell] = s_mass;
         }
         if (lane < 6) {  // two-float centres: s hi, s lo, com hi, com lo
             const double v = s_cen[lane];
@@ -1174,8 +1305,11 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __res
     }
     __syncthreads();
     const double s[3] = {s_cen[0], s_cen[1], s_cen[2]}, com[3] = {s_cen[3], s_cen[4], s_cen[5]};
-    if (c.count[cell] <= small) {
-        cell_radii(xm, xp, c, cell, s_q, s, com);
+    if (shared) {
+        if (kCluster) cg::this_cluster().sync();
+        cell_radii<kCluster>(xm, xp, c, cell, s_q, s, com);
+    } else if (count <= small) {
+        cell_radii<false>(xm, xp, c, cell, s_q, s, com);
     } else if (threadIdx.x < 12) {  // for the level's radii kernels; bounds and keys start at 0
         const RadTmp R(tmp, lev_end - lev_begin);
         const int k = cell - lev_begin;
@@ -1187,78 +1321,6 @@ __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __res
     }
 }
 
-// Exact radii of the internal cells of one level: max over their particles of |x - s|
-// and |x - com| (Sec. 4), taken in FP64, but only for the particles that can attain the
-// maximum.  A first pass bounds every distance in FP32 from the two-float positions and
-// the two-float centres: the difference of two-float values carries at most 2^-23 |d| +
-// 2^-46 (|x| + |s|) per coordinate, so with d_f the FP32 distance
-//   d_f (1 - 2^-20) - E <= d <= d_f (1 + 2^-20) + E,  E = 2^-44 sum_c (|x_c| + |s_c|)
-// (the FP32 square and square root stay inside the relative margin; below the coordinate
-// range 2^-18 an underflowed square would escape E and above 2^60 it would overflow, so
-// there every particle is a candidate).  The per-cell maximum LB of the lower bounds is
-// at most the largest distance, so the particle attaining it has an upper bound >= LB;
-// the second pass takes the FP64 distance of every particle whose upper bound reaches LB,
-// and the maximum over those is the maximum over all, bit for bit.
-// One block, its own cell (the centres in shared memory):
-__device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__ xp, const Cells& c, int cell,
-                           const float* q, const double (&s)[3], const double (&com)[3]) {
-    __shared__ int s_lb[2];
-    __shared__ unsigned long long s_key[2];
-    const int first = c.first[cell], end = first + c.count[cell], lane = threadIdx.x & 31;
-    if (threadIdx.x < 2) {
-        s_lb[threadIdx.x] = 0;
-        s_key[threadIdx.x] = 0ull;
-    }
-    __syncthreads();
-    float l0 = 0.f, l1 = 0.f;
-    for (int i = first + threadIdx.x; i < end; i += blockDim.x) {
-        float a, b, u;
-        dist_bounds_f(xp, i, q, a, u);
-        dist_bounds_f(xp, i, q + 6, b, u);
-        l0 = fmaxf(l0, a);
-        l1 = fmaxf(l1, b);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        l0 = fmaxf(l0, __shfl_xor_sync(0xffffffffu, l0, o));
-        l1 = fmaxf(l1, __shfl_xor_sync(0xffffffffu, l1, o));
-    }
-    if (lane == 0) {  // non-negative floats order as their bit patterns
-        atomicMax(&s_lb[0], __float_as_int(l0));
-        atomicMax(&s_lb[1], __float_as_int(l1));
-    }
-    __syncthreads();
-    l0 = __int_as_float(s_lb[0]);
-    l1 = __int_as_float(s_lb[1]);
-    double d2 = 0, e2 = 0;
-    for (int i = first + threadIdx.x; i < end; i += blockDim.x) {
-        float l, u0, u1;
-        dist_bounds_f(xp, i, q, l, u0);
-        dist_bounds_f(xp, i, q + 6, l, u1);
-        const bool want0 = u0 >= l0, want1 = u1 >= l1;
-        if (!want0 && !want1) continue;
-        const d4 p = xm[i];
-        if (want0) {
-            const double dx = p.x - s[0], dy = p.y - s[1], dz = p.z - s[2];
-            d2 = max_nonneg(d2, dx * dx + dy * dy + dz * dz);
-        }
-        if (want1) {
-            const double ex = p.x - com[0], ey = p.y - com[1], ez = p.z - com[2];
-            e2 = max_nonneg(e2, ex * ex + ey * ey + ez * ez);
-        }
-    }
-    d2 = warp_max_nonneg(d2);
-    e2 = warp_max_nonneg(e2);
-    if (lane == 0) {
-        atomicMax(&s_key[0], (unsigned long long)__double_as_longlong(d2));
-        atomicMax(&s_key[1], (unsigned long long)__double_as_longlong(e2));
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        const double r = sqrt(__longlong_as_double((long long)s_key[threadIdx.x]));
-        if (threadIdx.x == 0) c.sr[cell].w = r;
-        else c.cr[cell].w = r;
-    }
-}
 // All blocks, the cells of more than `small` particles of a level.
 // owner[i]: an ancestor of the particle at or below the level processed last (its leaf to begin with).
 // The levels are processed bottom-up, so at level L the owner moves up to the ancestor at or above L;
@@ -1400,9 +1462,16 @@ void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_b
                               bool keep_centre) {
     int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
-    const int small = ncl > kLevelCells ? 0 : largest <= kLevelRadii ? kLevelRadii : kCellRadii;
-    k_internal_meb<<<(unsigned)ncl, keep_centre && small == 0 ? 32 : kMebWarps * 32, 0, s>>>(
-        xm, xp, c, lev_begin, lev_end, status, rad_tmp, keep_centre, small);
+    const bool wide = ncl <= kWideCells && largest > kWideRadii;
+    const int small = wide              ? (largest <= kWideLevel ? kWideLevel : kWideCell)
+                      : ncl > kLevelCells ? 0
+                                          : (largest <= kLevelRadii ? kLevelRadii : kCellRadii);
+    if (wide)
+        launch_cluster8(k_internal_meb<true>, 8 * ncl, kMebWarps * 32, 0, s, xm, xp, c, lev_begin, lev_end, status,
+                        rad_tmp, keep_centre, small);
+    else
+        k_internal_meb<false><<<(unsigned)ncl, keep_centre && small == 0 ? 32 : kMebWarps * 32, 0, s>>>(
+            xm, xp, c, lev_begin, lev_end, status, rad_tmp, keep_centre, small);
     note_launch();
     if (largest <= small) return;
     k_internal_radii_lb<<<grid_for(n, kRadThreads, 16), kRadThreads, 0, s>>>(xp, n, c, lev_begin, lev_end, small,
