@@ -185,7 +185,7 @@ def m2l_flops(p):
 
 
 def m2l_rot_flops(p):
-    """FP32 flops per pair of the rotation-accelerated M2L (App. A.5), 2 per multiply-add:
+    """Flops per pair of the rotation-accelerated M2L (App. A.5), 2 per multiply-add:
     four z rotations (4 multiply-adds per m > 0 of each order), four swaps (one
     multiply-add per entry of the swap matrices' parity pattern: cosine block n+m+l even,
     sine block n+m+l odd; the restricted forward/backward swaps only the rows/columns
@@ -265,11 +265,12 @@ def roofline(g, a, prec, phase, full):
     src = (f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {mhz:.0f} MHz" if mixed
            else "nominal FP64 rate of the part (1.25 TFLOP/s)")
     if k_m2l >= k_p2p:
-        rot = mixed and 3 <= a.p <= 16
+        rot = 3 <= a.p <= 16 or not mixed
         work = full["n_m2l"] * (m2l_rot_flops(a.p) if rot else m2l_flops(a.p))
         t_k, t_ph = k_m2l, t_m2l
-        kern = ("k_m2l_rot (App. A.5 rotations and eq. A31, orders > 2 in FP32)" if rot
-                else "k_m2l_rounds (eq. 3b, orders > 2 in FP32)" if mixed else "k_m2l (eq. 3b, FP64)")
+        kern = ("k_m2l_f64 (App. A.5 rotations and eq. A31, FP64)" if not mixed
+                else "k_m2l_rot (App. A.5 rotations and eq. A31, orders > 2 in FP32)" if rot
+                else "k_m2l_rounds (eq. 3b, orders > 2 in FP32)")
     else:
         work = 20.0 * full["p2p_interactions"]
         t_k, t_ph = k_p2p, t_p2p
