@@ -11,9 +11,12 @@
 // scan of one to three kernels and a scatter), for long ones the traffic (the keys were read twice a
 // pass).  A 1e4 evaluation had 0.67 ms of sort and scan kernels in histogram, scan and scatter form and
 // has 0.27 ms so; whole calls 2.52 -> 2.22 ms (1e4), 4.97 -> 4.44 (1e5).
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 namespace gb3 {
+namespace cg = cooperative_groups;
 namespace {
 
 typedef unsigned long long u64;
@@ -342,6 +345,154 @@ int passes_of(K* keys, int* vals, K* keys_alt, int* vals_alt, long long n, const
     return passes & 1;
 }
 
+// ---------------------------------------------------------------- sort in one cluster
+// All passes of a short array in one cluster of eight blocks: the items stay in registers and shared
+// memory, a pass exchanges the blocks' digit counts and then the items through distributed shared memory.
+// lin != nullptr: the items are pairs, packed and unpacked as above; else kin (and vin).  Every index of
+// kClBlocks * 1024 * ITEMS is held; those from n on have all bits set and stay last (the order is stable).
+// What bounds it: the chain of a pass (ranking, two cluster barriers): 1e4 keys with values, eight passes,
+// 44 us (as launches 68 and the histogram), lists of 5.3e4, 1.2e4 and 6e3 pairs, three passes, 31, 15 and 12 us
+// (33, 27 and 27); calls of 1e4 particles 1.26 -> 1.21 ms, of 2000 without allocations 1.16 -> 1.07.  The lines:
+// 6.1e4 keys with values 129 us in the cluster and 78 as launches, 5.3e4 pairs as above.
+constexpr int kClBlocks = 8, kClThreads = 1024;
+constexpr long long kClMax = (long long)kClBlocks * kClThreads * 8, kClMaxVals = kClMax / 2;
+template <class K, bool VALS, int ITEMS>
+__global__ void __launch_bounds__(kClThreads) k_sort_cluster(const int2* lin, const K* kin, const int* vin, int n,
+                                                             int begin_bit, int passes, int xb, int2* lout, K* kout,
+                                                             int* vout) {
+    constexpr int kHold = kClThreads * ITEMS;  // items of a block (a power of two)
+    extern __shared__ __align__(16) unsigned char csm[];
+    K* buf = (K*)csm;
+    int* vbuf = (int*)(buf + kHold);
+    __shared__ unsigned wc[32][256], part[4][256], tot[256], at[256], sw[8];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, b = (int)blockIdx.x, d0 = t & 255, q = t >> 8;
+    const int local = w * ITEMS * 32 + lane;  // the thread's items: local + 32 i
+    K key[ITEMS];
+    int val[VALS ? ITEMS : 1];
+    unsigned rank[ITEMS];
+    for (int p = 0; p < passes; ++p) {
+        const int shift = begin_bit + 8 * p;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int j = local + 32 * i;
+            if (p) {
+                key[i] = buf[j];
+                if (VALS) val[i] = vbuf[j];
+            } else {
+                const int g = b * kHold + j;
+                key[i] = ~(K)0;
+                if (VALS) val[i] = 0;
+                if (g < n) {
+                    if (lin) {
+                        const int2 v = lin[g];
+                        key[i] = (K)(((u64)(unsigned)v.y << xb) | (u64)(unsigned)v.x);
+                    } else {
+                        key[i] = kin[g];
+                        if (VALS) val[i] = vin[g];
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) wc[8 * q + k][d0] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int d = (int)((key[i] >> shift) & 255);
+            unsigned peers = 0xffffffffu;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const unsigned on = (d >> k) & 1 ? 0xffffffffu : 0u;
+                peers &= ~(on ^ __ballot_sync(0xffffffffu, on != 0u));
+            }
+            const unsigned c = wc[w][d];
+            rank[i] = c + __popc(peers & ((1u << lane) - 1u));
+            __syncwarp();
+            if (lane == __ffs(peers) - 1) wc[w][d] = c + __popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        // digit d0: the warps' offsets (8 warps per thread) and the block's count
+        unsigned own = 0;
+        unsigned c8[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            c8[k] = own;
+            own += wc[8 * q + k][d0];
+        }
+        part[q][d0] = own;
+        __syncthreads();
+        unsigned off = 0;
+        for (int k = 0; k < q; ++k) off += part[k][d0];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) wc[8 * q + k][d0] = off + c8[k];
+        if (q == 3) tot[d0] = off + own;
+        cl.sync();  // all counts are there, and every block's items are in registers
+        unsigned x = 0, before = 0, all = 0;
+        if (t < 256) {
+            for (int r = 0; r < kClBlocks; ++r) {
+                const unsigned v = *cl.map_shared_rank(tot + d0, r);
+                if (r < b) before += v;
+                all += v;
+            }
+            x = all;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) sw[w] = x;
+        }
+        __syncthreads();
+        if (t < 256) {
+            for (int k = 0; k < w; ++k) x += sw[k];
+            at[d0] = x - all + before;
+        }
+        __syncthreads();
+        const bool last = p == passes - 1;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int d = (int)((key[i] >> shift) & 255);
+            const unsigned pos = at[d] + wc[w][d] + rank[i];
+            if (!last) {
+                const int r = (int)(pos / kHold), j = (int)(pos % kHold);
+                *cl.map_shared_rank(buf + j, r) = key[i];
+                if (VALS) *cl.map_shared_rank(vbuf + j, r) = val[i];
+            } else if (pos < (unsigned)n) {
+                if (lout) {
+                    const K mask = xb >= (int)(8 * sizeof(K)) ? ~(K)0 : (K)(((K)1 << xb) - 1);
+                    lout[pos] = make_int2((int)(unsigned)(key[i] & mask), (int)(key[i] >> xb));
+                } else {
+                    kout[pos] = key[i];
+                    if (VALS) vout[pos] = val[i];
+                }
+            }
+        }
+        cl.sync();  // the items of the next pass are there; the counts have been read
+    }
+}
+template <class K, bool VALS, int ITEMS>
+void go_cluster(int2* list, const K* kin, const int* vin, int n, int begin_bit, int passes, int xb, K* kout, int* vout,
+                cudaStream_t s) {
+    const size_t sm = (size_t)kClThreads * ITEMS * (sizeof(K) + (VALS ? sizeof(int) : 0));
+    auto kern = k_sort_cluster<K, VALS, ITEMS>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    launch_cluster8(kern, kClBlocks, kClThreads, sm, s, (const int2*)list, kin, vin, n, begin_bit, passes, xb, list,
+                    kout, vout);
+    note_launch();
+}
+// n <= kClMax (with values kClMaxVals); pairs in place in list, or kin, vin to kout, vout (which may be the same arrays)
+template <class K, bool VALS>
+void sort_cluster(int2* list, const K* kin, const int* vin, int n, int begin_bit, int passes, int xb, K* kout,
+                  int* vout, cudaStream_t s) {
+    const int per = kClBlocks * kClThreads;
+    if (n <= per) go_cluster<K, VALS, 1>(list, kin, vin, n, begin_bit, passes, xb, kout, vout, s);
+    else if (n <= 2 * per) go_cluster<K, VALS, 2>(list, kin, vin, n, begin_bit, passes, xb, kout, vout, s);
+    else if (n <= 4 * per) go_cluster<K, VALS, 4>(list, kin, vin, n, begin_bit, passes, xb, kout, vout, s);
+    else if constexpr (!VALS) go_cluster<K, VALS, 8>(list, kin, vin, n, begin_bit, passes, xb, kout, vout, s);
+}
+
 int bits_for(long long v) {
     int b = 1;
     while ((1LL << b) < v) ++b;
@@ -358,9 +509,17 @@ int radix_sort_pairs_bits(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx
                           int begin_bit, int end_bit, cudaStream_t s) {
     if (n <= 1) return 0;
     const int passes = (end_bit - begin_bit + 7) / 8;
+    u64 *ka = (u64*)keys, *kb = (u64*)keys_alt;
+    if (n <= (idx ? kClMaxVals : kClMax)) {
+        u64* out = passes & 1 ? kb : ka;
+        if (idx)
+            sort_cluster<u64, true>(nullptr, ka, idx, (int)n, begin_bit, passes, 64, out, passes & 1 ? idx_alt : idx, s);
+        else
+            sort_cluster<u64, false>(nullptr, ka, nullptr, (int)n, begin_bit, passes, 64, out, nullptr, s);
+        return passes & 1;
+    }
     const RsTmp T(tmp, n);
     cudaMemsetAsync(T.st, 0, T.bytes, s);
-    u64 *ka = (u64*)keys, *kb = (u64*)keys_alt;
     k_rs_hist<u64><<<grid_for(n, 256 * kRsItems, 4), 256, 0, s>>>(ka, n, begin_bit, passes, T.hist);
     note_launch();
     return idx ? passes_of<u64, true>(ka, idx, kb, idx_alt, n, T, begin_bit, passes, nullptr, 64, s)
@@ -383,10 +542,14 @@ size_t list_sort_tmp_bytes(long long npairs, int /*ncells*/) {
 // hold them), the last one writing pairs
 template <class K>
 static void sort_list(int2* list, long long npairs, int xb, int bits, void* tmp, cudaStream_t s) {
+    const int passes = (bits + 7) / 8;
+    if (npairs <= kClMax) {
+        sort_cluster<K, false>(list, nullptr, nullptr, (int)npairs, 0, passes, xb, nullptr, nullptr, s);
+        return;
+    }
     K* k0 = (K*)tmp;
     K* k1 = k0 + npairs;
     const RsTmp T(k1 + npairs, npairs);
-    const int passes = (bits + 7) / 8;
     cudaMemsetAsync(T.st, 0, T.bytes, s);
     k_rs_pack<K><<<grid_for(npairs, 256 * kRsItems, 4), 256, 0, s>>>(list, npairs, xb, passes, k0, T.hist);
     note_launch();

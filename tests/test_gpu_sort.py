@@ -49,3 +49,20 @@ def test_order_and_lists(g, n):
     for lst in (d["m2l"], d["p2p"]):
         key = lst[:, 1] * (1 << 32) + lst[:, 0]
         assert np.all(np.diff(key) > 0)
+
+
+@pytest.mark.parametrize("n", [8191, 8192, 8193, 16384, 16385, 32768, 32769, 65536, 65537])
+@pytest.mark.parametrize("leaf", [16, 256])
+def test_order_and_lists_in_one_cluster(g, n, leaf):
+    """Sizes at the edges of the sort in one cluster (items per thread 1, 2, 4, 8, then the passes as
+    launches); lists of about 1e4 to 1e6 pairs."""
+    x, mu = inputs.plummer(n, 400 + n)
+    x[7:900] = x[7]
+    ctx = g.Context(p=6, eps=1e-5, leaf_size=leaf, p2p_c=1.0)
+    ctx.fmm_evaluate(_dev(x), _dev(mu))
+    d = ctx.fmm_debug_dump()
+    ctx.close()
+    assert np.array_equal(d["perm"], np.argsort(_morton(x), kind="stable"))
+    for lst in (d["m2l"], d["p2p"]):
+        key = lst[:, 1] * (1 << 32) + lst[:, 0]
+        assert np.all(np.diff(key) > 0)
