@@ -10,7 +10,7 @@
 // What bounds them: for the short arrays of small systems the launches (a pass was a histogram, a
 // scan of one to three kernels and a scatter), for long ones the traffic (the keys were read twice a
 // pass).  A 1e4 evaluation had 0.67 ms of sort and scan kernels in histogram, scan and scatter form and
-// has 0.27 ms so; whole calls 2.52 -> 2.22 ms (1e4), 4.97 -> 4.44 (1e5).
+// had 0.27 ms so; whole calls 2.52 -> 2.22 ms (1e4), 4.97 -> 4.44 (1e5).  Short sorts now run in one cluster.
 #include <cooperative_groups.h>
 
 #include "kernels.cuh"
