@@ -11,9 +11,10 @@
 // warp in groups of 8 lanes.  A chunk's pairs are added in list order and a sink's chunks in chunk
 // order, whatever shares their warp, so a system gives the same bits in an ensemble as alone.
 // Shared memory holds, per warp, the rotated multipoles (entries |m| <= min(k, p - k) only, all that
-// eq. A31 reads: 113 of 225 at p = 14) and three work vectors: four warps an SM at p = 14, which is
-// what the pipe needs.  1e5 particles, p = 10 (598,127 pairs): 31.9 ms with eq. 3b term by term, 5.0 ms
-// so (2.9 ms at the pipe's rate); 6e4 cusp, p = 14 (143,081 pairs): 30.7 -> 3.5 ms (1.6).
+// eq. A31 reads: 113 of 225 at p = 14) and work vectors of 4 p + 3 rows: five warps an SM at p = 14,
+// eight at p = 10 (two more rows of 2 p + 1 left room for four and six, and for some of the latency:
+// 5.0 and 3.5 ms below).  1e5 particles, p = 10 (598,127 pairs): 31.9 ms with eq. 3b term by term, 4.36 ms
+// so (2.9 ms at the pipe's rate); 6e4 cusp, p = 14 (143,081 pairs): 30.7 -> 3.10 ms (1.6).
 #include <vector>
 
 #include "kernels.cuh"
@@ -147,7 +148,7 @@ __host__ __device__ inline int rot_entries(int p) {  // sum over k of 2 min(k, p
     return t;
 }
 __host__ inline size_t m2l_f64_smem(int p) {
-    return ((size_t)rot_entries(p) * 32 + 3 * (size_t)(2 * p + 1) * kPitch) * sizeof(double);
+    return ((size_t)rot_entries(p) * 32 + (size_t)(4 * p + 3) * kPitch) * sizeof(double);
 }
 
 // ---------------------------------------------------------------- work items
@@ -236,7 +237,6 @@ __global__ void __launch_bounds__(32) k_m2l_f64(const int2* __restrict__ list, c
     double* S = dsm + lane;
     double* const w0 = dsm + rot_entries(p) * 32;
     double* const w1 = w0 + (2 * p + 1) * kPitch;
-    double* const w2 = w1 + (2 * p + 1) * kPitch;
     const unsigned n0 = it.counts[0], n1 = it.counts[1], n2 = it.counts[2], n3 = it.counts[3];
     const unsigned i2 = (n2 + 1) / 2, i1 = n1 > n3 ? (n1 - n3 + 3) / 4 : 0;
     for (;;) {
@@ -356,12 +356,12 @@ __global__ void __launch_bounds__(32) k_m2l_f64(const int2* __restrict__ list, c
         };
         for (int n = 0; 2 * n <= P; ++n) {
             const int o = P - n;
-            back(n, w1);
-            if (o > n) back(o, w2);
+            back(n, w1);  // (its 2 n + 1 rows and those of o together are 2 P + 2)
+            if (o > n) back(o, w1 + (2 * n + 1) * kPitch);
             __syncwarp();
             const int ra = 2 * n + 1, rows = o > n ? 2 * P + 2 : ra;
             for (int r = lane; r < rows; r += 32) {
-                const double* x = r < ra ? w1 + r * kPitch : w2 + (r - ra) * kPitch;
+                const double* x = w1 + r * kPitch;
                 const int i = r < ra ? n * n + r : o * o + r - ra;
                 const double nm = __ldg(&g_tab.norm[i]);
                 for (int k = 0; k < nch; ++k) {

@@ -1345,8 +1345,12 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
         auto go = [&](auto kern) {
-            // eight warps per SM keep the FP64 pipe busy; more only take items early
-            const int nblocks = item_blocks(kern, kP2PWarpsD * 32, nitems, 2);
+            // Eight warps per SM keep the FP64 pipe busy, and with few items per warp more only take the long
+            // ones early (both P2P kernels of 4096 particles 0.99 ms, 0.95 with two blocks per SM).  With many items every
+            // resident block: two per SM crowd on the SMs that the M2L beside them leaves first (cusp of 6e4
+            // 28.6 ms, 21.5 so).
+            const bool few = nitems <= 4 * 2 * kP2PWarpsD * sm_count();
+            const int nblocks = item_blocks(kern, kP2PWarpsD * 32, nitems, few ? 2 : 32);
             kern<<<nblocks, kP2PWarpsD * 32, 0, s>>>(xm, c, leaves, ranges, pc, items, nitems, counter, psi, acc, part);
         };
         if (want_f) go(k_p2p_f64<true>);
