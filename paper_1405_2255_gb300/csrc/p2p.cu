@@ -1026,9 +1026,13 @@ __global__ void __launch_bounds__(kP2PWarpsD * 32)
 // sums.  30 packed FP32 operations and two rsqrt for the two pairs of a slot: bound by the FMA pipe.
 // The R groups of S lanes take tiles of their own, all in step: the source cells are cut into tiles 32
 // records at a time, the tiles ordered by length and dealt to the groups, so that the tiles of a round
-// are about equally long (the shorter ones are filled up with massless sources).  150,001 particles,
-// 1.16e9 pairs: 19.0 ms with one warp per leaf and one sink per lane (the longest leaf ran on alone),
-// 3.3 ms with groups that run through their tiles on their own (they diverge), 2.2 ms so.
+// are about equally long.  The shorter ones are filled up with massless sources beside the leaf: its first
+// particle moved by 4 units in x (the extent is below 2; of a system without extent, whose coordinates
+// are not scaled, the low part holds the move), so that 1 / r^2 and r^2 stay in range wherever the
+// leaf lies.  (A filler at a fixed place is no zero term: for a sink within 5e-20 of it 1 / r^2 overflows,
+// for one farther than 1.8e19 r^2 does, and 0 times infinity is NaN.)  150,001 particles, 1.16e9 pairs:
+// 19.0 ms with one warp per leaf and one sink per lane (the longest leaf ran on alone), 3.3 ms with
+// groups that run through their tiles on their own (they diverge), 2.2 ms so.
 constexpr int kTidWarps = 4;
 constexpr int kTidTile = 32;
 constexpr int kTidGroups = 4;  // PlanTidal's largest R
@@ -1077,6 +1081,7 @@ __global__ void __launch_bounds__(kTidWarps * 32)
                       unsigned* __restrict__ counter, double* __restrict__ T, double* __restrict__ part) {
     __shared__ __align__(16) float4 bufs[kTidWarps][2][kTidGroups][2 * kTidTile];
     __shared__ int2 tiles_all[kTidWarps][kTidBatch], sorted_all[kTidWarps][kTidBatch];
+    __shared__ __align__(16) float4 fill_all[kTidWarps][2];  // the record of the fillers
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const f2 zero = f2_pack(0.f, 0.f);
     for (;;) {
@@ -1107,6 +1112,12 @@ __global__ void __launch_bounds__(kTidWarps * 32)
 #pragma unroll
         for (int q = 0; q < 6; ++q) sh[q] = sl[q] = zero;
         int2 *tiles = tiles_all[wid], *sorted = sorted_all[wid];
+        float4* fill = fill_all[wid];
+        if (lane < 2) {
+            fill[lane] = xp[2 * (size_t)first + lane];
+            if (lane == 0) fill[0].w = 0.f;
+            else fill[1].x += 4.f;
+        }
         const int end = pc.r1[pv];
         int at = pc.r0[pv], off = 0;  // the next record and the tiles of it that are done
         while (at < end) {
@@ -1153,7 +1164,13 @@ __global__ void __launch_bounds__(kTidWarps * 32)
                 float4* buf = bufs[wid][b][g];
                 const float4* src = xp + 2 * (size_t)t.x;
                 for (int j = slot; j < 2 * t.y; j += S) cp_async16(buf + j, src + j);
-                for (int j = 2 * t.y + slot; j < 2 * nmax; j += S) buf[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (t.y < nmax) {
+                    const float4 fh = fill[0], fl = fill[1];
+                    for (int j = t.y + slot; j < nmax; j += S) {
+                        buf[2 * j] = fh;
+                        buf[2 * j + 1] = fl;
+                    }
+                }
             };
             fetch(0, 0);
             cp_async_commit();

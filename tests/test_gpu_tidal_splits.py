@@ -51,6 +51,42 @@ def test_mixed_near_tidal_splits(g, n, leaf):
     assert np.max(np.abs(T - ref) / mag[:, None]) < 4e-6
 
 
+def _near_ref(x, mu):
+    """Plain FP64 sums over all pairs, and the sums of the terms' magnitudes."""
+    d = x[None] - x[:, None]
+    r2 = (d * d).sum(2)
+    q3 = np.where(r2 > 0, mu / np.where(r2 > 0, r2, 1.0) ** 1.5, 0.0)
+    q5 = np.where(r2 > 0, q3 / np.where(r2 > 0, r2, 1.0), 0.0)
+    ref = [(3 * q5 * d[:, :, i] * d[:, :, j] - (q3 if i == j else 0.0)).sum(1)
+           for i, j in [(0, 0), (0, 1), (0, 2), (1, 1), (1, 2), (2, 2)]]
+    return np.stack(ref, 1), 3 * q3.sum(1)
+
+
+@pytest.mark.parametrize("r", [2.0 ** k for k in (-62, -64, -68, -71, -74, -77)])
+@pytest.mark.parametrize("leaf", [1, 9, 17, 40])
+def test_mixed_near_tidal_at_the_origin(g, leaf, r):
+    """A particle so near the origin that its squared distance from it is an FP32 subnormal (or 0): the
+    fillers of short tiles add nothing wherever it lies (bound as in test_mixed_near_tidal_splits)."""
+    x, mu = inputs.plummer(1200, 41)
+    x[7] = (r, 0.0, 0.0)
+    ctx = g.Context(p=3, eps=1e-30, leaf_size=leaf, p2p_c=1.0, precision=g.FMM_PREC_MIXED)
+    T = ctx.fmm_evaluate_active(_dev(x), _dev(mu), tidal=True)[2].cpu().numpy()
+    ctx.close()
+    ref, mag = _near_ref(x, mu)
+    assert np.max(np.abs(T - ref) / mag[:, None]) < 4e-6
+
+
+@pytest.mark.parametrize("n", [1, 2, 5])
+@pytest.mark.parametrize("at", [1e15, 1e19, 1e20, 1e30, 3e38])
+def test_mixed_near_tidal_of_one_place(g, n, at):
+    """All particles at one place (no extent to scale by): the tensor is 0 at any coordinates."""
+    x, mu = np.full((n, 3), at), np.ones(n)
+    ctx = g.Context(p=3, leaf_size=8, precision=g.FMM_PREC_MIXED)
+    T = ctx.fmm_evaluate_active(_dev(x), _dev(mu), tidal=True)[2].cpu().numpy()
+    ctx.close()
+    assert np.array_equal(T, np.zeros((n, 6)))
+
+
 @pytest.mark.parametrize("p", [1, 2, 3, 7, 14, 18])
 def test_far_tidal_orders(g, orc, p):
     """The far part alone differs from the oracle's only by FP64 rounding (FP64 mode, 1e-10 of the
