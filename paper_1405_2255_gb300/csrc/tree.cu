@@ -269,16 +269,22 @@ void launch_gather(const double* x, const double* mu, const int* idx, int n, d4*
 // The mixed-precision path works in units in which the system's extent and its largest mass
 // lie in [1, 2): positions and masses are scaled by powers of two (exact), so the FP32
 // parts (pair terms, high expansion orders, estimate) stay in range whatever the caller's
-// units, and the outputs are scaled back exactly.  One thread; e[0], e[1]: the exponents.
+// units, and the outputs are scaled back exactly.  Without extent (every system at one place, all results
+// 0) the lengths keep their units, unless the coordinates themselves are too large for FP32: then the
+// largest is scaled to [1, 2).  One thread; e[0], e[1]: the exponents.
 __global__ void k_work_units(const unsigned long long* __restrict__ b, int nsys, int* __restrict__ e) {
     if (blockIdx.x || threadIdx.x) return;
     const int ns = nsys > 0 ? nsys : 1;
-    double ext = 0.0;
+    double ext = 0.0, far = 0.0;
     for (int k = 0; k < ns; ++k)
         for (int d = 0; d < 3; ++d) {
             const double lo = key_dbl(b[6 * k + d]), hi = key_dbl(b[6 * k + 3 + d]);
-            if (hi >= lo) ext = fmax(ext, hi - lo);
+            if (hi >= lo) {
+                ext = fmax(ext, hi - lo);
+                far = fmax(far, fmax(fabs(lo), fabs(hi)));
+            }
         }
+    if (ext == 0.0 && far >= 0x1p127) ext = far;
     const double mmax = key_dbl(b[6 * ns]);
     const bool use_m = b[6 * ns] != 0ull && mmax > 0.0 && isfinite(mmax);
     int el = (ext > 0.0 && isfinite(ext)) ? ilogb(ext) : 0, em = use_m ? ilogb(mmax) : 0;

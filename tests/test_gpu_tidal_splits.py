@@ -87,6 +87,18 @@ def test_mixed_near_tidal_of_one_place(g, n, at):
     assert np.array_equal(T, np.zeros((n, 6)))
 
 
+@pytest.mark.parametrize("n", [1, 3, 20])
+@pytest.mark.parametrize("at", [2.0 ** 127, 1e39, -1e100, 1e300])
+def test_one_place_beyond_fp32(g, n, at):
+    """The same where the coordinates have no FP32 value: every result is 0."""
+    x, mu = np.full((n, 3), at), np.full(n, 0.5)
+    ctx = g.Context(p=3, leaf_size=8, precision=g.FMM_PREC_MIXED)
+    out = ctx.fmm_evaluate_active(_dev(x), _dev(mu), tidal=True)
+    ctx.close()
+    for t in out:
+        assert np.array_equal(t.cpu().numpy(), np.zeros(tuple(t.shape)))
+
+
 @pytest.mark.parametrize("p", [1, 2, 3, 7, 14, 18])
 def test_far_tidal_orders(g, orc, p):
     """The far part alone differs from the oracle's only by FP64 rounding (FP64 mode, 1e-10 of the
