@@ -59,14 +59,16 @@ __global__ void __launch_bounds__(kDirThreads) k_direct(const double* __restrict
             const double r2 = dx * dx + dy * dy + dz * dz;
             if (positive_bits(r2)) {
                 const double rinv = rsqrt(r2);
+                // (mu / r, mu / r^2, mu / r^3 in this order: 1 / r^2 alone overflows for a subnormal r^2,
+                // and a massless source would give NaN)
                 const double qm = q.w * rinv;
-                const double r2i = rinv * rinv;
-                const double q3 = qm * r2i;
+                const double q2 = qm * rinv;
+                const double q3 = q2 * rinv;
                 v[0] += qm;
                 v[1] = fma(q3, dx, v[1]);
                 v[2] = fma(q3, dy, v[2]);
                 v[3] = fma(q3, dz, v[3]);
-                if (WANT_F) v[NV - 1] = fma(q.w, r2i, v[NV - 1]);
+                if (WANT_F) v[NV - 1] += q2;
             }
         }
     }

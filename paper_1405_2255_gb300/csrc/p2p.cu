@@ -917,12 +917,12 @@ __device__ __forceinline__ void tile_f64(const d4* __restrict__ tile, int nt, in
             const double dx = a.x - b[u][0], dy = a.y - b[u][1], dz = a.z - b[u][2];
             const double r2 = dx * dx + dy * dy + dz * dz;
             if (positive_bits(r2)) {
-                const double rinv = rsqrt(r2);
-                const double r2i = rinv * rinv;
+                // (no 1 / r^2 by itself: it overflows for a subnormal r^2, and a massless source would give NaN)
+                const double rinv = rsqrt(r2), qm = a.w * rinv;
                 if (WANT_F) {
-                    v[u][0] = fma(a.w, r2i, v[u][0]);
+                    v[u][0] = fma(qm, rinv, v[u][0]);
                 } else {
-                    const double qm = a.w * rinv, q3 = qm * r2i;
+                    const double q3 = qm * rinv * rinv;
                     v[u][0] += qm;
                     v[u][1] = fma(q3, dx, v[u][1]);
                     v[u][2] = fma(q3, dy, v[u][2]);

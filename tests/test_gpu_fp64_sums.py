@@ -84,6 +84,29 @@ def test_fp64_p2p_splits(g, n, leaf, mac):
     ctx.close()
 
 
+@pytest.mark.parametrize("m", [0.0, 1e-20])
+def test_subnormal_squared_distance(g, m):
+    """Two light particles whose squared distance is subnormal (1e-310, with a dozen digits) and one of
+    mass 1: a massless source adds nothing, and mu / r^2 is finite where its value is."""
+    x = np.zeros((3, 3))
+    x[1, 0], x[2, 0] = 1e-155, 1.0
+    mu = np.array([m, m, 1.0])
+    near = m * 1e155 * 1e155  # mu / r^2
+    ctx = g.Context(p=3, leaf_size=8, mac=1, precision=g.FMM_PREC_FP64)
+    psi, acc, f = (t.cpu().numpy() for t in ctx.fmm_direct(_dev(x), _dev(mu), want_f=True))
+    psi2, acc2 = (t.cpu().numpy() for t in ctx.fmm_evaluate(_dev(x), _dev(mu)))
+    d = ctx.fmm_debug_dump()
+    f2 = np.empty(3)
+    f2[d["perm"]] = d["scale"]
+    ctx.close()
+    for p, a, ff in ((psi, acc, f), (psi2, acc2, f2)):
+        assert np.allclose(p, [1.0 + m * 1e155, 1.0 + m * 1e155, 2 * m], rtol=1e-12, atol=0)
+        assert np.allclose(ff, [1.0 + near, 1.0 + near, 2 * m], rtol=1e-12, atol=0)
+        assert np.allclose(a[2], [-2 * m, 0, 0], rtol=1e-12, atol=0)
+        if m == 0.0:
+            assert np.array_equal(a[:2], [[1.0, 0, 0], [1.0, 0, 0]])
+
+
 @pytest.mark.parametrize("p", [1, 2, 3, 9, 16, 17, 18])
 @pytest.mark.parametrize("shape", ["plummer", "z axis", "x axis", "plane"])
 def test_fp64_m2l_orders_and_directions(g, orc, p, shape):
