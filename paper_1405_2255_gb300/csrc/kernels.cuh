@@ -284,11 +284,16 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
                         bool shares = false, const int* off = nullptr, int nsys = 0);
 // whether a forest whose smallest system has this many particles has pieces to be shared
 bool p2p_shares(int smallest_system);
+// the partial sums of split items that a system of n particles may take in a work plan: base + per n bytes
+struct PlanBudget {
+    double base, per;
+};
+PlanBudget plan_budget(const fmm_params& prm);  // (capi.cu)
 // FP64 P2P with a work plan as launch_p2p_mixed's (the same scratch, return value and host read);
 // want_f: psi receives sum mu / r^2 instead (eq. 6; acc is scratch)
 size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,
-                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, void* tmp,
-                           size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
+                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, PlanBudget bg,
+                           void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
 // ordered pairs of distinct particles at distance 0 (sorted keys and positions); with
 // an ensemble (off != nullptr) only pairs inside one system count
 void launch_coincident(const d4* xm, const uint64_t* keys, int n, unsigned long long* coincident, cudaStream_t s,
@@ -331,7 +336,7 @@ void launch_p2p_tidal(const d4* xm, const float4* xp, int n, bool fp32, Cells c,
 // the near part in mixed precision with a work plan as launch_p2p_mixed's (same scratch, return value
 // and host read)
 size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
-                             const int* seg_end, const int* leaves, int nleaves, double* T, void* tmp,
+                             const int* seg_end, const int* leaves, int nleaves, double* T, PlanBudget bg, void* tmp,
                              size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s);
 void launch_finish_tidal(const double* Tf, const double* Tn, const int* perm, int n, double G,
                          const unsigned char* pact, double* T, cudaStream_t s, const int* e = nullptr);

@@ -154,11 +154,11 @@ int p2p_na(Run& r, const float4* xp, const int2* list, const int* seg_start, con
 }
 
 // the FP64 P2P (want_f: the near sums of f into psi) likewise; false when its plan does not fit there
-bool p2p_f64_na(Run& r, const int2* list, const int* seg_start, const int* seg_end, double* psi, double* acc,
-                bool want_f) {
+bool p2p_f64_na(Run& r, const fmm_params& prm, const int2* list, const int* seg_start, const int* seg_end, double* psi,
+                double* acc, bool want_f) {
     unsigned long long h_tot[6] = {0, 0, 0, 0, 0, 0};
     return launch_p2p_f64_plan(r.xm, r.n, r.c, list, seg_start, seg_end, r.leaves, r.nleaves, psi, acc, want_f,
-                               r.p2p_tmp, r.p2p_tmp_bytes, h_tot, r.s) <= r.p2p_tmp_bytes;
+                               plan_budget(prm), r.p2p_tmp, r.p2p_tmp_bytes, h_tot, r.s) <= r.p2p_tmp_bytes;
 }
 
 int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu, double G, double* psi, double* acc) {
@@ -282,7 +282,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
         if (want_f) {
             launch_f_m2l(est_m2l, m2l_seg_start, m2l_seg_end, nc, r.c, Ff, s);
             for (int L = 1; L < nl; ++L) launch_f_down_level(r.c, r.lev[L], r.lev[L + 1], Ff, s);
-            if (p2p_f64_na(r, est_p2p, seg_start, seg_end, psi_near, acc_near, true))
+            if (p2p_f64_na(r, prm, est_p2p, seg_start, seg_end, psi_near, acc_near, true))
                 launch_f_add(r.c, r.leaves, r.nleaves, Ff, psi_near, scale, s);
             else
                 launch_f_p2p(r.xm, r.c, est_p2p, seg_start, seg_end, r.leaves, r.nleaves, Ff, scale, s);
@@ -295,7 +295,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
             if (prm.precision == FMM_PREC_MIXED) {
                 rc = p2p_na(r, xp, est_p2p, seg_start, seg_end, psi_near, acc_near, 0);
                 if (rc) return rc;
-            } else if (!p2p_f64_na(r, est_p2p, seg_start, seg_end, psi_near, acc_near, false))
+            } else if (!p2p_f64_na(r, prm, est_p2p, seg_start, seg_end, psi_near, acc_near, false))
                 launch_p2p_fp64(r.xm, r.c, est_p2p, seg_start, seg_end, r.leaves, r.nleaves, psi_near, acc_near, s);
             launch_est_scale(r.c, r.leaves, r.nleaves, F1, acc_near, scale, s);
         }
@@ -354,7 +354,7 @@ int evaluate_na(Run& r, const fmm_params& prm, const double* x, const double* mu
     if (prm.precision == FMM_PREC_MIXED) {
         rc = p2p_na(r, xp, p2p, seg_start, seg_end, psi_near, acc_near, prm.p2p_two_float);
         if (rc) return rc;
-    } else if (!p2p_f64_na(r, p2p, seg_start, seg_end, psi_near, acc_near, false))
+    } else if (!p2p_f64_na(r, prm, p2p, seg_start, seg_end, psi_near, acc_near, false))
         launch_p2p_fp64(r.xm, r.c, p2p, seg_start, seg_end, r.leaves, r.nleaves, psi_near, acc_near, s);
     for (int L = 1; L < nl; ++L) {
         if (split) launch_l2l_split(r.c, r.c.sr, pw, r.lev[L], r.lev[L + 1], p, F, s);

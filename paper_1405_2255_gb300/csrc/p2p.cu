@@ -181,6 +181,7 @@ struct Chunk {
 // pair), then k = ceil(c / (2 S)) so that no item is empty.  Items longer than piece_steps steps
 // are split (see below).
 struct PlanMixed {
+    static constexpr bool budget = false;
     static constexpr unsigned piece_steps = 8192, sub_steps = 1024;
     static constexpr int sub_n = 16384;  // particles of the largest system whose pieces are shared
     static constexpr int max_pieces = 64;
@@ -209,8 +210,10 @@ struct PlanMixed {
 // The FP64 P2P is bound by the FP64 pipe alone (an instruction costs the same however many lanes
 // are active, staging runs beside it): the fewest steps k Q / R per source over S <= 32 slots and
 // Q <= 4 sinks per slot.  Short pieces (a step of 18 FP64 instructions holds a quarter of an SM for
-// 1152 cycles, so 256 steps are 0.14 ms) keep every SM busy to the end.
+// 1152 cycles, so 256 steps are 0.14 ms) keep every SM busy to the end; where there are many, longer
+// ones do too (k_p2p_pieces).
 struct PlanF64 {
+    static constexpr bool budget = true;
     static constexpr unsigned piece_steps = 256, sub_steps = 0;
     static constexpr int sub_n = 0;
     static constexpr int max_pieces = 1024;
@@ -246,6 +249,7 @@ struct PlanF64 {
 // The mixed tidal P2P: a slot holds two sinks as the halves of packed operations, and the R groups of
 // S lanes take shares of the source cells of their own: the fewest items k / R per source.
 struct PlanTidal {
+    static constexpr bool budget = true;
     static constexpr unsigned piece_steps = 1024, sub_steps = 0;
     static constexpr int sub_n = 0;
     static constexpr int max_pieces = 256;
@@ -279,7 +283,9 @@ __device__ inline bool p2p_near(const d4& a, const d4& b) {
 // (Q sources / R) has its stream of source cells cut into P = ceil(steps / piece_steps) <=
 // max_pieces pieces of about equal numbers of source cells, each with its own ranges, items
 // and FP64 partial sums, which k_p2p_reduce adds in piece order.  The split depends on the leaf
-// alone, so a system gives the same result in an ensemble as alone.
+// and its own system alone, so a system gives the same result in an ensemble as alone.
+// PL::budget: the pieces are short where that fills the device, and longer where their partial sums
+// would exceed the system's share of the workspace (k_p2p_pieces).
 // A piece of the mixed P2P of a small system is shared by U = its steps / sub_steps warps: its stream of
 // sources is cut at tile boundaries into U parts with ranges, items and partial sums of their own, so
 // the tiles and their FP32 sums are those of the whole piece.  With few leaves the longest item sets
@@ -292,19 +298,23 @@ __device__ inline bool p2p_near(const d4& a, const d4& b) {
 // at most: its own and its ancestors' segment lengths), its pieces P and their parts U as np[t] =
 // P | U << 16, its items per piece kc[t] and its sort key,
 // descending in the length of a piece's items (a lane's steps, Q source particles / R; 0 for a leaf
-// without active particles); tot[0] += nb
+// without active particles); tot[0] += nb.  work != nullptr: np[t] is the length of the leaf's items,
+// root[t] its system's root and work[root] the sum of length x sinks over the system; k_p2p_pieces follows
 template <class PL>
 __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* __restrict__ seg_start,
                             const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int sub_n,
                             int n, const int* __restrict__ off, int nsys, int* __restrict__ nb, int* __restrict__ np,
-                            int* __restrict__ kc, uint64_t* __restrict__ keys, unsigned long long* __restrict__ tot) {
+                            int* __restrict__ kc, uint64_t* __restrict__ keys, int* __restrict__ root,
+                            unsigned long long* __restrict__ work, unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long my = 0;
     for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nleaves; t += nw) {
         const int leaf = leaves[t];
         long long e = 0, src = 0;
+        int top = leaf;
         for (int cell = leaf; cell >= 0; cell = c.parent[cell]) {
+            top = cell;
             const int s0 = seg_start[cell], s1 = seg_end[cell];
             e += s1 - s0;
             for (int i = s0 + lane; i < s1; i += 32) src += c.count[list[i].x];
@@ -318,6 +328,12 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
             kc[t] = ch.k;
             const unsigned long long l = (unsigned long long)ch.Q * (unsigned long long)src / (unsigned long long)ch.R + 1;
             const unsigned len = !cell_active(c, leaf) ? 0u : (l > 0xfffffffeull ? 0xfffffffeu : (unsigned)l);
+            if (PL::budget && work) {
+                np[t] = (int)len;
+                root[t] = top;
+                atomicAdd(&work[top], (unsigned long long)len * (unsigned)c.count[leaf]);
+                continue;
+            }
             int P = (int)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
             const int cap = e < PL::max_pieces ? (int)e : PL::max_pieces;
             P = P < 1 ? 1 : (P > cap ? (cap > 0 ? cap : 1) : P);
@@ -336,6 +352,29 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
         }
     }
     if (lane == 0 && my) atomicAdd(&tot[0], my);
+}
+
+// The pieces of PL::budget's leaves.  A piece costs nv partial sums per sink, so pieces of L steps of a system
+// with the work A = sum of length x sinks take 8 nv A / L bytes: L is the shortest for which that is at most
+// base + per x the system's particles, and at least piece_steps.  (Of 256 steps in any system the FP64 plan's
+// partial sums took up to 10 KB per particle, of 1024 steps the tidal plan's up to 9 KB: 13 times the bound of the
+// whole workspace for leaves of 1024.)  A call takes 6 us longer, so it is left out where no system can
+// need it (an item has at most 4 steps per particle; 4096 particles).
+template <class PL>
+__global__ void k_p2p_pieces(Cells c, int nleaves, const int* __restrict__ nb, const int* __restrict__ root,
+                             const unsigned long long* __restrict__ work, PlanBudget bg, int* __restrict__ np,
+                             uint64_t* __restrict__ keys) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nleaves; t += gridDim.x * blockDim.x) {
+        const int r = root[t], e = nb[t];
+        const double L = ceil(8.0 * PL::nv * (double)work[r] / (bg.base + bg.per * (double)c.count[r]));
+        const unsigned len = (unsigned)np[t];
+        unsigned P;
+        if (L <= (double)PL::piece_steps) P = (unsigned)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
+        else P = (unsigned)((double)len / L);  // (rounded down: the sum stays within the share)
+        P = max(1u, min(P, (unsigned)max(1, min(e, PL::max_pieces))));
+        np[t] = (int)(P | 1u << 16);
+        keys[t] = ((uint64_t)(255u - qlen8((unsigned)(((unsigned long long)len + P - 1) / P))) << 32) | (unsigned)t;
+    }
 }
 
 // the warp's sum of v, and *before = the sum over the lanes below
@@ -1237,8 +1276,10 @@ PlanLayout plan_layout(void* base, int nleaves) {
         off += bytes;
         return r;
     };
-    L.k0 = (uint64_t*)take(nl * 8);
+    L.tot = (unsigned long long*)take(8 * 8);  // (tot, counter and k1 side by side: cleared together)
+    L.counter = (unsigned*)take(4 * 4);
     L.k1 = (uint64_t*)take(nl * 8);
+    L.k0 = (uint64_t*)take(nl * 8);
     L.order = (int*)take(nl * 4);
     L.nb = (int*)take(nl * 4);
     L.roff = (int*)take((nl + 1) * 4);
@@ -1252,8 +1293,6 @@ PlanLayout plan_layout(void* base, int nleaves) {
     L.split = (int2*)take(nl * 8);
     L.stmp = (int*)take(scan_tmp_ints((long long)nl + 1) * 4);
     L.rtmp = (int*)take(radix_tmp_ints((long long)nl) * 4);
-    L.tot = (unsigned long long*)take(8 * 8);
-    L.counter = (unsigned*)take(4 * 4);
     L.bytes = (off + 255) & ~(size_t)255;
     return L;
 }
@@ -1264,16 +1303,25 @@ PlanLayout plan_layout(void* base, int nleaves) {
 template <class PL, class RUN>
 size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, const int* seg_end, const int* leaves,
                     int nleaves, double* psi, double* acc, int mode, void* tmp, size_t tmp_bytes,
-                    unsigned long long* h_tot, bool shares, const int* off, int nsys, cudaStream_t s, RUN run) {
+                    unsigned long long* h_tot, bool shares, const int* off, int nsys, PlanBudget bg, cudaStream_t s,
+                    RUN run) {
     if (nleaves <= 0) return 0;
     if (n > kRangeMax) return ~(size_t)0;  // no range is ever cut: a leaf's region holds its source cells
     PlanLayout L = plan_layout(tmp, nleaves);
     if (tmp_bytes < L.bytes) return L.bytes;
-    cudaMemsetAsync(L.tot, 0, 8 * sizeof(unsigned long long), s);
-    cudaMemsetAsync(L.counter, 0, 4 * sizeof(unsigned), s);
+    const bool cut = PL::budget && 8.0 * PL::nv * n * (4.0 * n + 1.0) > (double)PL::piece_steps * (bg.base + bg.per * n);
+    unsigned long long* work = cut ? (unsigned long long*)L.k1 : nullptr;  // (k1 and voff have their own use later)
+    int* root = L.voff;
+    unsigned char* zero_end = cut ? (unsigned char*)(work + nleaves) : (unsigned char*)(L.counter + 4);  // (roots <= leaves)
+    cudaMemsetAsync(L.tot, 0, (size_t)(zero_end - (unsigned char*)L.tot), s);
     k_p2p_count<PL><<<grid_for((long long)nleaves * 32, 128, 16), 128, 0, s>>>(
-        c, list, seg_start, seg_end, leaves, nleaves, shares ? PL::sub_n : 0, n, off, nsys, L.nb, L.np, L.kc, L.k0, L.tot);
+        c, list, seg_start, seg_end, leaves, nleaves, shares ? PL::sub_n : 0, n, off, nsys, L.nb, L.np, L.kc, L.k0, root, work,
+        L.tot);
     note_launch();
+    if constexpr (PL::budget) if (cut) {
+        k_p2p_pieces<PL><<<grid_for(nleaves, 128), 128, 0, s>>>(c, nleaves, L.nb, root, work, bg, L.np, L.k0);
+        note_launch();
+    }
     scan_exclusive_i32(L.nb, L.roff, nleaves, L.roff + nleaves, L.stmp, s);
     // the low 32 bits are the leaf index, already in order: sort the 8 length bits only
     const int flip = radix_sort_pairs_bits(L.k0, nullptr, L.k1, nullptr, nleaves, L.rtmp, 32, 40, s);
@@ -1353,12 +1401,12 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
         note_launch();
     };
     return plan_and_run<PlanMixed>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, mode, tmp, tmp_bytes,
-                                   h_tot, shares, off, nsys, s, run);
+                                   h_tot, shares, off, nsys, PlanBudget{0.0, 0.0}, s, run);
 }
 
 size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const int* seg_start, const int* seg_end,
-                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, void* tmp,
-                           size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
+                           const int* leaves, int nleaves, double* psi, double* acc, bool want_f, PlanBudget bg,
+                           void* tmp, size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
         auto go = [&](auto kern) {
@@ -1375,11 +1423,11 @@ size_t launch_p2p_f64_plan(const d4* xm, int n, Cells c, const int2* list, const
         note_launch();
     };
     return plan_and_run<PlanF64>(n, c, list, seg_start, seg_end, leaves, nleaves, psi, acc, 0, tmp, tmp_bytes, h_tot,
-                                 false, nullptr, 0, s, run);
+                                 false, nullptr, 0, bg, s, run);
 }
 
 size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list, const int* seg_start,
-                             const int* seg_end, const int* leaves, int nleaves, double* T, void* tmp,
+                             const int* seg_end, const int* leaves, int nleaves, double* T, PlanBudget bg, void* tmp,
                              size_t tmp_bytes, unsigned long long* h_tot, cudaStream_t s) {
     auto run = [&](const int2* ranges, const Pieces& pc, const int2* items, int nitems, unsigned* counter,
                    double* part) {
@@ -1388,7 +1436,7 @@ size_t launch_p2p_tidal_plan(const float4* xp, int n, Cells c, const int2* list,
         note_launch();
     };
     return plan_and_run<PlanTidal>(n, c, list, seg_start, seg_end, leaves, nleaves, nullptr, T, 0, tmp, tmp_bytes,
-                                   h_tot, false, nullptr, 0, s, run);
+                                   h_tot, false, nullptr, 0, bg, s, run);
 }
 
 }  // namespace gb3
