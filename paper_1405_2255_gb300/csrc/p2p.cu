@@ -393,17 +393,18 @@ __device__ inline unsigned long long warp_total(unsigned long long v, unsigned l
 // per position q of the sorted order: its leaf index order[q], pieces npc[q] (their parts counted) and
 // items nit[q] (pieces x items per piece; 0 for a leaf without active particles); a split leaf (more than one
 // piece) takes the first of its partial-sum slots pbase[q] (pieces x sinks of them; -1: not split)
-// and an entry (leaf index, first slot) of the split list.  tot[1] items, tot[3] pieces, tot[4]
+// and an entry (leaf index, first slot) of the split list; a leaf with parts also the first of its nb + 2
+// npc places for their records, cbase[q].  tot[1] items, tot[2] those places, tot[3] pieces, tot[4]
 // slots, tot[5] split leaves; one atomic per warp and counter (a thread each took 60 us for 43,000
 // leaves).
 __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __restrict__ leaves, int nleaves, Cells c,
-                             const int* __restrict__ np, const int* __restrict__ kc, int* __restrict__ order, int* __restrict__ nit,
-                             int* __restrict__ npc, int* __restrict__ pbase, int2* __restrict__ split,
-                             unsigned long long* __restrict__ tot) {
+                             const int* __restrict__ np, const int* __restrict__ nb, const int* __restrict__ kc,
+                             int* __restrict__ order, int* __restrict__ nit, int* __restrict__ npc, int* __restrict__ pbase,
+                             int* __restrict__ cbase, int2* __restrict__ split, unsigned long long* __restrict__ tot) {
     const int lane = threadIdx.x & 31;
     for (int q0 = blockIdx.x * blockDim.x; q0 < nleaves; q0 += gridDim.x * blockDim.x) {
         const int q = q0 + threadIdx.x;
-        int t = 0, k = 0, P = 0, count = 0;
+        int t = 0, k = 0, P = 0, count = 0, places = 0;
         if (q < nleaves) {
             t = (int)(keys[q] & 0xffffffffu);
             order[q] = t;
@@ -412,19 +413,22 @@ __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __res
             if (cell_active(c, leaf)) {
                 k = kc[t];
                 P = (np[t] & 0xffff) * (np[t] >> 16);
+                if ((np[t] >> 16) > 1) places = nb[t] + 2 * P;
             }
             nit[q] = k * P;
             npc[q] = P;
         }
         const bool sp = P > 1;
         const unsigned long long slots = sp ? (unsigned long long)P * (unsigned long long)count : 0ull;
-        unsigned long long ex, sbefore, lbefore;
+        unsigned long long ex, sbefore, lbefore, cbefore = 0, tc = 0, cb = 0;
+        if (__any_sync(0xffffffffu, places)) tc = warp_total((unsigned long long)places, &cbefore);
         const unsigned long long ti = warp_total((unsigned long long)k * P, &ex), tp = warp_total(P, &ex);
         const unsigned long long ts = warp_total(slots, &sbefore), tl = warp_total(sp ? 1 : 0, &lbefore);
         unsigned long long sb = 0, lb = 0;
         if (lane == 0) {
             if (ti) atomicAdd(&tot[1], ti);
             if (tp) atomicAdd(&tot[3], tp);
+            if (tc) cb = atomicAdd(&tot[2], tc);
             if (tl) {
                 sb = atomicAdd(&tot[4], ts);
                 lb = atomicAdd(&tot[5], tl);
@@ -432,7 +436,9 @@ __global__ void k_p2p_nitems(const uint64_t* __restrict__ keys, const int* __res
         }
         sb = __shfl_sync(0xffffffffu, sb, 0) + sbefore;
         lb = __shfl_sync(0xffffffffu, lb, 0) + lbefore;
+        cb = __shfl_sync(0xffffffffu, cb, 0) + cbefore;
         if (q < nleaves) {
+            if (places) cbase[q] = (int)cb;
             pbase[q] = sp ? (int)sb : -1;
             if (sp) split[lb] = make_int2(t, (int)sb);
         }
@@ -467,8 +473,8 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
                const int* __restrict__ seg_end, const int* __restrict__ leaves, int nleaves, int mode,
                const int* __restrict__ order, const int* __restrict__ roff, const int* __restrict__ nb,
                const int* __restrict__ ioff, const int* __restrict__ nit, const int* __restrict__ voff,
-               const int* __restrict__ npc, const int* __restrict__ np, const int* __restrict__ pbase, int npieces,
-               Pieces pc, int2* __restrict__ ranges, int2* __restrict__ cuts, int2* __restrict__ items) {
+               const int* __restrict__ npc, const int* __restrict__ np, const int* __restrict__ pbase,
+               const int* __restrict__ cbase, int npieces, Pieces pc, int2* __restrict__ ranges, int2* __restrict__ cuts, int2* __restrict__ items) {
     constexpr bool MERGE = PL::merge;
     __shared__ int rsum_all[kEmitWarps][33], rg_all[kEmitWarps][33];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -593,11 +599,10 @@ __global__ void __launch_bounds__(kEmitWarps * 32)
         // The parts: the piece's tiles are cut (tiles of T sources of the near records, then of the far
         // ones); part u has the tiles u K .. (u + 1) K - 1, the last part the rest.  The records of a
         // class that overlap its interval of sources are copied, clipped, behind those of the part
-        // before it (a record cut in two is in both, hence one place more per part; U is at most the
-        // number of the piece's source cells, so three times its region hold them).
+        // before it (a record cut in two is in both, hence one place more per part and class).
         const int nr[2] = {__shfl_sync(0xffffffffu, cnt[1], 0), __shfl_sync(0xffffffffu, cnt[0], 0)};  // near, far
         const int rb[2] = {r0, r1 - nr[1]};
-        int2* cut = cuts + 3 * (size_t)r0;
+        int2* cut = cuts + (size_t)cbase[q] + (size_t)f0 + 2 * (size_t)pj * U;
         const int T = p2p_tile(PL::chunk(count).R), K = max(1, (int)PL::sub_steps * PL::chunk(count).R / (2 * T));
         long long total[2] = {0, 0};
         for (int k = 0; k < 2; ++k) {
@@ -1260,8 +1265,8 @@ struct PlanLayout {
     uint64_t *k0, *k1;
     int *order, *nb, *roff, *np, *kc, *npc, *voff, *nit, *ioff, *pbase, *stmp, *rtmp;
     int2* split;
-    unsigned long long* tot;  // [0] ranges, [1] items, [3] pieces, [4] partial slots, [5] split
-                              // leaves ([2] unused)
+    unsigned long long* tot;  // [0] ranges, [1] items, [2] parts' records, [3] pieces, [4] partial slots,
+                              // [5] split leaves
     unsigned* counter;
     size_t bytes;
 };
@@ -1325,23 +1330,25 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     scan_exclusive_i32(L.nb, L.roff, nleaves, L.roff + nleaves, L.stmp, s);
     // the low 32 bits are the leaf index, already in order: sort the 8 length bits only
     const int flip = radix_sort_pairs_bits(L.k0, nullptr, L.k1, nullptr, nleaves, L.rtmp, 32, 40, s);
-    k_p2p_nitems<<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.kc, L.order,
-                                                            L.nit, L.npc, L.pbase, L.split, L.tot);
+    int* cbase = (int*)(flip ? L.k0 : L.k1);  // (the sort's other buffer is free)
+    k_p2p_nitems<<<grid_for(nleaves, 256), 256, 0, s>>>(flip ? L.k1 : L.k0, leaves, nleaves, c, L.np, L.nb, L.kc,
+                                                        L.order, L.nit, L.npc, L.pbase, cbase, L.split, L.tot);
     note_launch();
     scan_exclusive_i32(L.nit, L.ioff, nleaves, L.ioff + nleaves, L.stmp, s);
     scan_exclusive_i32(L.npc, L.voff, nleaves, L.voff + nleaves, L.stmp, s);
     cudaMemcpyAsync(h_tot, L.tot, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
-    const unsigned long long nranges = h_tot[0], nitems = h_tot[1], npieces = h_tot[3], nslots = h_tot[4],
-                             nsplit = h_tot[5];
-    if (nranges > (unsigned long long)INT_MAX || nitems > (unsigned long long)INT_MAX ||
-        nslots > (unsigned long long)INT_MAX || (shares && 4 * (nranges + nitems + npieces) > (unsigned long long)INT_MAX))
+    const unsigned long long nranges = h_tot[0], nitems = h_tot[1], ncuts = h_tot[2], npieces = h_tot[3],
+                             nslots = h_tot[4], nsplit = h_tot[5], most = INT_MAX;
+    // (a part's records are indexed from the ranges, with the items and pieces between them)
+    if (nranges > most || nitems > most || nslots > most ||
+        (ncuts && nranges + nitems + 3 * npieces + ncuts + 128 > most))
         return ~(size_t)0;
     auto a256 = [](unsigned long long b) { return (size_t)((b + 255) & ~255ull); };
     const size_t o_ranges = L.bytes, o_items = o_ranges + a256(nranges * sizeof(int2)),
                  o_pieces = o_items + a256(nitems * sizeof(int2)),
                  o_cuts = o_pieces + a256(npieces * 6 * sizeof(int)),
-                 o_part = o_cuts + (shares ? a256(3 * nranges * sizeof(int2)) : 0),
+                 o_part = o_cuts + a256(ncuts * sizeof(int2)),
                  need = o_part + a256(nslots * PL::nv * sizeof(double)) + 256;
     if (tmp_bytes < need) return need;
     unsigned char* b = (unsigned char*)tmp;
@@ -1354,7 +1361,7 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     if (nitems == 0) return need;
     const unsigned g = grid_for((long long)npieces * 32, kEmitWarps * 32, 16);  // one warp per piece
     k_p2p_emit<PL><<<g, kEmitWarps * 32, 0, s>>>(c, list, seg_start, seg_end, leaves, nleaves, mode, L.order, L.roff,
-                                             L.nb, L.ioff, L.nit, L.voff, L.npc, L.np, L.pbase, (int)npieces, pc, ranges,
+                                             L.nb, L.ioff, L.nit, L.voff, L.npc, L.np, L.pbase, cbase, (int)npieces, pc, ranges,
                                              (int2*)(b + o_cuts), items);
     note_launch();
     run(ranges, pc, items, (int)nitems, L.counter, part);
