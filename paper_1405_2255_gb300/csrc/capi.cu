@@ -79,7 +79,8 @@ struct fmm_ctx {
     // walk
     Buf walkf;  // single-precision view of the cells for the walk's acceptance test
     Buf units;  // int[2]: the working units of the tree in use (launch_work_units)
-    Buf front0, front1, m2l, p2p, sort_tmp, sort_tmp2, m2l_tmp, p2p_tmp, seg_start, seg_end, est_m2l, est_p2p,
+    // sort_tmp also holds a P2P list's work plan once the list is sorted (on the sort's stream)
+    Buf front0, front1, m2l, p2p, sort_tmp, sort_tmp2, m2l_tmp, seg_start, seg_end, est_m2l, est_p2p,
         m2l_seg_start, m2l_seg_end;
     long long front_cap = 0, m2l_cap = 0, p2p_cap = 0, est_m2l_cap = 0, est_p2p_cap = 0;
     // per particle results (sorted order)
@@ -115,7 +116,7 @@ struct fmm_ctx {
         return {&hx, &hmu, &hpsi, &hacc, &bounds, &status, &counters, &coin, &keys, &keys_alt, &idx,
                 &idx_alt, &rtmp, &xm, &perm, &xp, &first, &count, &child, &nchild, &parent, &level, &sr,
                 &cr, &mass, &minscale, &tree_tmp, &shape, &leaves, &rad_tmp, &M, &F, &Pw, &pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
-                &sort_tmp, &sort_tmp2, &m2l_tmp, &p2p_tmp, &seg_start, &seg_end, &est_m2l, &est_p2p, &m2l_seg_start,
+                &sort_tmp, &sort_tmp2, &m2l_tmp, &seg_start, &seg_end, &est_m2l, &est_p2p, &m2l_seg_start,
                 &m2l_seg_end, &psi_far, &acc_far, &psi_near, &acc_near, &scale_sorted, &sys_off, &sys_G,
                 &sys_roots, &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
     }
@@ -345,7 +346,7 @@ static int run_walk(fmm_ctx* ctx, WalkParams wp, Buf& m2l, long long& m2l_cap, B
 static int sort_and_segment(fmm_ctx* ctx, Buf& list, long long npairs, Buf& seg_start, Buf& seg_end,
                             cudaStream_t s, bool wide = false, Buf* tmp = nullptr) {
     Buf& st = tmp ? *tmp : ctx->sort_tmp;
-    TRY(ensure(st, list_sort_tmp_bytes(npairs, ctx->ncells)));
+    TRY(ensure(st, list_sort_tmp_bytes(npairs, ctx->ncells, wide)));
     TRY(ensure(seg_start, sizeof(int) * ctx->ncells));
     TRY(ensure(seg_end, sizeof(int) * ctx->ncells));
     sort_pairs_by_sink(P<int2>(list), npairs, ctx->ncells, st.p, s, wide);
@@ -353,21 +354,21 @@ static int sort_and_segment(fmm_ctx* ctx, Buf& list, long long npairs, Buf& seg_
     return 0;
 }
 
-// mixed P2P over the segments in seg_start/seg_end of list: the work plan grows its scratch
-// once if the plan needs more than the context holds
+// mixed P2P over the segments in seg_start/seg_end of list: the work plan takes the scratch of the list's sort,
+// which runs before it on the stream, and grows it once if the plan needs more
 static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t s) {
     Cells c = cells_of(ctx);
-    TRY(ensure(ctx->p2p_tmp, p2p_plan_fixed_bytes(ctx->nleaves)));
+    TRY(ensure(ctx->sort_tmp, p2p_plan_fixed_bytes(ctx->nleaves)));
     for (int attempt = 0; attempt < 2; ++attempt) {
         const size_t need = launch_p2p_mixed(P<float4>(ctx->xp), ctx->n, c, list,
                                              P<int>(ctx->seg_start), P<int>(ctx->seg_end), P<int>(ctx->leaves),
                                              ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), mode,
-                                             ctx->p2p_tmp.p, ctx->p2p_tmp.bytes, ctx->h_counters + kWalkCounters, s,
+                                             ctx->sort_tmp.p, ctx->sort_tmp.bytes, ctx->h_counters + kWalkCounters, s,
                                              p2p_shares(ctx->nsys ? ctx->smallest : ctx->n),
                                              ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
         if (need == ~(size_t)0) return fail(ctx, FMM_E_OVERFLOW, "P2P plan beyond 2^31 source ranges or n >= 2^29");
-        if (need <= ctx->p2p_tmp.bytes) return 0;
-        TRY(ensure(ctx->p2p_tmp, need));
+        if (need <= ctx->sort_tmp.bytes) return 0;
+        TRY(ensure(ctx->sort_tmp, need));
     }
     return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
 }
@@ -379,13 +380,13 @@ static int run_p2p_fp64(fmm_ctx* ctx, const int2* list, bool want_f, bool* plann
     *planned = false;
     size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
     for (int attempt = 0; attempt < 2; ++attempt) {
-        if (ensure(ctx->p2p_tmp, need)) return 0;
+        if (ensure(ctx->sort_tmp, need)) return 0;
         need = launch_p2p_f64_plan(P<d4>(ctx->xm), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
                                    P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near),
-                                   P<double>(ctx->acc_near), want_f, plan_budget(ctx->prm), ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
+                                   P<double>(ctx->acc_near), want_f, plan_budget(ctx->prm), ctx->sort_tmp.p, ctx->sort_tmp.bytes,
                                    ctx->h_counters + kWalkCounters, s);
         if (need == ~(size_t)0) return 0;
-        if (need <= ctx->p2p_tmp.bytes) {
+        if (need <= ctx->sort_tmp.bytes) {
             *planned = true;
             return 0;
         }
@@ -407,12 +408,12 @@ static int run_p2p_tidal(fmm_ctx* ctx, cudaStream_t s) {
     const bool mixed = ctx->prm.precision == FMM_PREC_MIXED;
     size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
     for (int attempt = 0; mixed && attempt < 2; ++attempt) {
-        if (ensure(ctx->p2p_tmp, need)) break;
+        if (ensure(ctx->sort_tmp, need)) break;
         need = launch_p2p_tidal_plan(P<float4>(ctx->xp), ctx->n, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
                                      P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves,
-                                     P<double>(ctx->tid_near), plan_budget(ctx->prm), ctx->p2p_tmp.p, ctx->p2p_tmp.bytes,
+                                     P<double>(ctx->tid_near), plan_budget(ctx->prm), ctx->sort_tmp.p, ctx->sort_tmp.bytes,
                                      ctx->h_counters + kWalkCounters, s);
-        if (need <= ctx->p2p_tmp.bytes) return 0;
+        if (need <= ctx->sort_tmp.bytes) return 0;
         if (need == ~(size_t)0) break;
     }
     launch_p2p_tidal(P<d4>(ctx->xm), P<float4>(ctx->xp), ctx->n, mixed, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
@@ -1118,14 +1119,14 @@ int64_t fmm_footprint_bytes(const fmm_params* prm, int64_t n) {
 
 }  // extern "C"
 
-// What is left of the bound for the partial sums of the FP64 and tidal work plans: half of its constant
-// part and a tenth of what it grows by per particle.  With these the workspace stays within the bound for leaves
-// of 64 to 4096 particles; the plans of the benchmark's parameters are hardly cut (1e5 particles,
-// leaves of 64, p = 10: 61 MB, pieces of 512 steps).
+// The share of the bound for the partial sums of the FP64 and tidal work plans: half of its constant part and a
+// twentieth of what it grows by per particle.  With these the workspace stays within the bound for leaves of 64
+// to 4096 particles, and those of 8 to 32 at the orders 4 and 5, whose lists are the longest; pieces
+// of some 700 steps in place of 256 cost 1e5 particles nothing (leaves of 64, p = 10: 28.0 ms).
 gb3::PlanBudget gb3::plan_budget(const fmm_params& prm) {
     const double n = 1 << 20;
     const double per = ((double)fmm_footprint_bytes(&prm, 1 << 20) - (double)fmm_footprint_bytes(&prm, 0)) / n;
-    return PlanBudget{8.0 * n, 0.1 * per};
+    return PlanBudget{8.0 * n, 0.05 * per};
 }
 
 extern "C" {

@@ -203,8 +203,8 @@ struct WalkResult {
 WalkResult walk_result(const unsigned long long* h, int steps);
 // sort a pair list by (sink, first entry) -- the first entry taken as unsigned, so an adaptive
 // walk's M2L entries (wide: order bits above the source index) sort by (sink, order, source) --
-// then mark per-sink segments [seg_start, seg_end); tmp: list_sort_tmp_bytes(npairs, ncells)
-size_t list_sort_tmp_bytes(long long npairs, int ncells);
+// then mark per-sink segments [seg_start, seg_end); tmp: list_sort_tmp_bytes(npairs, ncells, wide)
+size_t list_sort_tmp_bytes(long long npairs, int ncells, bool wide = false);
 void sort_pairs_by_sink(int2* list, long long npairs, int ncells, void* tmp, cudaStream_t s, bool wide = false);
 void launch_segments(const int2* list, long long npairs, int ncells, int* seg_start, int* seg_end,
                      cudaStream_t s);
@@ -284,7 +284,8 @@ size_t launch_p2p_mixed(const float4* xp, int n, Cells c, const int2* list, cons
                         bool shares = false, const int* off = nullptr, int nsys = 0);
 // whether a forest whose smallest system has this many particles has pieces to be shared
 bool p2p_shares(int smallest_system);
-// the partial sums of split items that a system of n particles may take in a work plan: base + per n bytes
+// the partial sums of split items that a system of n particles may take in a work plan with four values per
+// sink: base + per n bytes
 struct PlanBudget {
     double base, per;
 };

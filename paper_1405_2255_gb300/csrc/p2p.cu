@@ -356,7 +356,7 @@ __global__ void k_p2p_count(Cells c, const int2* __restrict__ list, const int* _
 
 // The pieces of PL::budget's leaves.  A piece costs nv partial sums per sink, so pieces of L steps of a system
 // with the work A = sum of length x sinks take 8 nv A / L bytes: L is the shortest for which that is at most
-// base + per x the system's particles, and at least piece_steps.  (Of 256 steps in any system the FP64 plan's
+// nv / 4 (base + per x the system's particles), and at least piece_steps.  (Of 256 steps in any system the FP64 plan's
 // partial sums took up to 10 KB per particle, of 1024 steps the tidal plan's up to 9 KB: 13 times the bound of the
 // whole workspace for leaves of 1024.)  A call takes 6 us longer, so it is left out where no system can
 // need it (an item has at most 4 steps per particle; 4096 particles).
@@ -366,7 +366,7 @@ __global__ void k_p2p_pieces(Cells c, int nleaves, const int* __restrict__ nb, c
                              uint64_t* __restrict__ keys) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nleaves; t += gridDim.x * blockDim.x) {
         const int r = root[t], e = nb[t];
-        const double L = ceil(8.0 * PL::nv * (double)work[r] / (bg.base + bg.per * (double)c.count[r]));
+        const double L = ceil(32.0 * (double)work[r] / (bg.base + bg.per * (double)c.count[r]));
         const unsigned len = (unsigned)np[t];
         unsigned P;
         if (L <= (double)PL::piece_steps) P = (unsigned)(((unsigned long long)len + PL::piece_steps - 1) / PL::piece_steps);
@@ -1314,7 +1314,7 @@ size_t plan_and_run(int n, Cells c, const int2* list, const int* seg_start, cons
     if (n > kRangeMax) return ~(size_t)0;  // no range is ever cut: a leaf's region holds its source cells
     PlanLayout L = plan_layout(tmp, nleaves);
     if (tmp_bytes < L.bytes) return L.bytes;
-    const bool cut = PL::budget && 8.0 * PL::nv * n * (4.0 * n + 1.0) > (double)PL::piece_steps * (bg.base + bg.per * n);
+    const bool cut = PL::budget && 32.0 * n * (4.0 * n + 1.0) > (double)PL::piece_steps * (bg.base + bg.per * n);
     unsigned long long* work = cut ? (unsigned long long*)L.k1 : nullptr;  // (k1 and voff have their own use later)
     int* root = L.voff;
     unsigned char* zero_end = cut ? (unsigned char*)(work + nleaves) : (unsigned char*)(L.counter + 4);  // (roots <= leaves)

@@ -533,9 +533,17 @@ void radix_sort_pairs(uint64_t* keys, int* idx, uint64_t* keys_alt, int* idx_alt
 }
 
 // ---------------------------------------------------------------- list sort
-size_t list_sort_tmp_bytes(long long npairs, int /*ncells*/) {
+// bits of a key below the sink's, and all of them
+static int list_key_bits(int ncells, bool wide, int& xb) {
+    const int sb = bits_for(ncells);
+    xb = wide ? 32 : sb;
+    return xb + sb;
+}
+size_t list_sort_tmp_bytes(long long npairs, int ncells, bool wide) {
     const size_t n = (size_t)(npairs > 0 ? npairs : 1);
-    return n * 2 * sizeof(uint64_t) + radix_tmp_ints((long long)n) * sizeof(int) + 256;
+    int xb;
+    const size_t key = list_key_bits(ncells, wide, xb) <= 32 ? sizeof(unsigned) : sizeof(u64);
+    return n * 2 * key + radix_tmp_ints((long long)n) * sizeof(int) + 256;
 }
 
 // LSD passes over the keys alone (8 bits per pass over the xb + sb bits in use; 32-bit keys where they
@@ -557,9 +565,10 @@ static void sort_list(int2* list, long long npairs, int xb, int bits, void* tmp,
 }
 void sort_pairs_by_sink(int2* list, long long npairs, int ncells, void* tmp, cudaStream_t s, bool wide) {
     if (npairs <= 1) return;
-    const int sb = bits_for(ncells), xb = wide ? 32 : sb;
-    if (xb + sb <= 32) sort_list<unsigned>(list, npairs, xb, xb + sb, tmp, s);
-    else sort_list<u64>(list, npairs, xb, xb + sb, tmp, s);
+    int xb;
+    const int bits = list_key_bits(ncells, wide, xb);
+    if (bits <= 32) sort_list<unsigned>(list, npairs, xb, bits, tmp, s);
+    else sort_list<u64>(list, npairs, xb, bits, tmp, s);
 }
 
 }  // namespace gb3

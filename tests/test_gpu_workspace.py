@@ -42,6 +42,19 @@ def test_fp64_workspace_within_footprint(g, model, n, leaf, p, c, mac):
     ctx.close()
 
 
+@pytest.mark.parametrize("model", ["plummer", "dehnen"])
+@pytest.mark.parametrize("leaf,p", [(8, 4), (16, 5), (32, 5)])
+def test_fp64_workspace_of_long_lists(g, model, leaf, p):
+    """Low orders: the P2P lists are long, and so are the plan's ranges."""
+    n = 50_000
+    x, mu = getattr(inputs, model)(n, 77)
+    prm = dict(p=p, eps=1e-6, leaf_size=leaf, p2p_c=1.0, precision=g.FMM_PREC_FP64)
+    ctx = g.Context(**prm)
+    ctx.fmm_evaluate(_dev(x), _dev(mu))
+    assert ctx.fmm_workspace_bytes() <= g.fmm_footprint_bytes(n, **prm)
+    ctx.close()
+
+
 @pytest.mark.parametrize("leaf,p,c", SHAPES[:4])
 @pytest.mark.parametrize("mac", [0, 1])
 def test_tidal_workspace_within_footprint(g, leaf, p, c, mac):
@@ -57,7 +70,8 @@ def test_tidal_workspace_within_footprint(g, leaf, p, c, mac):
 
 @pytest.mark.parametrize("model", ["plummer", "dehnen"])
 @pytest.mark.parametrize("n", [9_000, 16_384])
-@pytest.mark.parametrize("leaf,p,c", [(8, 6, 1.0), (16, 6, 1.0), (32, 6, 1.0), (48, 14, 1.0), (512, 8, 8.0)])
+@pytest.mark.parametrize("leaf,p,c", [(8, 6, 1.0), (16, 6, 1.0), (32, 5, 1.0), (32, 6, 1.0), (48, 14, 1.0),
+                                      (512, 8, 8.0)])
 def test_small_mixed_workspace_within_footprint(g, model, n, leaf, p, c):
     """Systems whose pieces are shared by several warps (the parts have records of their own)."""
     x, mu = getattr(inputs, model)(n, 77)
