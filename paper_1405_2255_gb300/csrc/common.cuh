@@ -28,6 +28,14 @@ inline void once_per_device(DeviceOnce& o, F&& init) {
     o.done |= bit;
 }
 
+// Allow a kernel `bytes` of dynamic shared memory, once per device.  The limit belongs to the kernel, whatever
+// thread or context launches it, so it is set to the most any launch takes and never lowered: set per
+// call to that call's size, a thread of lower order could lower it between another's setting and launch.
+template <class K>
+inline void allow_smem(DeviceOnce& o, K kern, size_t bytes) {
+    once_per_device(o, [&] { cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
+}
+
 constexpr int kMaxP = 20;        // largest expansion order supported (p <= 20, Sec. 6.1)
 constexpr int kMaxLevel = 21;    // 21 bits per axis in a 63-bit Morton key
 constexpr int kWarp = 32;

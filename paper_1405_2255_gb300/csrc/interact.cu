@@ -398,7 +398,8 @@ static void m2l_rounds_launch(const int2* list, const int* seg_start, const int*
                               const int* item_start, unsigned* work, const d4* cen, const float2* Mf, const cd* M64,
                               int p, double* part, cudaStream_t s) {
     const size_t sm = RoundsSmem<kRB>(p).total;
-    cudaFuncSetAttribute(k_m2l_rounds<kRB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    static DeviceOnce once;
+    allow_smem(once, k_m2l_rounds<kRB>, RoundsSmem<kRB>(kMaxP).total);
     int dev = 0, nsm = 152, bps = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -672,8 +673,10 @@ void launch_l2p(const d4* xm, Cells c, const d4* cen, const int* leaves, int nle
                 double* psi, double* acc, cudaStream_t s) {
     if (nleaves <= 0) return;
     init_rec_tables();
-    const size_t sm = sizeof(L2PWeights) * (size_t)kL2PLeaves * out_count(p);
-    cudaFuncSetAttribute(k_l2p, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto smem = [](int order) { return sizeof(L2PWeights) * (size_t)kL2PLeaves * out_count(order); };
+    const size_t sm = smem(p);
+    static DeviceOnce once;
+    allow_smem(once, k_l2p, smem(kMaxP));
     const unsigned g = grid_for(((long long)nleaves + kL2PLeaves - 1) / kL2PLeaves * kL2PThreads, kL2PThreads, 16);
     k_l2p<<<g, kL2PThreads, sm, s>>>(xm, c, cen, leaves, nleaves, p, F, psi, acc);
     note_launch();

@@ -429,7 +429,8 @@ void launch_m2l_f64(const int2* list, const int* seg_start, const int* seg_end, 
     k_m2l_f64_items<<<grid_for(ncells, 256), 256, 0, s>>>(seg_start, seg_end, ncells, it);
     note_launch();
     const size_t sm = m2l_f64_smem(p);
-    cudaFuncSetAttribute(k_m2l_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    static DeviceOnce once;
+    allow_smem(once, k_m2l_f64, m2l_f64_smem(kMaxP));
     int bps = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_m2l_f64, 32, sm);
     k_m2l_f64<<<sm_count() * (bps > 0 ? bps : 1), 32, sm, s>>>(list, seg_start, seg_end, L.cnt, L.cstart, it, cen, L.Mn,

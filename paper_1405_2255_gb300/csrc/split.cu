@@ -389,7 +389,8 @@ void launch_m2m_split(Cells c, const d4* cen, const double* pw, int lev_begin, i
     if (ncl <= 6 * sm_count()) {
         launch_cluster8(k_m2m_split<true>, 8 * ncl, kM2MWarps * 32, per, s, c, cen, pw, lev_begin, p, M);
     } else {
-        cudaFuncSetAttribute(k_m2m_split<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * per));
+        static DeviceOnce once;
+        allow_smem(once, k_m2m_split<false>, 8 * m2m_smem_bytes(kMaxP));
         k_m2m_split<false><<<(unsigned)ncl, kM2MWarps * 32, 8 * per, s>>>(c, cen, pw, lev_begin, p, M);
     }
     note_launch();

@@ -152,8 +152,10 @@ void launch_l2p_tidal(const d4* xm, Cells c, const d4* cen, const int* leaves, i
                       double* T, cudaStream_t s) {
     if (nleaves <= 0) return;  // (p < 2: no terms and T_far = 0)
     init_tid_tab();
-    const size_t sm = sizeof(TidComb) * (size_t)kTidLeaves * (p >= 2 ? (p - 1) * p / 2 : 0);
-    cudaFuncSetAttribute(k_l2p_tidal, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto smem = [](int order) { return sizeof(TidComb) * (size_t)kTidLeaves * (order >= 2 ? (order - 1) * order / 2 : 0); };
+    const size_t sm = smem(p);
+    static DeviceOnce once;
+    allow_smem(once, k_l2p_tidal, smem(kMaxP));
     const unsigned g = grid_for(((long long)nleaves + kTidLeaves - 1) / kTidLeaves * kTidThreads, kTidThreads, 16);
     k_l2p_tidal<<<g, kTidThreads, sm, s>>>(xm, c, cen, leaves, nleaves, p, F, T);
     note_launch();
