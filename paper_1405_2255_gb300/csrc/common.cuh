@@ -11,8 +11,10 @@
 
 namespace gb3 {
 
-// Run an initialisation (an upload of __constant__ tables, which every device holds
-// separately) once per device, safely from several host threads.
+// Run an initialisation (an upload of tables, which every device holds separately) once per device,
+// safely from several host threads.  A copy from pageable memory may return before it has reached the
+// device, and the streams that read the tables do not wait for the legacy stream (they are non-blocking):
+// so the copies are waited for before anyone, this thread included, finds the initialisation done.
 struct DeviceOnce {
     std::mutex m;
     unsigned long long done = 0;
@@ -25,6 +27,7 @@ inline void once_per_device(DeviceOnce& o, F&& init) {
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
     if (o.done & bit) return;
     init();
+    cudaStreamSynchronize(0);
     o.done |= bit;
 }
 
