@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "plan_run.cuh"
 #include "serve.cuh"
 
 namespace gb3 {
@@ -354,22 +355,26 @@ static int sort_and_segment(fmm_ctx* ctx, Buf& list, long long npairs, Buf& seg_
     return 0;
 }
 
-// mixed P2P over the segments in seg_start/seg_end of list: the work plan takes the scratch of the list's sort,
-// which runs before it on the stream, and grows it once if the plan needs more
+// A work plan over the segments in seg_start/seg_end of a list: it takes the scratch of the list's sort, which
+// runs before it on the stream, and grows it once if it needs more
+template <class Run>
+static PlanEnd plan_in_sort_tmp(fmm_ctx* ctx, bool parts, Run run) {
+    return run_plan(
+        p2p_plan_fixed_bytes(ctx->nleaves), parts, run, [&](size_t bytes) { return ensure(ctx->sort_tmp, bytes); },
+        [&] { return ctx->sort_tmp.bytes; });
+}
+
 static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t s) {
     Cells c = cells_of(ctx);
-    TRY(ensure(ctx->sort_tmp, p2p_plan_fixed_bytes(ctx->nleaves)));
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        const size_t need = launch_p2p_mixed(P<float4>(ctx->xp), ctx->n, c, list,
-                                             P<int>(ctx->seg_start), P<int>(ctx->seg_end), P<int>(ctx->leaves),
-                                             ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near), mode,
-                                             ctx->sort_tmp.p, ctx->sort_tmp.bytes, ctx->h_counters + kWalkCounters, s,
-                                             p2p_shares(ctx->nsys ? ctx->smallest : ctx->n),
-                                             ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
-        if (need == ~(size_t)0) return fail(ctx, FMM_E_OVERFLOW, "P2P plan beyond 2^31 source ranges or n >= 2^29");
-        if (need <= ctx->sort_tmp.bytes) return 0;
-        TRY(ensure(ctx->sort_tmp, need));
-    }
+    const PlanEnd end = plan_in_sort_tmp(ctx, p2p_shares(ctx->nsys ? ctx->smallest : ctx->n), [&](bool parts) {
+        return launch_p2p_mixed(P<float4>(ctx->xp), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
+                                P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near), P<double>(ctx->acc_near),
+                                mode, ctx->sort_tmp.p, ctx->sort_tmp.bytes, ctx->h_counters + kWalkCounters, s, parts,
+                                ctx->nsys ? P<int>(ctx->sys_off) : nullptr, ctx->nsys);
+    });
+    if (end == kPlanRan) return 0;
+    if (end == kPlanNoRoom) return fail_cuda(ctx, FMM_E_OOM);
+    if (end == kPlanTooLarge) return fail(ctx, FMM_E_OVERFLOW, "P2P plan beyond 2^31 source ranges or n >= 2^29");
     return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
 }
 
@@ -377,21 +382,15 @@ static int run_p2p_mixed(fmm_ctx* ctx, const int2* list, int mode, cudaStream_t 
 // scratch, or beyond its index ranges, the form that needs none.  *planned: which one ran
 static int run_p2p_fp64(fmm_ctx* ctx, const int2* list, bool want_f, bool* planned, cudaStream_t s) {
     Cells c = cells_of(ctx);
-    *planned = false;
-    size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        if (ensure(ctx->sort_tmp, need)) return 0;
-        need = launch_p2p_f64_plan(P<d4>(ctx->xm), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
+    const PlanEnd end = plan_in_sort_tmp(ctx, false, [&](bool) {
+        return launch_p2p_f64_plan(P<d4>(ctx->xm), ctx->n, c, list, P<int>(ctx->seg_start), P<int>(ctx->seg_end),
                                    P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->psi_near),
-                                   P<double>(ctx->acc_near), want_f, plan_budget(ctx->prm), ctx->sort_tmp.p, ctx->sort_tmp.bytes,
-                                   ctx->h_counters + kWalkCounters, s);
-        if (need == ~(size_t)0) return 0;
-        if (need <= ctx->sort_tmp.bytes) {
-            *planned = true;
-            return 0;
-        }
-    }
-    return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
+                                   P<double>(ctx->acc_near), want_f, plan_budget(ctx->prm), ctx->sort_tmp.p,
+                                   ctx->sort_tmp.bytes, ctx->h_counters + kWalkCounters, s);
+    });
+    *planned = end == kPlanRan;
+    if (end == kPlanUnfit) return fail(ctx, FMM_E_CUDA, "P2P plan did not fit after growing its scratch");
+    return 0;
 }
 static int p2p_fp64(fmm_ctx* ctx, const int2* list, cudaStream_t s) {
     bool planned;
@@ -406,16 +405,13 @@ static int p2p_fp64(fmm_ctx* ctx, const int2* list, cudaStream_t s) {
 static int run_p2p_tidal(fmm_ctx* ctx, cudaStream_t s) {
     Cells c = cells_of(ctx);
     const bool mixed = ctx->prm.precision == FMM_PREC_MIXED;
-    size_t need = p2p_plan_fixed_bytes(ctx->nleaves);
-    for (int attempt = 0; mixed && attempt < 2; ++attempt) {
-        if (ensure(ctx->sort_tmp, need)) break;
-        need = launch_p2p_tidal_plan(P<float4>(ctx->xp), ctx->n, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
-                                     P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves,
-                                     P<double>(ctx->tid_near), plan_budget(ctx->prm), ctx->sort_tmp.p, ctx->sort_tmp.bytes,
-                                     ctx->h_counters + kWalkCounters, s);
-        if (need <= ctx->sort_tmp.bytes) return 0;
-        if (need == ~(size_t)0) break;
-    }
+    if (mixed && plan_in_sort_tmp(ctx, false, [&](bool) {
+            return launch_p2p_tidal_plan(P<float4>(ctx->xp), ctx->n, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
+                                         P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves,
+                                         P<double>(ctx->tid_near), plan_budget(ctx->prm), ctx->sort_tmp.p,
+                                         ctx->sort_tmp.bytes, ctx->h_counters + kWalkCounters, s);
+        }) == kPlanRan)
+        return 0;
     launch_p2p_tidal(P<d4>(ctx->xm), P<float4>(ctx->xp), ctx->n, mixed, c, P<int2>(ctx->p2p), P<int>(ctx->seg_start),
                      P<int>(ctx->seg_end), P<int>(ctx->leaves), ctx->nleaves, P<double>(ctx->tid_near), s);
     return 0;
