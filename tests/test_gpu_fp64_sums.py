@@ -68,6 +68,20 @@ def test_direct_splits(g, n, ns, want_f):
     ctx.close()
 
 
+@pytest.mark.parametrize("n", [2, 8, 112, 113, 224, 225, 448, 449, 897])
+@pytest.mark.parametrize("ns", [1, 40])
+def test_direct_slices_of_few_sources(g, n, ns):
+    """One, two, four and eight slices of the sources, warps without any among them."""
+    x, mu = inputs.plummer(n, 940 + n)
+    sinks = (np.arange(ns) * 7919) % n
+    ctx = g.Context()
+    out = ctx.fmm_direct(_dev(x), _dev(mu), 1.0, sinks=_dev(sinks.astype(np.int64)), want_f=True)
+    ctx.close()
+    ref = tuple(v[sinks] for v in _sums(x, mu, np.arange(n)))
+    _check(out[0].cpu().numpy(), out[1].cpu().numpy(), ref)
+    assert np.max(np.abs(out[2].cpu().numpy() - ref[2]) / np.maximum(ref[2], 1e-300)) < TOL
+
+
 @pytest.mark.parametrize("n,leaf", [(2, 1), (33, 1), (500, 3), (777, 17), (1500, 33), (2000, 65), (5001, 64),
                                     (4000, 130), (3000, 1000), (700, 4096)])
 @pytest.mark.parametrize("mac", [0, 1])
