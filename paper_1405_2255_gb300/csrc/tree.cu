@@ -1132,12 +1132,16 @@ __device__ void cell_radii(const d4* __restrict__ xm, const float4* __restrict__
 // of 8192: tree of 1e5 0.733 ms with 2048, 0.748 with 4096, 0.804 with 8192); with more cells 0 (a block
 // per cell has too little to do: block step of 1e6 1.1 % slower).
 // keep_centre: a reused tree keeps its centres (one warp per block where the block takes no radii).
-// kCluster, where a level of at most kWideCells cells has one of more than kWideRadii particles: eight blocks
+// kCluster, where a level of at most kWidePerSm cells per SM has one of more than kWideRadii particles: eight blocks
 // share the radii of such a cell (the first one has its ball), of up to kWideLevel particles if no cell is
 // larger and else kWideCell.  A block took 25 us for a cell of 1000 to 2000 particles and 51 us for one of
 // 1e4, the cluster takes 17 and 22; levels of 100 to 560 cells of a cusp of 6e4 46 to 70 us as blocks, 18 to
 // 23 us so (the blocks that have nothing to do return at once).  From 32768 particles on all blocks are
-// faster (a cell of 6e4 in a cluster 43 us, by the level's kernels 28).
+// faster (a cell of 6e4 in a cluster 43 us, by the level's kernels 28).  The line at six cells per SM: with more the
+// seven empty blocks of every small cell cost what the large ones gain.  Whole trees without clusters, with
+// the line at 6 and at 12 cells per SM: cusps of 6e4 0.625, 0.565, 0.563 ms and 1e5 0.716, 0.684, 0.699, spheres
+// of 6e4 0.594, 0.539, 0.537 and 3e5 1.008, 1.053, 1.062 (where the largest cells have the level's kernels
+// anyway, the clusters beside them lose).
 // What bounds a level of few cells: the chain of one cell's loads, balls and FP64 operations (64 cycles
 // each in a warp that is alone): 1e4 particles 25 to 30 us a level with every warp converting all daughters,
 // masks of all sizes in a warp and the mass summed behind them, 12 us so (without the radii).
@@ -1156,7 +1160,7 @@ struct MebMasks {
 };
 static __device__ const MebMasks g_meb_masks = MebMasks();
 constexpr int kLevelRadii = 16384, kCellRadii = 2048, kLevelCells = 2048;
-constexpr int kWideCells = 912, kWideRadii = 1024, kWideLevel = 32768, kWideCell = 16384;
+constexpr int kWidePerSm = 6, kWideRadii = 1024, kWideLevel = 32768, kWideCell = 16384;
 template <bool kCluster>
 __global__ void __launch_bounds__(kMebWarps * 32) k_internal_meb(const d4* __restrict__ xm,
                                                                  const float4* __restrict__ xp, Cells c,
@@ -1468,7 +1472,7 @@ void launch_internal_geometry(const d4* xm, const float4* xp, Cells c, int lev_b
                               bool keep_centre) {
     int ncl = lev_end - lev_begin;
     if (ncl <= 0) return;
-    const bool wide = ncl <= kWideCells && largest > kWideRadii;
+    const bool wide = ncl <= kWidePerSm * sm_count() && largest > kWideRadii;
     const int small = wide              ? (largest <= kWideLevel ? kWideLevel : kWideCell)
                       : ncl > kLevelCells ? 0
                                           : (largest <= kLevelRadii ? kLevelRadii : kCellRadii);
