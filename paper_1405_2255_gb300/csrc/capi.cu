@@ -102,10 +102,9 @@ struct fmm_ctx {
     bool timed = false;  // the events of the last evaluation were recorded
     bool marked_m2l = false, marked_p2p = false;  // ... and those around its main kernels
     gb3::Serve* serve = nullptr;  // the serving loop (serve.cu), created on first use
-    // ensemble of the current evaluation (nsys = 0: one system): system offsets and G
-    // on the device, roots (first, count) of the non-empty systems
-    Buf sys_off, sys_G, sys_roots, skey, skey_alt, spos, spos_alt;
-    int nsys = 0, nroots = 1, smallest = 0;  // (the smallest non-empty system's particles)
+    // ensemble of the current evaluation (nsys = 0: one system): system offsets and G on the device
+    Buf sys_off, sys_G, skey, skey_alt, spos, spos_alt;
+    int nsys = 0, nroots = 1, smallest = 0;  // (non-empty systems, the smallest one's particles)
     // force evaluation for a subset (Sec. 7.1): per sorted particle and per cell activity
     Buf pact, act, act_i, act_scan;
     bool active_mode = false;
@@ -119,7 +118,7 @@ struct fmm_ctx {
                 &cr, &mass, &minscale, &tree_tmp, &shape, &leaves, &rad_tmp, &M, &F, &Pw, &pw, &binom, &pascal, &M1, &F1, &Ff, &front0, &front1, &m2l, &p2p,
                 &sort_tmp, &sort_tmp2, &m2l_tmp, &seg_start, &seg_end, &est_m2l, &est_p2p, &m2l_seg_start,
                 &m2l_seg_end, &psi_far, &acc_far, &psi_near, &acc_near, &scale_sorted, &sys_off, &sys_G,
-                &sys_roots, &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
+                &skey, &skey_alt, &spos, &spos_alt, &pact, &act, &act_i, &act_scan, &tid_far, &tid_near, &walkf, &owner, &units};
     }
     // tree shape of the last evaluation
     std::vector<int> lev_start, lev_largest;  // first cell and largest cell's particles of every level
@@ -944,12 +943,16 @@ int fmm_evaluate_batch(fmm_ctx* ctx, int nsys, const int64_t* offsets, const dou
     for (int k = 0; k < nsys; ++k)
         if (!std::isfinite(G[k])) return fail(ctx, FMM_E_INVALID, "G is not finite");
     std::vector<int> off(nsys + 1);
-    std::vector<int2> roots;
+    int nroots = 0;
+    int64_t smallest = INT32_MAX;
     for (int k = 0; k < nsys; ++k) {
         if (offsets[k + 1] < offsets[k]) return fail(ctx, FMM_E_INVALID, "offsets not increasing");
         if (offsets[k + 1] > (int64_t)INT32_MAX) return fail(ctx, FMM_E_INVALID, "more than 2^31-1 particles in all");
         off[k] = (int)offsets[k];
-        if (offsets[k + 1] > offsets[k]) roots.push_back(make_int2((int)offsets[k], (int)(offsets[k + 1] - offsets[k])));
+        if (offsets[k + 1] > offsets[k]) {
+            ++nroots;
+            smallest = std::min(smallest, offsets[k + 1] - offsets[k]);
+        }
     }
     off[nsys] = (int)offsets[nsys];
     const int n = off[nsys];
@@ -959,16 +962,12 @@ int fmm_evaluate_batch(fmm_ctx* ctx, int nsys, const int64_t* offsets, const dou
     if (cudaSetDevice(ctx->device) != cudaSuccess) return fail(ctx, FMM_E_CUDA, "cudaSetDevice failed");
     TRY(ensure(ctx->sys_off, sizeof(int) * (nsys + 1)));
     TRY(ensure(ctx->sys_G, sizeof(double) * nsys));
-    TRY(ensure(ctx->sys_roots, sizeof(int2) * std::max<size_t>(1, roots.size())));
     CU(cudaMemcpyAsync(ctx->sys_off.p, off.data(), sizeof(int) * (nsys + 1), cudaMemcpyHostToDevice, s));
     CU(cudaMemcpyAsync(ctx->sys_G.p, G, sizeof(double) * nsys, cudaMemcpyHostToDevice, s));
-    if (!roots.empty())
-        CU(cudaMemcpyAsync(ctx->sys_roots.p, roots.data(), sizeof(int2) * roots.size(), cudaMemcpyHostToDevice, s));
     // the host arrays above are pageable and local: wait for the copies before returning
     ctx->nsys = nsys;
-    ctx->nroots = (int)roots.size();
-    ctx->smallest = n;
-    for (const int2& r : roots) ctx->smallest = std::min(ctx->smallest, r.y);
+    ctx->nroots = nroots;
+    ctx->smallest = (int)smallest;
     int rc = evaluate_device(ctx, n, x, mu, 1.0, nullptr, psi, acc, s, stats);
     cudaError_t e = cudaStreamSynchronize(s);
     ctx->nsys = 0;
