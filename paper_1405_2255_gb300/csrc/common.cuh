@@ -14,20 +14,21 @@ namespace gb3 {
 // Run an initialisation (an upload of tables, which every device holds separately) once per device,
 // safely from several host threads.  A copy from pageable memory may return before it has reached the
 // device, and the streams that read the tables do not wait for the legacy stream (they are non-blocking):
-// so the copies are waited for before anyone, this thread included, finds the initialisation done.
+// so the copies are waited for before anyone, this thread included, finds the initialisation done (uploads
+// = false: there are none).
 struct DeviceOnce {
     std::mutex m;
     unsigned long long done = 0;
 };
 template <class F>
-inline void once_per_device(DeviceOnce& o, F&& init) {
+inline void once_per_device(DeviceOnce& o, F&& init, bool uploads = true) {
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(o.m);
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
     if (o.done & bit) return;
     init();
-    cudaStreamSynchronize(0);
+    if (uploads) cudaStreamSynchronize(0);
     o.done |= bit;
 }
 
@@ -36,7 +37,8 @@ inline void once_per_device(DeviceOnce& o, F&& init) {
 // call to that call's size, a thread of lower order could lower it between another's setting and launch.
 template <class K>
 inline void allow_smem(DeviceOnce& o, K kern, size_t bytes) {
-    once_per_device(o, [&] { cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
+    once_per_device(
+        o, [&] { cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); }, false);
 }
 
 constexpr int kMaxP = 20;        // largest expansion order supported (p <= 20, Sec. 6.1)

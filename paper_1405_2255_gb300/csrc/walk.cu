@@ -317,9 +317,8 @@ void launch_walk(Cells c, WalkParams wp, WalkBuffers wb, int nroots, int ncells,
     cudaMemsetAsync(wb.counters, 0, kWalkCounters * sizeof(unsigned long long), s);
     if (ncells <= (wp.mac == kMacEstimate ? kWalkClusterCellsEst : kWalkClusterCells)) {
         static DeviceOnce once;
-        once_per_device(once, [] {
-            cudaFuncSetAttribute(k_walk_all, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        });
+        once_per_device(
+            once, [] { cudaFuncSetAttribute(k_walk_all, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); }, false);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at;
         at.id = cudaLaunchAttributeClusterDimension;
