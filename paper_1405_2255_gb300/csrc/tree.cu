@@ -275,16 +275,21 @@ void launch_gather(const double* x, const double* mu, const int* idx, int n, d4*
 __global__ void k_work_units(const unsigned long long* __restrict__ b, int nsys, int* __restrict__ e) {
     if (blockIdx.x || threadIdx.x) return;
     const int ns = nsys > 0 ? nsys : 1;
-    double ext = 0.0, far = 0.0;
+    double ext = 0.0;
     for (int k = 0; k < ns; ++k)
         for (int d = 0; d < 3; ++d) {
             const double lo = key_dbl(b[6 * k + d]), hi = key_dbl(b[6 * k + 3 + d]);
-            if (hi >= lo) {
-                ext = fmax(ext, hi - lo);
-                far = fmax(far, fmax(fabs(lo), fabs(hi)));
-            }
+            if (hi >= lo) ext = fmax(ext, hi - lo);
         }
-    if (ext == 0.0 && far >= 0x1p127) ext = far;
+    if (ext == 0.0) {  // (a loop of its own: in the one above it took 0.3 us a system)
+        double far = 0.0;
+        for (int k = 0; k < ns; ++k)
+            for (int d = 0; d < 3; ++d) {
+                const double lo = key_dbl(b[6 * k + d]), hi = key_dbl(b[6 * k + 3 + d]);
+                if (hi >= lo) far = fmax(far, fmax(fabs(lo), fabs(hi)));
+            }
+        if (far >= 0x1p127) ext = far;
+    }
     const double mmax = key_dbl(b[6 * ns]);
     const bool use_m = b[6 * ns] != 0ull && mmax > 0.0 && isfinite(mmax);
     int el = (ext > 0.0 && isfinite(ext)) ? ilogb(ext) : 0, em = use_m ? ilogb(mmax) : 0;
