@@ -1203,17 +1203,15 @@ __global__ void __launch_bounds__(kTidWarps * 32)
             // copy the tiles of round i (one per group), filled up to the longest of them
             auto fetch = [&](int i, int b) {
                 if (i * R >= ntl || !in) return;
+                const float4 fh = fill[0], fl = fill[1];  // (here, so that the copies' issue hides the reads)
                 const int nmax = sorted[i * R].y, k = i * R + g;
                 const int2 t = k < ntl ? sorted[k] : make_int2(0, 0);
                 float4* buf = bufs[wid][b][g];
                 const float4* src = xp + 2 * (size_t)t.x;
                 for (int j = slot; j < 2 * t.y; j += S) cp_async16(buf + j, src + j);
-                if (t.y < nmax) {
-                    const float4 fh = fill[0], fl = fill[1];
-                    for (int j = t.y + slot; j < nmax; j += S) {
-                        buf[2 * j] = fh;
-                        buf[2 * j + 1] = fl;
-                    }
+                for (int j = t.y + slot; j < nmax; j += S) {
+                    buf[2 * j] = fh;
+                    buf[2 * j + 1] = fl;
                 }
             };
             fetch(0, 0);
