@@ -77,12 +77,9 @@ def dist_env():
     return int(os.environ.get("RANK", 0)), int(os.environ.get("WORLD_SIZE", 1)), int(os.environ.get("LOCAL_RANK", 0))
 
 
-# ALU peaks derived from the unit counts and the maximum SM clock: SMs x 128 FP32 lanes x
+# FP32 peak derived from the unit counts and the maximum SM clock: SMs x 128 FP32 lanes x
 # 2 flops (FFMA) x the maximum SM clock (the SM count and clock are read from the device);
-# FP64 is the part's nominal 1.25 TFLOP/s
-FP64_PEAK_TFLOPS = 1.25
-
-
+# the FP64 peak is measured (fmm_alu_peaks)
 def fp32_peak(dev=None):
     """(TFLOP/s, SM count, max SM MHz) of the FP32 FMA pipes of the device."""
     import torch
@@ -261,9 +258,9 @@ def roofline(g, a, prec, phase, full):
     loop64, loop32 = g.fmm_alu_peaks()
     mixed = prec == g.FMM_PREC_MIXED
     p32, sms, mhz = fp32_peak()
-    pk, loop = (p32, loop32) if mixed else (FP64_PEAK_TFLOPS, loop64)
+    pk, loop = (p32, loop32) if mixed else (loop64, loop64)
     src = (f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {mhz:.0f} MHz" if mixed
-           else "nominal FP64 rate of the part (1.25 TFLOP/s)")
+           else "measured: FP64 multiply-adds alone on this device (fmm_alu_peaks)")
     if k_m2l >= k_p2p:
         rot = 3 <= a.p <= 16 or not mixed
         work = full["n_m2l"] * (m2l_rot_flops(a.p) if rot else m2l_flops(a.p))
@@ -274,7 +271,7 @@ def roofline(g, a, prec, phase, full):
     else:
         work = 20.0 * full["p2p_interactions"]
         t_k, t_ph = k_p2p, t_p2p
-        kern = "k_p2p_mixed (eq. 1, FP32 two-float)" if mixed else "k_p2p_fp64 (eq. 1)"
+        kern = "k_p2p_mixed (eq. 1, FP32 two-float)" if mixed else "k_p2p_f64 (eq. 1, FP64)"
     achieved = work / t_k / 1e12
     key = (a.workload, a.n, a.p, a.eps, a.leaf, a.c, a.precision)
     traffic = MEASURED_TRAFFIC.get(key, {}).get(kern.split(" ")[0])
